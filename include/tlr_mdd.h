@@ -47,7 +47,7 @@ extern "C" {
 #define TLR_ERR_STATE       -8  /* call out of order (e.g. destroyed handle) */
 
 /* ---- precision of the complex contractions ---- */
-#define TLR_PREC_FP32   0  /* FP32 SIMT (CUDA cores), FP32 accumulation */
+#define TLR_PREC_FP32   0  /* FP32: exact three-way BF16 split on the tensor cores, FP32 accumulation */
 #define TLR_PREC_BF16X3 1  /* tcgen05 tensor cores: BF16 hi/lo split (3 products), 4M complex, FP32 accumulation */
 #define TLR_PREC_TF32   2  /* tcgen05 tensor cores: operands rounded to TF32 (RN, ties away; 10 mantissa bits),
                               4M complex, FP32 accumulation.  The dense adjoint (tlr_mdd_adjoint) and the
@@ -357,8 +357,8 @@ int tlr_mdd_set_stream(tlr_mdd_t* h, void* stream);
 
 /* ---- allocation-free dense adjoint ----
  * G = V Dt^H (nr x nr) for receiver-major V and Dt (nr x ns), all complex64
- * DEVICE buffers owned by the caller; FP32 CUDA-core arithmetic, the same
- * kernels as tlr_mdd_adjoint.  The paper has no counterpart: this entry point
+ * DEVICE buffers owned by the caller; FP32, the same kernels as
+ * tlr_mdd_adjoint on an FP32 handle.  The paper has no counterpart: this entry point
  * exists for callers that cannot allocate device memory -- a process that
  * hands all device memory to its own pool allocator (an allocation from this
  * library would fail or fragment that pool), or a latency-critical path on

@@ -32,6 +32,18 @@ using namespace tlr;
 
 std::atomic<long long> tlr::g_launches{0};
 
+int tlr::device_sms() {
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+            return v;
+        (void)cudaGetLastError();
+        return 152;
+    }();
+    return n;
+}
+
 namespace {
 
 thread_local std::string g_last_error;
@@ -621,7 +633,13 @@ void carve(tlr_mdd_s* h, Arena& a) {
     const size_t nz = std::max<size_t>(1, (size_t)(L.nth - L.nlr));
     h->Zs = a.take<cf>(nz);
     h->Zsd = a.take<cf>(nz);
-    h->part = a.take<cf>((size_t)h->nsplit * L.nth);
+    // split-K partials of the projection.  FP32 path: over A1 and A2, which are
+    // adjacent and dead between the step that uses them and the next line search
+    // (where a single partial does not fit there, a buffer of its own)
+    if (!tensor_core(h->d.precision) && (size_t)h->nsplit * L.nth <= 2 * nrs)
+        h->part = h->A1;
+    else
+        h->part = a.take<cf>((size_t)h->nsplit * L.nth);
     h->dpart = a.take<double>(16 * kRedBlocks);
     // the fused residual step works on 16-row tiles of one block each: every
     // tile size a multiple of 16
@@ -688,21 +706,9 @@ long long packed_estimate(const Layout& L) {
     return t;
 }
 
-int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            n = v;
-        else
-            n = 152;
-    }
-    return n;
-}
-
-// Split of the contraction over ns in the gradient projection.  SIMT path:
-// enough 64 x 64 tiles for a few waves.  Tensor-core path: the split s that
+// Split of the contraction over ns in the gradient projection.  FP32 path:
+// gemm_f32_split, as many partials as fit where they are kept (A1 and A2, see
+// carve).  Packed tensor-core path: the split s that
 // minimises the modelled time ceil(tiles s / SMs) (ns / s + c0) of 128 x 128
 // tiles, c0 = 128 standing for a tile's fixed cost (set-up, pipeline fill,
 // epilogue) in units of contraction depth; this avoids a short last wave.
@@ -716,7 +722,7 @@ int split_for(const Layout& L, int prec) {
             if (L.dense[i]) tiles += ((b + kPackTRA - 1) / kPackTRA) * ((b + kPackTRB - 1) / kPackTRB);
         }
         tiles = std::max(1LL, tiles);
-        const long long sms = sm_count(), smax = std::max(1LL, std::min(16LL, (long long)L.ns / 256));
+        const long long sms = device_sms(), smax = std::max(1LL, std::min(16LL, (long long)L.ns / 256));
         long long best = 1;
         double tbest = 1e300;
         for (long long sp = 1; sp <= smax; ++sp) {
@@ -729,13 +735,10 @@ int split_for(const Layout& L, int prec) {
         return (int)best;
     }
     long long tiles = 0;
-    for (int i = 0; i < L.N; ++i) {
-        const long long b = L.d[i];
-        tiles += ((b + 63) / 64) * ((L.Kb[i] + 63) / 64);
-        if (L.general) tiles += ((b + 63) / 64) * ((L.KbB[i] + 63) / 64);
-        if (L.dense[i]) tiles += ((b + 63) / 64) * ((b + 63) / 64);
-    }
-    return choose_split(std::max(1LL, tiles), L.ns);
+    auto t128 = [](long long n) { return (n + 127) / 128; };
+    for (int i = 0; i < L.N; ++i)
+        tiles += t128(L.d[i]) * (t128(L.Kb[i]) + (L.general ? t128(L.KbB[i]) : 0) + (L.dense[i] ? t128(L.d[i]) : 0));
+    return gemm_f32_split(tiles, L.ns, std::max(1LL, 2LL * L.nr * L.ns / std::max<long long>(1, L.nth)));
 }
 
 GTerm term(const cf* A, long long lda, const cf* B, long long ldb, const int* g, int K, bool conjA, bool conjB) {
@@ -1354,6 +1357,7 @@ int64_t tlr_mdd_workspace_bytes(const tlr_mdd_desc_t* d) {
     tlr_mdd_s tmp;
     std::string e;
     if (build_layout(d, tmp.L, e)) return -1;
+    tmp.d.precision = d->precision;
     tmp.nsplit = split_for(tmp.L, d->precision);
     Arena a;
     carve(&tmp, a);
@@ -1498,7 +1502,10 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
     CKF(cudaEventCreate(&h->ev0));
     CKF(cudaEventCreate(&h->ev1));
     CKF(cudaMallocHost((void**)&h->hstats, sizeof(HostStats)));
-    if (tensor_core(d->precision)) CKF(gemm_tc_prepare());
+    if (tensor_core(d->precision))
+        CKF(gemm_tc_prepare());
+    else
+        CKF(gemm_f32_prepare());
     CKF(cudaStreamSynchronize(h->st));
     CKF(cudaMemcpy(&h->alpha, h->scal, sizeof(double), cudaMemcpyDeviceToHost));
 #undef CKF
@@ -1586,8 +1593,9 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     if (!V || !G) FAIL(h, TLR_ERR_ARG, "V or G is NULL");
     const Layout& L = h->L;
     const long long nr = L.nr, ns = L.ns;
-    const long long tiles = ((nr + 63) / 64) * ((nr + 63) / 64);
-    const int ns_split = choose_split(tiles, ns);
+    const bool tc = tensor_core(h->d.precision);
+    const long long t128 = (nr + 127) / 128, t64 = (nr + 63) / 64;
+    int ns_split = tc ? choose_split(t64 * t64, ns) : gemm_f32_split(t128 * t128, ns, 32);
     GProb p;
     memset(&p, 0, sizeof(p));
     p.t[0] = term((const cf*)V, ns, h->Dt, ns, nullptr, (int)ns, false, true);
@@ -1595,19 +1603,31 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     p.M = (int)nr;
     p.N = (int)nr;
     p.ldc = nr;
-    GProb* dp = nullptr;
+    // table and partials in the handle's work panels (R .. T_p, dead outside a
+    // forward product, gradient or solve, all of them on this stream); only
+    // partials that do not fit there are allocated.  Allocating them on each
+    // call cost 0.5 ms at nr = 2048 (fresh mappings), as much as the product.
+    Arena w;
+    w.base = reinterpret_cast<char*>(h->R);
+    w.cap = (size_t)(reinterpret_cast<char*>(h->Zs) - w.base);
+    GProb* dp = w.take<GProb>(1);
     cf* part = nullptr;
-    CK(h, cudaMallocAsync((void**)&dp, sizeof(GProb), h->st));
-    if (ns_split > 1) {
-        cudaError_t e = cudaMallocAsync((void**)&part, (size_t)ns_split * nr * nr * sizeof(cf), h->st);
-        if (e != cudaSuccess) {
-            cudaFreeAsync(dp, h->st);
+    bool own = false;
+    const size_t npart = (size_t)ns_split * nr * nr;
+    if (ns_split > 1 && w.used + npart * sizeof(cf) <= w.cap) {
+        part = w.take<cf>(npart);
+    } else if (ns_split > 1) {
+        cudaError_t e = cudaMallocAsync((void**)&part, npart * sizeof(cf), h->st);
+        own = e == cudaSuccess;
+        if (e == cudaErrorMemoryAllocation && !tc) {
+            (void)cudaGetLastError();   // no room for the partials: one pass over ns
+            part = nullptr;
+            ns_split = 1;
+        } else {
             CK(h, e);
         }
-        p.C = part;
-    } else {
-        p.C = (cf*)G;
     }
+    p.C = part ? part : (cf*)G;
     GemmLaunch G1;
     G1.d_probs = dp;
     G1.nprob = 1;
@@ -1621,12 +1641,11 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     cudaError_t e = cudaMemcpyAsync(dp, &p, sizeof(GProb), cudaMemcpyHostToDevice, h->st);
     G1.flops = 8.0 * nr * (double)nr * ns;
     G1.cls = 2;
-    G1.prec = tensor_core(h->d.precision) ? TLR_PREC_BF16X3 : TLR_PREC_FP32;   // operands split on the fly
+    G1.prec = tc ? TLR_PREC_BF16X3 : TLR_PREC_FP32;   // operands split on the fly
     G1.err = h->ints + SI_COUNT + 1;
     if (e == cudaSuccess) e = run_gemm(G1, h->st);
     if (e == cudaSuccess && ns_split > 1) e = reduce_grad(part, ns_split, nr * nr, nr * nr, 0, 1, (cf*)G, h->st);
-    if (part) cudaFreeAsync(part, h->st);
-    cudaFreeAsync(dp, h->st);
+    if (own) cudaFreeAsync(part, h->st);
     CK(h, e);
     CK(h, cudaStreamSynchronize(h->st));  // p lives on this stack frame
     return TLR_OK;

@@ -47,7 +47,7 @@ inline cudaError_t launch_pass(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
 }
 
 // ---------------------------------------------------------------------------
-// Grouped complex GEMM descriptors (FP32 SIMT and tensor-core paths).
+// Grouped complex GEMM descriptors (FP32 and packed tensor-core paths).
 //
 // One problem computes C[m, n] (M x N) = sum over terms t of
 //   sum_k opA_t[m, k] * opB_t[k, n]
@@ -147,7 +147,7 @@ struct GemmLaunch {
     int amode = 0, bmode = 0, epi = 0;
     double flops = 0.0;         // algorithmic flops of one launch (8 per complex MAC)
     int cls = 0;                // diagnostics class (0 compress, 1 expand, 2 project)
-    int prec = 0;               // TLR_PREC_FP32 (SIMT), TLR_PREC_BF16X3 or TLR_PREC_TF32 (tcgen05)
+    int prec = 0;               // TLR_PREC_FP32 (three-way BF16 split), TLR_PREC_BF16X3 or TLR_PREC_TF32 (tcgen05)
     bool persistent = false;    // packed path: the persistent, double-buffered kernel
     const ZItem* d_zmap = nullptr;   // persistent only: per-slice problem, split and partial offset
     int nz = 0;                      // slices in d_zmap (replaces nprob x nsplit)
@@ -257,14 +257,20 @@ cudaError_t gemm_tcp_prepare();
 cudaError_t wait_selftest(int* status, unsigned long long limit_ns, unsigned long long* waited_ns, cudaStream_t st);
 cudaError_t gemm_tcp(const GemmLaunch& L, cudaStream_t st);
 
-// SIMT path (k_gemm_simt.cu)
-cudaError_t gemm_simt(const GemmLaunch& L, cudaStream_t st);
+// FP32 path (k_gemm_f32.cu): exact three-way BF16 split on the tensor cores, FP32
+// operands in place.  gemm_f32_split: the split of a contraction of depth K over
+// `tiles` 128 x 128 output tiles, at most `most`.
+cudaError_t gemm_f32(const GemmLaunch& L, cudaStream_t st);
+cudaError_t gemm_f32_prepare();
+int gemm_f32_split(long long tiles, long long K, long long most);
+// SMs of the current device (api.cu)
+int device_sms();
 // tcgen05 path (k_gemm_tc.cu): BF16x3 split, 3M complex, FP32 accumulation in TMEM
 cudaError_t gemm_tc(const GemmLaunch& L, cudaStream_t st);
 // one-time kernel attributes (shared-memory size), outside any stream capture
 cudaError_t gemm_tc_prepare();
 inline cudaError_t gemm_any(const GemmLaunch& L, cudaStream_t st) {
-    if (!tensor_core(L.prec)) return gemm_simt(L, st);
+    if (!tensor_core(L.prec)) return gemm_f32(L, st);
     if (!L.d_pprobs) return gemm_tc(L, st);
     cudaError_t e = cudaSuccess;
     if (L.n_gpack) e = tpack(L.d_gpack, L.n_gpack, L.gpack_src, nullptr, nullptr, L.gpack_ns, st);

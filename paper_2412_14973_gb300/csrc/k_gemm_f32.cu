@@ -1,0 +1,714 @@
+// FP32 grouped complex GEMM on the tensor cores (tcgen05, sm_103a): the
+// default-precision path of the TLR contractions -- compress T = F^T Dfrak,
+// expand Y = F T~ (+ P Z Dfrak), the factor-gradient projections (eq. 25-27)
+// and the dense adjoint G = V Dfrak^H, on FP32 operands in place.
+//
+// Arithmetic.  Every FP32 value is split exactly into three BF16 values
+// x = h + m + l (h = RN(x), m = RN(x - h), l = x - h - m: 8 + 8 + 8 significant
+// bits), and every real product takes the six of the nine BF16 products that
+// are not below 2^-24 of it: hh, hm, mh, hl, mm, lh.  A complex product is four
+// real ones (4M), so a 16-deep chunk of a 128 x 128 tile takes 24 MMAs.
+// The tensor core adds into its FP32 accumulator without rounding to nearest
+// (about half an ulp toward zero per MMA), so the accumulator never carries
+// more than one chunk: the smallest products are issued first (while the
+// accumulator is still small) and every 16-deep chunk is drained and added to
+// FP32 registers, rounding to nearest.  Measured against 64 bits this is at or
+// below the error of FP32 fused multiply-adds over the whole contraction
+// (see tests/test_gpu_gemm_f32.py).
+//
+// What bounds it: the MMA rate, 24 BF16 products per complex multiply-add of
+// 16-deep chunks, 8/48 of the BF16 peak.  Everything else runs beside the
+// MMAs: three warps copy chunks from global memory into a raw shared-memory ring
+// (cp.async, gather applied, zeros from the k tail on), 16 worker warps split
+// chunk c into the tensor core's canonical K-major no-swizzle layout (8-row x
+// 16-byte core matrices) and drain chunk c - 2 from one of two TMEM accumulator
+// pairs, while the tensor core works on chunk c - 1 and another warp issues chunk
+// c's MMAs.  The split takes fewer issue slots than the SM has under 24 MMAs (it
+// bounded the 12-MMA form), so no operand is packed in memory and the kernel
+// needs no workspace.  The roles are apart because a worker's 64 accumulators
+// leave no registers for cursors, and beside this much shared memory the L1
+// holds no spills.  Tried on nr = ns = 4096 (dense adjoint, TFLOP/s; the MMAs
+// alone: 285): copies and cursors in the workers 58 to 83 (spills) and 176, the
+// MMAs issued by a worker 125, one copy warp per operand 191 to 204 (65 cycles
+// per copy instruction), bulk copies of 128 bytes 74 (31 cycles each); this form
+// 225, bound by the workers' split and drain (the FP32 FMA kernel before: 34).
+// Persistent: one CTA per SM walks the output tiles, its pipeline running
+// across tile ends.
+//
+// Values beyond the split (Inf, NaN, or a magnitude that rounds to Inf in BF16)
+// make a tile's results non-finite; every non-finite result is recomputed with
+// plain FP32 fused multiply-adds before it is stored, so Inf and NaN come out
+// as FP32 arithmetic gives them.
+//
+// Every barrier wait is bounded (2 s); a timeout is recorded in the error word.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "internal.h"
+
+namespace tlr {
+
+namespace {
+
+constexpr int TM = 128, TN = 128, KC = 16;
+constexpr int NW = 16;                              // worker warps
+constexpr int WMMA = NW, WCOPY = NW + 1, NCOPY = 3; // the MMA warp, the copy warps
+constexpr int NTHR = (NW + 4) * 32;                 // whole warps per scheduler
+constexpr int PLANE = 128 * KC * 2;                 // one BF16 plane of a 128 x 16 operand tile
+constexpr int TILE = 6 * PLANE;                     // Re h, m, l, Im h, m, l
+constexpr int STAGE = 2 * TILE;                     // A and B
+constexpr int NSTAGE = 3;
+constexpr int LAG = 2;                              // chunks between split and drain
+constexpr int RAW_OP = 128 * KC * 8;                // one operand's raw chunk: 128 rows x 128 B, or 16 k x 1 KB
+constexpr int NRAW = 2;
+constexpr int RAW_OFF = NSTAGE * STAGE;
+constexpr int ROW_OFF = RAW_OFF + NRAW * 2 * RAW_OP;   // per copy warp: element offsets of A's and B's 128 rows
+constexpr int CTRL_OFF = ROW_OFF + NCOPY * 2 * 128 * 8;
+constexpr int SMEM_BYTES = CTRL_OFF + 256;
+constexpr uint32_t TMEM_COLS = 512;                 // two pairs of 2 x 128 columns
+constexpr unsigned long long WAIT_NS = 2000000000ull;
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
+
+// instruction descriptor: FP32 accumulator, BF16 x BF16, M 128; N / 8 goes to bits 17-22
+constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TM >> 4) << 24);
+constexpr uint32_t NEG_A = 1u << 13;
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// shared-memory matrix descriptor, K-major no-swizzle: core matrices 128 B
+// apart along K and 256 B apart along rows
+__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
+    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(256u >> 4) << 32) |
+           ((uint64_t)1 << 46);
+}
+
+__device__ __forceinline__ unsigned long long now_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const volatile int* abort_flag) {
+    unsigned long long t0 = 0;
+    for (unsigned it = 0;; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if ((it & 255u) == 255u) {
+            if (*abort_flag) return false;
+            const unsigned long long t = now_ns();
+            if (t0 == 0)
+                t0 = t;
+            else if (t - t0 > WAIT_NS)
+                return false;
+        }
+    }
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        :
+        : "r"(tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr));
+}
+
+// two FP32 operations per instruction
+__device__ __forceinline__ uint64_t pair(float lo, float hi) {
+    return ((uint64_t)__float_as_uint(hi) << 32) | __float_as_uint(lo);
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// h, m, l of two FP32 values as BF16 pairs (x0 in the low half)
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t* w) {
+    uint64_t x = pair(x0, x1);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float((uint32_t)x), __uint_as_float((uint32_t)(x >> 32)));
+        const uint32_t u = *reinterpret_cast<const uint32_t*>(&b);
+        w[p] = u;
+        // minus the BF16 values (their sign bits flipped)
+        if (p < 2)
+            x = add2(x, ((uint64_t)((u & 0xffff0000u) ^ 0x80000000u) << 32) | ((u << 16) ^ 0x80000000u));
+    }
+}
+
+// ---------------------------------------------------------------------------
+// work items: (M tile fastest, N tile, problem and split)
+// ---------------------------------------------------------------------------
+struct Item {
+    const GProb* P;
+    int m0, n0, chunk;
+};
+
+struct Launch {
+    const GProb* probs;
+    int nsplit, kchunk, nx, ny;
+    int nitems;         // below 2^31 - grid (gemm_f32)
+};
+
+__device__ __forceinline__ bool item_at(const Launch& L, int i, Item& it) {
+    const int xy = L.nx * L.ny;
+    const int z = i / xy, r = i - z * xy;
+    const int prob = z / L.nsplit;
+    it.chunk = z - prob * L.nsplit;
+    it.m0 = (r % L.ny) * TM;
+    it.n0 = (r / L.ny) * TN;
+    it.P = L.probs + prob;
+    return it.m0 < it.P->M && it.n0 < it.P->N;
+}
+
+// the K range [kb, ke) of a term (kb a multiple of 16)
+__device__ __forceinline__ void k_range(const Launch& L, const Item& it, int K, int& kb, int& ke) {
+    kb = 0;
+    ke = K;
+    if (L.nsplit > 1) {
+        kb = it.chunk * L.kchunk;
+        ke = min(K, kb + L.kchunk);
+    }
+}
+
+__device__ __forceinline__ int chunks_of(const Launch& L, const Item& it) {
+    int C = 0;
+    for (int t = 0; t < it.P->nt; ++t) {
+        int kb, ke;
+        k_range(L, it, it.P->t[t].K, kb, ke);
+        if (ke > kb) C += (ke - kb + KC - 1) / KC;
+    }
+    return C;
+}
+
+// ---------------------------------------------------------------------------
+// copying and splitting one operand's 16-deep chunk
+// ---------------------------------------------------------------------------
+
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copy8(uint32_t dst, const void* src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(in ? 8 : 0) : "memory");
+}
+
+// one operand of one term as a copy warp sees it
+struct Opnd {
+    const cf* base;      // k contiguous: row r at base + rowoff[r]; rows contiguous: base + k ld (k through g)
+    const int* g;
+    const long long* rowoff;
+    long long ld;
+    int rows;            // valid rows of the tile
+    bool vec;            // every row piece starts on 16 bytes
+};
+
+template <bool KCONTIG>
+__device__ __forceinline__ Opnd make_opnd(const cf* base, long long ld, const int* g, int R, int r0,
+                                          long long* rowoff, int lane) {
+    Opnd o;
+    o.g = g;
+    o.ld = ld;
+    o.rows = min(128, R - r0);
+    o.rowoff = rowoff;
+    o.vec = (ld & 1) == 0;
+    if (KCONTIG) {
+        __syncwarp();
+        for (int r = lane; r < o.rows; r += 32) rowoff[r] = (long long)(g ? g[r0 + r] : r0 + r) * ld;
+        __syncwarp();
+    } else {
+        base += r0;
+        o.vec = o.vec && (o.rows & 1) == 0;
+    }
+    o.base = base;
+    o.vec = o.vec && (reinterpret_cast<uintptr_t>(base) & 15) == 0;
+    return o;
+}
+
+// raw position of 16-byte column q (two k) of row r, k contiguous: columns
+// rotated by the row so that 8 rows of one column lie in 8 different ones
+__device__ __forceinline__ int raw_pos(int r, int q) { return r * 128 + ((q ^ (r & 7)) << 4); }
+
+// Copy warp w of NCOPY starts its copies of chunk k0 .. k0 + 15, zeros from ke on.
+// Rows beyond the operand keep what the ring held: they reach only results that
+// are not stored.  k contiguous: 8 lanes take a row's 128 bytes; rows contiguous:
+// 512 bytes of one k per instruction.
+template <bool KCONTIG>
+__device__ __forceinline__ void copy_chunk(const Opnd& o, int k0, int ke, int w, uint32_t raw, int lane) {
+    if (KCONTIG) {
+        if (o.vec) {
+            const int q = lane & 7, n = max(0, min(2, ke - k0 - 2 * q)) * 8;   // bytes
+            const cf* p = n ? o.base + k0 + 2 * q : o.base;
+#pragma unroll
+            for (int i = 0; i < 11; ++i) {
+                const int r = (i * NCOPY + w) * 4 + (lane >> 3);
+                if (r < o.rows) copy16(raw + raw_pos(r, q), p + o.rowoff[r], n);
+            }
+        } else {
+            const int q = lane & 15;
+            const bool in = k0 + q < ke;
+            const cf* p = o.base + (in ? k0 + q : 0);
+#pragma unroll 4
+            for (int i = w; i < 64; i += NCOPY) {
+                const int r = i * 2 + (lane >> 4);
+                if (r < o.rows) copy8(raw + raw_pos(r, q >> 1) + (q & 1) * 8, p + o.rowoff[r], in);
+            }
+        }
+    } else {
+        const int k = k0 + (lane & 15);
+        const int gi = k < ke ? (o.g ? o.g[k] : k) : -1;
+#pragma unroll
+        for (int i = 0; i < 11; ++i) {
+            const int e = i * NCOPY + w;   // half (e & 1) of k e >> 1
+            const int row = __shfl_sync(0xffffffffu, gi, (e >> 1) & 15);
+            const bool in = row >= 0;
+            const int r = (e & 1) * 64 + lane * 2;
+            if (e < 2 * KC && r < o.rows) {
+                const cf* p = in ? o.base + (long long)row * o.ld + r : o.base;
+                const uint32_t d = raw + (e >> 1) * 1024 + r * 8;
+                if (o.vec) {
+                    copy16(d, p, in ? 16 : 0);
+                } else {
+                    copy8(d, p, in);
+                    if (r + 1 < o.rows) copy8(d + 8, in ? p + 1 : o.base, in);
+                }
+            }
+        }
+    }
+}
+
+// Splits a raw chunk into the operand tile, four k at a time (8 values and 12
+// words live beside the 64 accumulators).  Both the reads (8 rows of a phase in
+// 8 different columns, or consecutive rows) and the 8-byte stores (rows 8 to 15
+// of 16 take the other half of the k-group: together all banks) are free of
+// bank conflicts.  k contiguous: thread = (row, half of each k-group); rows
+// contiguous: thread = (row, k-group).
+template <bool KCONTIG>
+__device__ __forceinline__ void split_chunk(char* tile, const char* raw, int t8) {
+    const int r = KCONTIG ? (t8 >> 5) * 16 + (t8 & 15) : t8 & 127;
+    const int odd = (r >> 3) & 1;
+    char* const d = tile + (r >> 3) * 256 + (r & 7) * 16;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        float2 v[4];
+        const int kg = KCONTIG ? j : t8 >> 7;
+        const int h = (KCONTIG ? (t8 >> 4) & 1 : j) ^ odd;   // k 8 kg + 4 h ..
+        if (KCONTIG) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float4 x = *reinterpret_cast<const float4*>(raw + raw_pos(r, kg * 4 + h * 2 + i));
+                v[2 * i] = make_float2(x.x, x.y);
+                v[2 * i + 1] = make_float2(x.z, x.w);
+            }
+        } else {
+            const char* q = raw + (kg * 8 + h * 4) * 1024 + r * 8;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = *reinterpret_cast<const float2*>(q + i * 1024);
+        }
+        char* const o = d + kg * 128 + h * 8;
+        uint32_t w[2][3];
+        split2(v[0].x, v[1].x, w[0]);
+        split2(v[2].x, v[3].x, w[1]);
+#pragma unroll
+        for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(o + p * PLANE) = make_uint2(w[0][p], w[1][p]);
+        split2(v[0].y, v[1].y, w[0]);
+        split2(v[2].y, v[3].y, w[1]);
+#pragma unroll
+        for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(o + (3 + p) * PLANE) = make_uint2(w[0][p], w[1][p]);
+    }
+}
+
+// one output by plain FP32 fused multiply-adds
+template <int AM, int BMD>
+__device__ __forceinline__ float2 plain_dot(const Launch& L, const Item& it, int m, int n) {
+    float2 c = make_float2(0.f, 0.f);
+    for (int ti = 0; ti < it.P->nt; ++ti) {
+        const GTerm& t = it.P->t[ti];
+        int kb, ke;
+        k_range(L, it, t.K, kb, ke);
+        for (int k = kb; k < ke; ++k) {
+            float2 a = AM == A_KM ? t.A[(long long)k * t.lda + m] : t.A[(long long)m * t.lda + k];
+            const long long row = BMD == B_KN ? (t.g ? t.g[k] : k) : (t.g ? t.g[n] : n);
+            float2 b = BMD == B_KN ? t.B[row * t.ldb + n] : t.B[row * t.ldb + k];
+            a.y *= t.sa;
+            b.y *= t.sb;
+            c.x = fmaf(a.x, b.x, c.x);
+            c.x = fmaf(-a.y, b.y, c.x);
+            c.y = fmaf(a.x, b.y, c.y);
+            c.y = fmaf(a.y, b.x, c.y);
+        }
+    }
+    return c;
+}
+
+__device__ __forceinline__ bool finite2(float2 v) { return isfinite(v.x) && isfinite(v.y); }
+
+// Recomputes the non-finite results among a thread's row of 32 columns just
+// written (not inlined: called once the accumulators are dead).
+template <int AM, int BMD>
+__device__ __noinline__ void mend_row(const Launch& L, int item, int epi, long long part_stride, int lg, int cg,
+                                      int lane) {
+    Item it;
+    item_at(L, item, it);
+    const GProb& P = *it.P;
+    const int m = it.m0 + lg * 32 + lane, nb = it.n0 + cg * 32;
+    if (m >= P.M) return;
+    cf* const Cp = P.C + (epi == EPI_PARTIAL ? it.chunk * part_stride : 0) + (long long)m * P.ldc;
+    for (int n = nb; n < min(P.N, nb + 32); ++n) {
+        if (finite2(Cp[n])) continue;
+        float2 v = plain_dot<AM, BMD>(L, it, m, n);
+        if (epi == EPI_SUB) {
+            const float2 s = P.S[(long long)m * P.ldc + n];
+            v.x -= s.x;
+            v.y -= s.y;
+        }
+        Cp[n] = v;
+    }
+}
+
+// Writes a thread's row of 32 columns (real parts of pairs of columns, then
+// imaginary parts) to the tile's destination, 16 bytes at a time; consecutive
+// stores fill the row's 32-byte sectors.  (No room for a staging transpose in
+// shared memory; the stores run beside the next tile's first MMAs.)  True if
+// any value is not finite.
+__device__ __forceinline__ bool write_tile(const Item& it, int epi, long long part_stride, const uint64_t* acc, int lg,
+                                           int cg, int lane) {
+    const GProb& P = *it.P;
+    const int m = it.m0 + lg * 32 + lane, nb = it.n0 + cg * 32, N = P.N;
+    if (m >= P.M) return false;
+    cf* const Cp = P.C + (epi == EPI_PARTIAL ? it.chunk * part_stride : 0) + (long long)m * P.ldc + nb;
+    const cf* const Sp = epi == EPI_SUB ? P.S + (long long)m * P.ldc + nb : nullptr;
+    const bool vec = ((reinterpret_cast<uintptr_t>(Cp) | reinterpret_cast<uintptr_t>(Sp)) & 15) == 0;
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        if (nb + 2 * q < N) {
+            const bool two = nb + 2 * q + 1 < N;
+            float4 v = make_float4(__uint_as_float((uint32_t)acc[q]), __uint_as_float((uint32_t)acc[16 + q]),
+                                   __uint_as_float((uint32_t)(acc[q] >> 32)),
+                                   __uint_as_float((uint32_t)(acc[16 + q] >> 32)));
+            if (epi == EPI_SUB) {
+                if (vec && two) {
+                    const float4 s = *reinterpret_cast<const float4*>(Sp + 2 * q);
+                    v.x -= s.x;
+                    v.y -= s.y;
+                    v.z -= s.z;
+                    v.w -= s.w;
+                } else {
+                    v.x -= Sp[2 * q].x;
+                    v.y -= Sp[2 * q].y;
+                    if (two) {
+                        v.z -= Sp[2 * q + 1].x;
+                        v.w -= Sp[2 * q + 1].y;
+                    }
+                }
+            }
+            bad |= !(isfinite(v.x) && isfinite(v.y)) || (two && !(isfinite(v.z) && isfinite(v.w)));
+            if (vec && two) {
+                *reinterpret_cast<float4*>(Cp + 2 * q) = v;
+            } else {
+                Cp[2 * q] = make_float2(v.x, v.y);
+                if (two) Cp[2 * q + 1] = make_float2(v.z, v.w);
+            }
+        }
+    }
+    return bad;
+}
+
+template <int AM, int BMD>
+__global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ Launch L, int epi,
+                                                       long long part_stride, int* err) {
+    extern __shared__ __align__(1024) char smem[];
+    if (*(volatile int*)err != 0) return;   // an earlier contraction gave up: do no more work
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + CTRL_OFF);   // operand stage split (one arrival per worker warp)
+    uint64_t* empty = full + NSTAGE;        // operand stage read by its MMAs
+    uint64_t* tfull = empty + NSTAGE;       // [2] accumulator pair holds a chunk
+    uint64_t* tempty = tfull + 2;           // [2] accumulator pair drained (one arrival per worker warp)
+    uint64_t* rfull = tempty + 2;           // [NRAW] raw chunk landed (every copy lane's copies)
+    uint64_t* rempty = rfull + NRAW;        // [NRAW] raw chunk read (one arrival per worker warp)
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(rempty + NRAW);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < NSTAGE; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])), "r"(NW) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[s])) : "memory");
+        }
+        for (int b = 0; b < 2; ++b) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&tfull[b])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&tempty[b])), "r"(NW) : "memory");
+        }
+        for (int r = 0; r < NRAW; ++r) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&rfull[r])), "r"(NCOPY * 32) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&rempty[r])), "r"(NW) : "memory");
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        *abort_flag = 0;
+    }
+    if (warp == WMMA) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tslot;
+
+    if (warp == WMMA) {
+        if (lane == 0) {
+            // ---------------- MMA issuer: one chunk after the other, across tiles ----------------
+            int c = 0;
+            for (int i = blockIdx.x; i < L.nitems && !*abort_flag; i += gridDim.x) {
+                Item it;
+                if (!item_at(L, i, it)) continue;
+                // a ragged last N tile computes only its 16-column groups
+                const uint32_t idesc = IDESC | ((uint32_t)(min(TN, (it.P->N - it.n0 + 15) & ~15) >> 3) << 17);
+                for (int t = 0; t < it.P->nt && !*abort_flag; ++t) {
+                    int k0, ke;
+                    k_range(L, it, it.P->t[t].K, k0, ke);
+                    // Cr = Ar Br - sa sb Ai Bi, Ci = sb Ar Bi + sa Ai Br (sa, sb: -1 for a conjugated operand)
+                    const bool ca = it.P->t[t].sa < 0.f, cb = it.P->t[t].sb < 0.f;
+                    const uint32_t id_ii = idesc | (ca == cb ? NEG_A : 0u), id_ri = idesc | (cb ? NEG_A : 0u),
+                                   id_ir = idesc | (ca ? NEG_A : 0u);
+                    for (; k0 < ke; k0 += KC, ++c) {
+                        const int s = c % NSTAGE, b = c & 1;
+                        if (!mbar_wait(smem_u32(&full[s]), (uint32_t)((c / NSTAGE) & 1), abort_flag) ||
+                            (c >= 2 && !mbar_wait(smem_u32(&tempty[b]), (uint32_t)(((c >> 1) - 1) & 1), abort_flag))) {
+                            *abort_flag = 1;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t a0 = smem_u32(smem + s * STAGE);
+                        const uint64_t ar = sdesc(a0), br = sdesc(a0 + TILE);
+                        constexpr uint64_t D = PLANE >> 4;   // one plane further (0 h, 1 m, 2 l; + 3: Im)
+                        const uint64_t ai = ar + 3 * D, bi = br + 3 * D;
+                        const uint32_t dr = tmem + b * 2 * TN, di = dr + TN;
+                        // products of the order of 2^-16, then 2^-8, then 1
+#pragma unroll
+                        for (int order = 2; order >= 0; --order)
+#pragma unroll
+                            for (int p = 0; p <= order; ++p) {
+                                const int q = order - p;
+                                mma(dr, ar + p * D, br + q * D, idesc, order == 2 && p == 0 ? 0u : 1u);
+                                mma(di, ar + p * D, bi + q * D, id_ri, order == 2 && p == 0 ? 0u : 1u);
+                                mma(dr, ai + p * D, bi + q * D, id_ii, 1u);
+                                mma(di, ai + p * D, br + q * D, id_ir, 1u);
+                            }
+                        commit(smem_u32(&empty[s]));
+                        commit(smem_u32(&tfull[b]));
+                    }
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp >= WCOPY) {
+        // ---------------- copies, across tiles ----------------
+        const int w = warp - WCOPY;
+        long long* const rowoff = reinterpret_cast<long long*>(smem + ROW_OFF) + w * 256;
+        int c = 0;
+        for (int i = blockIdx.x; i < L.nitems && !*abort_flag; i += gridDim.x) {
+            Item it;
+            if (!item_at(L, i, it)) continue;
+            for (int t = 0; t < it.P->nt && !*abort_flag; ++t) {
+                const GTerm& T = it.P->t[t];
+                int k0, ke;
+                k_range(L, it, T.K, k0, ke);
+                if (k0 >= ke) continue;
+                const Opnd oa = make_opnd<AM == A_MK>(T.A, T.lda, nullptr, it.P->M, it.m0, rowoff, lane);
+                const Opnd ob = make_opnd<BMD == B_NK>(T.B, T.ldb, T.g, it.P->N, it.n0, rowoff + 128, lane);
+                for (; k0 < ke; k0 += KC, ++c) {
+                    const int s = c % NRAW;
+                    if (c >= NRAW && !mbar_wait(smem_u32(&rempty[s]), (uint32_t)((c / NRAW - 1) & 1), abort_flag)) {
+                        *abort_flag = 1;
+                        break;
+                    }
+                    const uint32_t raw = smem_u32(smem + RAW_OFF) + s * 2 * RAW_OP;
+                    copy_chunk<AM == A_MK>(oa, k0, ke, w, raw, lane);
+                    copy_chunk<BMD == B_NK>(ob, k0, ke, w, raw + RAW_OP, lane);
+                    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&rfull[s]))
+                                 : "memory");
+                }
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if (warp < NW) {
+        // ---------------- workers ----------------
+        const bool isB = warp >= NW / 2;
+        const int t8 = threadIdx.x & 255;
+        const int lg = warp & 3, cg = warp >> 2;   // TMEM lanes 32 lg .., columns 32 cg ..
+        const uint32_t tm0 = tmem + ((uint32_t)(lg * 32) << 16) + cg * 32;
+        uint64_t acc[32];   // real parts of 32 columns in pairs, then imaginary parts
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[j] = 0;
+        // the item whose chunks are being added up, its chunks still to split and to drain
+        int ci = (int)blockIdx.x - (int)gridDim.x;
+        bool cols = false;   // it has columns in this warp's group
+        // moves to the next item with chunks (returns their number, 0 at the
+        // end); items without chunks are written as zeros on the way
+        auto next_item = [&]() -> int {
+            for (;;) {
+                ci += gridDim.x;
+                if (ci >= L.nitems) return 0;
+                Item it;
+                if (!item_at(L, ci, it)) continue;
+                const int C = chunks_of(L, it);
+                cols = it.n0 + cg * 32 < it.P->N;
+                if (C > 0) return C;
+                write_tile(it, epi, part_stride, acc, lg, cg, lane);
+            }
+        };
+        // chunks of this CTA in all (the split runs ahead of the drain, across items)
+        int total = 0;
+        for (int i = blockIdx.x; i < L.nitems; i += gridDim.x) {
+            Item it;
+            if (item_at(L, i, it)) total += chunks_of(L, it);
+        }
+        int left = next_item();
+        int produced = 0, drained = 0;
+        while (drained < total) {
+            if (produced < total) {
+                const int s = produced % NSTAGE, r = produced % NRAW;
+                if (!mbar_wait(smem_u32(&rfull[r]), (uint32_t)((produced / NRAW) & 1), abort_flag) ||
+                    (produced >= NSTAGE &&
+                     !mbar_wait(smem_u32(&empty[s]), (uint32_t)((produced / NSTAGE - 1) & 1), abort_flag))) {
+                    *abort_flag = 1;
+                    break;
+                }
+                char* tile = smem + s * STAGE + (isB ? TILE : 0);
+                const char* raw = smem + RAW_OFF + (2 * r + (isB ? 1 : 0)) * RAW_OP;
+                if (isB)
+                    split_chunk<BMD == B_NK>(tile, raw, t8);
+                else
+                    split_chunk<AM == A_MK>(tile, raw, t8);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(smem_u32(&full[s]));
+                    mbar_arrive(smem_u32(&rempty[r]));
+                }
+                ++produced;
+                if (produced < total && produced - drained <= LAG) continue;
+            }
+            const int b = drained & 1;
+            if (!mbar_wait(smem_u32(&tfull[b]), (uint32_t)((drained >> 1) & 1), abort_flag)) {
+                *abort_flag = 1;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (cols) {
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {   // Re columns 0-15, 16-31, Im columns 0-15, 16-31
+                    uint32_t r[16];
+                    tmem_ld16(tm0 + b * 2 * TN + (h >> 1) * TN + (h & 1) * 16, r);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        acc[h * 8 + j] =
+                            add2(acc[h * 8 + j], pair(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1])));
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&tempty[b]));
+            ++drained;
+            if (--left == 0) {
+                Item it;
+                item_at(L, ci, it);
+                const bool bad = write_tile(it, epi, part_stride, acc, lg, cg, lane);
+                if (__any_sync(0xffffffffu, bad)) mend_row<AM, BMD>(L, ci, epi, part_stride, lg, cg, lane);
+#pragma unroll
+                for (int j = 0; j < 32; ++j) acc[j] = 0;
+                left = next_item();
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (*abort_flag && threadIdx.x == 0) atomicExch(err, TLR_ERR_TIMEOUT);
+    if (warp == WMMA) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+template <int AM, int BMD>
+cudaError_t launch(const GemmLaunch& G, const Launch& L, unsigned grid, cudaStream_t st) {
+    k_cgemm_f32<AM, BMD><<<grid, NTHR, SMEM_BYTES, st>>>(L, G.epi, G.part_stride, G.err);
+    counted(1);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+int gemm_f32_split(long long tiles, long long K, long long most) {
+    // the split s that minimises ceil(tiles s / SMs) (K / s + 48): whole waves of
+    // tiles, each with a fixed cost (start of the pipeline, write-out) of about
+    // 48 units of depth; at least 64 deep, so that a partial is worth its write
+    const long long sms = device_sms(), smax = std::max(1LL, std::min({32LL, most, K / 64}));
+    long long best = 1;
+    double tbest = 1e300;
+    for (long long s = 1; s <= smax; ++s) {
+        const double t = (double)((std::max(1LL, tiles) * s + sms - 1) / sms) * ((double)K / s + 48.0);
+        if (t < tbest * 0.98) {
+            tbest = t;
+            best = s;
+        }
+    }
+    return (int)best;
+}
+
+cudaError_t gemm_f32_prepare() {
+    cudaError_t e = cudaFuncSetAttribute(k_cgemm_f32<A_KM, B_KN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_cgemm_f32<A_MK, B_KN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_cgemm_f32<A_MK, B_NK>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    return e;
+}
+
+cudaError_t gemm_f32(const GemmLaunch& G, cudaStream_t st) {
+    if (G.nprob == 0 || G.maxM == 0 || G.maxN == 0) return cudaSuccess;
+    if (!G.err) return cudaErrorInvalidValue;
+    Launch L;
+    L.probs = G.d_probs;
+    L.nsplit = G.nsplit;
+    L.kchunk = G.kchunk;
+    L.nx = (G.maxN + TN - 1) / TN;
+    L.ny = (G.maxM + TM - 1) / TM;
+    const long long nitems = (long long)L.nx * L.ny * G.nprob * G.nsplit;
+    if (nitems > 0x7fff0000LL) return cudaErrorInvalidValue;
+    L.nitems = (int)nitems;
+    const unsigned grid = (unsigned)std::min<long long>(device_sms(), nitems);
+    if (G.amode == A_KM && G.bmode == B_KN) return launch<A_KM, B_KN>(G, L, grid, st);
+    if (G.amode == A_MK && G.bmode == B_KN) return launch<A_MK, B_KN>(G, L, grid, st);
+    if (G.amode == A_MK && G.bmode == B_NK) return launch<A_MK, B_NK>(G, L, grid, st);
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace tlr

@@ -1,5 +1,5 @@
 // Tensor-core (tcgen05, sm_103a) grouped complex GEMM for the TLR contractions,
-// same problem tables as the FP32 SIMT path (compress, expand, projection,
+// same problem tables as the FP32 path (compress, expand, projection,
 // adjoint).
 //
 // Arithmetic.  Every complex product C = A B is formed from four real

@@ -7,7 +7,6 @@
 // latency-critical path where an allocation call may synchronise the device)
 // can still use the kernel.  The array is TLR_NOALLOC_SCRATCH_BYTES per GPU
 // that loads the library and is held until the process exits.
-#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -18,6 +17,7 @@ namespace {
 
 constexpr size_t kScratchBytes = TLR_NOALLOC_SCRATCH_BYTES;
 constexpr size_t kProbBytes = 256;  // problem descriptor slot at the start of the array
+constexpr size_t kErrOffset = 240;  // the contraction's error word, at the slot's end
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -76,12 +76,9 @@ extern "C" int tlr_mdd_adjoint_noalloc(const void* V, const void* Dt, int64_t nr
     if (scratch_address(&base) != cudaSuccess) return TLR_ERR_CUDA;
 
     // split-K over ns into as many partial slabs as fit (deterministic reduction)
-    const long long tiles = ((nr + 63) / 64) * ((nr + 63) / 64);
-    long long want = (4LL * 152 * 2 + tiles - 1) / tiles;
-    want = std::min(want, std::max(1LL, (long long)ns / 256));
-    want = std::max(1LL, std::min(want, 64LL));
+    const long long tiles = ((nr + 127) / 128) * ((nr + 127) / 128);
     const long long fit = (long long)((kScratchBytes - kProbBytes) / slab);
-    const int nsplit = (int)std::max(1LL, std::min(want, fit));
+    const int nsplit = gemm_f32_split(tiles, ns, fit);
 
     GProb p;
     memset(&p, 0, sizeof(p));
@@ -99,7 +96,9 @@ extern "C" int tlr_mdd_adjoint_noalloc(const void* V, const void* Dt, int64_t nr
     p.ldc = nr;
     cf* part = reinterpret_cast<cf*>(reinterpret_cast<char*>(base) + kProbBytes);
     p.C = part;
-    static_assert(sizeof(GProb) <= kProbBytes, "descriptor slot too small");
+    static_assert(sizeof(GProb) <= kErrOffset && kErrOffset + sizeof(int) <= kProbBytes, "descriptor slot too small");
+    int* const err = reinterpret_cast<int*>(reinterpret_cast<char*>(base) + kErrOffset);
+    if (gemm_f32_prepare() != cudaSuccess) return TLR_ERR_CUDA;
 
     GemmLaunch L;
     L.d_probs = reinterpret_cast<GProb*>(base);
@@ -116,10 +115,14 @@ extern "C" int tlr_mdd_adjoint_noalloc(const void* V, const void* Dt, int64_t nr
     // Every partial slab is written in full by the GEMM before the reduction
     // reads it, so no part of the array has to start at zero.
     if (cudaMemcpyAsync(base, &p, sizeof(GProb), cudaMemcpyHostToDevice, st) != cudaSuccess) return TLR_ERR_CUDA;
+    L.err = err;
+    if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) return TLR_ERR_CUDA;
     if (run_gemm(L, st) != cudaSuccess) return TLR_ERR_CUDA;
     if (reduce_grad(part, nsplit, nr * nr, nr * nr, 0, 1, (cf*)G, st) != cudaSuccess) return TLR_ERR_CUDA;
     // p lives on this stack frame; the copy above was staged before return,
     // but wait for the stream so the caller may reuse V, Dt and G at once.
+    int werr = 0;
+    if (cudaMemcpyAsync(&werr, err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return TLR_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return TLR_ERR_CUDA;
-    return TLR_OK;
+    return werr == 0 ? TLR_OK : TLR_ERR_TIMEOUT;
 }
