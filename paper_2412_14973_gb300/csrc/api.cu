@@ -1610,7 +1610,23 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     Arena w;
     w.base = reinterpret_cast<char*>(h->R);
     w.cap = (size_t)(reinterpret_cast<char*>(h->Zs) - w.base);
-    GProb* dp = w.take<GProb>(1);
+    struct AdjTab {
+        GProb g;
+        PProb p;
+        PackJob j[2];
+    };
+    AdjTab tab;
+    memset(&tab, 0, sizeof(tab));
+    AdjTab* dtab = w.take<AdjTab>(1);
+    GProb* dp = &dtab->g;
+    // tensor-core handles: V and conj(Dfrak) packed first, then the packed
+    // contraction (the same MMAs in the same order as the on-the-fly kernel, which
+    // its split of the operands in every tile holds to 109 TFLOP/s at nr = ns =
+    // 4096; the two packs cost 2 x 268 MB there), where both operands fit
+    const size_t pk = (size_t)packed_bytes(nr, ns, kPackTRA);
+    const bool packed = tc && h->tcp_tables && w.used + 2 * (pk + 256) <= w.cap;
+    char* pka = packed ? w.take<char>(pk) : nullptr;
+    char* pkb = packed ? w.take<char>(pk) : nullptr;
     cf* part = nullptr;
     bool own = false;
     const size_t npart = (size_t)ns_split * nr * nr;
@@ -1638,16 +1654,40 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     G1.kchunk = (int)(((ns + ns_split - 1) / ns_split + 15) / 16 * 16);
     G1.part_stride = nr * nr;
     G1.epi = ns_split > 1 ? EPI_PARTIAL : EPI_STORE;
-    cudaError_t e = cudaMemcpyAsync(dp, &p, sizeof(GProb), cudaMemcpyHostToDevice, h->st);
+    tab.g = p;
+    if (packed) {
+        for (int i = 0; i < 2; ++i) {
+            PackJob& J = tab.j[i];
+            J.src = i == 0 ? (const cf*)V : h->Dt;
+            J.ld = ns;
+            J.kcontig = 1;
+            J.sgn = i == 0 ? 1.f : -1.f;
+            J.R = (int)nr;
+            J.K = (int)ns;
+            J.TR = i == 0 ? kPackTRA : kPackTRB;
+            J.dst = i == 0 ? pka : pkb;
+            J.fmt = kFmtBF16X3;
+        }
+        tab.p.t[0] = PTerm{pka, pkb, (int)ns};
+        tab.p.nt = 1;
+        tab.p.M = tab.p.N = (int)nr;
+        tab.p.C = p.C;
+        tab.p.ldc = nr;
+        G1.d_pprobs = &dtab->p;
+        G1.d_jobs = dtab->j;
+        G1.njobs = 2;
+        G1.max_items = ((nr + 127) / 128 * 128) << 32 | ((ns + 15) / 16 * 2);
+    }
+    cudaError_t e = cudaMemcpyAsync(dtab, &tab, sizeof(tab), cudaMemcpyHostToDevice, h->st);
     G1.flops = 8.0 * nr * (double)nr * ns;
     G1.cls = 2;
-    G1.prec = tc ? TLR_PREC_BF16X3 : TLR_PREC_FP32;   // operands split on the fly
+    G1.prec = tc ? TLR_PREC_BF16X3 : TLR_PREC_FP32;
     G1.err = h->ints + SI_COUNT + 1;
     if (e == cudaSuccess) e = run_gemm(G1, h->st);
     if (e == cudaSuccess && ns_split > 1) e = reduce_grad(part, ns_split, nr * nr, nr * nr, 0, 1, (cf*)G, h->st);
     if (own) cudaFreeAsync(part, h->st);
     CK(h, e);
-    CK(h, cudaStreamSynchronize(h->st));  // p lives on this stack frame
+    CK(h, cudaStreamSynchronize(h->st));  // tab lives on this stack frame
     return TLR_OK;
 }
 
