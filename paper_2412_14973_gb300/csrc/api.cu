@@ -96,6 +96,50 @@ cudaError_t ws_alloc(void** ptr, size_t bytes, cudaStream_t st) {
     return cudaMallocFromPoolAsync(ptr, bytes, p, st);
 }
 
+// Per-call scratch, from the same pool: mapping fresh device memory on every
+// call cost as much as the work it served (0.9 of 5.9 ms of a benchmark solve at
+// nr = 2048).  When it is given back the pool keeps at most kScratchKeep bytes
+// more than it held reserved before the call.
+constexpr unsigned long long kScratchKeep = 256ull << 20;
+
+class Scratch {
+public:
+    Scratch() = default;
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+    cudaError_t get(size_t bytes, cudaStream_t st) {
+        st_ = st;
+        cudaError_t e = ws_pool(&pool_);
+        if (e == cudaSuccess) e = cudaMemPoolGetAttribute(pool_, cudaMemPoolAttrReservedMemCurrent, &before_);
+        if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)&p_, bytes, pool_, st);
+        if (e != cudaSuccess) p_ = nullptr;
+        return e;
+    }
+    char* ptr() const { return p_; }
+    // stream-ordered release; the trim takes effect on memory whose release the
+    // device has reached (call after a synchronisation where there is one)
+    void release() {
+        if (!p_) return;
+        cudaFreeAsync(p_, st_);
+        p_ = nullptr;
+        freed_ = true;
+    }
+    ~Scratch() {
+        release();
+        unsigned long long now = 0;
+        if (freed_ && cudaMemPoolGetAttribute(pool_, cudaMemPoolAttrReservedMemCurrent, &now) == cudaSuccess &&
+            now > before_ + kScratchKeep)
+            cudaMemPoolTrimTo(pool_, (size_t)(before_ + kScratchKeep));
+    }
+
+private:
+    cudaMemPool_t pool_ = nullptr;
+    cudaStream_t st_ = nullptr;
+    unsigned long long before_ = 0;
+    char* p_ = nullptr;
+    bool freed_ = false;
+};
+
 // environment switch set to "0"
 bool getenv_off(const char* name) {
     const char* e = getenv(name);
@@ -1708,20 +1752,21 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
     const size_t n2 = (size_t)n * n;
     const bool tc = tensor_core(h->d.precision);   // BF16x3 packed products for both tensor-core modes
     const int np = cg_partials(n);
-    // work arrays: G, x, r, p, y, Ap; partials; scalars; tables; packed operands (tensor cores)
+    // work arrays: G, r, p, y and (FP32) Ap, which takes G's place once G is packed;
+    // x is built in X; partials; scalars; tables; packed operands (tensor cores)
     const size_t pk = tc ? (size_t)std::max(packed_bytes(n, ns, kPackTRA), packed_bytes(n, n, kPackTRA)) : 0;
     const size_t tab = 4096;
-    const size_t bytes = 6 * n2 * sizeof(cf) + (size_t)np * sizeof(double) + 64 + tab + 2 * pk + 16 * 256;
-    char* buf = nullptr;
-    CK(h, cudaMallocAsync((void**)&buf, bytes, h->st));
+    const size_t bytes = (tc ? 4 : 5) * n2 * sizeof(cf) + (size_t)np * sizeof(double) + 64 + tab + 2 * pk + 16 * 256;
+    Scratch buf;
+    CK(h, buf.get(bytes, h->st));
     Arena a;
-    a.base = buf;
+    a.base = buf.ptr();
     cf* G = a.take<cf>(n2);
-    cf* x = a.take<cf>(n2);
+    cf* x = (cf*)X;
     cf* r = a.take<cf>(n2);
     cf* pv = a.take<cf>(n2);
     cf* y = a.take<cf>(n2);
-    cf* Ap = a.take<cf>(n2);
+    cf* Ap = tc ? G : a.take<cf>(n2);
     double* part = a.take<double>(np);
     double* sc = a.take<double>(8);
     char* tables = a.take<char>(tab);
@@ -1799,7 +1844,7 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
         auto items = [](long long R, long long K, int TR) {
             return (((R + TR - 1) / TR * TR) << 32) | ((K + 15) / 16 * 2);
         };
-        const int first[3] = {0, 2, 4}, cnt[3] = {2, 1, 1};
+        const int first[3] = {0, 2, 4}, cnt[3] = {2, 1, 0};   // p is packed where it is made
         for (int i = 0; i < 3; ++i) {
             GL[i].d_pprobs = dq + i;
             GL[i].d_jobs = dj + first[i];
@@ -1819,26 +1864,30 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
     if (e == cudaSuccess) e = cudaEventRecord(e0, h->st);
     if (e == cudaSuccess) e = gemm_any(GL[0], h->st);                          // G
     if (e == cudaSuccess) e = gemm_any(GL[1], h->st);                          // Bm -> y
-    if (e == cudaSuccess) e = cg_sym(y, nullptr, 0.f, r, n, nullptr, h->st);   // b = P(Bm) -> r
+    if (e == cudaSuccess) e = cg_sym(y, nullptr, 0.f, r, n, nullptr, sc, h->st);   // b = P(Bm) -> r
     if (e == cudaSuccess && tc) {                                              // G packed once, as A
         PackJob* dj = reinterpret_cast<PackJob*>(tables + 1024);
         e = pack_operands(dj + 3, 1, (((long long)(n + kPackTRA - 1) / kPackTRA * kPackTRA) << 32) | ((n + 15) / 16 * 2),
                           h->st);
     }
     if (e == cudaSuccess) e = cg_start(x, r, pv, n, part, sc, h->st);
+    if (e == cudaSuccess && tc) {                                              // the first p; later ones by cg_iteration_tail
+        PackJob* dj = reinterpret_cast<PackJob*>(tables + 1024);
+        e = pack_operands(dj + 4, 1, (((long long)(n + kPackTRB - 1) / kPackTRB * kPackTRB) << 32) | ((n + 15) / 16 * 2),
+                          h->st);
+    }
     const float s2 = (float)(2.0 * lambda);
     for (int it = 0; it < iters && e == cudaSuccess; ++it) {
         e = gemm_any(GL[2], h->st);                                            // y = G p
-        if (e == cudaSuccess) e = cg_sym(y, pv, s2, Ap, n, part, h->st);       // Ap = P(y) + 2 lambda p
-        if (e == cudaSuccess) e = cg_iteration_tail(x, r, pv, Ap, n, tol, part, sc, h->st);
+        if (e == cudaSuccess) e = cg_sym(y, pv, s2, Ap, n, part, sc, h->st);   // Ap = P(y) + 2 lambda p, alpha
+        if (e == cudaSuccess) e = cg_iteration_tail(x, r, pv, Ap, n, tol, part, sc, pkB, h->st);
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(X, x, n2 * sizeof(cf), cudaMemcpyDeviceToDevice, h->st);
     if (e == cudaSuccess) e = cudaEventRecord(e1, h->st);
     double hs[8] = {0};
     int werr = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(hs, sc, sizeof(hs), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&werr, h->ints + SI_COUNT + 1, sizeof(int), cudaMemcpyDeviceToHost, h->st);
-    cudaFreeAsync(buf, h->st);
+    buf.release();
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
@@ -1882,14 +1931,14 @@ int tile_ranks_impl(const cf* X, int64_t nr, int64_t b, double eps, std::vector<
     a.take<SvdTile>(nt);
     a.take<int>(nt);
     a.take<double>(1);
-    char* buf = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&buf, a.used, st);
+    Scratch buf;
+    cudaError_t e = buf.get(a.used, st);
     if (e != cudaSuccess) {
         err = std::string("tile ranks: ") + cudaGetErrorString(e);
         return e == cudaErrorMemoryAllocation ? TLR_ERR_NOMEM : TLR_ERR_CUDA;
     }
     Arena w;
-    w.base = buf;
+    w.base = buf.ptr();
     cf* work = w.take<cf>(tile_svd_work_bytes(nt, (int)b, false) / sizeof(cf));
     float* sig = w.take<float>((size_t)nt * b);
     SvdTile* dtl = w.take<SvdTile>(nt);
@@ -1902,7 +1951,7 @@ int tile_ranks_impl(const cf* X, int64_t nr, int64_t b, double eps, std::vector<
     if (e == cudaSuccess) e = rank_rule(sig, nt, (int)b, eps, dr, dv0, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ranks.data(), dr, nt * sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hv0, dv0, sizeof(double), cudaMemcpyDeviceToHost, st);
-    cudaFreeAsync(buf, st);
+    buf.release();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         err = std::string("tile ranks: ") + cudaGetErrorString(e);
@@ -2029,10 +2078,10 @@ int tlr_mdd_warm_start(tlr_mdd_t* h, const void* X, void* theta) {
     a.take<int>((size_t)std::max(1, nsvd) * bmax);
     a.take<SvdTile>(std::max(1, nsvd));
     a.take<WarmTile>(std::max(1, nw));
-    char* buf = nullptr;
-    CK(h, cudaMallocAsync((void**)&buf, a.used, h->st));
+    Scratch buf;
+    CK(h, buf.get(a.used, h->st));
     Arena w;
-    w.base = buf;
+    w.base = buf.ptr();
     cf* work = w.take<cf>(tile_svd_work_bytes(std::max(1, nsvd), bmax, true) / sizeof(cf));
     float* sig = w.take<float>((size_t)std::max(1, nsvd) * bmax);
     int* ord = w.take<int>((size_t)std::max(1, nsvd) * bmax);
@@ -2044,7 +2093,7 @@ int tlr_mdd_warm_start(tlr_mdd_t* h, const void* X, void* theta) {
     if (e == cudaSuccess)
         e = tile_svd((const cf*)X, L.nr, dtl, nsvd, bmax, work, true, 30, 1e-5f, sig, ord, nullptr, h->st);
     if (e == cudaSuccess) e = warm_fill((const cf*)X, L.nr, dwt, nw, bmax, work, sig, ord, (cf*)theta, h->st);
-    cudaFreeAsync(buf, h->st);
+    buf.release();
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);   // the host tables above go out of scope
     CK(h, e);
     return TLR_OK;
@@ -2169,16 +2218,18 @@ int tlr_mdd_unpermute_dense(tlr_mdd_t* h, const void* theta, void* X) {
                 }
             }
     }
-    cf* Xh = nullptr;
-    AsmTile* dt = nullptr;
-    CK(h, cudaMallocAsync((void**)&Xh, (size_t)nr * nr * sizeof(cf), h->st));
-    cudaError_t e = cudaMallocAsync((void**)&dt, tiles.size() * sizeof(AsmTile), h->st);
+    Scratch buf;
+    CK(h, buf.get((size_t)nr * nr * sizeof(cf) + 512 + tiles.size() * sizeof(AsmTile), h->st));
+    Arena w;
+    w.base = buf.ptr();
+    cf* Xh = w.take<cf>((size_t)nr * nr);
+    AsmTile* dt = w.take<AsmTile>(tiles.size());
+    cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = cudaMemcpyAsync(dt, tiles.data(), tiles.size() * sizeof(AsmTile), cudaMemcpyHostToDevice, h->st);
     if (e == cudaSuccess)
         e = assemble_dense((const cf*)theta, nr, L.dmax, L.N, dt, Xh, h->st, L.general, L.b > 0 ? nullptr : h->d_roff);
     if (e == cudaSuccess) e = unpermute_dense(Xh, nr, h->perm, (cf*)X, h->st);
-    if (dt) cudaFreeAsync(dt, h->st);
-    cudaFreeAsync(Xh, h->st);
+    buf.release();
     CK(h, e);
     CK(h, cudaStreamSynchronize(h->st));
     return TLR_OK;

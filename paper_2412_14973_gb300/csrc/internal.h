@@ -203,15 +203,16 @@ cudaError_t dots6_packed(char* const* kn, const cf* A1, const cf* A2, int nr, in
 cudaError_t rstep(cf* R, const cf* A1, const cf* A2, const double* alpha, int nr, int ns, int b, char* const* kn,
                   char* const* mk, double* part, cudaStream_t st, const long long* roff, int nblk, int fmt);
 // Benchmark solver of eq. (4) (k_cg.cu): the symmetrising pass
-// out = P(y) + s2 p (with partials of <p, out> when part != nullptr; p may be
-// nullptr: out = P(y)), the start (x = 0, r = p = b with b in r on entry),
-// and the CG tail of one iteration (alpha, step, beta, direction) on device
-// scalars sc[8] (slots in k_cg.cu: rr, <p,Ap>, alpha, beta, ||b||^2, done,
-// iterations).  cg_partials(n) = partial slots needed.
+// out = P(y) + s2 p with alpha from <p, out> (p may be nullptr: out = P(y)),
+// the start (x = 0, r = p = b with b in r on entry), and the CG tail of one
+// iteration (step, beta, direction; pk != nullptr: the new p as a packed BF16x3
+// B operand, its padding untouched) on device scalars sc[8] (slots in k_cg.cu:
+// rr, <p,Ap>, alpha, beta, ||b||^2, done, iterations, a block counter).
+// cg_partials(n) = partial slots needed.
 int cg_partials(int n);
-cudaError_t cg_sym(const cf* y, const cf* p, float s2, cf* out, int n, double* part, cudaStream_t st);
+cudaError_t cg_sym(const cf* y, const cf* p, float s2, cf* out, int n, double* part, double* sc, cudaStream_t st);
 cudaError_t cg_start(cf* x, cf* r, cf* p, int n, double* part, double* sc, cudaStream_t st);
-cudaError_t cg_iteration_tail(cf* x, cf* r, cf* p, const cf* Ap, int n, double tol, double* part, double* sc,
+cudaError_t cg_iteration_tail(cf* x, cf* r, cf* p, const cf* Ap, int n, double tol, double* part, double* sc, char* pk,
                               cudaStream_t st);
 // Tile SVDs (k_svd.cu) for the rank rule and the warm start.  tile_svd: one
 // one-sided Jacobi SVD per listed tile (rows r0 .. r0+m-1, columns c0 ..

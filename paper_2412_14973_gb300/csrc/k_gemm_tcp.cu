@@ -27,6 +27,7 @@
 #include <cstdlib>
 
 #include "internal.h"
+#include "pack.h"
 #include "reduce.h"
 
 namespace tlr {
@@ -61,7 +62,7 @@ constexpr uint32_t IDESC_NEG_A = IDESC | (1u << 13);
 constexpr uint32_t IDESC_TF32 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TN >> 3) << 17) |
                                 ((uint32_t)(TM >> 4) << 24);
 constexpr uint32_t IDESC_TF32_NEG_A = IDESC_TF32 | (1u << 13);
-constexpr int PK_TILE = 16384;   // bytes of one packed 128 x 16 tile (both formats)
+constexpr int PK_TILE = kPackTile;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -129,88 +130,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, float* v) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// byte offset of row r's first 16-byte group (k 0 .. 7 for BF16, k 0 .. 3
-// for TF32) inside a packed tile's first plane
-__device__ __forceinline__ int row_off(int fmt, int r) {
-    return (r >> 3) * (fmt == kFmtTF32 ? 512 : 256) + (r & 7) * 16;
-}
-
-// TF32 bit pattern of x rounded to nearest, ties away from zero
-__device__ __forceinline__ uint32_t tf32_rna(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
-}
-
-// The 8 complex values of k-group kg (k = 8 kg .. 8 kg + 7) of one row of a
-// packed tile, row = tile + row_off(fmt, r); the imaginary parts times sgn.
-__device__ __forceinline__ void pk_store8(char* row, int fmt, int kg, const float2* v, float sgn) {
-    if (fmt == kFmtTF32) {
-        uint32_t re[8], im[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            re[j] = tf32_rna(v[j].x);
-            im[j] = tf32_rna(v[j].y * sgn);
-        }
-        char* p = row + kg * 256;
-        *reinterpret_cast<uint4*>(p) = make_uint4(re[0], re[1], re[2], re[3]);
-        *reinterpret_cast<uint4*>(p + 128) = make_uint4(re[4], re[5], re[6], re[7]);
-        *reinterpret_cast<uint4*>(p + 8192) = make_uint4(im[0], im[1], im[2], im[3]);
-        *reinterpret_cast<uint4*>(p + 8192 + 128) = make_uint4(im[4], im[5], im[6], im[7]);
-        return;
-    }
-    uint32_t w[4][4];
-#pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-        const float x[2][2] = {{v[j].x, v[j + 1].x}, {v[j].y * sgn, v[j + 1].y * sgn}};
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            const __nv_bfloat162 hi = __floats2bfloat162_rn(x[p][0], x[p][1]);
-            const float2 hf = __bfloat1622float2(hi);
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(x[p][0] - hf.x, x[p][1] - hf.y);
-            w[2 * p][j >> 1] = *reinterpret_cast<const uint32_t*>(&hi);
-            w[2 * p + 1][j >> 1] = *reinterpret_cast<const uint32_t*>(&lo);
-        }
-    }
-    char* dst = row + kg * 128;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<uint4*>(dst + q * 4096) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
-}
-
-// The inverse: the 8 complex values of k-group kg of a packed row (BF16:
-// hi + lo of each part, the BF16 halves widened by moving their bits into the
-// high half of an FP32 word; TF32: the stored words).
-__device__ __forceinline__ void pk_load8(const char* row, int fmt, int kg, float2* v) {
-    if (fmt == kFmtTF32) {
-        const char* p = row + kg * 256;
-        const uint4 r0 = *reinterpret_cast<const uint4*>(p), r1 = *reinterpret_cast<const uint4*>(p + 128);
-        const uint4 i0 = *reinterpret_cast<const uint4*>(p + 8192),
-                    i1 = *reinterpret_cast<const uint4*>(p + 8192 + 128);
-        const uint32_t re[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-        const uint32_t im[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = make_float2(__uint_as_float(re[j]), __uint_as_float(im[j]));
-        return;
-    }
-    const char* src = row + kg * 128;
-    uint4 w[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) w[q] = *reinterpret_cast<const uint4*>(src + q * 4096);
-    const uint32_t* wr = reinterpret_cast<const uint32_t*>(&w[0]);
-    const uint32_t* wl = reinterpret_cast<const uint32_t*>(&w[1]);
-    const uint32_t* wi = reinterpret_cast<const uint32_t*>(&w[2]);
-    const uint32_t* wm = reinterpret_cast<const uint32_t*>(&w[3]);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const uint32_t sh = (j & 1) * 16;
-        v[j] = make_float2(__uint_as_float(((wr[j >> 1] >> sh) & 0xffffu) << 16) +
-                               __uint_as_float(((wl[j >> 1] >> sh) & 0xffffu) << 16),
-                           __uint_as_float(((wi[j >> 1] >> sh) & 0xffffu) << 16) +
-                               __uint_as_float(((wm[j >> 1] >> sh) & 0xffffu) << 16));
-    }
 }
 
 // ---------------------------------------------------------------------------

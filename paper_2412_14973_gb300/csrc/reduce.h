@@ -27,6 +27,47 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return r;
 }
 
+// Block-wide sums of K values per thread (256 threads); thread k < K returns sum k,
+// the others 0.  FP64 adds run at 2 lanes per cycle and SM on this part, so the
+// tree is folded through shared memory first (8 values per thread, 32 lanes per
+// sum): 12 warp-wide adds per value in all, where a shuffle tree in every warp
+// takes 45 (the six line-search products: 4300 -> 1150 cycles per block).
+// Every call sums in the same order.
+template <int K>
+__device__ __forceinline__ double block_sums(const double (&v)[K], double (*sh)[256]) {
+    static_assert(K <= 8, "one warp per sum");
+    const int t = threadIdx.x, w = t >> 5, l = t & 31;
+#pragma unroll
+    for (int k = 0; k < K; ++k) sh[k][t] = v[k];
+    __syncthreads();
+    double r = 0.0;
+    if (w < K) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) r += sh[w][j * 32 + l];
+        r = warp_sum(r);
+        if (l == 0) sh[w][0] = r;
+    }
+    __syncthreads();
+    r = t < K ? sh[t][0] : 0.0;
+    return r;
+}
+
+// True in every thread of the last block of a grid of `blocks` to arrive at *ctr
+// (zero before the launch, zero again after it); what the other blocks wrote
+// before the call is then visible to it.
+__device__ __forceinline__ bool last_block(unsigned* ctr, unsigned blocks) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(ctr, 1u) == blocks - 1;
+        if (last) *ctr = 0;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
 // Per-thread partial sum: FP32 terms accumulated with Knuth's two-sum
 // compensation (error-free transformation), so a thread's partial is as good
 // as an FP64 sum of its FP32 terms while costing FP32 adds only; partials are
