@@ -12,13 +12,32 @@
 // |gamma| <= tol sqrt(alpha beta) (or after max_sweeps): then
 // A_0 = U Sigma V^H with sigma_c = |a_c| and u_c = a_c / sigma_c (columns that
 // end at zero, n - m of them at least when n > m, have sigma_c = 0).
+//
+// What bounds it: instruction issue -- per pair the sums and rotation of 2 m
+// values, and a scalar part (five square roots, four divisions) that a warp per
+// pair spends on 32 lanes.  So a warp takes P pairs at a time: their 4 P sums go
+// down one butterfly that halves the values per lane at each step (16 shuffles
+// for 4 pairs instead of 80; the same tree of additions), the scalar parts run
+// side by side in groups of lanes, and each pair's two columns stay in registers
+// from the sums to the rotation.  As many columns of A, then of V, as fit live in
+// shared memory (all of A and 94 of V's 128 columns for a 128 x 128 tile; 111 of
+// A's for 256 x 256), the rest in global memory (L2).  With a warp per pair,
+// every column in L2 and read twice, 78 tiles of 128 x 128 took 8.2 ms (singular
+// values) and 9.5 ms (with V); now 5.3 and 7.1 (256 x 256, 136 tiles, values only:
+// 52.6 and 37.1).  The order of pairs, sums and
+// operations does not depend on P or on where a column lives, and the products
+// that are fused are written out, so the results are the same bits.
+#include <algorithm>
+
 #include "internal.h"
 
 namespace tlr {
 
 namespace {
 
-constexpr int SVD_THREADS = 1024;   // 32 warps: the pairs of a round run in parallel
+constexpr int SVD_SMEM = 222 * 1024;   // columns of A and V in shared memory, at most
+
+constexpr int SVD_THREADS = 512;       // at most; 128 registers
 
 __device__ __forceinline__ float warp_sumf(float v) {
 #pragma unroll
@@ -26,86 +45,217 @@ __device__ __forceinline__ float warp_sumf(float v) {
     return v;
 }
 
-// player at position m of round r (circle method; position 0 is fixed)
-__device__ __forceinline__ int player(int m, int r, int nb) { return m == 0 ? 0 : ((m - 1 + r) % (nb - 1)) + 1; }
+// player at position m of round r (circle method; position 0 is fixed):
+// ((m - 1 + r) mod (nb - 1)) + 1 with m, r < nb
+__device__ __forceinline__ int player(int m, int r, int nb) {
+    const int i = m + r;
+    return m == 0 ? 0 : (i > nb - 1 ? i - (nb - 1) : i);
+}
 
+// two FP32 operations per instruction, on (re, im) pairs
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(float x, float y) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// The rotation of one pair of values by (c, s) and the phase (er, ei); the first
+// product of each sum is the fused one:
+//   b = y (er + i ei),  x <- c x - s b,  y <- s x + c b
+__device__ __forceinline__ void rotate(f2& x, f2& y, f2 cc, f2 ss, f2 ns, f2 e, f2 ie) {
+    const float2 v = unpack2(y);
+    const f2 b = fma2(pack2(v.x, v.x), e, mul2(pack2(v.y, v.y), ie));   // e = (er, ei), ie = (-ei, er)
+    y = fma2(ss, x, mul2(cc, b));
+    x = fma2(cc, x, mul2(ns, b));
+}
+
+// R = ceil(max rows / 32): values of a column per lane; P pairs per warp (1, 2
+// or 4)
+template <int R, int P>
 __global__ void __launch_bounds__(SVD_THREADS) k_tile_svd(const cf* __restrict__ X, long long ldx,
                                                           const SvdTile* __restrict__ tiles, int bmax,
                                                           cf* __restrict__ work, int want_vec, int max_sweeps,
                                                           float tol, float* __restrict__ sig,
-                                                          int* __restrict__ order, int* __restrict__ sweeps_out) {
+                                                          int* __restrict__ order, int* __restrict__ sweeps_out,
+                                                          int smem_bytes) {
+    extern __shared__ __align__(16) cf cols[];
     const int t = blockIdx.x;
     const SvdTile tg = tiles[t];
     // the matrix the sweeps work on: the tile (m x n) or its transpose
     const int m = tg.trans ? tg.n : tg.m, n = tg.trans ? tg.m : tg.n, nb = n + (n & 1);
     const long long slot = (long long)bmax * bmax;
-    cf* A = work + (long long)t * (want_vec ? 2 : 1) * slot;   // column-major m x n
-    cf* V = A + slot;                                          // column-major n x n
+    cf* const Ag = work + (long long)t * (want_vec ? 2 : 1) * slot;   // column-major m x n
+    cf* const Vg = Ag + slot;                                         // column-major n x n
+    // columns in shared memory: the first sa of A, then the first sv of V
+    const int room = smem_bytes / (int)sizeof(cf);
+    const int sa = min(n, room / m), sv = want_vec ? min(n, (room - sa * m) / n) : 0;
+    cf* const Vs = cols + sa * m;
+    auto colA = [&](int c) { return c < sa ? cols + c * m : Ag + (long long)c * m; };
+    auto colV = [&](int c) { return c < sv ? Vs + c * n : Vg + (long long)c * n; };
     __shared__ unsigned int smax;
     __shared__ float snorm[512];
     // load the tile (reads coalesced along the rows of X), V = I
-    for (long long e = threadIdx.x; e < (long long)m * n; e += blockDim.x) {
+    for (int e = threadIdx.x; e < m * n; e += blockDim.x) {
         if (tg.trans) {
-            const int r = (int)(e % m), c = (int)(e / m);   // A[r][c] = X tile[c][r]
-            A[(long long)c * m + r] = X[((long long)tg.r0 + c) * ldx + (long long)tg.c0 + r];
+            const int r = e % m, c = e / m;   // A[r][c] = X tile[c][r]
+            colA(c)[r] = X[((long long)tg.r0 + c) * ldx + (long long)tg.c0 + r];
         } else {
-            const int r = (int)(e / n), c = (int)(e % n);
-            A[(long long)c * m + r] = X[((long long)tg.r0 + r) * ldx + (long long)tg.c0 + c];
+            const int r = e / n, c = e % n;
+            colA(c)[r] = X[((long long)tg.r0 + r) * ldx + (long long)tg.c0 + c];
         }
     }
     if (want_vec)
-        for (long long e = threadIdx.x; e < (long long)n * n; e += blockDim.x)
-            V[e] = make_float2((e / n) == (e % n) ? 1.f : 0.f, 0.f);
+        for (int e = threadIdx.x; e < n * n; e += blockDim.x)
+            colV(e / n)[e % n] = make_float2((e / n) == (e % n) ? 1.f : 0.f, 0.f);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+    constexpr int NV = 4 * P, GRP = 32 / P;   // sums of a batch; lanes per pair in the scalar part
     int sw = 0;
     for (; sw < max_sweeps; ++sw) {
         if (threadIdx.x == 0) smax = 0u;
         __syncthreads();
+        float mx = 0.f;
         for (int r = 0; r < nb - 1; ++r) {
-            for (int k = warp; k < nb / 2; k += nwarp) {
-                const int p = player(k, r, nb), q = player(nb - 1 - k, r, nb);
-                if (p >= n || q >= n) continue;   // the dummy player of an odd n
-                cf* ap = A + (long long)p * m;
-                cf* aq = A + (long long)q * m;
-                float al = 0.f, be = 0.f, gr = 0.f, gi = 0.f;
-                for (int i = lane; i < m; i += 32) {
-                    const cf x = ap[i], y = aq[i];
-                    al = fmaf(x.x, x.x, fmaf(x.y, x.y, al));
-                    be = fmaf(y.x, y.x, fmaf(y.y, y.y, be));
-                    gr = fmaf(x.x, y.x, fmaf(x.y, y.y, gr));    // Re(conj(x) y)
-                    gi = fmaf(x.x, y.y, fmaf(-x.y, y.x, gi));   // Im(conj(x) y)
-                }
-                al = warp_sumf(al);
-                be = warp_sumf(be);
-                gr = warp_sumf(gr);
-                gi = warp_sumf(gi);
-                const float g = sqrtf(gr * gr + gi * gi);
-                if (!(al > 0.f) || !(be > 0.f) || !(g > tol * sqrtf(al) * sqrtf(be))) continue;
-                if (lane == 0) atomicMax(&smax, __float_as_uint(g / (sqrtf(al) * sqrtf(be))));
-                const float zeta = (be - al) / (2.f * g);
-                const float tt = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
-                const float c = rsqrtf(1.f + tt * tt), s = c * tt;
-                const float er = gr / g, ei = -gi / g;   // e^{-i phi}
-                for (int i = lane; i < m; i += 32) {
-                    const cf x = ap[i], y = aq[i];
-                    const cf yb = make_float2(y.x * er - y.y * ei, y.x * ei + y.y * er);
-                    ap[i] = make_float2(c * x.x - s * yb.x, c * x.y - s * yb.y);
-                    aq[i] = make_float2(s * x.x + c * yb.x, s * x.y + c * yb.y);
-                }
-                if (want_vec) {
-                    cf* vp = V + (long long)p * n;
-                    cf* vq = V + (long long)q * n;
-                    for (int i = lane; i < n; i += 32) {
-                        const cf x = vp[i], y = vq[i];
-                        const cf yb = make_float2(y.x * er - y.y * ei, y.x * ei + y.y * er);
-                        vp[i] = make_float2(c * x.x - s * yb.x, c * x.y - s * yb.y);
-                        vq[i] = make_float2(s * x.x + c * yb.x, s * x.y + c * yb.y);
+            for (int k0 = warp * P; k0 < nb / 2; k0 += nwarp * P) {
+                f2 x[P][R], y[P][R];
+                f2 *ap[P], *aq[P];
+                int pp[P], qq[P];
+                float sum[NV];   // |a_p|^2, |a_q|^2, Re and Im of a_p^H a_q of each pair
+#pragma unroll
+                for (int u = 0; u < P; ++u) {
+                    const int k = k0 + u;
+                    const int p = player(k, r, nb), q = player(nb - 1 - k, r, nb);
+                    const bool on = k < nb / 2 && p < n && q < n;   // not the dummy player of an odd n
+                    pp[u] = on ? p : 0;
+                    qq[u] = on ? q : 0;
+                    ap[u] = reinterpret_cast<f2*>(colA(pp[u]));
+                    aq[u] = reinterpret_cast<f2*>(colA(qq[u]));
+#pragma unroll
+                    for (int j = 0; j < R; ++j) {
+                        const int i = lane + 32 * j;
+                        x[u][j] = on && i < m ? ap[u][i] : 0;
+                        y[u][j] = on && i < m ? aq[u][i] : 0;
                     }
+                }
+#pragma unroll
+                for (int u = 0; u < P; ++u) {
+                    float al = 0.f, be = 0.f;
+                    f2 gg = 0;   // Re and Im of conj(x) y
+#pragma unroll
+                    for (int j = 0; j < R; ++j) {
+                        const float2 v = unpack2(x[u][j]), w = unpack2(y[u][j]);
+                        al = fmaf(v.x, v.x, fmaf(v.y, v.y, al));
+                        be = fmaf(w.x, w.x, fmaf(w.y, w.y, be));
+                        gg = fma2(pack2(v.x, v.x), y[u][j], fma2(pack2(v.y, -v.y), pack2(w.y, w.x), gg));
+                    }
+                    sum[4 * u] = al;
+                    sum[4 * u + 1] = be;
+                    sum[4 * u + 2] = unpack2(gg).x;
+                    sum[4 * u + 3] = unpack2(gg).y;
+                }
+                // butterfly over the lanes; while more than one value is left, a
+                // lane keeps the half that its bit says and sends the other
+                int left = NV;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    if (left > 1) {
+                        left >>= 1;
+                        const bool hi = (lane & o) != 0;
+#pragma unroll
+                        for (int v = 0; v < NV / 2; ++v)
+                            if (v < left) {
+                                const float keep = hi ? sum[v + left] : sum[v], send = hi ? sum[v] : sum[v + left];
+                                sum[v] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                            }
+                    } else {
+                        sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], o);
+                    }
+                }
+                // the lane group of pair u: lanes u GRP ..; kind t in its quarter t
+                const int g0 = lane & ~(GRP - 1);
+                const float al = __shfl_sync(0xffffffffu, sum[0], g0);
+                const float be = __shfl_sync(0xffffffffu, sum[0], g0 + GRP / 4);
+                const float gr = __shfl_sync(0xffffffffu, sum[0], g0 + GRP / 2);
+                const float gi = __shfl_sync(0xffffffffu, sum[0], g0 + 3 * GRP / 4);
+                const float g = sqrtf(fmaf(gr, gr, __fmul_rn(gi, gi)));
+                const bool turn = al > 0.f && be > 0.f && g > tol * sqrtf(al) * sqrtf(be);
+                const unsigned turns = __ballot_sync(0xffffffffu, turn);
+                if (turns == 0) continue;
+                float c = 1.f, s = 0.f, er = 1.f, ei = 0.f;
+                if (turn) {
+                    mx = fmaxf(mx, g / (sqrtf(al) * sqrtf(be)));
+                    const float zeta = (be - al) / (2.f * g);
+                    const float tt = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
+                    c = rsqrtf(fmaf(tt, tt, 1.f));
+                    s = c * tt;
+                    er = gr / g;
+                    ei = -gi / g;   // e^{-i phi}
+                }
+                // the pairs' rotations, from their lane groups to the warp
+                f2 cc[P], ss[P], e[P];
+#pragma unroll
+                for (int u = 0; u < P; ++u) {
+                    const float cu = __shfl_sync(0xffffffffu, c, u * GRP), su = __shfl_sync(0xffffffffu, s, u * GRP);
+                    cc[u] = pack2(cu, cu);
+                    ss[u] = pack2(su, su);
+                    e[u] = pack2(__shfl_sync(0xffffffffu, er, u * GRP), __shfl_sync(0xffffffffu, ei, u * GRP));
+                }
+                auto turned = [&](int u) { return ((turns >> (u * GRP)) & 1) != 0; };
+                auto turn_rows = [&](int u, f2* p, f2* q, int rows) {
+                    const float2 ev = unpack2(e[u]);
+                    const f2 ie = pack2(-ev.y, ev.x), ns = pack2(-unpack2(ss[u]).x, -unpack2(ss[u]).x);
+#pragma unroll
+                    for (int j = 0; j < R; ++j) {
+                        const int i = lane + 32 * j;
+                        rotate(x[u][j], y[u][j], cc[u], ss[u], ns, e[u], ie);
+                        if (i < rows) {
+                            p[i] = x[u][j];
+                            q[i] = y[u][j];
+                        }
+                    }
+                };
+#pragma unroll
+                for (int u = 0; u < P; ++u)
+                    if (turned(u)) turn_rows(u, ap[u], aq[u], m);
+                if (want_vec) {
+#pragma unroll
+                    for (int u = 0; u < P; ++u) {
+                        if (!turned(u)) continue;
+                        const f2* vp = reinterpret_cast<const f2*>(colV(pp[u]));
+                        const f2* vq = reinterpret_cast<const f2*>(colV(qq[u]));
+#pragma unroll
+                        for (int j = 0; j < R; ++j) {
+                            const int i = lane + 32 * j;
+                            x[u][j] = i < n ? vp[i] : 0;
+                            y[u][j] = i < n ? vq[i] : 0;
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < P; ++u)
+                        if (turned(u))
+                            turn_rows(u, reinterpret_cast<f2*>(colV(pp[u])), reinterpret_cast<f2*>(colV(qq[u])), n);
                 }
             }
             __syncthreads();
         }
+        if (mx > 0.f) atomicMax(&smax, __float_as_uint(mx));
+        __syncthreads();
         if (__uint_as_float(smax) <= tol) {
             ++sw;
             break;
@@ -115,7 +265,7 @@ __global__ void __launch_bounds__(SVD_THREADS) k_tile_svd(const cf* __restrict__
     // sigma_c = |a_c|, then the order of decreasing sigma (ties by column);
     // slots n .. bmax-1 get sigma = -1 (below every threshold)
     for (int c = warp; c < n; c += nwarp) {
-        const cf* ac = A + (long long)c * m;
+        const cf* ac = colA(c);
         float s2 = 0.f;
         for (int i = lane; i < m; i += 32) s2 = fmaf(ac[i].x, ac[i].x, fmaf(ac[i].y, ac[i].y, s2));
         s2 = warp_sumf(s2);
@@ -135,6 +285,10 @@ __global__ void __launch_bounds__(SVD_THREADS) k_tile_svd(const cf* __restrict__
     for (int c = n + threadIdx.x; c < bmax; c += blockDim.x) {
         sig[(long long)t * bmax + c] = -1.f;
         if (order) order[(long long)t * bmax + c] = 0;
+    }
+    if (want_vec) {   // the columns kept in shared memory go where the warm start reads them
+        for (int e = threadIdx.x; e < sa * m; e += blockDim.x) Ag[e] = cols[e];
+        for (int e = threadIdx.x; e < sv * n; e += blockDim.x) Vg[e] = Vs[e];
     }
     if (threadIdx.x == 0 && sweeps_out) sweeps_out[t] = sw;
 }
@@ -237,8 +391,31 @@ cudaError_t tile_svd(const cf* X, long long ldx, const SvdTile* tiles, int ntile
                      int max_sweeps, float tol, float* sig, int* order, int* sweeps, cudaStream_t st) {
     if (ntiles == 0) return cudaSuccess;
     if (bmax < 1 || bmax > 512) return cudaErrorInvalidValue;
-    k_tile_svd<<<ntiles, SVD_THREADS, 0, st>>>(X, ldx, tiles, bmax, work, vec ? 1 : 0, max_sweeps, tol, sig, order,
-                                               sweeps);
+    // shared memory for the columns of the largest tile (or what there is of it);
+    // a warp per pair of a round
+    const long long want = (long long)bmax * bmax * (vec ? 2 : 1) * (long long)sizeof(cf);
+    const int smem = (int)std::min<long long>(want, SVD_SMEM);
+    const int R = (bmax + 31) / 32, pairs = (bmax + 1) / 2;
+#define TLR_SVD(Rv, Pv)                                                                                         \
+    do {                                                                                                        \
+        cudaError_t e =                                                                                         \
+            cudaFuncSetAttribute(k_tile_svd<Rv, Pv>, cudaFuncAttributeMaxDynamicSharedMemorySize, SVD_SMEM);    \
+        if (e != cudaSuccess) return e;                                                                         \
+        k_tile_svd<Rv, Pv><<<ntiles, std::min(SVD_THREADS, 32 * ((pairs + Pv - 1) / Pv)), smem, st>>>(          \
+            X, ldx, tiles, bmax, work, vec ? 1 : 0, max_sweeps, tol, sig, order, sweeps, smem);                 \
+    } while (0)
+    // P pairs of 2 R values per warp: 64 registers
+    if (R <= 1)
+        TLR_SVD(1, 4);
+    else if (R <= 2)
+        TLR_SVD(2, 4);
+    else if (R <= 4)
+        TLR_SVD(4, 4);
+    else if (R <= 8)
+        TLR_SVD(8, 2);
+    else
+        TLR_SVD(16, 1);
+#undef TLR_SVD
     counted(1);
     return cudaGetLastError();
 }
