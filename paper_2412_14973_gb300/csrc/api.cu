@@ -2159,7 +2159,10 @@ int tlr_mdd_time_to_freq(const float* x_t, int64_t ntr, int64_t nt, int64_t f0, 
     std::string err;
     int rc = check_stack(ntr, nt, f0, nf, err);
     if (rc) FAIL(h, rc, err);
-    rc = fft_stack(true, x_t, nullptr, ntr, nt, f0, nf, (cf*)X_w, nullptr, (cudaStream_t)stream, err);
+    Scratch buf;   // the transform's tables
+    const size_t need = fft_scratch_bytes(nt);
+    if (need) CK(h, buf.get(need, (cudaStream_t)stream));
+    rc = fft_stack(true, x_t, nullptr, ntr, nt, f0, nf, (cf*)X_w, nullptr, buf.ptr(), (cudaStream_t)stream, err);
     if (rc) FAIL(h, rc, err);
     return TLR_OK;
 }
@@ -2171,7 +2174,10 @@ int tlr_mdd_freq_to_time(const void* X_w, int64_t ntr, int64_t nt, int64_t f0, i
     std::string err;
     int rc = check_stack(ntr, nt, f0, nf, err);
     if (rc) FAIL(h, rc, err);
-    rc = fft_stack(false, nullptr, (const cf*)X_w, ntr, nt, f0, nf, nullptr, x_t, (cudaStream_t)stream, err);
+    Scratch buf;   // the transform's tables
+    const size_t need = fft_scratch_bytes(nt);
+    if (need) CK(h, buf.get(need, (cudaStream_t)stream));
+    rc = fft_stack(false, nullptr, (const cf*)X_w, ntr, nt, f0, nf, nullptr, x_t, buf.ptr(), (cudaStream_t)stream, err);
     if (rc) FAIL(h, rc, err);
     return TLR_OK;
 }

@@ -6,12 +6,26 @@
 // Traces are stored trace-major, x_t[tr][t] (tr = s nr + r for data, a nr +
 // b for X), nt samples each.  X(omega_k) = sum_t x(t) exp(-2 pi i k t / nt)
 // (unnormalised), k = 0 .. nt/2; the inverse puts the band [f0, f0 + nf) back
-// (zero elsewhere) and divides by nt.  The real FFTs are cuFFT plans over a
-// chunk of traces; the band gather / scatter between the trace-major spectrum
-// and the frequency-major stack (stack[f][tr], one ns x nr panel per
-// frequency) are transposes through shared memory, coalesced on both sides.
+// (zero elsewhere) and divides by nt.
+//
+// Lengths up to 4096 with prime factors up to 13, and any length up to 2048, take
+// one kernel per direction: a CTA transforms a few pairs of traces (a pair as the
+// real and imaginary part of one complex transform) in shared memory and writes
+// the band of the frequency-major stack (stack[f][tr], one ns x nr panel per
+// frequency) or the traces themselves, so a trace is read once and its band
+// written once: 244 MB each way for 40000 traces of 1125 samples, 200 bins,
+// where a library transform between a spectrum in memory and a gather moved
+// 1.5 GB and its plans were made (and destroyed) on every call: 3.55 ms for both
+// directions against 0.46 here (kernels 233 + 189 us).  Bound by shared-memory
+// traffic (two passes per factor); the bytes alone would take 72 us.
+//
+// Other lengths: cuFFT plans over a chunk of traces, with the band gather /
+// scatter between the trace-major spectrum and the stack as transposes through
+// shared memory, coalesced on both sides.
 #include <cufft.h>
 
+#include <algorithm>
+#include <cstring>
 #include <string>
 
 #include "internal.h"
@@ -68,6 +82,475 @@ __global__ void k_scale(float* x, long long n, float s) {
         x[i] *= s;
 }
 
+// ---------------------------------------------------------------------------
+// transforms in shared memory
+// ---------------------------------------------------------------------------
+// A plan of length n: the complex transform has length M = n, factors fac[], or,
+// for n with a prime factor above 13, M = a power of two >= 2 n - 1 (Bluestein
+// 1970: the transform of n points as a convolution with a chirp).
+constexpr int FFT_T = 256;
+constexpr int FFT_MAXF = 12;
+struct FftPlan {
+    int n, M, nfac, B;             // B: trace pairs per CTA
+    int fac[FFT_MAXF];
+    unsigned magic[FFT_MAXF];      // ceil(2^32 / L) of the stage's L = product of the factors before it
+    unsigned magic_m[FFT_MAXF];    // ceil(2^32 / m), m = M / factor
+    bool chirp;
+};
+
+// The tables of a plan: W_M^j = exp(-2 pi i j / M), j < M, then (chirp) c_t =
+// exp(-pi i t^2 / n), t < n, then the transform of conj(c) wrapped to M (filled by
+// k_fft_chirp).  FP64 angles, rounded once.
+__global__ void k_fft_tables(FftPlan P, cf* __restrict__ tab) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    double s, c;
+    if (e < P.M) {
+        sincospi(-2.0 * e / P.M, &s, &c);
+        tab[e] = make_float2((float)c, (float)s);
+    } else if (P.chirp && e < P.M + P.n) {
+        const long long t = e - P.M;
+        sincospi(-(double)(t * t % (2LL * P.n)) / P.n, &s, &c);
+        tab[e] = make_float2((float)c, (float)s);
+    }
+}
+
+__device__ __forceinline__ cf cmul(cf a, cf b) {
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ cf cadd(cf a, cf b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ cf csub(cf a, cf b) { return make_float2(a.x - b.x, a.y - b.y); }
+
+// the transform of R values in place; W_R^1 = w[step] for the sizes without a
+// closed form here
+template <int R>
+__device__ __forceinline__ void dft(cf* v, const cf* __restrict__ w, int step) {
+    if (R == 2) {
+        const cf a = v[0];
+        v[0] = cadd(a, v[1]);
+        v[1] = csub(a, v[1]);
+    } else if (R == 4) {
+        const cf a = cadd(v[0], v[2]), b = csub(v[0], v[2]), c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
+        v[0] = cadd(a, c);
+        v[1] = make_float2(b.x + d.y, b.y - d.x);
+        v[2] = csub(a, c);
+        v[3] = make_float2(b.x - d.y, b.y + d.x);
+    } else if (R == 3) {
+        const cf s = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+        constexpr float h = 0.86602540378443864676f;   // sin(2 pi / 3)
+        const cf m = make_float2(fmaf(-0.5f, s.x, v[0].x), fmaf(-0.5f, s.y, v[0].y));
+        v[0] = cadd(v[0], s);
+        v[1] = make_float2(fmaf(h, d.y, m.x), fmaf(-h, d.x, m.y));
+        v[2] = make_float2(fmaf(-h, d.y, m.x), fmaf(h, d.x, m.y));
+    } else if (R == 5) {
+        constexpr float c1 = 0.30901699437494742410f, c2 = -0.80901699437494742410f;   // cos(2 pi / 5), cos(4 pi / 5)
+        constexpr float s1 = 0.95105651629515357212f, s2 = 0.58778525229247312917f;    // sin(2 pi / 5), sin(4 pi / 5)
+        const cf a = cadd(v[1], v[4]), b = csub(v[1], v[4]), c = cadd(v[2], v[3]), d = csub(v[2], v[3]);
+        const cf p = make_float2(fmaf(c2, c.x, fmaf(c1, a.x, v[0].x)), fmaf(c2, c.y, fmaf(c1, a.y, v[0].y)));
+        const cf q = make_float2(fmaf(c1, c.x, fmaf(c2, a.x, v[0].x)), fmaf(c1, c.y, fmaf(c2, a.y, v[0].y)));
+        const cf r = make_float2(fmaf(s2, d.x, s1 * b.x), fmaf(s2, d.y, s1 * b.y));
+        const cf t = make_float2(fmaf(-s1, d.x, s2 * b.x), fmaf(-s1, d.y, s2 * b.y));
+        v[0] = cadd(v[0], cadd(a, c));
+        v[1] = make_float2(p.x + r.y, p.y - r.x);
+        v[4] = make_float2(p.x - r.y, p.y + r.x);
+        v[2] = make_float2(q.x + t.y, q.y - t.x);
+        v[3] = make_float2(q.x - t.y, q.y + t.x);
+    } else {
+        // pairs v_j +- v_{R-j}: real parts from the cosines, imaginary from the sines
+        cf a[R / 2], b[R / 2], o[R];
+        o[0] = v[0];
+#pragma unroll
+        for (int j = 0; j < R / 2; ++j) {
+            a[j] = cadd(v[j + 1], v[R - 1 - j]);
+            b[j] = csub(v[j + 1], v[R - 1 - j]);
+            o[0] = cadd(o[0], a[j]);
+        }
+#pragma unroll
+        for (int k = 1; k <= R / 2; ++k) {
+            cf p = v[0], q = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < R / 2; ++j) {
+                const cf t = w[(k * (j + 1) % R) * step];   // cos, -sin
+                p = make_float2(fmaf(t.x, a[j].x, p.x), fmaf(t.x, a[j].y, p.y));
+                q = make_float2(fmaf(-t.y, b[j].x, q.x), fmaf(-t.y, b[j].y, q.y));
+            }
+            o[k] = make_float2(p.x + q.y, p.y - q.x);
+            o[R - k] = make_float2(p.x - q.y, p.y + q.x);
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[k] = o[k];
+    }
+}
+
+// one factor of `count` transforms of length M (rows of ld values): Stockham's
+// autosort step, src to dst.  The butterflies of all rows share the threads.
+// up != nullptr: the two parts of row b's values times up[2 b], up[2 b + 1] first.
+template <int R>
+__device__ __forceinline__ void fft_stage(const cf* __restrict__ src, cf* __restrict__ dst, int M, int ld, int count,
+                                          int L, unsigned magic, unsigned magic_m, const cf* __restrict__ w,
+                                          const float* up) {
+    const int m = M / R, step = m / L;   // step: W_{L R}^1 = W_M^step
+    for (int e = threadIdx.x; e < count * m; e += FFT_T) {
+        const int b = m == 1 ? e : (int)__umulhi((unsigned)e, magic_m), j = e - b * m;
+        const int g = L == 1 ? j : (int)__umulhi((unsigned)j, magic), k = j - g * L;
+        const cf* s = src + b * ld + j;
+        cf v[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = s[q * m];
+        if (up) {
+            const float ux = up[2 * b], uy = up[2 * b + 1];
+#pragma unroll
+            for (int q = 0; q < R; ++q) v[q] = make_float2(v[q].x * ux, v[q].y * uy);
+        }
+        if (k) {
+#pragma unroll
+            for (int q = 1; q < R; ++q) v[q] = cmul(v[q], __ldg(w + k * q * step));
+        }
+        dft<R>(v, w, m);
+        cf* d = dst + b * ld + g * L * R + k;
+#pragma unroll
+        for (int q = 0; q < R; ++q) d[q * L] = v[q];
+    }
+    __syncthreads();
+}
+
+// `count` transforms of length M in a (scratch b), their parts times up[] first
+// (up != nullptr); returns where they end up
+__device__ __forceinline__ cf* fft_rows(const FftPlan& P, cf* a, cf* b, int ld, int count, const cf* __restrict__ w,
+                                        const float* up) {
+    int L = 1;
+    for (int f = 0; f < P.nfac; ++f) {
+        const unsigned mg = P.magic[f], mm = P.magic_m[f];
+        switch (P.fac[f]) {
+            case 2: fft_stage<2>(a, b, P.M, ld, count, L, mg, mm, w, up); break;
+            case 3: fft_stage<3>(a, b, P.M, ld, count, L, mg, mm, w, up); break;
+            case 4: fft_stage<4>(a, b, P.M, ld, count, L, mg, mm, w, up); break;
+            case 5: fft_stage<5>(a, b, P.M, ld, count, L, mg, mm, w, up); break;
+            case 7: fft_stage<7>(a, b, P.M, ld, count, L, mg, mm, w, up); break;
+            case 11: fft_stage<11>(a, b, P.M, ld, count, L, mg, mm, w, up); break;
+            default: fft_stage<13>(a, b, P.M, ld, count, L, mg, mm, w, up); break;
+        }
+        up = nullptr;
+        L *= P.fac[f];
+        cf* t = a;
+        a = b;
+        b = t;
+    }
+    return a;
+}
+
+// the n-point transforms of the rows of a (n values each, zeros beyond them when
+// P.chirp): plain, or by the chirp convolution
+__device__ __forceinline__ cf* fft_any(const FftPlan& P, cf* a, cf* b, int ld, const cf* __restrict__ tab,
+                                       const float* up) {
+    if (!P.chirp && (P.nfac || !up)) return fft_rows(P, a, b, ld, P.B, tab, up);
+    if (!P.chirp) {   // one point
+        const int r = threadIdx.x;
+        if (r < P.B) a[r * ld] = make_float2(a[r * ld].x * up[2 * r], a[r * ld].y * up[2 * r + 1]);
+        __syncthreads();
+        return a;
+    }
+    const cf* c = tab + P.M;
+    const cf* bt = c + P.n;
+    cf* y = fft_rows(P, a, b, ld, P.B, tab, nullptr);
+    for (int r = 0; r < P.B; ++r)
+        for (int k = threadIdx.x; k < P.M; k += FFT_T) {
+            const cf t = cmul(y[r * ld + k], __ldg(bt + k));
+            y[r * ld + k] = make_float2(t.x, -t.y);   // conjugated: the inverse by a forward transform
+        }
+    __syncthreads();
+    y = fft_rows(P, y, y == a ? b : a, ld, P.B, tab, nullptr);
+    const float s = 1.f / (float)P.M;
+    for (int r = 0; r < P.B; ++r)
+        for (int k = threadIdx.x; k < P.n; k += FFT_T) {
+            const cf t = y[r * ld + k];
+            y[r * ld + k] = cmul(make_float2(t.x * s, -t.y * s), __ldg(c + k));
+        }
+    __syncthreads();
+    return y;
+}
+
+// the transform of the wrapped conjugate chirp, for P.chirp (one CTA)
+__global__ void __launch_bounds__(FFT_T) k_fft_chirp(const __grid_constant__ FftPlan P, cf* __restrict__ tab) {
+    extern __shared__ __align__(16) cf sm[];
+    const int ld = P.M + 1;
+    const cf* c = tab + P.M;
+    for (int k = threadIdx.x; k < P.M; k += FFT_T) {
+        const int t = min(k, P.M - k);
+        cf v = make_float2(0.f, 0.f);
+        if (t < P.n) v = make_float2(c[t].x, -c[t].y);
+        sm[k] = v;
+    }
+    __syncthreads();
+    const cf* y = fft_rows(P, sm, sm + ld, ld, 1, tab, nullptr);
+    for (int k = threadIdx.x; k < P.M; k += FFT_T) tab[P.M + P.n + k] = y[k];
+}
+
+// The two traces of a pair share a transform, so each is scaled by a power of
+// two to about unit 2-norm first (exact, undone on the results: the error of
+// either stays relative to its own norm, and a trace of zeros stays zeros).
+// From every thread's squared norms s1, s2 over values of its pair (n1, n2: any
+// of them not zero): the scales up[], down[] per trace of the CTA.  Lanes `b` apart
+// share a pair (warp: one pair per warp).  Returns whether a trace cannot be
+// scaled (Inf, NaN, or a squared norm outside 1e-30 .. 1e30): then the traces are
+// transformed one at a time.
+__device__ __forceinline__ bool pair_scales(float s1, float s2, bool n1, bool n2, int pair, int apart_by, int B,
+                                            float* up, float* down) {
+    __shared__ float red[FFT_T / 32][16], nzr[FFT_T / 32][16];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane < 16) red[w][lane] = nzr[w][lane] = 0.f;
+    __syncwarp();
+    float z1 = n1 ? 1.f : 0.f, z2 = n2 ? 1.f : 0.f;
+    for (int o = 16; o >= apart_by; o >>= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        z1 += __shfl_xor_sync(0xffffffffu, z1, o);
+        z2 += __shfl_xor_sync(0xffffffffu, z2, o);
+    }
+    if (lane < apart_by) {
+        red[w][2 * pair] = s1;
+        red[w][2 * pair + 1] = s2;
+        nzr[w][2 * pair] = z1;
+        nzr[w][2 * pair + 1] = z2;
+    }
+    __syncthreads();
+    bool odd = false;
+    if (threadIdx.x < 2 * B) {
+        float ss = 0.f, nz = 0.f;
+        for (int i = 0; i < FFT_T / 32; ++i) {
+            ss += red[i][threadIdx.x];
+            nz += nzr[i][threadIdx.x];
+        }
+        odd = nz != 0.f && !(ss > 1e-30f && ss < 1e30f);
+        const int e = nz != 0.f && !odd ? ilogbf(ss) / 2 : 0;
+        up[threadIdx.x] = ldexpf(1.f, -e);
+        down[threadIdx.x] = nz != 0.f ? ldexpf(1.f, e) : 0.f;
+    }
+    return __syncthreads_or(odd) != 0;
+}
+
+// stack[f][tr] = the bins f0 .. f0 + nf - 1 of the traces; a CTA takes P.B pairs
+__global__ void __launch_bounds__(FFT_T, 3) k_fft_forward(const __grid_constant__ FftPlan P, const float* __restrict__ x,
+                                                          long long ntr, int f0, int nf, const cf* __restrict__ tab,
+                                                          cf* __restrict__ out) {
+    extern __shared__ __align__(16) cf sm[];
+    __shared__ float up[16], down[16];
+    const int n = P.n, ld = P.M + 1, B = P.B;   // odd row length: a bin's rows lie in different banks
+    const long long t0 = (long long)blockIdx.x * 2 * B;
+    cf* a = sm;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // a warp loads one pair (8 / B warps share it).  pass -1: both traces; 0, 1:
+    // the first, the second alone
+    const int pr = warp & (B - 1);
+    float s1 = 0.f, s2 = 0.f;
+    bool n1 = false, n2 = false;
+    auto load = [&](int pass) {
+        const long long tr = t0 + 2 * pr;
+        const bool in1 = tr < ntr && pass != 1, in2 = tr + 1 < ntr && pass != 0;
+        const float* xa = x + tr * n;
+        const float* xb = xa + n;
+#pragma unroll 4
+        for (int t = warp / B * 32 + lane; t < P.M; t += FFT_T / B) {
+            cf v = make_float2(in1 && t < n ? xa[t] : 0.f, in2 && t < n ? xb[t] : 0.f);
+            s1 = fmaf(v.x, v.x, s1);
+            s2 = fmaf(v.y, v.y, s2);
+            n1 = n1 || v.x != 0.f;
+            n2 = n2 || v.y != 0.f;
+            if (pass == 1) v = make_float2(v.y, 0.f);
+            a[pr * ld + t] = v;
+        }
+    };
+    load(-1);
+    const bool apart = pair_scales(s1, s2, n1, n2, pr, 1, B, up, down);
+    const bool vec = (ntr & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    for (int pass = apart ? 0 : -1; pass < (apart ? 2 : 0); ++pass) {
+        if (apart) {
+            load(pass);
+            __syncthreads();
+        }
+        if (P.chirp) {
+            for (int b = 0; b < B; ++b)
+                for (int t = threadIdx.x; t < n; t += FFT_T) {
+                    cf v = a[b * ld + t];
+                    if (!apart) v = make_float2(v.x * up[2 * b], v.y * up[2 * b + 1]);
+                    a[b * ld + t] = cmul(v, __ldg(tab + P.M + t));
+                }
+            __syncthreads();
+        }
+        const cf* z = fft_any(P, a, sm + B * ld, ld, tab, apart ? nullptr : up);
+        for (int e = threadIdx.x; e < nf * B; e += FFT_T) {
+            const int b = e & (B - 1), f = e / B;   // B is 8, 4 or 2
+            const int k = f0 + f, kc = k == 0 ? 0 : n - k;
+            const cf u = z[b * ld + k], v = z[b * ld + kc];
+            const long long tr = t0 + 2 * b, o = (long long)f * ntr + tr;
+            if (apart) {
+                if (tr + pass < ntr) out[o + pass] = u;
+                continue;
+            }
+            // z = x1 + i x2: X1 = (Z_k + conj Z_{n-k}) / 2, X2 = (Z_k - conj Z_{n-k}) / 2i
+            const float h1 = 0.5f * down[2 * b], h2 = 0.5f * down[2 * b + 1];
+            const cf p = make_float2(h1 * (u.x + v.x), h1 * (u.y - v.y));
+            const cf q = make_float2(h2 * (u.y + v.y), h2 * (v.x - u.x));
+            if (vec && tr < ntr) {
+                *reinterpret_cast<float4*>(out + o) = make_float4(p.x, p.y, q.x, q.y);
+            } else {
+                if (tr < ntr) out[o] = p;
+                if (tr + 1 < ntr) out[o + 1] = q;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// traces from the bins f0 .. f0 + nf - 1 (zero elsewhere, the imaginary parts of
+// bins 0 and n / 2 ignored), times 1 / n.  The band is read twice, once for the
+// norms (the second time from L2).
+__global__ void __launch_bounds__(FFT_T, 3) k_fft_inverse(const __grid_constant__ FftPlan P, const cf* __restrict__ in,
+                                                       long long ntr, int f0, int nf, const cf* __restrict__ tab,
+                                                       float* __restrict__ x) {
+    extern __shared__ __align__(16) cf sm[];
+    __shared__ float up[16], down[16];
+    const int n = P.n, ld = P.M + 1, B = P.B;
+    const long long t0 = (long long)blockIdx.x * 2 * B;
+    const int b = threadIdx.x & (B - 1), fs = FFT_T / B;   // a thread's pair and its step over bins
+    const long long tr = t0 + 2 * b;
+    const bool vec = (ntr & 1) == 0 && (reinterpret_cast<uintptr_t>(in) & 15) == 0;
+    auto bin = [&](int f, cf& p, cf& q) {
+        const long long o = (long long)f * ntr + tr;
+        p = q = make_float2(0.f, 0.f);
+        if (vec && tr < ntr) {
+            const float4 v = *reinterpret_cast<const float4*>(in + o);
+            p = make_float2(v.x, v.y);
+            q = make_float2(v.z, v.w);
+        } else {
+            if (tr < ntr) p = in[o];
+            if (tr + 1 < ntr) q = in[o + 1];
+        }
+        const int k = f0 + f;
+        if (k == 0 || 2 * k == n) p.y = q.y = 0.f;
+    };
+    bool apart;
+    {
+        float s1 = 0.f, s2 = 0.f;
+        bool n1 = false, n2 = false;
+#pragma unroll 4
+        for (int f = threadIdx.x / B; f < nf; f += fs) {
+            cf p, q;
+            bin(f, p, q);
+            s1 = fmaf(p.x, p.x, fmaf(p.y, p.y, s1));
+            s2 = fmaf(q.x, q.x, fmaf(q.y, q.y, s2));
+            n1 = n1 || p.x != 0.f || p.y != 0.f;
+            n2 = n2 || q.x != 0.f || q.y != 0.f;
+        }
+        apart = pair_scales(s1, s2, n1, n2, b, B, B, up, down);
+    }
+    const float s = 1.f / (float)n;
+    for (int pass = apart ? 0 : -1; pass < (apart ? 2 : 0); ++pass) {
+        for (int e = threadIdx.x; e < B * ld; e += FFT_T) sm[e] = make_float2(0.f, 0.f);
+        __syncthreads();
+        for (int f = threadIdx.x / B; f < nf; f += fs) {
+            cf p, q;
+            bin(f, p, q);
+            if (apart) {
+                if (pass == 1) p = q;
+                q = make_float2(0.f, 0.f);
+            } else {   // the spectra are scaled here: a bin mixes both traces
+                p = make_float2(p.x * up[2 * b], p.y * up[2 * b]);
+                q = make_float2(q.x * up[2 * b + 1], q.y * up[2 * b + 1]);
+            }
+            const int k = f0 + f;
+            // conj(Z_k) with Z = X1 + i X2, and conj(Z_{n-k}) from X_{n-k} = conj X_k
+            cf u = make_float2(p.x - q.y, -(p.y + q.x)), w = make_float2(p.x + q.y, p.y - q.x);
+            if (P.chirp) u = cmul(u, __ldg(tab + P.M + k));
+            sm[b * ld + k] = u;
+            if (k > 0 && 2 * k < n) {
+                if (P.chirp) w = cmul(w, __ldg(tab + P.M + n - k));
+                sm[b * ld + n - k] = w;
+            }
+        }
+        __syncthreads();
+        const cf* z = fft_any(P, sm, sm + B * ld, ld, tab, nullptr);
+        for (int r = 0; r < B; ++r) {
+            float* xa = x + (t0 + 2 * r) * n;
+            float* xb = xa + n;
+            const bool in1 = t0 + 2 * r < ntr, in2 = t0 + 2 * r + 1 < ntr;
+            for (int t = threadIdx.x; t < n; t += FFT_T) {
+                const cf v = z[r * ld + t];   // the conjugate of n (x1 + i x2)
+                if (apart) {
+                    if (pass ? in2 : in1) (pass ? xb : xa)[t] = v.x * s;
+                } else {
+                    if (in1) xa[t] = v.x * s * down[2 * r];
+                    if (in2) xb[t] = -v.y * s * down[2 * r + 1];
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// The plan of length n; false: not a length for these kernels.
+bool fft_plan(long long n, FftPlan& P) {
+    if (n < 1 || n > 4096) return false;
+    memset(&P, 0, sizeof(P));
+    P.n = (int)n;
+    auto factor = [&](int m) {
+        P.nfac = 0;
+        unsigned long long L = 1;
+        for (int f : {13, 11, 7, 5, 3, 4, 2})   // odd factors first: their strides meet no bank conflicts
+            while (m % f == 0) {
+                P.fac[P.nfac] = f;
+                P.magic[P.nfac++] = L == 1 ? 0u : (unsigned)(((1ull << 32) + L - 1) / L);
+                m /= f;
+                L *= f;
+            }
+        for (int f = 0; m == 1 && f < P.nfac; ++f) {
+            const unsigned long long k = L / P.fac[f];
+            P.magic_m[f] = k == 1 ? 0u : (unsigned)(((1ull << 32) + k - 1) / k);
+        }
+        return m == 1;
+    };
+    P.M = P.n;
+    if (!factor(P.n)) {
+        if (n > 2048) return false;
+        P.chirp = true;
+        P.M = 1;
+        while (P.M < 2 * P.n - 1) P.M *= 2;
+        factor(P.M);
+    }
+    // trace pairs per CTA: the most of 8, 4 that leave room for three CTAs per SM, else 2
+    P.B = 8;
+    while (P.B > 2 && 2 * P.B * (P.M + 1) * (int)sizeof(cf) > 74 * 1024) P.B /= 2;
+    return true;
+}
+
+// both directions in shared memory (see the top of this file)
+int fft_shared(const FftPlan& P, bool forward, const float* x_in, const cf* X_in, long long ntr, long long f0,
+               long long nf, cf* X_out, float* x_out, char* scratch, cudaStream_t st, std::string& err) {
+    cf* tab = reinterpret_cast<cf*>(scratch);
+    const int smem = 2 * P.B * (P.M + 1) * (int)sizeof(cf);
+    const int entries = P.M + (P.chirp ? P.n : 0);
+    const long long ctas = (ntr + 2 * P.B - 1) / (2 * P.B);
+    constexpr int most = 2 * 2 * 4097 * (int)sizeof(cf);
+    cudaError_t e = cudaFuncSetAttribute(forward ? (const void*)k_fft_forward : (const void*)k_fft_inverse,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_chirp, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) {
+        k_fft_tables<<<(entries + 63) / 64, 64, 0, st>>>(P, tab);
+        if (P.chirp) k_fft_chirp<<<1, FFT_T, 2 * (P.M + 1) * (int)sizeof(cf), st>>>(P, tab);
+        if (forward)
+            k_fft_forward<<<(unsigned)ctas, FFT_T, smem, st>>>(P, x_in, ntr, (int)f0, (int)nf, tab, X_out);
+        else
+            k_fft_inverse<<<(unsigned)ctas, FFT_T, smem, st>>>(P, X_in, ntr, (int)f0, (int)nf, tab, x_out);
+        counted(P.chirp ? 3 : 2);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        err = cudaGetErrorString(e);
+        return TLR_ERR_CUDA;
+    }
+    return TLR_OK;
+}
+
 const char* cufft_msg(cufftResult r) {
     switch (r) {
         case CUFFT_SUCCESS: return "success";
@@ -89,8 +572,16 @@ long long chunk_traces(long long ntr, long long nt) {
 
 }  // namespace
 
+size_t fft_scratch_bytes(long long nt) {
+    FftPlan P;
+    return fft_plan(nt, P) ? (size_t)(2 * P.M + P.n) * sizeof(cf) : 0;
+}
+
 int fft_stack(bool forward, const float* x_t_in, const cf* X_in, long long ntr, long long nt, long long f0,
-              long long nf, cf* X_out, float* x_t_out, cudaStream_t st, std::string& err) {
+              long long nf, cf* X_out, float* x_t_out, char* scratch, cudaStream_t st, std::string& err) {
+    FftPlan P;
+    if (scratch && fft_plan(nt, P) && ntr <= 0x7fffffffLL)
+        return fft_shared(P, forward, x_t_in, X_in, ntr, f0, nf, X_out, x_t_out, scratch, st, err);
     const long long nh = nt / 2 + 1;
     const long long C = chunk_traces(ntr, nt);
     cf* spec = nullptr;
