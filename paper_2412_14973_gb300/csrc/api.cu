@@ -1579,9 +1579,28 @@ static int forward(tlr_mdd_s* h, bool plain_apply) {
     if (h->n_tpack) CK(h, tpack(h->d_tpack, h->n_tpack, h->T, h->Tp, nullptr, (int)L.ns, h->st));
     CK(h, run_gemm(plain_apply ? h->Le_apply : h->Le_fwd, h->st));
     if (!plain_apply && h->rstep_on)
-        CK(h, rstep(h->R, h->A1, h->A2, nullptr, (int)L.nr, (int)L.ns, (int)L.b, h->d_rkn, h->d_rmk, nullptr, h->st,
+        CK(h, rstep(h->R, h->A1, h->A2, nullptr, (int)L.nr, (int)L.ns, (int)L.b, h->d_rkn, h->d_rmk, h->rpart, h->st,
                     L.b > 0 ? nullptr : h->d_roff, L.N, pack_fmt(h->d.precision)));
     return TLR_OK;
+}
+
+// partials of ||R||^2: the fused residual step leaves one per tile, the plain
+// passes red_blocks(nr ns) of them
+static const double* norm_parts(const tlr_mdd_s* h, long long* n) {
+    *n = h->rstep_on ? h->n_rpart : red_blocks((long long)h->L.nr * h->L.ns);
+    return h->rstep_on ? h->rpart : h->dpart + 14 * kRedBlocks;
+}
+// those of a fresh residual (forward() leaves them when the residual step is fused)
+static cudaError_t norm_pass(tlr_mdd_s* h, cudaStream_t st) {
+    if (h->rstep_on) return cudaSuccess;
+    return sv_norm_part(h->R, (long long)h->L.nr * h->L.ns, h->dpart + 14 * kRedBlocks, st);
+}
+static cudaError_t gradient_pair(tlr_mdd_s* h, const SolverDev& S, double rho, cudaStream_t st) {
+    const Layout& L = h->L;
+    long long nf;
+    const double* pf = norm_parts(h, &nf);
+    return sv_gradient_pair(S, h->part, h->nsplit, L.nlr, L.ndense, L.dmax, L.general, h->pm.zoff, h->pm.zdim, rho, pf, nf,
+                            st);
 }
 
 static int gradient(tlr_mdd_s* h) {
@@ -1615,8 +1634,10 @@ int tlr_mdd_grad(tlr_mdd_t* h, const void* theta, void* grad, double* f) {
     if (rc) return rc;
     CK(h, panel_to_theta(h->pm, h->gf, (cf*)grad, h->st));
     if (f) {
-        CK(h, sv_norm_part(h->R, (long long)L.nr * L.ns, h->dpart, h->st));
-        CK(h, finalize(h->dpart, kRedBlocks, 1, 1, h->scal + 1, h->st));
+        CK(h, norm_pass(h, h->st));
+        long long np;
+        const double* pf = norm_parts(h, &np);
+        CK(h, sum_partials(pf, np, 1.0, h->scal + 1, h->st));
         double rr = 0;
         int werr = 0;
         CK(h, cudaMemcpyAsync(&rr, h->scal + 1, sizeof(double), cudaMemcpyDeviceToHost, h->st));
@@ -2386,18 +2407,16 @@ static SolverDev solver_dev(tlr_mdd_s* h, int m) {
     S.sc = h->sc;
     S.ints = h->ints;
     S.fhist = h->fhist;
-    S.part = h->dpart;   // 2 slabs
+    S.part3 = h->dpart;
+    S.part6 = h->dpart + 3 * kRedBlocks;
+    S.partp = h->dpart + 9 * kRedBlocks;
     return S;
 }
 
 static int enqueue_solve(tlr_mdd_s* h, const tlr_mdd_solve_opts_t* o) {
     const Layout& L = h->L;
     const long long nrs = (long long)L.nr * L.ns;
-    SolverDev S = solver_dev(h, o->memory);
-    double* part6 = h->dpart + 2 * kRedBlocks;    // 6 slabs
-    double* part3 = h->dpart + 8 * kRedBlocks;    // 3 slabs
-    double* part3b = h->dpart + 11 * kRedBlocks;  // 3 slabs
-    double* partf = h->dpart + 14 * kRedBlocks;   // 1 slab
+    const SolverDev S = solver_dev(h, o->memory);
     const double rho = o->rho;
 
     CK(h, theta_to_panel(h->pm, h->th_io, h->x, h->st));
@@ -2407,8 +2426,10 @@ static int enqueue_solve(tlr_mdd_s* h, const tlr_mdd_solve_opts_t* o) {
         CK(h, sv_admm_init(S, h->st));
     int rc = forward(h, false);
     if (rc) return rc;
-    CK(h, sv_norm_part(h->R, nrs, partf, h->st));
-    CK(h, sv_record_f0(S, partf, h->st));
+    CK(h, norm_pass(h, h->st));
+    long long np;
+    const double* pf = norm_parts(h, &np);
+    CK(h, sv_record_f0(S, pf, np, h->st));
     rc = gradient(h);
     if (rc) return rc;
     int xu = 0;   // x-updates of this call
@@ -2429,35 +2450,26 @@ static int enqueue_solve(tlr_mdd_s* h, const tlr_mdd_solve_opts_t* o) {
                 CK(h, sym_dense(h->dd, L.nlr, L.ndense, L.dmax, h->Zsd, h->st, L.general, h->pm.zoff, h->pm.zdim));
                 CK(h, run_gemm(h->Le_a1, h->st));
                 CK(h, run_gemm(h->Le_a2, h->st));
-                if (h->rstep_on) {
-                    // the carried residual lives in its packed forms
-                    CK(h, dots6_packed(h->d_rkn, h->A1, h->A2, (int)L.nr, (int)L.ns, (int)L.b, part6, h->st,
-                                       L.b > 0 ? nullptr : h->d_roff, L.N, pack_fmt(h->d.precision)));
-                    CK(h, sv_dots3(S, part3, h->st));
-                    CK(h, sv_line_search(S, part6, kRedBlocks, part3, rho, h->st));
-                } else {
-                    CK(h, dots6_part(h->R, h->A1, h->A2, nrs, part6, h->st));
-                    CK(h, sv_dots3(S, part3, h->st));
-                    CK(h, sv_line_search(S, part6, kRedBlocks, part3, rho, h->st));
-                }
+                if (h->rstep_on)   // the carried residual lives in its packed forms
+                    CK(h, sv_line_search_packed(S, h->d_rkn, h->A1, h->A2, (int)L.nr, (int)L.ns, (int)L.b,
+                                                L.b > 0 ? nullptr : h->d_roff, L.N, pack_fmt(h->d.precision), rho,
+                                                h->st));
+                else
+                    CK(h, sv_line_search(S, h->R, h->A1, h->A2, nrs, rho, h->st));
                 if (h->rstep_on)
                     CK(h, rstep(h->R, h->A1, h->A2, h->sc + SC_ALPHA, (int)L.nr, (int)L.ns, (int)L.b, h->d_rkn,
                                 h->d_rmk, h->rpart, h->st, L.b > 0 ? nullptr : h->d_roff, L.N,
                                 pack_fmt(h->d.precision)));
                 else
-                    CK(h, sv_step_residual(h->R, h->A1, h->A2, nrs, h->sc + SC_ALPHA, partf, h->st));
+                    CK(h, sv_step_residual(h->R, h->A1, h->A2, nrs, h->sc + SC_ALPHA, h->dpart + 14 * kRedBlocks, h->st));
                 if (h->n_tpack)
                     CK(h, tpack(h->d_tpack, h->n_tpack, h->T, h->Tp, h->sc + SC_ALPHA, (int)L.ns, h->st));
                 else if (L.KtotB > 0)
                     CK(h, axpy_dev((float*)h->T, (const float*)h->Tp, 2LL * L.KtotB * L.ns, h->sc + SC_ALPHA, h->st));
                 CK(h, sv_step_theta(S, h->st));
-                rc = gradient(h);
-                if (rc) return rc;
-                CK(h, sv_pair_prep(S, rho, part3b, h->st));
-                if (h->rstep_on)
-                    CK(h, sv_pair_accept(S, part3b, h->rpart, (int)h->n_rpart, h->st));
-                else
-                    CK(h, sv_pair_accept(S, part3b, partf, kRedBlocks, h->st));
+                CK(h, run_gemm(h->Lc_v, h->st));
+                CK(h, run_gemm(h->Lp, h->st));
+                CK(h, gradient_pair(h, S, rho, h->st));
             }
             CK(h, sv_admm_zu(S, lam, rho, h->st));
         }
@@ -2798,16 +2810,19 @@ int b_forward(tlr_mdd_batch_s* b) {
         tlr_mdd_s* h = b->hs[m];
         const Layout& L = h->L;
         if (h->rstep_on)
-            BCK(rstep(h->R, h->A1, h->A2, nullptr, (int)L.nr, (int)L.ns, (int)L.b, h->d_rkn, h->d_rmk, nullptr,
+            BCK(rstep(h->R, h->A1, h->A2, nullptr, (int)L.nr, (int)L.ns, (int)L.b, h->d_rkn, h->d_rmk, h->rpart,
                       b->ms[m], L.b > 0 ? nullptr : h->d_roff, L.N, pack_fmt(h->d.precision)));
     }
     return TLR_OK;
 }
 
+int b_products(tlr_mdd_batch_s* b) {
+    const int rc = b_gemm(b, 2);    // Lc_v
+    return rc ? rc : b_gemm(b, 5);  // Lp
+}
+
 int b_gradient(tlr_mdd_batch_s* b) {
-    int rc = b_gemm(b, 2);   // Lc_v
-    if (rc) return rc;
-    rc = b_gemm(b, 5);       // Lp
+    const int rc = b_products(b);
     if (rc) return rc;
     for (size_t m = 0; m < b->hs.size(); ++m) {
         tlr_mdd_s* h = b->hs[m];
@@ -2824,7 +2839,6 @@ int b_enqueue(tlr_mdd_batch_s* b, const tlr_mdd_solve_opts_t* o) {
     const size_t n = b->hs.size();
     std::vector<SolverDev> S(n);
     for (size_t m = 0; m < n; ++m) S[m] = solver_dev(b->hs[m], o->memory);
-    auto part = [&](size_t m, int slab) { return b->hs[m]->dpart + (size_t)slab * kRedBlocks; };
     const double rho = o->rho;
     for (size_t m = 0; m < n; ++m) {
         tlr_mdd_s* h = b->hs[m];
@@ -2838,8 +2852,10 @@ int b_enqueue(tlr_mdd_batch_s* b, const tlr_mdd_solve_opts_t* o) {
     if (rc) return rc;
     for (size_t m = 0; m < n; ++m) {
         tlr_mdd_s* h = b->hs[m];
-        BCK(sv_norm_part(h->R, (long long)h->L.nr * h->L.ns, part(m, 14), b->ms[m]));
-        BCK(sv_record_f0(S[m], part(m, 14), b->ms[m]));
+        BCK(norm_pass(h, b->ms[m]));
+        long long np;
+        const double* pf = norm_parts(h, &np);
+        BCK(sv_record_f0(S[m], pf, np, b->ms[m]));
     }
     rc = b_gradient(b);
     if (rc) return rc;
@@ -2872,34 +2888,26 @@ int b_enqueue(tlr_mdd_batch_s* b, const tlr_mdd_solve_opts_t* o) {
                     const long long nrs = (long long)L.nr * L.ns;
                     cudaStream_t st = b->ms[m];
                     if (h->rstep_on)
-                        BCK(dots6_packed(h->d_rkn, h->A1, h->A2, (int)L.nr, (int)L.ns, (int)L.b, part(m, 2), st,
-                                         L.b > 0 ? nullptr : h->d_roff, L.N, pack_fmt(h->d.precision)));
+                        BCK(sv_line_search_packed(S[m], h->d_rkn, h->A1, h->A2, (int)L.nr, (int)L.ns, (int)L.b,
+                                                  L.b > 0 ? nullptr : h->d_roff, L.N, pack_fmt(h->d.precision), rho,
+                                                  st));
                     else
-                        BCK(dots6_part(h->R, h->A1, h->A2, nrs, part(m, 2), st));
-                    BCK(sv_dots3(S[m], part(m, 8), st));
-                    BCK(sv_line_search(S[m], part(m, 2), kRedBlocks, part(m, 8), rho, st));
+                        BCK(sv_line_search(S[m], h->R, h->A1, h->A2, nrs, rho, st));
                     if (h->rstep_on)
                         BCK(rstep(h->R, h->A1, h->A2, h->sc + SC_ALPHA, (int)L.nr, (int)L.ns, (int)L.b, h->d_rkn,
                                   h->d_rmk, h->rpart, st, L.b > 0 ? nullptr : h->d_roff, L.N,
                                   pack_fmt(h->d.precision)));
                     else
-                        BCK(sv_step_residual(h->R, h->A1, h->A2, nrs, h->sc + SC_ALPHA, part(m, 14), st));
+                        BCK(sv_step_residual(h->R, h->A1, h->A2, nrs, h->sc + SC_ALPHA, h->dpart + 14 * kRedBlocks, st));
                     if (h->n_tpack)
                         BCK(tpack(h->d_tpack, h->n_tpack, h->T, h->Tp, h->sc + SC_ALPHA, (int)L.ns, st));
                     else if (L.KtotB > 0)
                         BCK(axpy_dev((float*)h->T, (const float*)h->Tp, 2LL * L.KtotB * L.ns, h->sc + SC_ALPHA, st));
                     BCK(sv_step_theta(S[m], st));
                 }
-                rc = b_gradient(b);
+                rc = b_products(b);
                 if (rc) return rc;
-                for (size_t m = 0; m < n; ++m) {
-                    tlr_mdd_s* h = b->hs[m];
-                    BCK(sv_pair_prep(S[m], rho, part(m, 11), b->ms[m]));
-                    if (h->rstep_on)
-                        BCK(sv_pair_accept(S[m], part(m, 11), h->rpart, (int)h->n_rpart, b->ms[m]));
-                    else
-                        BCK(sv_pair_accept(S[m], part(m, 11), part(m, 14), kRedBlocks, b->ms[m]));
-                }
+                for (size_t m = 0; m < n; ++m) BCK(gradient_pair(b->hs[m], S[m], rho, b->ms[m]));
             }
             for (size_t m = 0; m < n; ++m) BCK(sv_admm_zu(S[m], lam, rho, b->ms[m]));
         }

@@ -113,7 +113,7 @@ constexpr int kPackTRA = 128, kPackTRB = 128;
 // 128 columns keep their shared memory at 16.5 KB, so one of their CTAs fits
 // beside the two GEMM CTAs an SM holds (2 x 97 KB) and they overlap
 // contractions of other streams; the tiles of rstep need 16 | d_i for every tile
-constexpr int kFuseRows = 16;
+constexpr int kFuseRows = 16, kFuseCols = 128;
 struct PTerm {
     const void* A;   // packed A of this problem (TR = kPackTRA), all row blocks
     const void* B;   // packed B of this problem (TR = kPackTRB)
@@ -195,11 +195,6 @@ cudaError_t tpack(const TPackTile* d_tiles, int ntiles, cf* T, const cf* Tp, con
 // [nblk + 1]); every block size a multiple of kFuseRows.  rstep_ctas gives the
 // number of tiles (and partials).
 long long rstep_ctas(int nr, int ns);
-// The six line-search inner products with R read from its KN packing (kn[i],
-// as rstep writes it), over rstep's tiles: part[blk * 6 + k], kRedBlocks
-// partials (a fixed grid, so the sums are reproducible).
-cudaError_t dots6_packed(char* const* kn, const cf* A1, const cf* A2, int nr, int ns, int b, double* part,
-                         cudaStream_t st, const long long* roff, int nblk, int fmt);
 cudaError_t rstep(cf* R, const cf* A1, const cf* A2, const double* alpha, int nr, int ns, int b, char* const* kn,
                   char* const* mk, double* part, cudaStream_t st, const long long* roff, int nblk, int fmt);
 // Benchmark solver of eq. (4) (k_cg.cu): the symmetrising pass
@@ -341,16 +336,9 @@ cudaError_t reduce_grad(const cf* part, int nsplit, long long stride, long long 
                         long long b, cf* grad, cudaStream_t st, int general = 0, const long long* zoff = nullptr,
                         const int* zdim = nullptr);
 
-// partial FP64 real dot sums over float arrays (2 per complex) -> part[kRedBlocks]
-cudaError_t dot_part(const float* a, const float* b, long long n2, double* part, cudaStream_t st);
-// out[k] = sum_{blk} part[blk * stride + k], k < cnt, one block, fixed order
-cudaError_t finalize(const double* part, int nblk, int stride, int cnt, double* out, cudaStream_t st);
-// six partials of the line-search inner products over Rf, A1, A2 (n complex)
-cudaError_t dots6_part(const cf* R, const cf* A1, const cf* A2, long long n, double* part, cudaStream_t st);
-// elementwise step: R += a A1 + a^2 A2 (n complex); alpha read from device
-cudaError_t step_residual(cf* R, const cf* A1, const cf* A2, long long n, const double* alpha, cudaStream_t st);
+// *out = scale * sum of part[0 .. n), one block, fixed order
+cudaError_t sum_partials(const double* part, long long n, double scale, double* out, cudaStream_t st);
 // x += a * y over n2 floats, a = alpha[0] (device)
 cudaError_t axpy_dev(float* x, const float* y, long long n2, const double* alpha, cudaStream_t st);
-
 
 }  // namespace tlr

@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256) k_pack(const PackJob* __restrict__ jobs) 
 // CTAs as registers allow.  Padding of the packed buffers (k >= K_i, rows >=
 // ns) is zero from the buffer's creation; whole padding groups are never
 // written, and the padding inside a written group is written as zeros.
-constexpr int TP_K = kFuseRows, TP_N = 128;
+constexpr int TP_K = kFuseRows, TP_N = kFuseCols;
 static_assert(kPackTRB == 128 && KC == 16 && TP_K == 16,
               "the passes take 16-deep, 128-row packed tiles with two k-groups of 8");
 
@@ -316,35 +316,6 @@ __global__ void __launch_bounds__(256) k_tpack(const TPackTile* __restrict__ til
 // receiver row to the MK packing (rows = receivers, k = n).  No shared
 // memory besides the block sum.
 
-// Block of the 16-row residual tile starting at row r0: r0 / b for equal
-// tiles, else the largest i with roff[i] <= r0 (every roff[i] is a multiple
-// of TP_K, so the tile lies in it); rl0 = its first row in the block, bK =
-// the block's size.
-struct RTile {
-    int blk, rl0, bK;
-};
-__device__ __forceinline__ RTile rtile(int r0, int b, const long long* roff, int nblk) {
-    RTile t;
-    if (roff) {
-        int lo = 0, hi = nblk - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (roff[mid] <= r0)
-                lo = mid;
-            else
-                hi = mid - 1;
-        }
-        t.blk = lo;
-        t.rl0 = r0 - (int)roff[lo];
-        t.bK = (int)(roff[lo + 1] - roff[lo]);
-    } else {
-        t.blk = r0 / b;
-        t.rl0 = r0 - t.blk * b;
-        t.bK = b;
-    }
-    return t;
-}
-
 __global__ void __launch_bounds__(256) k_rstep(cf* __restrict__ R, const cf* __restrict__ A1,
                                                const cf* __restrict__ A2, const double* __restrict__ alpha, int ns,
                                                int b, char* const* __restrict__ kn, char* const* __restrict__ mk,
@@ -413,56 +384,6 @@ __global__ void __launch_bounds__(256) k_rstep(cf* __restrict__ R, const cf* __r
             char* dst = mk[blk] + ((long long)(rl >> 7) * nkcN + (nb >> 4)) * 4 * plane + row_off(fmt, rl & 127);
             pk_store8(dst, fmt, (nb >> 3) & 1, r, 1.f);
         }
-    }
-}
-
-// The six line-search inner products Re<R,R>, Re<R,A1>, Re<R,A2>, Re<A1,A1>,
-// Re<A1,A2>, Re<A2,A2> over rstep's 16-row x 128-column tiles, with R read
-// from its KN packing (the form it is carried in between forward products)
-// and A1, A2 in FP32; products of four elements summed in FP32 before each
-// compensated add.  A fixed grid walks the tiles in a fixed order and leaves
-// one partial per dot and CTA (few partials for the one-block finaliser).
-__global__ void __maxnreg__(48) k_dots6p(char* const* __restrict__ kn, const cf* __restrict__ A1,
-                                                const cf* __restrict__ A2, int ns, int nr, int b,
-                                                const long long* __restrict__ roff, int nblk,
-                                                double* __restrict__ part, int fmt) {
-    __shared__ double sh[32];
-    constexpr int plane = 128 * 16 * 2;
-    const int gx = (ns + TP_N - 1) / TP_N;
-    const long long ntiles = (long long)gx * (nr / TP_K);
-    const int n = threadIdx.x & (TP_N - 1), kg = threadIdx.x >> 7;
-    Acc acc[6];
-    for (long long tt = blockIdx.x; tt < ntiles; tt += gridDim.x) {
-        const int n0 = (int)(tt % gx) * TP_N, r0 = (int)(tt / gx) * TP_K;
-        if (n0 + n >= ns) continue;
-        const RTile tl = rtile(r0, b, roff, nblk);
-        float2 v[8];
-        pk_load8(kn[tl.blk] + ((long long)(n0 >> 7) * (tl.bK >> 4) + (tl.rl0 >> 4)) * 4 * plane + row_off(fmt, n), fmt,
-                 kg, v);
-        float g[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const long long o = (long long)(r0 + kg * 8 + j) * ns + n0 + n;
-            const float2 r = v[j], x = A1[o], c = A2[o];
-            g[0] += fmaf(r.x, r.x, r.y * r.y);
-            g[1] += fmaf(r.x, x.x, r.y * x.y);
-            g[2] += fmaf(r.x, c.x, r.y * c.y);
-            g[3] += fmaf(x.x, x.x, x.y * x.y);
-            g[4] += fmaf(x.x, c.x, x.y * c.y);
-            g[5] += fmaf(c.x, c.x, c.y * c.y);
-            if ((j & 3) == 3) {
-#pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    acc[k].add(g[k]);
-                    g[k] = 0.f;
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const double t = block_sum(acc[k].val(), sh);
-        if (threadIdx.x == 0) part[(long long)blockIdx.x * 6 + k] = t;
     }
 }
 
@@ -1112,18 +1033,6 @@ cudaError_t rstep(cf* R, const cf* A1, const cf* A2, const double* alpha, int nr
     const long long nt = (long long)gx * (nr / TP_K);
     const cudaError_t e = launch_pass(k_rstep, dim3((unsigned)pass_grid(nt)), dim3(256), st, R, A1, A2, alpha, ns, b, kn,
                                       mk, part, roff, nblk, fmt, gx, nt);
-    counted(1);
-    return e;
-}
-
-cudaError_t dots6_packed(char* const* kn, const cf* A1, const cf* A2, int nr, int ns, int b, double* part,
-                         cudaStream_t st, const long long* roff, int nblk, int fmt) {
-    if (nr == 0 || ns == 0) return cudaSuccess;
-    if (nr % TP_K != 0) return cudaErrorInvalidValue;
-    if (!roff && (b <= 0 || b % TP_K != 0 || nr % b != 0)) return cudaErrorInvalidValue;
-    if (roff && nblk <= 0) return cudaErrorInvalidValue;
-    const cudaError_t e = launch_pass(k_dots6p, dim3(kRedBlocks), dim3(256), st, kn, A1, A2, ns, nr, b, roff, nblk,
-                                      part, fmt);
     counted(1);
     return e;
 }

@@ -4,28 +4,61 @@
 // the exact line search on the quartic phi(alpha), and the L-BFGS direction
 // (compact form) / ADMM updates (eq. 19-24) with every scalar kept on the device.
 //
-// All reductions run on a fixed grid (kRedBlocks x kRedThreads) and sum their
-// per-block partials in a fixed order, so results are bitwise reproducible.
+// All reductions run on a grid that depends on the length alone (red_blocks) and
+// sum their per-block partials in a fixed order, so results are bitwise
+// reproducible.  An iteration of a small solve is a chain of launches, so the
+// passes are few and finish their own sums: the last block to arrive adds the
+// partials up and makes the scalar decision (direction coefficients, step length,
+// pair acceptance), where each was a launch of its own with one block.
+#include <algorithm>
+
 #include "internal.h"
-#include "solver_dev.h"
+#include "pack.h"
 #include "reduce.h"
+#include "solver_dev.h"
 
 namespace tlr {
 
 // ---------------------------------------------------------------------------
 // helpers
 // ---------------------------------------------------------------------------
-// Sum of part[i * stride + k] over i < nblk by warp 0 in a fixed order; every
-// block that calls this obtains the same value.  Result broadcast via shared.
-__device__ __forceinline__ double sum_partials(const double* part, int nblk, int stride, int k, double* sh1) {
-    if (threadIdx.x < 32) {
-        double v = 0.0;
-        for (int i = threadIdx.x; i < nblk; i += 32) v += part[(long long)i * stride + k];
-        v = warp_sum(v);
-        if (threadIdx.x == 0) sh1[0] = v;
+// Sum of n partials by a block of 256 threads in a fixed order, in every thread;
+// four independent sums per thread keep the loads in flight.
+__device__ __forceinline__ double sum_part(const double* part, long long n, double (*sh)[256]) {
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    long long i = threadIdx.x;
+    for (; i + 768 < n; i += 1024) {
+        a0 += part[i];
+        a1 += part[i + 256];
+        a2 += part[i + 512];
+        a3 += part[i + 768];
+    }
+    for (; i < n; i += 256) a0 += part[i];
+    const double v[1] = {(a0 + a1) + (a2 + a3)};
+    (void)block_sums(v, sh);
+    const double r = sh[0][0];
+    __syncthreads();
+    return r;
+}
+
+// Sums of K interleaved partial slabs (part[i K + k], i < n) by a block of 256
+// threads: one warp per sum, lanes over i.  Thread k < K returns sum k.
+template <int K>
+__device__ __forceinline__ double sum_slabs(const double* part, int n, double* sh) {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (w < K) {
+        double a0 = 0.0, a1 = 0.0;
+        int i = l;
+        for (; i + 32 < n; i += 64) {
+            a0 += part[i * K + w];
+            a1 += part[(i + 32) * K + w];
+        }
+        if (i < n) a0 += part[i * K + w];
+        const double r = warp_sum(a0 + a1);
+        if (l == 0) sh[w] = r;
     }
     __syncthreads();
-    const double r = sh1[0];
+    const double r = threadIdx.x < K ? sh[threadIdx.x] : 0.0;
     __syncthreads();
     return r;
 }
@@ -113,37 +146,46 @@ cudaError_t sym_dense(const cf* pan, long long zbase, long long ndense, long lon
     return cudaGetLastError();
 }
 
-// grad = sum of split-K partials (FP64, fixed order); dense tiles: (G + G^T)/2
-// (reciprocal form) or G^T (general form)
+// one gradient entry: its split-K partials (compensated, fixed order) ...
+__device__ __forceinline__ cf split_sum(const cf* __restrict__ part, int nsplit, long long stride, long long e) {
+    Acc x, y;
+#pragma unroll 4
+    for (int c = 0; c < nsplit; ++c) {
+        const cf v = part[c * stride + e];
+        x.add(v.x);
+        y.add(v.y);
+    }
+    return make_float2((float)x.val(), (float)y.val());
+}
+// ... of a dense tile: (G + G^T)/2 (reciprocal form) or G^T (general form); e1 the
+// entry, e2 its mirror
+__device__ __forceinline__ cf split_sum_dense(const cf* __restrict__ part, int nsplit, long long stride, long long e1,
+                                              long long e2, int general) {
+    Acc x, y;
+    for (int c = 0; c < nsplit; ++c) {
+        const cf v = part[c * stride + e2];
+        if (!general) {
+            const cf u = part[c * stride + e1];
+            x.add(u.x);
+            y.add(u.y);
+        }
+        x.add(v.x);
+        y.add(v.y);
+    }
+    const double s = general ? 1.0 : 0.5;
+    return make_float2((float)(s * x.val()), (float)(s * y.val()));
+}
+
+// grad = sum of split-K partials
 __global__ void k_reduce_grad(const cf* __restrict__ part, int nsplit, long long stride, long long nlr,
                               long long ndense, long long b, cf* __restrict__ grad, int general,
                               const long long* __restrict__ zoff, const int* __restrict__ zdim) {
-    GRID_STRIDE(e, nlr) {
-        Acc x, y;
-        for (int c = 0; c < nsplit; ++c) {
-            const cf v = part[c * stride + e];
-            x.add(v.x);
-            y.add(v.y);
-        }
-        grad[e] = make_float2((float)x.val(), (float)y.val());
-    }
+    GRID_STRIDE(e, nlr) grad[e] = split_sum(part, nsplit, stride, e);
     GRID_STRIDE(e, ndense * b * b) {
         long long base, n, r, q;
         if (!dense_tile(e, b, zoff, zdim, base, n, r, q)) continue;
         const long long e1 = nlr + base + r * n + q, e2 = nlr + base + q * n + r;
-        Acc x, y;
-        for (int c = 0; c < nsplit; ++c) {
-            const cf v = part[c * stride + e2];
-            if (!general) {
-                const cf u = part[c * stride + e1];
-                x.add(u.x);
-                y.add(u.y);
-            }
-            x.add(v.x);
-            y.add(v.y);
-        }
-        const double s = general ? 1.0 : 0.5;
-        grad[e1] = make_float2((float)(s * x.val()), (float)(s * y.val()));
+        grad[e1] = split_sum_dense(part, nsplit, stride, e1, e2, general);
     }
 }
 
@@ -159,38 +201,19 @@ cudaError_t reduce_grad(const cf* part, int nsplit, long long stride, long long 
 // ---------------------------------------------------------------------------
 // FP64 inner products
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kRedThreads) k_dot_part(const float* __restrict__ a, const float* __restrict__ b,
-                                                         long long n2, double* part) {
-    __shared__ double sh[32];
-    Acc s;
-    GRID_STRIDE(i, n2) s.add(a[i] * b[i]);
-    const double r = block_sum(s.val(), sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = r;
+__global__ void __launch_bounds__(256) k_sum_partials(const double* part, long long n, double scale, double* out) {
+    __shared__ double sh[1][256];
+    const double v = sum_part(part, n, sh);
+    if (threadIdx.x == 0) out[0] = scale * v;
 }
 
-cudaError_t dot_part(const float* a, const float* b, long long n2, double* part, cudaStream_t st) {
-    (void)launch_pass(k_dot_part, dim3(kRedBlocks), dim3(kRedThreads), st, a, b, n2, part);
+cudaError_t sum_partials(const double* part, long long n, double scale, double* out, cudaStream_t st) {
+    (void)launch_pass(k_sum_partials, dim3(1), dim3(256), st, part, n, scale, out);
     counted(1);
     return cudaGetLastError();
 }
 
-__global__ void k_finalize(const double* part, int nblk, int stride, int cnt, double* out) {
-    __shared__ double sh1[1];
-    for (int k = 0; k < cnt; ++k) {
-        const double v = sum_partials(part, nblk, stride, k, sh1);
-        if (threadIdx.x == 0) out[k] = v;
-    }
-}
-
-cudaError_t finalize(const double* part, int nblk, int stride, int cnt, double* out, cudaStream_t st) {
-    (void)launch_pass(k_finalize, dim3(1), dim3(32), st, part, nblk, stride, cnt, out);
-    counted(1);
-    return cudaGetLastError();
-}
-
-// Re<R,R>, Re<R,A1>, Re<R,A2>, Re<A1,A1>, Re<A1,A2>, Re<A2,A2>  -> part[blk*6 + k]
-// (two complex values per 16-byte load when n is even; the buffers start
-// 256-byte aligned)
+// Re<R,R>, Re<R,A1>, Re<R,A2>, Re<A1,A1>, Re<A1,A2>, Re<A2,A2>
 __device__ __forceinline__ void dots6_add(Acc* s, float rx, float ry, float ax, float ay, float cx, float cy) {
     s[0].add(fmaf(rx, rx, ry * ry));
     s[1].add(fmaf(rx, ax, ry * ay));
@@ -212,9 +235,480 @@ __device__ __forceinline__ void dots6_group(float* t, float rx, float ry, float 
     t[5] += fmaf(cx, cx, cy * cy);
 }
 
-__global__ void __launch_bounds__(kRedThreads) k_dots6(const cf* __restrict__ R, const cf* __restrict__ A1,
-                                                      const cf* __restrict__ A2, long long n, double* part) {
-    __shared__ double sh[32];
+// R += a A1 + a^2 A2 ; partial of ||R_new||^2 -> part[blk]
+__global__ void __launch_bounds__(kRedThreads) k_step_residual(cf* __restrict__ R, const cf* __restrict__ A1,
+                                                              const cf* __restrict__ A2, long long n,
+                                                              const double* __restrict__ alpha, double* part) {
+    __shared__ double sh[1][256];
+    const float a = (float)alpha[0];
+    const float a2 = (float)(alpha[0] * alpha[0]);
+    Acc s;
+    GRID_STRIDE(i, n) {
+        cf r = R[i];
+        if (a != 0.f) {
+            const cf u = A1[i], w = A2[i];
+            r.x = fmaf(a2, w.x, fmaf(a, u.x, r.x));
+            r.y = fmaf(a2, w.y, fmaf(a, u.y, r.y));
+            R[i] = r;
+        }
+        s.add(fmaf(r.x, r.x, r.y * r.y));
+    }
+    const double v[1] = {s.val()};
+    const double t = block_sums(v, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = t;
+}
+
+__global__ void k_axpy_dev(float* __restrict__ x, const float* __restrict__ y, long long n2,
+                           const double* __restrict__ alpha) {
+    const float a = (float)alpha[0];
+    if (a == 0.f) return;
+    GRID_STRIDE(i, n2) x[i] = fmaf(a, y[i], x[i]);
+}
+
+cudaError_t axpy_dev(float* x, const float* y, long long n2, const double* alpha, cudaStream_t st) {
+    (void)launch_pass(k_axpy_dev, dim3(1024), dim3(256), st, x, y, n2, alpha);
+    counted(1);
+    return cudaGetLastError();
+}
+
+// ===========================================================================
+// Solver kernels (L-BFGS two-loop recursion, exact line search, ADMM).
+// ===========================================================================
+
+// partials of ||R||^2
+__global__ void __launch_bounds__(kRedThreads) k_norm_part(const cf* __restrict__ R, long long n, double* part) {
+    __shared__ double sh[1][256];
+    Acc s;
+    GRID_STRIDE(i, n) {
+        const cf r = R[i];
+        s.add(fmaf(r.x, r.x, r.y * r.y));
+    }
+    const double v[1] = {s.val()};
+    const double t = block_sums(v, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = t;
+}
+
+// g = gf + rho (x - v); history cleared (start of an x-update)
+__global__ void k_xupdate_start(SolverDev S, double rho) {
+    const float r = (float)rho;
+    GRID_STRIDE(i, S.n2) S.g[i] = S.gf[i] + r * (S.x[i] - S.v[i]);
+    if (blockIdx.x == 0 && threadIdx.x == 0) S.ints[SI_CNT] = 0;
+}
+
+__device__ __forceinline__ int ring_idx(const SolverDev& S, int j) {
+    // j-th newest pair (0 = newest)
+    const int R = S.ring;
+    return ((S.ints[SI_NEWEST] - j) % R + R) % R;
+}
+
+// L-BFGS direction d = -H g in the compact form of the inverse BFGS update
+// (Byrd, Nocedal and Schnabel 1994): with the k stored pairs ordered oldest
+// first, S = [s_1 .. s_k], Y = [y_1 .. y_k], R = triu(S^T Y), D = diag(S^T Y),
+// H0 = gamma I and gamma = <s,y>/<y,y> of the newest pair,
+//   H g = gamma g + S a - gamma Y u,  u = R^-1 S^T g,
+//   a = R^-T ((D + gamma Y^T Y) u - gamma Y^T g).
+// This is the matrix the two-loop recursion applies, evaluated in three
+// steps: the inner products (passes over groups of pairs; they also fill the
+// newest pair's row and column of S^T Y and Y^T Y, which are kept by slot),
+// the small FP64 triangular solves in one block, and one combination pass.
+
+// partials per block: for pair j of the group, <s_j,g>, <y_j,g>, <s_j,y_n>,
+// <s_n,y_j>, <y_j,y_n> (n = the newest pair).  Per-thread sums are plain FP32
+// multiply-adds (a thread sums a few dozen terms at these sizes), combined in FP64
+// across threads and blocks: these products only set the direction's coefficients,
+// whose rounding the exact line search and the descent test absorb.
+// 128 threads of <= 128 registers: a CTA fits beside the two GEMM CTAs of an SM
+constexpr int kLbThreads = 128;
+constexpr int kLbVals = 5 * kLbGroup + 1;
+constexpr int kLbLd = kLbThreads + 8;   // row length of the block's sums: 4 rows read together lie in different banks
+
+__device__ void lb_solve(const SolverDev& S, int cnt, int nblk, double* val, double* mat);
+
+// Blocks of the direction's inner products: 8 values of each vector per thread
+inline int lb_blocks(long long n2) {
+    const long long b = (n2 + 8 * kLbThreads - 1) / (8 * kLbThreads);
+    return (int)(b < 1 ? 1 : b > kRedBlocks ? kRedBlocks : b);
+}
+
+// last != 0: the launch over the last group of pairs, whose last block finishes
+// the direction's coefficients (lb_solve).  FP64 adds run at 2 lanes per cycle on
+// this part, so the block sums its 51 values 8 lanes each (72 cycles a value; a
+// shuffle tree per warp and value took 320).
+__global__ void __launch_bounds__(kLbThreads, 4) k_lb_dots(SolverDev S, int j0, int last) {
+    __shared__ __align__(16) float shv[kLbVals * kLbLd];
+    const int cnt = S.ints[SI_CNT];
+    if (j0 < cnt) {
+        const int jc = min(kLbGroup, cnt - j0);
+        const float* sp[kLbGroup];
+        const float* yp[kLbGroup];
+#pragma unroll
+        for (int jj = 0; jj < kLbGroup; ++jj) {
+            const int idx = ring_idx(S, jj < jc ? j0 + jj : j0);
+            sp[jj] = S.sh + (long long)idx * S.n2;
+            yp[jj] = S.yh + (long long)idx * S.n2;
+        }
+        const int nw = ring_idx(S, 0);
+        const float* sn = S.sh + (long long)nw * S.n2;
+        const float* yn = S.yh + (long long)nw * S.n2;
+        float acc[kLbGroup][5];
+#pragma unroll
+        for (int jj = 0; jj < kLbGroup; ++jj)
+#pragma unroll
+            for (int t = 0; t < 5; ++t) acc[jj][t] = 0.f;
+        float gg = 0.f;   // <g, g> for the descent test (first group only)
+        GRID_STRIDE(i, S.n2) {
+            const float gi = S.g[i], sni = sn[i], yni = yn[i];
+            gg = fmaf(gi, gi, gg);
+#pragma unroll
+            for (int jj = 0; jj < kLbGroup; ++jj) {
+                if (jj < jc) {
+                    const float s = sp[jj][i], y = yp[jj][i];
+                    acc[jj][0] = fmaf(s, gi, acc[jj][0]);
+                    acc[jj][1] = fmaf(y, gi, acc[jj][1]);
+                    acc[jj][2] = fmaf(s, yni, acc[jj][2]);
+                    acc[jj][3] = fmaf(sni, y, acc[jj][3]);
+                    acc[jj][4] = fmaf(y, yni, acc[jj][4]);
+                }
+            }
+        }
+#pragma unroll
+        for (int jj = 0; jj < kLbGroup; ++jj)
+#pragma unroll
+            for (int t = 0; t < 5; ++t) shv[(jj * 5 + t) * kLbLd + threadIdx.x] = acc[jj][t];
+        shv[5 * kLbGroup * kLbLd + threadIdx.x] = gg;
+        __syncthreads();
+        const int lane = threadIdx.x & 31, l8 = lane & 7;
+        for (int v0 = 0; v0 < kLbVals; v0 += kLbThreads / 8) {
+            const int v = v0 + (threadIdx.x >> 3);   // 8 lanes per value
+            const float* row = shv + min(v, kLbVals - 1) * kLbLd;
+            double r = 0.0;
+#pragma unroll
+            for (int i = 0; i < kLbThreads / 8; ++i) r += (double)row[l8 + 8 * i];
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o, 8);
+            if (l8 == 0) {
+                if (v < 5 * jc)
+                    S.lbpart[((long long)(j0 / kLbGroup) * 5 * kLbGroup + v) * kRedBlocks + blockIdx.x] = r;
+                else if (v == kLbVals - 1 && j0 == 0)
+                    S.lbpart[kLbGGOff + blockIdx.x] = r;
+            }
+        }
+    }
+    if (!last || !last_block(reinterpret_cast<unsigned*>(S.ints + CT_DIR), gridDim.x)) return;
+    double* const mat = reinterpret_cast<double*>(shv);   // 2 x 32 x 33 doubles and 161 values
+    lb_solve(S, cnt, gridDim.x, mat + 2 * 32 * 33, mat);
+}
+static_assert(sizeof(double) * (2 * 32 * 33 + 161) <= sizeof(float) * kLbVals * kLbLd, "lb_solve's storage");
+
+// One block: finalise the partials (a warp per two values, fixed order), update the
+// newest pair's row / column of S^T Y and Y^T Y, then (warp 0, a lane per
+// pair) the triangular solves; coefficients to acoef, gamma to sc[SC_GAMMA].
+__device__ void lb_solve(const SolverDev& S, int cnt, int nblk, double* val, double* mat) {
+    double* const Rm = mat;
+    double* const Ym = mat + 32 * 33;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (cnt == 0) {
+        // d = -g, a descent direction unless g = 0 (which the line search meets)
+        if (threadIdx.x == 0) {
+            S.ints[SI_RFLAG] = 0;
+            S.sc[SC_GAMMA] = 1.0;
+        }
+        return;
+    }
+    const int nval = 5 * cnt + 1;   // the last value is <g, g>
+    auto row = [&](int v) {
+        return v == 5 * cnt ? S.lbpart + kLbGGOff : S.lbpart + (long long)v * kRedBlocks;
+    };
+    for (int v = 2 * w; v < nval; v += 2 * (kLbThreads / 32)) {
+        const double* r0 = row(v);
+        const double* r1 = row(min(v + 1, nval - 1));
+        double a0 = 0.0, a1 = 0.0;
+#pragma unroll 5
+        for (int b = l; b < nblk; b += 32) {
+            a0 += r0[b];
+            a1 += r1[b];
+        }
+        a0 = warp_sum(a0);
+        a1 = warp_sum(a1);
+        if (l == 0) {
+            val[v] = a0;
+            if (v + 1 < nval) val[v + 1] = a1;
+        }
+    }
+    __syncthreads();
+    const int R = S.ring, k = cnt;
+    const int nw = ring_idx(S, 0);
+    if (threadIdx.x < cnt) {
+        const int j = threadIdx.x, a = ring_idx(S, j);
+        S.SYm[a * R + nw] = val[j * 5 + 2];
+        if (j > 0) S.SYm[nw * R + a] = val[j * 5 + 3];
+        S.YYm[a * R + nw] = val[j * 5 + 4];
+        S.YYm[nw * R + a] = val[j * 5 + 4];
+    }
+    __syncthreads();
+    // oldest first: position i holds the (cnt - 1 - i)-th newest pair
+    for (int e = threadIdx.x; e < k * k; e += kLbThreads) {
+        const int i = e / k, j = e - i * k;
+        const int si = ring_idx(S, k - 1 - i), sj = ring_idx(S, k - 1 - j);
+        Rm[i * 33 + j] = S.SYm[si * R + sj];
+        Ym[i * 33 + j] = S.YYm[si * R + sj];
+    }
+    __syncthreads();
+    if (w != 0) return;
+    // lane i holds position i
+    const bool on = l < k;
+    const double p = on ? val[(k - 1 - l) * 5] : 0.0, q = on ? val[(k - 1 - l) * 5 + 1] : 0.0;
+    const double dia = on ? Rm[l * 33 + l] : 1.0, inv = 1.0 / dia;
+    const double gamma = Rm[(k - 1) * 33 + (k - 1)] / Ym[(k - 1) * 33 + (k - 1)];
+    // u = R^-1 p (R upper triangular)
+    double u = p;
+    for (int i = k - 1; i >= 0; --i) {
+        const double ui = __shfl_sync(0xffffffffu, u * inv, i);
+        if (l == i) u = ui;
+        if (l < i) u -= Rm[l * 33 + i] * ui;
+    }
+    // t = D u + gamma Y^T Y u - gamma q
+    double t = dia * u - gamma * q;
+    for (int j = 0; j < k; ++j) {
+        const double uj = __shfl_sync(0xffffffffu, u, j);
+        if (on) t += gamma * Ym[l * 33 + j] * uj;
+    }
+    // a = R^-T t (R^T lower triangular)
+    for (int i = 0; i < k; ++i) {
+        const double ai = __shfl_sync(0xffffffffu, t * inv, i);
+        if (l == i) t = ai;
+        if (on && l > i) t -= Rm[i * 33 + l] * ai;
+    }
+    // descent test: <g, d> = -(gamma <g,g> + sum_i a_i <s_i,g> - gamma sum_i u_i <y_i,g>)
+    double gd = warp_sum(on ? t * p - gamma * u * q : 0.0);
+    gd = -(gamma * val[5 * k] + __shfl_sync(0xffffffffu, gd, 0));
+    if (!(gd < 0.0)) {
+        // not a descent direction: clear the memory and take d = -g in this
+        // same iteration (the restart of L-BFGS)
+        if (l == 0) {
+            S.ints[SI_CNT] = 0;
+            S.ints[SI_RESTARTS] += 1;
+            S.ints[SI_RFLAG] = 1;
+            S.sc[SC_GAMMA] = 1.0;
+        }
+        return;
+    }
+    if (on) {
+        S.acoef[k - 1 - l] = t;   // j-th newest
+        S.acoef[32 + k - 1 - l] = -gamma * u;
+    }
+    if (l == 0) {
+        S.ints[SI_RFLAG] = 0;
+        S.sc[SC_GAMMA] = gamma;
+    }
+}
+
+// d = -(gamma g + sum_j a_j s_j + sum_j c_j y_j), with the partials of the
+// theta-space line-search inner products <x - v, x - v>, <x - v, d>, <d, d> (blk *
+// 3 + k); four floats per thread and four pairs per step in flight (the vectors
+// start 16-byte aligned when n2 is a multiple of 4, else a scalar loop)
+__global__ void __launch_bounds__(kRedThreads) k_lb_dir(SolverDev S) {
+    __shared__ float cs[32], cy[32];
+    __shared__ const float* ps[32];
+    __shared__ const float* py[32];
+    __shared__ double sh[3][256];
+    const int cnt = S.ints[SI_CNT];
+    if (threadIdx.x < cnt) {
+        const int idx = ring_idx(S, threadIdx.x);
+        cs[threadIdx.x] = (float)S.acoef[threadIdx.x];
+        cy[threadIdx.x] = (float)S.acoef[32 + threadIdx.x];
+        ps[threadIdx.x] = S.sh + (long long)idx * S.n2;
+        py[threadIdx.x] = S.yh + (long long)idx * S.n2;
+    }
+    __syncthreads();
+    const float gamma = (float)S.sc[SC_GAMMA];
+    Acc s0, s1, s2;
+    auto dots = [&](float x, float v, float d) {
+        const float w = x - v;
+        s0.add(w * w);
+        s1.add(w * d);
+        s2.add(d * d);
+    };
+    if ((S.n2 & 3) == 0) {
+        const long long n4 = S.n2 >> 2;
+        const float4* g4 = reinterpret_cast<const float4*>(S.g);
+        float4* d4 = reinterpret_cast<float4*>(S.d);
+        GRID_STRIDE(i, n4) {
+            const float4 gv = g4[i];
+            const float4 xv = reinterpret_cast<const float4*>(S.x)[i], vv = reinterpret_cast<const float4*>(S.v)[i];
+            float4 r = make_float4(gamma * gv.x, gamma * gv.y, gamma * gv.z, gamma * gv.w);
+            int j = 0;
+            for (; j + 4 <= cnt; j += 4) {
+                float4 sv[4], yv[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    sv[u] = reinterpret_cast<const float4*>(ps[j + u])[i];
+                    yv[u] = reinterpret_cast<const float4*>(py[j + u])[i];
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float a = cs[j + u], c = cy[j + u];
+                    r.x = fmaf(c, yv[u].x, fmaf(a, sv[u].x, r.x));
+                    r.y = fmaf(c, yv[u].y, fmaf(a, sv[u].y, r.y));
+                    r.z = fmaf(c, yv[u].z, fmaf(a, sv[u].z, r.z));
+                    r.w = fmaf(c, yv[u].w, fmaf(a, sv[u].w, r.w));
+                }
+            }
+            for (; j < cnt; ++j) {
+                const float4 sv = reinterpret_cast<const float4*>(ps[j])[i];
+                const float4 yv = reinterpret_cast<const float4*>(py[j])[i];
+                const float a = cs[j], c = cy[j];
+                r.x = fmaf(c, yv.x, fmaf(a, sv.x, r.x));
+                r.y = fmaf(c, yv.y, fmaf(a, sv.y, r.y));
+                r.z = fmaf(c, yv.z, fmaf(a, sv.z, r.z));
+                r.w = fmaf(c, yv.w, fmaf(a, sv.w, r.w));
+            }
+            d4[i] = make_float4(-r.x, -r.y, -r.z, -r.w);
+            dots(xv.x, vv.x, -r.x);
+            dots(xv.y, vv.y, -r.y);
+            dots(xv.z, vv.z, -r.z);
+            dots(xv.w, vv.w, -r.w);
+        }
+    } else {
+        GRID_STRIDE(i, S.n2) {
+            float r = gamma * S.g[i];
+            for (int j = 0; j < cnt; ++j) r = fmaf(cy[j], py[j][i], fmaf(cs[j], ps[j][i], r));
+            S.d[i] = -r;
+            dots(S.x[i], S.v[i], -r);
+        }
+    }
+    const double v[3] = {s0.val(), s1.val(), s2.val()};
+    const double r = block_sums(v, sh);
+    if (threadIdx.x < 3) S.part3[blockIdx.x * 3 + threadIdx.x] = r;
+}
+
+__device__ double quartic_val(const double* c, double a) {
+    return c[0] + a * (c[1] + a * (c[2] + a * (c[3] + a * c[4])));
+}
+
+// a candidate root of phi', polished by two Newton steps: false if it is none
+__device__ __forceinline__ bool polish(const double* c, double& a) {
+    for (int it = 0; it < 2; ++it) {
+        const double d1 = c[1] + a * (2 * c[2] + a * (3 * c[3] + a * 4 * c[4]));
+        const double d2 = 2 * c[2] + a * (6 * c[3] + a * 12 * c[4]);
+        if (d2 != 0.0) a -= d1 / d2;
+    }
+    return a > 0.0 && isfinite(a);
+}
+
+// Minimiser over a > 0 of the quartic, by the lanes of a warp: real roots of
+// phi'(a) = 4 c4 a^3 + 3 c3 a^2 + 2 c2 a + c1 in closed form (depressed cubic:
+// trigonometric form for three real roots, Cardano otherwise), polished.  Lane k
+// takes the k-th root (the two cube roots of Cardano's form, the three cosines and
+// the polishing are long FP64 chains); ties go to the smaller root.
+__device__ __forceinline__ bool quartic_argmin(const double* c, int lane, double* out) {
+    const double A = 4 * c[4], B = 3 * c[3], C = 2 * c[2], D = c[1];
+    double a = 0.0;
+    bool have = false;
+    if (A != 0.0) {
+        const double p = B / A, q = C / A, r = D / A;
+        const double P = q - p * p / 3.0;
+        const double Q = 2.0 * p * p * p / 27.0 - p * q / 3.0 + r;
+        const double disc = 0.25 * Q * Q + P * P * P / 27.0;
+        const double sh = -p / 3.0;
+        if (disc > 0.0) {
+            const double sq = sqrt(disc);
+            const double t = cbrt(-0.5 * Q + (lane == 0 ? sq : -sq));
+            a = t + __shfl_sync(0xffffffffu, t, 1) + sh;   // lane 0
+            have = lane == 0;
+        } else if (P == 0.0) {
+            a = cbrt(-Q) + sh;
+            have = lane == 0;
+        } else {
+            const double m = 2.0 * sqrt(-P / 3.0);
+            double arg = 3.0 * Q / (P * m);
+            arg = fmin(1.0, fmax(-1.0, arg));
+            const double th = acos(arg) / 3.0;
+            const double tpi = 2.0943951023931954923;  // 2 pi / 3
+            a = m * cos(th - tpi * (lane < 3 ? lane : 0)) + sh;
+            have = lane < 3;
+        }
+    } else if (B != 0.0) {
+        const double dsc = C * C - 4 * B * D;
+        if (dsc >= 0.0) {
+            const double s = sqrt(dsc);
+            a = (-C + (lane == 0 ? s : -s)) / (2 * B);
+            have = lane < 2;
+        }
+    } else if (C != 0.0) {
+        a = -D / C;
+        have = lane == 0;
+    }
+    have = polish(c, a) && have;
+    const double v = quartic_val(c, a);
+    double best_a = 0.0, best_v = 0.0;
+    bool any = false;
+    for (int k = 0; k < 3; ++k) {
+        const bool hk = __shfl_sync(0xffffffffu, (int)have, k) != 0;
+        const double ak = __shfl_sync(0xffffffffu, a, k), vk = __shfl_sync(0xffffffffu, v, k);
+        if (hk && (!any || vk < best_v || (vk == best_v && ak < best_a))) {
+            any = true;
+            best_a = ak;
+            best_v = vk;
+        }
+    }
+    *out = best_a;
+    return any;
+}
+
+// The last block (256 threads) of a line-search pass: finalise the 6 + 3 inner
+// products, form phi's coefficients, check descent, pick alpha; alpha = 0 and a
+// memory reset when no step.
+__device__ __forceinline__ void line_search_last(const SolverDev& S, int nb6, int nb3, double rho, double (*sh)[256]) {
+    const double d6 = sum_slabs<6>(S.part6, nb6, sh[0]);
+    const double d3 = sum_slabs<3>(S.part3, nb3, sh[0]);
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    double e6[6], e3[3];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) e6[k] = __shfl_sync(0xffffffffu, d6, k);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) e3[k] = __shfl_sync(0xffffffffu, d3, k);
+    double c[5];
+    c[0] = 0.5 * e6[0] + 0.5 * rho * e3[0];
+    c[1] = e6[1] + rho * e3[1];
+    c[2] = 0.5 * e6[3] + e6[2] + 0.5 * rho * e3[2];
+    c[3] = e6[4];
+    c[4] = 0.5 * e6[5];
+    double a = 0.0;
+    bool ok = false;
+    if (c[1] < 0.0) ok = quartic_argmin(c, lane, &a);
+    if (lane != 0) return;
+    for (int k = 0; k < 5; ++k) S.sc[SC_C0 + k] = c[k];
+    if (!ok) {
+        // no minimiser on a > 0 along d: no step, memory cleared; counted as a
+        // restart unless the direction test already counted this iteration
+        a = 0.0;
+        S.ints[SI_CNT] = 0;
+        if (!S.ints[SI_RFLAG]) S.ints[SI_RESTARTS] += 1;
+    }
+    bool finite = isfinite(c[0]) && isfinite(c[1]) && isfinite(c[2]) && isfinite(c[3]) && isfinite(c[4]);
+    if (!finite) {
+        a = 0.0;
+        S.ints[SI_STATUS] = TLR_ERR_NONFINITE;
+    }
+    S.sc[SC_ALPHA] = a;
+}
+
+// the end of a line-search pass: the block's six sums, then the search by the last block
+__device__ __forceinline__ void dots6_end(const SolverDev& S, const Acc* s, int nb3, double rho, double (*sh)[256]) {
+    const double v[6] = {s[0].val(), s[1].val(), s[2].val(), s[3].val(), s[4].val(), s[5].val()};
+    const double r = block_sums(v, sh);
+    if (threadIdx.x < 6) S.part6[blockIdx.x * 6 + threadIdx.x] = r;
+    if (last_block(reinterpret_cast<unsigned*>(S.ints + CT_LINE), gridDim.x))
+        line_search_last(S, gridDim.x, nb3, rho, sh);
+}
+
+// the six products over FP32 arrays (two complex values per 16-byte load when n
+// is even; the buffers start 256-byte aligned)
+__global__ void __launch_bounds__(kRedThreads) k_dots6(SolverDev S, const cf* __restrict__ R, const cf* __restrict__ A1,
+                                                      const cf* __restrict__ A2, long long n, int nb3, double rho) {
+    __shared__ double sh[6][256];
     Acc s[6];
     if ((n & 1) == 0) {
         const float4* R4 = reinterpret_cast<const float4*>(R);
@@ -247,533 +741,133 @@ __global__ void __launch_bounds__(kRedThreads) k_dots6(const cf* __restrict__ R,
             dots6_add(s, r.x, r.y, a.x, a.y, c.x, c.y);
         }
     }
+    dots6_end(S, s, nb3, rho, sh);
+}
+
+// The same over rstep's 16-row x 128-column tiles, with R read from its KN packing
+// (the form it is carried in between forward products) and A1, A2 in FP32; products
+// of four elements summed in FP32 before each compensated add.  A grid fixed by the
+// number of tiles walks them in a fixed order and leaves one partial per product
+// and CTA.  Its 12 KB of shared memory and 48 registers fit beside two contraction
+// CTAs of another stream.
+__global__ void __maxnreg__(48) k_dots6p(SolverDev S, char* const* __restrict__ kn, const cf* __restrict__ A1,
+                                         const cf* __restrict__ A2, int ns, int nr, int b,
+                                         const long long* __restrict__ roff, int nblk, int fmt, int nb3, double rho) {
+    __shared__ double sh[6][256];
+    constexpr int plane = 128 * 16 * 2;
+    const int gx = (ns + kFuseCols - 1) / kFuseCols;
+    const long long ntiles = (long long)gx * (nr / kFuseRows);
+    const int n = threadIdx.x & (kFuseCols - 1), kg = threadIdx.x >> 7;
+    Acc acc[6];
+    for (long long tt = blockIdx.x; tt < ntiles; tt += gridDim.x) {
+        const int n0 = (int)(tt % gx) * kFuseCols, r0 = (int)(tt / gx) * kFuseRows;
+        if (n0 + n >= ns) continue;
+        const RTile tl = rtile(r0, b, roff, nblk);
+        float2 v[8];
+        pk_load8(kn[tl.blk] + ((long long)(n0 >> 7) * (tl.bK >> 4) + (tl.rl0 >> 4)) * 4 * plane + row_off(fmt, n), fmt,
+                 kg, v);
+        float g[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const double v = block_sum(s[k].val(), sh);
-        if (threadIdx.x == 0) part[blockIdx.x * 6 + k] = v;
-    }
-}
-
-cudaError_t dots6_part(const cf* R, const cf* A1, const cf* A2, long long n, double* part, cudaStream_t st) {
-    (void)launch_pass(k_dots6, dim3(kRedBlocks), dim3(kRedThreads), st, R, A1, A2, n, part);
-    counted(1);
-    return cudaGetLastError();
-}
-
-// R += a A1 + a^2 A2 ; partial of ||R_new||^2 -> part[blk]
-__global__ void __launch_bounds__(kRedThreads) k_step_residual(cf* __restrict__ R, const cf* __restrict__ A1,
-                                                              const cf* __restrict__ A2, long long n,
-                                                              const double* __restrict__ alpha, double* part) {
-    __shared__ double sh[32];
-    const float a = (float)alpha[0];
-    const float a2 = (float)(alpha[0] * alpha[0]);
-    Acc s;
-    GRID_STRIDE(i, n) {
-        cf r = R[i];
-        if (a != 0.f) {
-            const cf u = A1[i], w = A2[i];
-            r.x = fmaf(a2, w.x, fmaf(a, u.x, r.x));
-            r.y = fmaf(a2, w.y, fmaf(a, u.y, r.y));
-            R[i] = r;
-        }
-        s.add(fmaf(r.x, r.x, r.y * r.y));
-    }
-    const double t = block_sum(s.val(), sh);
-    if (part && threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
-cudaError_t step_residual(cf* R, const cf* A1, const cf* A2, long long n, const double* alpha, cudaStream_t st) {
-    (void)launch_pass(k_step_residual, dim3(kRedBlocks), dim3(kRedThreads), st, R, A1, A2, n, alpha, nullptr);
-    counted(1);
-    return cudaGetLastError();
-}
-
-__global__ void k_axpy_dev(float* __restrict__ x, const float* __restrict__ y, long long n2,
-                           const double* __restrict__ alpha) {
-    const float a = (float)alpha[0];
-    if (a == 0.f) return;
-    GRID_STRIDE(i, n2) x[i] = fmaf(a, y[i], x[i]);
-}
-
-cudaError_t axpy_dev(float* x, const float* y, long long n2, const double* alpha, cudaStream_t st) {
-    (void)launch_pass(k_axpy_dev, dim3(1024), dim3(256), st, x, y, n2, alpha);
-    counted(1);
-    return cudaGetLastError();
-}
-
-// ===========================================================================
-// Solver kernels (L-BFGS two-loop recursion, exact line search, ADMM).
-// ===========================================================================
-
-// f = 0.5 ||R||^2 from a fresh norm pass: part[blk] -> sc[SC_F]
-__global__ void __launch_bounds__(kRedThreads) k_norm_part(const cf* __restrict__ R, long long n, double* part) {
-    __shared__ double sh[32];
-    Acc s;
-    GRID_STRIDE(i, n) {
-        const cf r = R[i];
-        s.add(fmaf(r.x, r.x, r.y * r.y));
-    }
-    const double t = block_sum(s.val(), sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
-// g = gf + rho (x - v); history cleared (start of an x-update)
-__global__ void k_xupdate_start(SolverDev S, double rho) {
-    const float r = (float)rho;
-    GRID_STRIDE(i, S.n2) S.g[i] = S.gf[i] + r * (S.x[i] - S.v[i]);
-    if (blockIdx.x == 0 && threadIdx.x == 0) S.ints[SI_CNT] = 0;
-}
-
-__device__ __forceinline__ int ring_idx(const SolverDev& S, int j) {
-    // j-th newest pair (0 = newest)
-    const int R = S.ring;
-    return ((S.ints[SI_NEWEST] - j) % R + R) % R;
-}
-
-// L-BFGS direction d = -H g in the compact form of the inverse BFGS update
-// (Byrd, Nocedal and Schnabel 1994): with the k stored pairs ordered oldest
-// first, S = [s_1 .. s_k], Y = [y_1 .. y_k], R = triu(S^T Y), D = diag(S^T Y),
-// H0 = gamma I and gamma = <s,y>/<y,y> of the newest pair,
-//   H g = gamma g + S a - gamma Y u,  u = R^-1 S^T g,
-//   a = R^-T ((D + gamma Y^T Y) u - gamma Y^T g).
-// This is the matrix the two-loop recursion applies, evaluated in three
-// steps: the inner products (passes over groups of pairs; they also fill the
-// newest pair's row and column of S^T Y and Y^T Y, which are kept by slot),
-// the small FP64 triangular solves in one block, and one combination pass.
-
-// partials per block: for pair j of the group, <s_j,g>, <y_j,g>, <s_j,y_n>,
-// <s_n,y_j>, <y_j,y_n> (n = the newest pair).  Per-thread sums are plain FP32
-// multiply-adds (a thread sums n2 / (kRedBlocks kRedThreads) terms, a few
-// dozen at these sizes), combined in FP64 across threads and blocks: these
-// products only set the direction's coefficients, whose rounding the exact
-// line search and the descent test absorb.
-// 128 threads of <= 128 registers: a CTA fits beside the two GEMM CTAs of an SM
-constexpr int kLbThreads = 128;
-__global__ void __launch_bounds__(kLbThreads, 4) k_lb_dots(SolverDev S, int j0) {
-    __shared__ double sh[32];
-    const int cnt = S.ints[SI_CNT];
-    if (j0 >= cnt) return;
-    const int jc = min(kLbGroup, cnt - j0);
-    const float* sp[kLbGroup];
-    const float* yp[kLbGroup];
+        for (int j = 0; j < 8; ++j) {
+            const long long o = (long long)(r0 + kg * 8 + j) * ns + n0 + n;
+            const float2 r = v[j], x = A1[o], c = A2[o];
+            dots6_group(g, r.x, r.y, x.x, x.y, c.x, c.y);
+            if ((j & 3) == 3) {
 #pragma unroll
-    for (int jj = 0; jj < kLbGroup; ++jj) {
-        const int idx = ring_idx(S, jj < jc ? j0 + jj : j0);
-        sp[jj] = S.sh + (long long)idx * S.n2;
-        yp[jj] = S.yh + (long long)idx * S.n2;
-    }
-    const int nw = ring_idx(S, 0);
-    const float* sn = S.sh + (long long)nw * S.n2;
-    const float* yn = S.yh + (long long)nw * S.n2;
-    float acc[kLbGroup][5];
-#pragma unroll
-    for (int jj = 0; jj < kLbGroup; ++jj)
-#pragma unroll
-        for (int t = 0; t < 5; ++t) acc[jj][t] = 0.f;
-    float gg = 0.f;   // <g, g> for the descent test (first group only)
-    GRID_STRIDE(i, S.n2) {
-        const float gi = S.g[i], sni = sn[i], yni = yn[i];
-        gg = fmaf(gi, gi, gg);
-#pragma unroll
-        for (int jj = 0; jj < kLbGroup; ++jj) {
-            if (jj < jc) {
-                const float s = sp[jj][i], y = yp[jj][i];
-                acc[jj][0] = fmaf(s, gi, acc[jj][0]);
-                acc[jj][1] = fmaf(y, gi, acc[jj][1]);
-                acc[jj][2] = fmaf(s, yni, acc[jj][2]);
-                acc[jj][3] = fmaf(sni, y, acc[jj][3]);
-                acc[jj][4] = fmaf(y, yni, acc[jj][4]);
-            }
-        }
-    }
-    double* out = S.lbpart + (long long)(j0 / kLbGroup) * kRedBlocks * (5 * kLbGroup) +
-                  (long long)blockIdx.x * (5 * kLbGroup);
-#pragma unroll
-    for (int jj = 0; jj < kLbGroup; ++jj) {
-        if (jj >= jc) break;
-#pragma unroll
-        for (int t = 0; t < 5; ++t) {
-            const double r = block_sum((double)acc[jj][t], sh);
-            if (threadIdx.x == 0) out[jj * 5 + t] = r;
-        }
-    }
-    if (j0 == 0) {
-        const double r = block_sum((double)gg, sh);
-        if (threadIdx.x == 0) S.lbpart[kLbGGOff + blockIdx.x] = r;
-    }
-}
-
-// One block: finalise the partials (warp per value, fixed order), update the
-// newest pair's row / column of S^T Y and Y^T Y, then (thread 0) the
-// triangular solves; coefficients to acoef, gamma to sc[SC_GAMMA].
-// single-block finalisers on the solve's critical path: 256 threads sum the
-// partial slabs (fixed order per thread, then the block tree); at 256 threads
-// (56 registers at most) a finaliser fits on an SM beside two contraction
-// CTAs, so with several solves in flight it never waits for a free SM
-constexpr int kFinThreads = 256;
-
-__global__ void __launch_bounds__(kFinThreads) k_lb_solve(SolverDev S) {
-    __shared__ double val[32 * 5 + 1];
-    __shared__ double Rm[32 * 33];
-    __shared__ double Ym[32 * 33];
-    __shared__ double p[32], q[32], u[32], t[32];
-    const int cnt = S.ints[SI_CNT];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    const int nval = cnt > 0 ? 5 * cnt + 1 : 0;   // the last value is <g, g>
-    for (int v = w; v < nval; v += kFinThreads / 32) {
-        const double* base;
-        long long stride;
-        if (v == 5 * cnt) {
-            base = S.lbpart + kLbGGOff;
-            stride = 1;
-        } else {
-            const int j = v / 5, kind = v % 5;
-            base = S.lbpart + (long long)(j / kLbGroup) * kRedBlocks * (5 * kLbGroup) + (j % kLbGroup) * 5 + kind;
-            stride = 5 * kLbGroup;
-        }
-        double a = 0.0;
-        for (int b = l; b < kRedBlocks; b += 32) a += base[(long long)b * stride];
-        a = warp_sum(a);
-        if (l == 0) val[v] = a;
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    S.ints[SI_RFLAG] = 0;
-    if (cnt == 0) {
-        // d = -g, a descent direction unless g = 0 (which the line search meets)
-        S.sc[SC_GAMMA] = 1.0;
-        return;
-    }
-    const int R = S.ring;
-    const int nw = ring_idx(S, 0);
-    for (int j = 0; j < cnt; ++j) {
-        const int a = ring_idx(S, j);
-        S.SYm[a * R + nw] = val[j * 5 + 2];
-        S.SYm[nw * R + a] = val[j * 5 + 3];
-        S.YYm[a * R + nw] = val[j * 5 + 4];
-        S.YYm[nw * R + a] = val[j * 5 + 4];
-    }
-    // oldest first: position i holds the (cnt - 1 - i)-th newest pair
-    const int k = cnt;
-    for (int i = 0; i < k; ++i) {
-        const int si = ring_idx(S, k - 1 - i);
-        p[i] = val[(k - 1 - i) * 5 + 0];
-        q[i] = val[(k - 1 - i) * 5 + 1];
-        for (int j = 0; j < k; ++j) {
-            const int sj = ring_idx(S, k - 1 - j);
-            Rm[i * 33 + j] = S.SYm[si * R + sj];
-            Ym[i * 33 + j] = S.YYm[si * R + sj];
-        }
-    }
-    const double gamma = Rm[(k - 1) * 33 + (k - 1)] / Ym[(k - 1) * 33 + (k - 1)];
-    // u = R^-1 p (R upper triangular)
-    for (int i = k - 1; i >= 0; --i) {
-        double a = p[i];
-        for (int j = i + 1; j < k; ++j) a -= Rm[i * 33 + j] * u[j];
-        u[i] = a / Rm[i * 33 + i];
-    }
-    // t = D u + gamma Y^T Y u - gamma q
-    for (int i = 0; i < k; ++i) {
-        double a = Rm[i * 33 + i] * u[i] - gamma * q[i];
-        for (int j = 0; j < k; ++j) a += gamma * Ym[i * 33 + j] * u[j];
-        t[i] = a;
-    }
-    // a = R^-T t (R^T lower triangular), written over t
-    for (int i = 0; i < k; ++i) {
-        double a = t[i];
-        for (int j = 0; j < i; ++j) a -= Rm[j * 33 + i] * t[j];
-        t[i] = a / Rm[i * 33 + i];
-    }
-    // descent test: <g, d> = -(gamma <g,g> + sum_i a_i <s_i,g> - gamma sum_i u_i <y_i,g>)
-    double gd = gamma * val[5 * k];
-    for (int i = 0; i < k; ++i) gd += t[i] * p[i] - gamma * u[i] * q[i];
-    gd = -gd;
-    if (!(gd < 0.0)) {
-        // not a descent direction: clear the memory and take d = -g in this
-        // same iteration (the restart of L-BFGS)
-        S.ints[SI_CNT] = 0;
-        S.ints[SI_RESTARTS] += 1;
-        S.ints[SI_RFLAG] = 1;
-        S.sc[SC_GAMMA] = 1.0;
-        return;
-    }
-    for (int i = 0; i < k; ++i) {
-        const int j = k - 1 - i;   // j-th newest
-        S.acoef[j] = t[i];
-        S.acoef[32 + j] = -gamma * u[i];
-    }
-    S.sc[SC_GAMMA] = gamma;
-}
-
-// d = -(gamma g + sum_j a_j s_j + sum_j c_j y_j); four floats per thread and
-// four pairs per step in flight (the vectors start 16-byte aligned when n2 is
-// a multiple of 4, else a scalar loop)
-__global__ void __launch_bounds__(256) k_lb_dir(SolverDev S) {
-    __shared__ float cs[32], cy[32];
-    __shared__ const float* ps[32];
-    __shared__ const float* py[32];
-    const int cnt = S.ints[SI_CNT];
-    if (threadIdx.x < cnt) {
-        const int idx = ring_idx(S, threadIdx.x);
-        cs[threadIdx.x] = (float)S.acoef[threadIdx.x];
-        cy[threadIdx.x] = (float)S.acoef[32 + threadIdx.x];
-        ps[threadIdx.x] = S.sh + (long long)idx * S.n2;
-        py[threadIdx.x] = S.yh + (long long)idx * S.n2;
-    }
-    __syncthreads();
-    const float gamma = (float)S.sc[SC_GAMMA];
-    if ((S.n2 & 3) == 0) {
-        const long long n4 = S.n2 >> 2;
-        const float4* g4 = reinterpret_cast<const float4*>(S.g);
-        float4* d4 = reinterpret_cast<float4*>(S.d);
-        GRID_STRIDE(i, n4) {
-            const float4 gv = g4[i];
-            float4 r = make_float4(gamma * gv.x, gamma * gv.y, gamma * gv.z, gamma * gv.w);
-            int j = 0;
-            for (; j + 4 <= cnt; j += 4) {
-                float4 sv[4], yv[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    sv[u] = reinterpret_cast<const float4*>(ps[j + u])[i];
-                    yv[u] = reinterpret_cast<const float4*>(py[j + u])[i];
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float a = cs[j + u], c = cy[j + u];
-                    r.x = fmaf(c, yv[u].x, fmaf(a, sv[u].x, r.x));
-                    r.y = fmaf(c, yv[u].y, fmaf(a, sv[u].y, r.y));
-                    r.z = fmaf(c, yv[u].z, fmaf(a, sv[u].z, r.z));
-                    r.w = fmaf(c, yv[u].w, fmaf(a, sv[u].w, r.w));
+                for (int k = 0; k < 6; ++k) {
+                    acc[k].add(g[k]);
+                    g[k] = 0.f;
                 }
             }
-            for (; j < cnt; ++j) {
-                const float4 sv = reinterpret_cast<const float4*>(ps[j])[i];
-                const float4 yv = reinterpret_cast<const float4*>(py[j])[i];
-                const float a = cs[j], c = cy[j];
-                r.x = fmaf(c, yv.x, fmaf(a, sv.x, r.x));
-                r.y = fmaf(c, yv.y, fmaf(a, sv.y, r.y));
-                r.z = fmaf(c, yv.z, fmaf(a, sv.z, r.z));
-                r.w = fmaf(c, yv.w, fmaf(a, sv.w, r.w));
-            }
-            d4[i] = make_float4(-r.x, -r.y, -r.z, -r.w);
-        }
-    } else {
-        GRID_STRIDE(i, S.n2) {
-            float r = gamma * S.g[i];
-            for (int j = 0; j < cnt; ++j) r = fmaf(cy[j], py[j][i], fmaf(cs[j], ps[j][i], r));
-            S.d[i] = -r;
         }
     }
+    dots6_end(S, acc, nb3, rho, sh);
 }
 
-// theta-space line-search inner products: <x - v, x - v>, <x - v, d>, <d, d>
-__global__ void __launch_bounds__(kRedThreads) k_dots3(SolverDev S, double* part) {
-    __shared__ double sh[32];
-    Acc s0, s1, s2;
-    GRID_STRIDE(i, S.n2) {
-        const float w = S.x[i] - S.v[i];
-        const float d = S.d[i];
-        s0.add(w * w);
-        s1.add(w * d);
-        s2.add(d * d);
-    }
-    double r;
-    r = block_sum(s0.val(), sh);
-    if (threadIdx.x == 0) part[blockIdx.x * 3 + 0] = r;
-    r = block_sum(s1.val(), sh);
-    if (threadIdx.x == 0) part[blockIdx.x * 3 + 1] = r;
-    r = block_sum(s2.val(), sh);
-    if (threadIdx.x == 0) part[blockIdx.x * 3 + 2] = r;
-}
-
-__device__ double quartic_val(const double* c, double a) {
-    return c[0] + a * (c[1] + a * (c[2] + a * (c[3] + a * c[4])));
-}
-
-__device__ void consider(const double* c, double a, double& best_a, double& best_v, bool& have) {
-    // two Newton polishes on phi'
-    for (int it = 0; it < 2; ++it) {
-        const double d1 = c[1] + a * (2 * c[2] + a * (3 * c[3] + a * 4 * c[4]));
-        const double d2 = 2 * c[2] + a * (6 * c[3] + a * 12 * c[4]);
-        if (d2 != 0.0) a -= d1 / d2;
-    }
-    if (!(a > 0.0) || !isfinite(a)) return;
-    const double v = quartic_val(c, a);
-    if (!have || v < best_v || (v == best_v && a < best_a)) {
-        have = true;
-        best_a = a;
-        best_v = v;
-    }
-}
-
-// Minimiser over a > 0 of the quartic: real roots of phi'(a) =
-// 4 c4 a^3 + 3 c3 a^2 + 2 c2 a + c1 in closed form (depressed cubic:
-// trigonometric form for three real roots, Cardano otherwise), polished.
-__device__ bool quartic_argmin(const double* c, double* out) {
-    double best_a = 0.0, best_v = 0.0;
-    bool have = false;
-    const double A = 4 * c[4], B = 3 * c[3], C = 2 * c[2], D = c[1];
-    if (A != 0.0) {
-        const double p = B / A, q = C / A, r = D / A;
-        const double P = q - p * p / 3.0;
-        const double Q = 2.0 * p * p * p / 27.0 - p * q / 3.0 + r;
-        const double disc = 0.25 * Q * Q + P * P * P / 27.0;
-        const double sh = -p / 3.0;
-        if (disc > 0.0) {
-            const double sq = sqrt(disc);
-            const double t = cbrt(-0.5 * Q + sq) + cbrt(-0.5 * Q - sq);
-            consider(c, t + sh, best_a, best_v, have);
-        } else if (P == 0.0) {
-            consider(c, cbrt(-Q) + sh, best_a, best_v, have);
-        } else {
-            const double m = 2.0 * sqrt(-P / 3.0);
-            double arg = 3.0 * Q / (P * m);
-            arg = fmin(1.0, fmax(-1.0, arg));
-            const double th = acos(arg) / 3.0;
-            const double tpi = 2.0943951023931954923;  // 2 pi / 3
-            for (int k = 0; k < 3; ++k) consider(c, m * cos(th - tpi * k) + sh, best_a, best_v, have);
-        }
-    } else if (B != 0.0) {
-        const double dsc = C * C - 4 * B * D;
-        if (dsc >= 0.0) {
-            const double s = sqrt(dsc);
-            consider(c, (-C + s) / (2 * B), best_a, best_v, have);
-            consider(c, (-C - s) / (2 * B), best_a, best_v, have);
-        }
-    } else if (C != 0.0) {
-        consider(c, -D / C, best_a, best_v, have);
-    }
-    *out = best_a;
-    return have;
-}
-
-// One thread: finalise the 6 + 3 inner products, form phi's coefficients,
-// check descent, pick alpha; alpha = 0 and a memory reset when no step.
-__global__ void __launch_bounds__(kFinThreads) k_line_search(SolverDev S, const double* part6, int nb6,
-                                                             const double* part3, double rho) {
-    __shared__ double sh[32];
-    double d6[6], d3[3];
-    for (int k = 0; k < 6; ++k) {
-        double v = 0.0;
-        for (int i = threadIdx.x; i < nb6; i += blockDim.x) v += part6[i * 6 + k];
-        d6[k] = block_sum(v, sh);
-    }
-    for (int k = 0; k < 3; ++k) {
-        double v = 0.0;
-        for (int i = threadIdx.x; i < kRedBlocks; i += blockDim.x) v += part3[i * 3 + k];
-        d3[k] = block_sum(v, sh);
-    }
-    if (threadIdx.x != 0) return;
-    double c[5];
-    c[0] = 0.5 * d6[0] + 0.5 * rho * d3[0];
-    c[1] = d6[1] + rho * d3[1];
-    c[2] = 0.5 * d6[3] + d6[2] + 0.5 * rho * d3[2];
-    c[3] = d6[4];
-    c[4] = 0.5 * d6[5];
-    for (int k = 0; k < 5; ++k) S.sc[SC_C0 + k] = c[k];
-    double a = 0.0;
-    bool ok = false;
-    if (c[1] < 0.0) ok = quartic_argmin(c, &a);
-    if (!ok) {
-        // no minimiser on a > 0 along d: no step, memory cleared; counted as a
-        // restart unless the direction test already counted this iteration
-        a = 0.0;
-        S.ints[SI_CNT] = 0;
-        if (!S.ints[SI_RFLAG]) S.ints[SI_RESTARTS] += 1;
-    }
-    bool finite = isfinite(c[0]) && isfinite(c[1]) && isfinite(c[2]) && isfinite(c[3]) && isfinite(c[4]);
-    if (!finite) {
-        a = 0.0;
-        S.ints[SI_STATUS] = TLR_ERR_NONFINITE;
-    }
-    S.sc[SC_ALPHA] = a;
-}
-
-// x += a d ; s_free = a d
+// x += a d ; s_free = a d (two floats at a time: n2 is even)
 __global__ void k_step_theta(SolverDev S) {
     const double ad = S.sc[SC_ALPHA];
     const float a = (float)ad;
     const int R = S.ring;
     const int fr = (S.ints[SI_NEWEST] + 1) % R;
-    float* s = S.sh + (long long)fr * S.n2;
-    GRID_STRIDE(i, S.n2) {
-        const float st = a * S.d[i];
+    float2* s = reinterpret_cast<float2*>(S.sh + (long long)fr * S.n2);
+    float2* x = reinterpret_cast<float2*>(S.x);
+    const float2* d = reinterpret_cast<const float2*>(S.d);
+    GRID_STRIDE(i, S.n2 >> 1) {
+        const float2 dv = d[i];
+        float2 xv = x[i];
+        const float2 st = make_float2(a * dv.x, a * dv.y);
         s[i] = st;
-        S.x[i] += st;
+        xv.x += st.x;
+        xv.y += st.y;
+        x[i] = xv;
     }
 }
 
-// y_free = (gf + rho (x - v)) - g ; g <- gf + rho (x - v); partials ss, sy, yy
-__global__ void __launch_bounds__(kRedThreads) k_pair_prep(SolverDev S, double rho, double* part) {
-    __shared__ double sh[32];
+// gf from the split-K partials, y_free = (gf + rho (x - v)) - g, g <- gf + rho (x -
+// v), with partials of ss, sy, yy; the last block accepts the pair (s, y) when
+// alpha > 0 and <s,y> > 1e-12 |s||y| and records f = 0.5 ||R||^2 from the nf
+// residual-norm partials.
+__global__ void __launch_bounds__(kRedThreads) k_gradient_pair(SolverDev S, const cf* __restrict__ part, int nsplit,
+                                                              long long nlr, long long ndense, long long b, int general,
+                                                              const long long* __restrict__ zoff,
+                                                              const int* __restrict__ zdim, double rho,
+                                                              const double* __restrict__ partf, long long nf) {
+    __shared__ double sh[3][256];
     const float r = (float)rho;
     const int R = S.ring;
     const int fr = (S.ints[SI_NEWEST] + 1) % R;
-    const float* s = S.sh + (long long)fr * S.n2;
-    float* y = S.yh + (long long)fr * S.n2;
+    const cf* s = reinterpret_cast<const cf*>(S.sh + (long long)fr * S.n2);
+    cf* y = reinterpret_cast<cf*>(S.yh + (long long)fr * S.n2);
+    const cf* x = reinterpret_cast<const cf*>(S.x);
+    const cf* v = reinterpret_cast<const cf*>(S.v);
+    cf* g = reinterpret_cast<cf*>(S.g);
+    cf* gf = reinterpret_cast<cf*>(S.gf);
+    const long long stride = S.n2 >> 1;
     Acc ss, sy, yy;
-    GRID_STRIDE(i, S.n2) {
-        const float gn = S.gf[i] + r * (S.x[i] - S.v[i]);
-        const float yi = gn - S.g[i];
-        y[i] = yi;
-        S.g[i] = gn;
-        const float si = s[i];
-        ss.add(si * si);
-        sy.add(si * yi);
-        yy.add(yi * yi);
+    auto entry = [&](long long e, cf gv) {
+        const cf xe = x[e], ve = v[e], go = g[e], se = s[e];
+        const cf gn = make_float2(gv.x + r * (xe.x - ve.x), gv.y + r * (xe.y - ve.y));
+        const cf ye = make_float2(gn.x - go.x, gn.y - go.y);
+        gf[e] = gv;
+        y[e] = ye;
+        g[e] = gn;
+        ss.add(se.x * se.x);
+        ss.add(se.y * se.y);
+        sy.add(se.x * ye.x);
+        sy.add(se.y * ye.y);
+        yy.add(ye.x * ye.x);
+        yy.add(ye.y * ye.y);
+    };
+    GRID_STRIDE(e, nlr) entry(e, split_sum(part, nsplit, stride, e));
+    GRID_STRIDE(e, ndense * b * b) {
+        long long base, n, row, col;
+        if (!dense_tile(e, b, zoff, zdim, base, n, row, col)) continue;
+        entry(nlr + base + row * n + col, split_sum_dense(part, nsplit, stride, nlr + base + row * n + col,
+                                                          nlr + base + col * n + row, general));
     }
-    double t;
-    t = block_sum(ss.val(), sh);
-    if (threadIdx.x == 0) part[blockIdx.x * 3 + 0] = t;
-    t = block_sum(sy.val(), sh);
-    if (threadIdx.x == 0) part[blockIdx.x * 3 + 1] = t;
-    t = block_sum(yy.val(), sh);
-    if (threadIdx.x == 0) part[blockIdx.x * 3 + 2] = t;
-}
-
-// one thread: accept the pair (s, y) when alpha > 0 and <s,y> > 1e-12 |s||y|;
-// record f = 0.5 ||R||^2 from the nf residual-norm partials.
-__global__ void __launch_bounds__(kFinThreads) k_pair_accept(SolverDev S, const double* part3, const double* partf,
-                                                             int nf) {
-    __shared__ double sh[32];
-    double v[4];
-    for (int k = 0; k < 3; ++k) {
-        double a = 0.0;
-        for (int i = threadIdx.x; i < kRedBlocks; i += blockDim.x) a += part3[i * 3 + k];
-        v[k] = block_sum(a, sh);
-    }
-    {
-        // the residual-norm partials can number tens of thousands (one per
-        // fused residual-step CTA): four independent sums per thread in a
-        // fixed order keep the loads in flight
-        const int bd = blockDim.x;
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        int i = threadIdx.x;
-        for (; i + 3 * bd < nf; i += 4 * bd) {
-            a0 += partf[i];
-            a1 += partf[i + bd];
-            a2 += partf[i + 2 * bd];
-            a3 += partf[i + 3 * bd];
-        }
-        for (; i < nf; i += bd) a0 += partf[i];
-        v[3] = block_sum((a0 + a1) + (a2 + a3), sh);
-    }
+    const double w[3] = {ss.val(), sy.val(), yy.val()};
+    const double t = block_sums(w, sh);
+    if (threadIdx.x < 3) S.partp[blockIdx.x * 3 + threadIdx.x] = t;
+    if (!last_block(reinterpret_cast<unsigned*>(S.ints + CT_PAIR), gridDim.x)) return;
+    const double d = sum_slabs<3>(S.partp, gridDim.x, sh[0]);
+    const double rr = sum_part(partf, nf, sh);
+    if (threadIdx.x >= 32) return;
+    const double dss = __shfl_sync(0xffffffffu, d, 0), dsy = __shfl_sync(0xffffffffu, d, 1),
+                 dyy = __shfl_sync(0xffffffffu, d, 2);
     if (threadIdx.x != 0) return;
-    const double ss = v[0], sy = v[1], yy = v[2], rr = v[3];
     const double f = 0.5 * rr;
     S.sc[SC_F] = f;
     const int it = S.ints[SI_ITERS];
     if (it < TLR_MAX_HIST) S.fhist[it] = f;
     S.ints[SI_ITERS] = it + 1;
     if (!isfinite(f)) S.ints[SI_STATUS] = TLR_ERR_NONFINITE;
-    if (S.sc[SC_ALPHA] > 0.0 && sy > 1e-12 * sqrt(ss * yy)) {
-        const int R = S.ring;
-        const int fr = (S.ints[SI_NEWEST] + 1) % R;
+    if (S.sc[SC_ALPHA] > 0.0 && dsy > 1e-12 * sqrt(dss * dyy)) {
         S.ints[SI_NEWEST] = fr;
         S.ints[SI_CNT] = min(S.ints[SI_CNT] + 1, S.m);
-        S.rho_h[fr] = 1.0 / sy;
-        S.sy_h[fr] = sy;
-        S.yy_h[fr] = yy;
+        S.rho_h[fr] = 1.0 / dsy;
+        S.sy_h[fr] = dsy;
+        S.yy_h[fr] = dyy;
     }
 }
 
@@ -821,11 +915,11 @@ __global__ void k_admm_resume(SolverDev S) {
     }
 }
 
-// record f0 = 0.5 ||R||^2
-__global__ void k_record_f0(SolverDev S, const double* partf) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double rr = 0;
-    for (int i = 0; i < kRedBlocks; ++i) rr += partf[i];
+// f0 = f = 0.5 ||R||^2
+__global__ void __launch_bounds__(256) k_record_f0(SolverDev S, const double* partf, long long np) {
+    __shared__ double sh[1][256];
+    const double rr = sum_part(partf, np, sh);
+    if (threadIdx.x != 0) return;
     S.sc[SC_F0] = 0.5 * rr;
     S.sc[SC_F] = 0.5 * rr;
 }
@@ -834,12 +928,12 @@ __global__ void k_record_f0(SolverDev S, const double* partf) {
 // host wrappers
 // ---------------------------------------------------------------------------
 cudaError_t sv_norm_part(const cf* R, long long n, double* part, cudaStream_t st) {
-    (void)launch_pass(k_norm_part, dim3(kRedBlocks), dim3(kRedThreads), st, R, n, part);
+    (void)launch_pass(k_norm_part, dim3(red_blocks(n)), dim3(kRedThreads), st, R, n, part);
     counted(1);
     return cudaGetLastError();
 }
-cudaError_t sv_record_f0(const SolverDev& S, const double* partf, cudaStream_t st) {
-    (void)launch_pass(k_record_f0, dim3(1), dim3(32), st, S, partf);
+cudaError_t sv_record_f0(const SolverDev& S, const double* partf, long long np, cudaStream_t st) {
+    (void)launch_pass(k_record_f0, dim3(1), dim3(256), st, S, partf, np);
     counted(1);
     return cudaGetLastError();
 }
@@ -860,44 +954,46 @@ cudaError_t sv_xupdate_start(const SolverDev& S, double rho, cudaStream_t st) {
 }
 cudaError_t sv_direction(const SolverDev& S, cudaStream_t st) {
     for (int j0 = 0; j0 < S.m; j0 += kLbGroup) {
-        (void)launch_pass(k_lb_dots, dim3(kRedBlocks), dim3(kLbThreads), st, S, j0);
+        (void)launch_pass(k_lb_dots, dim3(lb_blocks(S.n2)), dim3(kLbThreads), st, S, j0, j0 + kLbGroup >= S.m ? 1 : 0);
         counted(1);
     }
-    (void)launch_pass(k_lb_solve, dim3(1), dim3(kFinThreads), st, S);
-    counted(1);
-    (void)launch_pass(k_lb_dir, dim3(1024), dim3(256), st, S);
+    (void)launch_pass(k_lb_dir, dim3(red_blocks(S.n2)), dim3(kRedThreads), st, S);
     counted(1);
     return cudaGetLastError();
 }
-cudaError_t sv_dots3(const SolverDev& S, double* part, cudaStream_t st) {
-    (void)launch_pass(k_dots3, dim3(kRedBlocks), dim3(kRedThreads), st, S, part);
-    counted(1);
-    return cudaGetLastError();
-}
-cudaError_t sv_line_search(const SolverDev& S, const double* part6, int nb6, const double* part3, double rho,
+cudaError_t sv_line_search(const SolverDev& S, const cf* R, const cf* A1, const cf* A2, long long n, double rho,
                            cudaStream_t st) {
-    (void)launch_pass(k_line_search, dim3(1), dim3(kFinThreads), st, S, part6, nb6, part3, rho);
+    (void)launch_pass(k_dots6, dim3(red_blocks(n)), dim3(kRedThreads), st, S, R, A1, A2, n, red_blocks(S.n2), rho);
+    counted(1);
+    return cudaGetLastError();
+}
+cudaError_t sv_line_search_packed(const SolverDev& S, char* const* kn, const cf* A1, const cf* A2, int nr, int ns, int b,
+                                  const long long* roff, int nblk, int fmt, double rho, cudaStream_t st) {
+    if (nr <= 0 || ns <= 0 || nr % kFuseRows != 0) return cudaErrorInvalidValue;
+    if (!roff && (b <= 0 || b % kFuseRows != 0 || nr % b != 0)) return cudaErrorInvalidValue;
+    if (roff && nblk <= 0) return cudaErrorInvalidValue;
+    const long long tiles = rstep_ctas(nr, ns);
+    (void)launch_pass(k_dots6p, dim3((unsigned)std::min<long long>(tiles, kRedBlocks)), dim3(256), st, S, kn, A1, A2, ns,
+                      nr, b, roff, nblk, fmt, red_blocks(S.n2), rho);
     counted(1);
     return cudaGetLastError();
 }
 cudaError_t sv_step_residual(cf* R, const cf* A1, const cf* A2, long long n, const double* alpha,
                              double* partf, cudaStream_t st) {
-    (void)launch_pass(k_step_residual, dim3(kRedBlocks), dim3(kRedThreads), st, R, A1, A2, n, alpha, partf);
+    (void)launch_pass(k_step_residual, dim3(red_blocks(n)), dim3(kRedThreads), st, R, A1, A2, n, alpha, partf);
     counted(1);
     return cudaGetLastError();
 }
 cudaError_t sv_step_theta(const SolverDev& S, cudaStream_t st) {
-    (void)launch_pass(k_step_theta, dim3(1024), dim3(256), st, S);
+    (void)launch_pass(k_step_theta, dim3(2 * red_blocks(S.n2)), dim3(256), st, S);
     counted(1);
     return cudaGetLastError();
 }
-cudaError_t sv_pair_prep(const SolverDev& S, double rho, double* part, cudaStream_t st) {
-    (void)launch_pass(k_pair_prep, dim3(kRedBlocks), dim3(kRedThreads), st, S, rho, part);
-    counted(1);
-    return cudaGetLastError();
-}
-cudaError_t sv_pair_accept(const SolverDev& S, const double* part3, const double* partf, int nf, cudaStream_t st) {
-    (void)launch_pass(k_pair_accept, dim3(1), dim3(kFinThreads), st, S, part3, partf, nf);
+cudaError_t sv_gradient_pair(const SolverDev& S, const cf* part, int nsplit, long long nlr, long long ndense,
+                             long long b, int general, const long long* zoff, const int* zdim, double rho,
+                             const double* partf, long long nf, cudaStream_t st) {
+    (void)launch_pass(k_gradient_pair, dim3(red_blocks(S.n2)), dim3(kRedThreads), st, S, part, nsplit, nlr, ndense, b,
+                      general, zoff, zdim, rho, partf, nf);
     counted(1);
     return cudaGetLastError();
 }

@@ -105,4 +105,33 @@ __device__ __forceinline__ void pk_load8(const char* row, int fmt, int kg, float
     }
 }
 
+// Block of the 16-row residual tile starting at row r0: r0 / b for equal
+// tiles, else the largest i with roff[i] <= r0 (every roff[i] is a multiple
+// of kFuseRows, so the tile lies in it); rl0 = its first row in the block, bK =
+// the block's size.
+struct RTile {
+    int blk, rl0, bK;
+};
+__device__ __forceinline__ RTile rtile(int r0, int b, const long long* roff, int nblk) {
+    RTile t;
+    if (roff) {
+        int lo = 0, hi = nblk - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (roff[mid] <= r0)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        t.blk = lo;
+        t.rl0 = r0 - (int)roff[lo];
+        t.bK = (int)(roff[lo + 1] - roff[lo]);
+    } else {
+        t.blk = r0 / b;
+        t.rl0 = r0 - t.blk * b;
+        t.bK = b;
+    }
+    return t;
+}
+
 }  // namespace tlr

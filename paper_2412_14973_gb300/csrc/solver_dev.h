@@ -13,8 +13,13 @@ enum ScalarSlot { SC_ALPHA = 0, SC_F, SC_F0, SC_C0, SC_C1, SC_C2, SC_C3, SC_C4, 
 // replaced by -g (the iteration already counts as a restart)
 enum IntSlot { SI_CNT = 0, SI_NEWEST, SI_ITERS, SI_RESTARTS, SI_STATUS, SI_RFLAG, SI_COUNT };
 
+// after the counters: [SI_COUNT + 1] the contractions' error word, then the block
+// counters of the passes whose last block finishes their sums (zero between launches)
+enum CounterSlot { CT_DIR = SI_COUNT + 2, CT_LINE, CT_PAIR, CT_NORM };
+
 // compact L-BFGS: pairs per inner-product pass, and the partial storage for
-// the largest memory (32 pairs), followed by one slab of <g, g> partials
+// the largest memory (32 pairs; value by value, kRedBlocks partials each), followed
+// by one slab of <g, g> partials
 constexpr int kLbGroup = 10;
 constexpr long long kLbGGOff = (long long)kRedBlocks * 5 * kLbGroup * ((32 + kLbGroup - 1) / kLbGroup);
 constexpr long long kLbPartDoubles = kLbGGOff + kRedBlocks;
@@ -31,29 +36,48 @@ struct SolverDev {
     double* acoef;       // [64] direction coefficients: [j] of s_j, [32 + j] of y_j (j-th newest)
     double* SYm;         // [ring * ring] <s_a, y_b> by slot
     double* YYm;         // [ring * ring] <y_a, y_b> by slot
-    double* lbpart;      // kRedBlocks * 5 * kLbGroup partials per group of pairs (direction inner products)
+    double* lbpart;      // partials of the direction's inner products
     double* sc;          // ScalarSlot values
     int* ints;           // IntSlot values
     double* fhist;       // [TLR_MAX_HIST]
-    double* part;        // 2 * kRedBlocks partial slabs
+    double* part3;       // 3 * kRedBlocks: <x-v,x-v>, <x-v,d>, <d,d> partials of the direction pass
+    double* part6;       // 6 * kRedBlocks: line-search inner products
+    double* partp;       // 3 * kRedBlocks: the new pair's inner products
 };
 
+// blocks of a reduction over n values: enough work for 256 threads each, at most
+// kRedBlocks (a function of n alone, so the order of every sum is fixed)
+inline int red_blocks(long long n) {
+    const long long b = (n + 2047) / 2048;
+    return (int)(b < 1 ? 1 : b > kRedBlocks ? kRedBlocks : b);
+}
+
+// partials of ||R||^2 (n complex) into part[red_blocks(n)]
 cudaError_t sv_norm_part(const cf* R, long long n, double* part, cudaStream_t st);
-cudaError_t sv_record_f0(const SolverDev& S, const double* partf, cudaStream_t st);
+// f0 = f = 0.5 sum of the np partials
+cudaError_t sv_record_f0(const SolverDev& S, const double* partf, long long np, cudaStream_t st);
 cudaError_t sv_admm_init(const SolverDev& S, cudaStream_t st);
 cudaError_t sv_admm_resume(const SolverDev& S, cudaStream_t st);
 cudaError_t sv_xupdate_start(const SolverDev& S, double rho, cudaStream_t st);
+// the direction d, and the partials of the theta-space line-search products
 cudaError_t sv_direction(const SolverDev& S, cudaStream_t st);
-cudaError_t sv_dots3(const SolverDev& S, double* part, cudaStream_t st);
-// part6: nb6 blocks of 6 partial sums (kRedBlocks from dots6_part, or one per
-// CTA of the packed-residual inner products)
-cudaError_t sv_line_search(const SolverDev& S, const double* part6, int nb6, const double* part3, double rho,
+// The line search: the six inner products of Rf, A1, A2 (n complex, FP32), or with
+// Rf read from its KN packing (kn[i], as rstep writes it, over rstep's tiles), then
+// phi's minimiser by the last block.
+cudaError_t sv_line_search(const SolverDev& S, const cf* R, const cf* A1, const cf* A2, long long n, double rho,
                            cudaStream_t st);
+cudaError_t sv_line_search_packed(const SolverDev& S, char* const* kn, const cf* A1, const cf* A2, int nr, int ns, int b,
+                                  const long long* roff, int nblk, int fmt, double rho, cudaStream_t st);
+// R += a A1 + a^2 A2 (a = *alpha) with partials of ||R||^2 into partf[red_blocks(n)]
 cudaError_t sv_step_residual(cf* R, const cf* A1, const cf* A2, long long n, const double* alpha,
                              double* partf, cudaStream_t st);
 cudaError_t sv_step_theta(const SolverDev& S, cudaStream_t st);
-cudaError_t sv_pair_prep(const SolverDev& S, double rho, double* part, cudaStream_t st);
-cudaError_t sv_pair_accept(const SolverDev& S, const double* part3, const double* partf, int nf, cudaStream_t st);
+// The gradient's split-K partials summed into gf (as reduce_grad does), the new
+// pair (s, y) and g from it, and, by the last block, f from the nf residual-norm
+// partials and the acceptance of the pair.
+cudaError_t sv_gradient_pair(const SolverDev& S, const cf* part, int nsplit, long long nlr, long long ndense,
+                             long long b, int general, const long long* zoff, const int* zdim, double rho,
+                             const double* partf, long long nf, cudaStream_t st);
 cudaError_t sv_admm_zu(const SolverDev& S, double lam, double rho, cudaStream_t st);
 
 }  // namespace tlr
