@@ -221,6 +221,8 @@ void account_replay(const std::vector<TimedLaunch>& v) {
     }
 }
 
+constexpr int kIntSlots = CT_DIR + 1 + kLbClusters;   // solver counters, error word, block counters
+
 struct HostStats {
     int ints[SI_COUNT + 2];
     double sc[SC_COUNT];
@@ -677,10 +679,10 @@ void carve(tlr_mdd_s* h, Arena& a) {
     const size_t nz = std::max<size_t>(1, (size_t)(L.nth - L.nlr));
     h->Zs = a.take<cf>(nz);
     h->Zsd = a.take<cf>(nz);
-    // split-K partials of the projection.  FP32 path: over A1 and A2, which are
-    // adjacent and dead between the step that uses them and the next line search
-    // (where a single partial does not fit there, a buffer of its own)
-    if (!tensor_core(h->d.precision) && (size_t)h->nsplit * L.nth <= 2 * nrs)
+    // split-K partials of the projection: over A1 and A2, which are adjacent and
+    // dead between the step that uses them and the next line search (where they do
+    // not fit there, a buffer of their own)
+    if ((size_t)h->nsplit * L.nth <= 2 * nrs)
         h->part = h->A1;
     else
         h->part = a.take<cf>((size_t)h->nsplit * L.nth);
@@ -721,7 +723,7 @@ void carve(tlr_mdd_s* h, Arena& a) {
     h->yy_h = a.take<double>(64);
     h->acoef = a.take<double>(64);
     h->sc = a.take<double>(SC_COUNT + 8);
-    h->ints = a.take<int>(SI_COUNT + 8);
+    h->ints = a.take<int>(kIntSlots);
     h->fhist = a.take<double>(TLR_MAX_HIST);
     h->lbm = a.take<double>(2 * 33 * 33);
     h->lbpart = a.take<double>((size_t)kLbPartDoubles);
@@ -776,6 +778,11 @@ int split_for(const Layout& L, int prec) {
                 best = sp;
             }
         }
+        // a small problem leaves most SMs idle: split on, down to 64 sources a split,
+        // while all of it still is one wave and the partials fit over A1 and A2
+        // (nr = ns = 256, tile 64: 1 -> 4, the projection 21.7 -> 11 us)
+        const long long fit = 2LL * L.nr * L.ns / std::max<long long>(1, L.nth);
+        while (best < 16 && tiles * (best + 1) <= sms && L.ns / (best + 1) >= 64 && best + 1 <= fit) ++best;
         return (int)best;
     }
     long long tiles = 0;
@@ -1528,7 +1535,7 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
     }
     CKF(cudaMemcpyAsync(h->d_roff, L.roff.data(), (L.N + 1) * sizeof(long long), cudaMemcpyHostToDevice, h->st));
     // solver counters and the contraction kernels' error word start at zero
-    CKF(cudaMemsetAsync(h->ints, 0, (SI_COUNT + 8) * sizeof(int), h->st));
+    CKF(cudaMemsetAsync(h->ints, 0, kIntSlots * sizeof(int), h->st));
     std::vector<HostTable> tabs;
     if (build_tables(h, h->tab_base, &tabs)) {
         h->err = "uploading GEMM tables failed";
@@ -2404,6 +2411,8 @@ static SolverDev solver_dev(tlr_mdd_s* h, int m) {
     S.SYm = h->lbm;
     S.YYm = h->lbm + 33 * 33;
     S.lbpart = h->lbpart;
+    S.lbsum = h->lbpart + kLbSumOff;
+    S.lbctr = reinterpret_cast<unsigned*>(h->ints + CT_DIR);
     S.sc = h->sc;
     S.ints = h->ints;
     S.fhist = h->fhist;

@@ -1,6 +1,8 @@
 // Data-preparation kernels: Hilbert receiver order (eq. 10), normalisation
 // alpha (Hyper-parameter selection section), receiver-major reordered panels
 // (eq. 14) and the natural-order back-mapping X = S X_h S^T (eq. 11).
+#include <algorithm>
+
 #include "internal.h"
 
 namespace tlr {
@@ -83,13 +85,43 @@ cudaError_t hilbert_perm(int nx, int ny, int32_t* perm, int32_t* slot, cudaStrea
 // ---------------------------------------------------------------------------
 // alpha = max |D| : per-block maxima of re^2 + im^2 in FP64, then one block.
 // ---------------------------------------------------------------------------
-__global__ void k_max_abs2_part(const cf* __restrict__ D, long long n, double* part) {
+// An FP64 square per entry takes FP64 time (46 us for 34 MB; 2 lanes per cycle and
+// SM), so a warp squares its 32 entries in FP64 only if an FP32 square among them
+// comes within 2^-21 of the largest the warp has met (a margin above the rounding of
+// both): every entry that could be the maximum is, the result is the same double,
+// and of m such groups about ln m are.  NaN entries are passed over and an Inf
+// gives Inf, as the FP64 comparison does.
+__global__ void __launch_bounds__(256) k_max_abs2_part(const cf* __restrict__ D, long long n, double* part) {
     double m = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const cf v = D[i];
-        const double a = (double)v.x * v.x + (double)v.y * v.y;
+    float mf = 0.f;   // the warp's largest FP32 square, less the margin
+    auto take = [&](float x, float y) {
+        const float f = fmaf(x, x, y * y);
+        // not below the margin, or possibly an underflow
+        if (!__any_sync(0xffffffffu, f >= mf && f > 0.f || (f < 1e-30f && mf < 1e-29f && (x != 0.f || y != 0.f)))) return;
+        const double a = (double)x * x + (double)y * y;
         m = a > m ? a : m;
+        // near overflow all of them go to FP64
+        const float g = f < 1e38f ? f * (1.f - 4.8e-7f) : 0.f;
+        mf = fmaxf(mf, __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(g))));
+    };
+    const long long stride = (long long)gridDim.x * blockDim.x, i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const bool vec = (reinterpret_cast<uintptr_t>(D) & 15) == 0;
+    const long long n4 = vec ? n >> 1 : 0;
+    const float4* D4 = reinterpret_cast<const float4*>(D);
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (long long i = i0; i - i0 < n4; i += 4 * stride) {   // the same trips for every lane
+        float4 v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = i + j * stride < n4 ? D4[i + j * stride] : z;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            take(v[j].x, v[j].y);
+            take(v[j].z, v[j].w);
+        }
+    }
+    for (long long i = 2 * n4 + i0; i - i0 < n; i += stride) {   // what the pairs leave (all of it when D is not 16-byte aligned)
+        const cf v = i < n ? D[i] : make_float2(0.f, 0.f);
+        take(v.x, v.y);
     }
     __shared__ double sh[256];
     sh[threadIdx.x] = m;
@@ -189,97 +221,151 @@ __device__ __forceinline__ int block_of(long long r, long long b, const long lon
     return lo;
 }
 
-// X_h = C(theta) assembled entry by entry from the stacked unknown (eq. 6-9,
-// 15).  An entry of a super-diagonal tile evaluates exactly the expression of
-// its mirror in the sub-diagonal tile (same products, same order), so the
-// result is bitwise symmetric, as X_ji = X_ij^T demands.
-// General form (general != 0): the tiles are listed row-major (i N + j) and
-// every entry is its own tile's L R^T (or Z entry), without mirroring.
-// roff == nullptr: N tiles of size b; else block i covers rows roff[i] ..
-// roff[i + 1] - 1.
-__global__ void k_assemble(const cf* __restrict__ th, long long nr, long long b, int N, const AsmTile* __restrict__ t,
-                           cf* __restrict__ Xh, int general, const long long* __restrict__ roff) {
-    const long long n2 = nr * nr;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n2;
-         e += (long long)gridDim.x * blockDim.x) {
-        long long r = e / nr, c = e % nr;
-        int i = block_of(r, b, roff, N), j = block_of(c, b, roff, N);
-        if (general) {
-            const AsmTile& a = t[i * N + j];
-            const long long rr = r - (roff ? roff[i] : i * b), cc = c - (roff ? roff[j] : j * b);
-            const long long di = roff ? roff[i + 1] - roff[i] : b;
-            float x = 0.f, y = 0.f;
-            if (i == j && a.dense) {
-                const cf u = th[a.off_l + rr * di + cc];
-                x = u.x;
-                y = u.y;
-            } else {
-                const cf* L = th + a.off_l + rr * a.k;
-                const cf* R = th + a.off_r + cc * a.k;
-                for (int q = 0; q < a.k; ++q) {
-                    const cf l = L[q], m = R[q];
-                    x = fmaf(l.x, m.x, fmaf(-l.y, m.y, x));
-                    y = fmaf(l.x, m.y, fmaf(l.y, m.x, y));
+// X_h = C(theta) assembled from the stacked unknown (eq. 6-9, 15).  A block of 256
+// threads takes 64 x 64 entries of one tile (r, c), 4 x 4 per thread, with the
+// factors' rows staged 32 columns at a time (an entry at a time read 2 k values
+// from L1 per entry: 782 us at nr = 4096, rank 26; about 70 us now).  In the reciprocal
+// form the mirror entry is written with it, so the result is bitwise symmetric, as
+// X_ji = X_ij^T demands; a low-rank diagonal tile evaluates its upper triangle.
+// General form (general != 0): the tiles are listed row-major (i N + j) and every
+// tile is its own L R^T (or Z).  The sum over the rank runs in order, one fused
+// multiply-add after the other.  roff == nullptr: N tiles of size b; else block i
+// covers rows roff[i] .. roff[i + 1] - 1.
+constexpr int AS_T = 64, AS_K = 32;
+__global__ void __launch_bounds__(256) k_assemble(const cf* __restrict__ th, long long nr, long long b, int N,
+                                                  const AsmTile* __restrict__ t, cf* __restrict__ Xh, int general,
+                                                  const long long* __restrict__ roff, int sub, int t0) {
+    // blockIdx.x: sub-block of the tile (sub x sub of them), blockIdx.y: the tile
+    int i, j;
+    const int e = t0 + blockIdx.y;
+    if (general) {
+        i = e / N;
+        j = e - i * N;
+    } else if (e < N) {
+        i = j = e;
+    } else {   // pair p = e - N: column j is the last with j N - j (j + 1) / 2 <= p
+        const int p = e - N;
+        int lo = 0, hi = N - 2;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if ((long long)mid * N - (long long)mid * (mid + 1) / 2 <= p)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        j = lo;
+        i = p - (j * N - j * (j + 1) / 2) + j + 1;
+    }
+    const AsmTile a = t[e];
+    const long long ri = roff ? roff[i] : i * b, rj = roff ? roff[j] : j * b;
+    const int di = (int)((roff ? roff[i + 1] : ri + b) - ri), dj = (int)((roff ? roff[j + 1] : rj + b) - rj);
+    const int r0 = blockIdx.x / sub * AS_T, c0 = blockIdx.x % sub * AS_T;
+    if (r0 >= di || c0 >= dj) return;
+    const bool diag = i == j && !general;
+    if (diag && r0 > c0) return;   // written as a mirror
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    float2 acc[4][4];
+    // the factors' rows (two of 64 x 33), then the mirrored block (64 x 65)
+    __shared__ cf buf[2 * AS_T * (AS_K + 1)];
+    static_assert(2 * (AS_K + 1) >= AS_T + 1, "the mirrored block fits");
+    if (i == j && a.dense) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int r = r0 + ty + 16 * u, c = c0 + tx + 16 * v;
+                acc[u][v] = make_float2(0.f, 0.f);
+                if (r >= di || c >= dj) continue;
+                const cf x = th[a.off_l + (long long)r * di + c];
+                acc[u][v] = x;
+                if (diag) {
+                    const cf y = th[a.off_l + (long long)c * di + r];
+                    acc[u][v] = make_float2(0.5f * (x.x + y.x), 0.5f * (x.y + y.y));
                 }
             }
-            Xh[e] = make_float2(x, y);
-            continue;
-        }
-        if (i < j) {  // mirror into the sub-diagonal tile
-            const long long tr = r;
-            r = c;
-            c = tr;
-            const int ti = i;
-            i = j;
-            j = ti;
-        }
-        long long rr = r - (roff ? roff[i] : i * b), cc = c - (roff ? roff[j] : j * b);
-        if (i == j && rr > cc) {  // low-rank diagonal: evaluate the upper triangle's entry
-            const long long t2 = rr;
-            rr = cc;
-            cc = t2;
-        }
-        const AsmTile& a = t[i == j ? i : N + (j * N - j * (j + 1) / 2 + (i - j - 1))];
-        float x = 0.f, y = 0.f;
-        if (i == j && a.dense) {
-            const long long di = roff ? roff[i + 1] - roff[i] : b;
-            const cf u = th[a.off_l + rr * di + cc], v = th[a.off_l + cc * di + rr];
-            x = 0.5f * (u.x + v.x);
-            y = 0.5f * (u.y + v.y);
-        } else {
-            const cf* L = th + a.off_l + rr * a.k;
-            const cf* R = th + a.off_r + cc * a.k;
-            for (int q = 0; q < a.k; ++q) {
-                const cf l = L[q], m = R[q];
-                x = fmaf(l.x, m.x, fmaf(-l.y, m.y, x));
-                y = fmaf(l.x, m.y, fmaf(l.y, m.x, y));
+    } else {
+        cf(*Ls)[AS_K + 1] = reinterpret_cast<cf(*)[AS_K + 1]>(buf);
+        cf(*Rs)[AS_K + 1] = Ls + AS_T;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[u][v] = make_float2(0.f, 0.f);
+        for (int k0 = 0; k0 < a.k; k0 += AS_K) {
+            const int kn = min(AS_K, a.k - k0);
+            __syncthreads();
+            for (int q = threadIdx.x; q < AS_T * AS_K; q += 256) {
+                const int r = q / AS_K, k = q % AS_K;
+                const bool in = k < kn;
+                Ls[r][k] = in && r0 + r < di ? th[a.off_l + (long long)(r0 + r) * a.k + k0 + k] : make_float2(0.f, 0.f);
+                Rs[r][k] = in && c0 + r < dj ? th[a.off_r + (long long)(c0 + r) * a.k + k0 + k] : make_float2(0.f, 0.f);
+            }
+            __syncthreads();
+            for (int k = 0; k < kn; ++k) {
+                cf l[4], m[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) l[u] = Ls[ty + 16 * u][k];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) m[v] = Rs[tx + 16 * v][k];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        acc[u][v].x = fmaf(l[u].x, m[v].x, fmaf(-l[u].y, m[v].y, acc[u][v].x));
+                        acc[u][v].y = fmaf(l[u].x, m[v].y, fmaf(l[u].y, m[v].x, acc[u][v].y));
+                    }
             }
         }
-        Xh[e] = make_float2(x, y);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int r = r0 + ty + 16 * u, c = c0 + tx + 16 * v;
+            if (r < di && c < dj && !(diag && r > c)) Xh[(ri + r) * nr + rj + c] = acc[u][v];
+        }
+    if (general) return;
+    // the mirror, through shared memory so that its rows are written whole
+    cf(*M)[AS_T + 1] = reinterpret_cast<cf(*)[AS_T + 1]>(buf);
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) M[tx + 16 * v][ty + 16 * u] = acc[u][v];
+    __syncthreads();
+    for (int q = threadIdx.x; q < AS_T * AS_T; q += 256) {
+        const int c = q / AS_T, r = q % AS_T;   // entry (r0 + r, c0 + c) to (c0 + c, r0 + r)
+        if (r0 + r < di && c0 + c < dj && !(diag && r0 + r >= c0 + c)) Xh[(rj + c0 + c) * nr + ri + r0 + r] = M[c][r];
     }
 }
 
 cudaError_t assemble_dense(const cf* theta, long long nr, long long b, int N, const AsmTile* tiles, cf* Xh,
                            cudaStream_t st, int general, const long long* roff) {
-    k_assemble<<<1024, 256, 0, st>>>(theta, nr, b, N, tiles, Xh, general, roff);
-    counted(1);
+    const int sub = (int)((b + AS_T - 1) / AS_T);   // b: the largest tile
+    const long long nt = general ? (long long)N * N : (long long)N * (N + 1) / 2;
+    for (long long t0 = 0; t0 < nt; t0 += 65535) {
+        const unsigned cnt = (unsigned)std::min<long long>(65535, nt - t0);
+        k_assemble<<<dim3((unsigned)(sub * sub), cnt), 256, 0, st>>>(theta, nr, b, N, tiles, Xh, general, roff, sub,
+                                                                     (int)t0);
+        counted(1);
+    }
     return cudaGetLastError();
 }
 
-// X[r, q] = Xh[inv[r], inv[q]]  (X = S X_h S^T)
-__global__ void k_unpermute(const cf* __restrict__ Xh, long long nr, const int32_t* __restrict__ inv,
-                            cf* __restrict__ X) {
-    const long long n2 = nr * nr;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n2;
-         e += (long long)gridDim.x * blockDim.x) {
-        const long long r = e / nr, q = e % nr;
-        X[e] = Xh[(long long)inv[r] * nr + inv[q]];
+// X[r, q] = Xh[inv[r], inv[q]]  (X = S X_h S^T): rows of X whole, the gather along
+// a row of X_h that fits L1
+__global__ void __launch_bounds__(256) k_unpermute(const cf* __restrict__ Xh, long long nr,
+                                                   const int32_t* __restrict__ inv, cf* __restrict__ X) {
+    for (long long r = blockIdx.x; r < nr; r += gridDim.x) {
+        const cf* src = Xh + (long long)inv[r] * nr;
+        cf* dst = X + r * nr;
+#pragma unroll 4
+        for (long long q = threadIdx.x; q < nr; q += blockDim.x) dst[q] = src[inv[q]];
     }
 }
 
 cudaError_t unpermute_dense(const cf* Xh, long long nr, const int32_t* perm, cf* X, cudaStream_t st) {
     const int32_t* inv = perm + nr;
-    k_unpermute<<<1024, 256, 0, st>>>(Xh, nr, inv, X);
+    k_unpermute<<<(unsigned)std::min<long long>(nr, 152 * 16), 256, 0, st>>>(Xh, nr, inv, X);
     counted(1);
     return cudaGetLastError();
 }

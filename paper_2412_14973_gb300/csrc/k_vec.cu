@@ -69,50 +69,78 @@ __device__ __forceinline__ double sum_slabs(const double* part, int n, double* s
 // ---------------------------------------------------------------------------
 // layout maps
 // ---------------------------------------------------------------------------
-__global__ void k_theta_to_panel(PanelMap m, const cf* __restrict__ th, cf* __restrict__ pan) {
-    const long long nlr = m.Ktot * m.b;
-    GRID_STRIDE(e, nlr) {
-        const long long g = e % m.Ktot, a = e / m.Ktot;
-        if (a < m.colrows[g]) pan[m.colpan[g] + a * m.panstride[g]] = th[m.colsrc[g] + a * m.colstride[g]];
+// Row a of panel column g, one block row of threads over 32 columns and 8 rows
+// (the columns' maps are read once per thread and 64 rows; a grid-stride loop with
+// a 64-bit division and a map lookup per value took 64 us for 64 MB).
+template <bool TO_PANEL>
+__global__ void __launch_bounds__(256) k_panel_map(PanelMap m, const cf* __restrict__ src, cf* __restrict__ dst,
+                                                   int gcols, int grows) {
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const long long nlb = (long long)gcols * grows;
+    for (long long e = blockIdx.x; e < nlb; e += gridDim.x) {
+        const long long g = e % gcols * 32 + tx;
+        const int a0 = (int)(e / gcols) * 64 + ty;
+        if (g >= m.Ktot) continue;
+        const int rows = min(m.colrows[g], a0 - ty + 64);
+        const long long tb = m.colsrc[g], pb = m.colpan[g];
+        const int ts = m.colstride[g], ps = m.panstride[g];
+#pragma unroll 8
+        for (int a = a0; a < rows; a += 8) {
+            const long long t = tb + (long long)a * ts, p = pb + (long long)a * ps;
+            if (TO_PANEL)
+                dst[p] = src[t];
+            else
+                dst[t] = src[p];
+        }
     }
     const long long bb = m.b * m.b;
     GRID_STRIDE(e, m.ndense * bb) {
         const long long t = e / bb, r = (e % bb) / m.b, c = e % m.b, n = m.zdim[t];
-        if (r < n && c < n) pan[m.zbase + m.zoff[t] + r * n + c] = th[m.zsrc[t] + r * n + c];
+        if (r < n && c < n) {
+            const long long th = m.zsrc[t] + r * n + c, pa = m.zbase + m.zoff[t] + r * n + c;
+            if (TO_PANEL)
+                dst[pa] = src[th];
+            else
+                dst[th] = src[pa];
+        }
     }
 }
 
-__global__ void k_panel_to_theta(PanelMap m, const cf* __restrict__ pan, cf* __restrict__ th) {
-    const long long nlr = m.Ktot * m.b;
-    GRID_STRIDE(e, nlr) {
-        const long long g = e % m.Ktot, a = e / m.Ktot;
-        if (a < m.colrows[g]) th[m.colsrc[g] + a * m.colstride[g]] = pan[m.colpan[g] + a * m.panstride[g]];
-    }
-    const long long bb = m.b * m.b;
-    GRID_STRIDE(e, m.ndense * bb) {
-        const long long t = e / bb, r = (e % bb) / m.b, c = e % m.b, n = m.zdim[t];
-        if (r < n && c < n) th[m.zsrc[t] + r * n + c] = pan[m.zbase + m.zoff[t] + r * n + c];
-    }
+static cudaError_t panel_map(const PanelMap& m, bool to_panel, const cf* src, cf* dst, cudaStream_t st) {
+    const long long gc = (m.Ktot + 31) / 32, gr = (m.b + 63) / 64;
+    const long long want = std::max(gc * gr, (m.ndense * m.b * m.b + 1023) / 1024);
+    const unsigned grid = (unsigned)std::max(1LL, std::min(want, 152LL * 64));
+    if (to_panel)
+        (void)launch_pass(k_panel_map<true>, dim3(grid), dim3(256), st, m, src, dst, (int)gc, (int)gr);
+    else
+        (void)launch_pass(k_panel_map<false>, dim3(grid), dim3(256), st, m, src, dst, (int)gc, (int)gr);
+    counted(1);
+    return cudaGetLastError();
 }
 
 cudaError_t theta_to_panel(const PanelMap& m, const cf* theta, cf* pan, cudaStream_t st) {
-    (void)launch_pass(k_theta_to_panel, dim3(1024), dim3(256), st, m, theta, pan);
-    counted(1);
-    return cudaGetLastError();
+    return panel_map(m, true, theta, pan, st);
 }
 cudaError_t panel_to_theta(const PanelMap& m, const cf* pan, cf* theta, cudaStream_t st) {
-    (void)launch_pass(k_panel_to_theta, dim3(1024), dim3(256), st, m, pan, theta);
-    counted(1);
-    return cudaGetLastError();
+    return panel_map(m, false, pan, theta, st);
 }
 
 // Dense tile t of a panel-ordered region: (offset, size) from the per-tile
 // tables, or the t-th of equal tiles of size b.
 __device__ __forceinline__ bool dense_tile(long long e, long long b, const long long* zoff, const int* zdim,
                                            long long& base, long long& n, long long& r, long long& c) {
-    const long long bb = b * b, t = e / bb;
-    r = (e % bb) / b;
-    c = e % b;
+    const long long bb = b * b;
+    long long t;
+    if (e < 0x7fffffffLL && bb < 0x7fffffffLL) {   // 64-bit divisions are long sequences
+        const unsigned ue = (unsigned)e, ub = (unsigned)b, ubb = (unsigned)bb, ut = ue / ubb, q = ue - ut * ubb;
+        t = ut;
+        r = q / ub;
+        c = q - (unsigned)r * ub;
+    } else {
+        t = e / bb;
+        r = (e % bb) / b;
+        c = e % b;
+    }
     if (!zoff) {
         base = t * bb;
         n = b;
@@ -319,14 +347,15 @@ __device__ __forceinline__ int ring_idx(const SolverDev& S, int j) {
 // whose rounding the exact line search and the descent test absorb.
 // 128 threads of <= 128 registers: a CTA fits beside the two GEMM CTAs of an SM
 constexpr int kLbThreads = 128;
-constexpr int kLbVals = 5 * kLbGroup + 1;
 constexpr int kLbLd = kLbThreads + 8;   // row length of the block's sums: 4 rows read together lie in different banks
 
-__device__ void lb_solve(const SolverDev& S, int cnt, int nblk, double* val, double* mat);
+__device__ void lb_solve(const SolverDev& S, int cnt, int ncl, double* val, double* mat);
 
-// Blocks of the direction's inner products: 8 values of each vector per thread
+// Blocks of the direction's inner products: 4 values of each vector per thread (a
+// round of its 23 loads is a memory latency, a block's sums are 2 us of FP64 adds)
+// until there are kRedBlocks
 inline int lb_blocks(long long n2) {
-    const long long b = (n2 + 8 * kLbThreads - 1) / (8 * kLbThreads);
+    const long long b = (n2 + 4 * kLbThreads - 1) / (4 * kLbThreads);
     return (int)(b < 1 ? 1 : b > kRedBlocks ? kRedBlocks : b);
 }
 
@@ -377,7 +406,8 @@ __global__ void __launch_bounds__(kLbThreads, 4) k_lb_dots(SolverDev S, int j0, 
             for (int t = 0; t < 5; ++t) shv[(jj * 5 + t) * kLbLd + threadIdx.x] = acc[jj][t];
         shv[5 * kLbGroup * kLbLd + threadIdx.x] = gg;
         __syncthreads();
-        const int lane = threadIdx.x & 31, l8 = lane & 7;
+        const int l8 = threadIdx.x & 7;
+        double* const mine = S.lbpart + ((long long)(j0 / kLbGroup) * kRedBlocks + blockIdx.x) * kLbRow;
         for (int v0 = 0; v0 < kLbVals; v0 += kLbThreads / 8) {
             const int v = v0 + (threadIdx.x >> 3);   // 8 lanes per value
             const float* row = shv + min(v, kLbVals - 1) * kLbLd;
@@ -386,24 +416,34 @@ __global__ void __launch_bounds__(kLbThreads, 4) k_lb_dots(SolverDev S, int j0, 
             for (int i = 0; i < kLbThreads / 8; ++i) r += (double)row[l8 + 8 * i];
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o, 8);
-            if (l8 == 0) {
-                if (v < 5 * jc)
-                    S.lbpart[((long long)(j0 / kLbGroup) * 5 * kLbGroup + v) * kRedBlocks + blockIdx.x] = r;
-                else if (v == kLbVals - 1 && j0 == 0)
-                    S.lbpart[kLbGGOff + blockIdx.x] = r;
-            }
+            if (l8 == 0 && v < kLbVals) mine[v] = r;
         }
     }
-    if (!last || !last_block(reinterpret_cast<unsigned*>(S.ints + CT_DIR), gridDim.x)) return;
+    // The last block of every 16 adds its cluster's partials up, the last of those
+    // finishes: a thread per value, and 16 (38) additions each on as many SMs, where
+    // one block adding 608 x 51 doubles took 10 us.
+    const int cl = blockIdx.x / kLbCluster, ncl = (gridDim.x + kLbCluster - 1) / kLbCluster;
+    const int in_cl = min(kLbCluster, (int)gridDim.x - cl * kLbCluster);
+    unsigned* const ctr = reinterpret_cast<unsigned*>(S.lbctr);
+    if (!last_block(ctr + 1 + cl, in_cl)) return;
+    const int grp = j0 / kLbGroup, t = threadIdx.x;
+    if (j0 < cnt && t < kLbVals) {
+        const double* q = S.lbpart + ((long long)grp * kRedBlocks + cl * kLbCluster) * kLbRow + t;
+        double a = 0.0;
+#pragma unroll 4
+        for (int i = 0; i < in_cl; ++i) a += q[(long long)i * kLbRow];
+        S.lbsum[((long long)grp * kLbClusters + cl) * kLbRow + t] = a;
+    }
+    if (!last || !last_block(ctr, ncl)) return;
     double* const mat = reinterpret_cast<double*>(shv);   // 2 x 32 x 33 doubles and 161 values
-    lb_solve(S, cnt, gridDim.x, mat + 2 * 32 * 33, mat);
+    lb_solve(S, cnt, ncl, mat + 2 * 32 * 33, mat);
 }
 static_assert(sizeof(double) * (2 * 32 * 33 + 161) <= sizeof(float) * kLbVals * kLbLd, "lb_solve's storage");
 
-// One block: finalise the partials (a warp per two values, fixed order), update the
+// One block: finalise the cluster sums (a thread per value, fixed order), update the
 // newest pair's row / column of S^T Y and Y^T Y, then (warp 0, a lane per
 // pair) the triangular solves; coefficients to acoef, gamma to sc[SC_GAMMA].
-__device__ void lb_solve(const SolverDev& S, int cnt, int nblk, double* val, double* mat) {
+__device__ void lb_solve(const SolverDev& S, int cnt, int ncl, double* val, double* mat) {
     double* const Rm = mat;
     double* const Ym = mat + 32 * 33;
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -415,43 +455,43 @@ __device__ void lb_solve(const SolverDev& S, int cnt, int nblk, double* val, dou
         }
         return;
     }
-    const int nval = 5 * cnt + 1;   // the last value is <g, g>
-    auto row = [&](int v) {
-        return v == 5 * cnt ? S.lbpart + kLbGGOff : S.lbpart + (long long)v * kRedBlocks;
-    };
-    for (int v = 2 * w; v < nval; v += 2 * (kLbThreads / 32)) {
-        const double* r0 = row(v);
-        const double* r1 = row(min(v + 1, nval - 1));
-        double a0 = 0.0, a1 = 0.0;
-#pragma unroll 5
-        for (int b = l; b < nblk; b += 32) {
-            a0 += r0[b];
-            a1 += r1[b];
-        }
-        a0 = warp_sum(a0);
-        a1 = warp_sum(a1);
-        if (l == 0) {
-            val[v] = a0;
-            if (v + 1 < nval) val[v + 1] = a1;
-        }
-    }
-    __syncthreads();
     const int R = S.ring, k = cnt;
     const int nw = ring_idx(S, 0);
-    if (threadIdx.x < cnt) {
-        const int j = threadIdx.x, a = ring_idx(S, j);
-        S.SYm[a * R + nw] = val[j * 5 + 2];
-        if (j > 0) S.SYm[nw * R + a] = val[j * 5 + 3];
-        S.YYm[a * R + nw] = val[j * 5 + 4];
-        S.YYm[nw * R + a] = val[j * 5 + 4];
+    // val[5 j + kind] of the j-th newest pair, val[5 cnt] = <g, g>
+    for (int v = threadIdx.x; v <= 5 * cnt; v += kLbThreads) {
+        const int grp = v == 5 * cnt ? 0 : v / (5 * kLbGroup), t = v == 5 * cnt ? kLbVals - 1 : v % (5 * kLbGroup);
+        const double* q = S.lbsum + (long long)grp * kLbClusters * kLbRow + t;
+        double a0 = 0.0, a1 = 0.0;
+#pragma unroll 4
+        for (int i = 0; i + 1 < ncl; i += 2) {
+            a0 += q[(long long)i * kLbRow];
+            a1 += q[(long long)(i + 1) * kLbRow];
+        }
+        if (ncl & 1) a0 += q[(long long)(ncl - 1) * kLbRow];
+        val[v] = a0 + a1;
     }
-    __syncthreads();
-    // oldest first: position i holds the (cnt - 1 - i)-th newest pair
+    // oldest first: position i holds the (cnt - 1 - i)-th newest pair; the newest
+    // pair's row and column come from val below
     for (int e = threadIdx.x; e < k * k; e += kLbThreads) {
         const int i = e / k, j = e - i * k;
         const int si = ring_idx(S, k - 1 - i), sj = ring_idx(S, k - 1 - j);
-        Rm[i * 33 + j] = S.SYm[si * R + sj];
-        Ym[i * 33 + j] = S.YYm[si * R + sj];
+        if (si != nw && sj != nw) {
+            Rm[i * 33 + j] = S.SYm[si * R + sj];
+            Ym[i * 33 + j] = S.YYm[si * R + sj];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < cnt) {
+        const int j = threadIdx.x, a = ring_idx(S, j), i = k - 1 - j;
+        const double sy = val[j * 5 + 2], ys = val[j * 5 + 3], yy = val[j * 5 + 4];   // <s_j,y_n>, <s_n,y_j>, <y_j,y_n>
+        S.SYm[a * R + nw] = sy;
+        if (j > 0) S.SYm[nw * R + a] = ys;
+        S.YYm[a * R + nw] = yy;
+        S.YYm[nw * R + a] = yy;
+        Rm[i * 33 + k - 1] = sy;
+        if (j > 0) Rm[(k - 1) * 33 + i] = ys;
+        Ym[i * 33 + k - 1] = yy;
+        Ym[(k - 1) * 33 + i] = yy;
     }
     __syncthreads();
     if (w != 0) return;
@@ -850,8 +890,8 @@ __global__ void __launch_bounds__(kRedThreads) k_gradient_pair(SolverDev S, cons
     const double t = block_sums(w, sh);
     if (threadIdx.x < 3) S.partp[blockIdx.x * 3 + threadIdx.x] = t;
     if (!last_block(reinterpret_cast<unsigned*>(S.ints + CT_PAIR), gridDim.x)) return;
-    const double d = sum_slabs<3>(S.partp, gridDim.x, sh[0]);
     const double rr = sum_part(partf, nf, sh);
+    const double d = sum_slabs<3>(S.partp, gridDim.x, sh[0]);
     if (threadIdx.x >= 32) return;
     const double dss = __shfl_sync(0xffffffffu, d, 0), dsy = __shfl_sync(0xffffffffu, d, 1),
                  dyy = __shfl_sync(0xffffffffu, d, 2);

@@ -15,14 +15,15 @@ enum IntSlot { SI_CNT = 0, SI_NEWEST, SI_ITERS, SI_RESTARTS, SI_STATUS, SI_RFLAG
 
 // after the counters: [SI_COUNT + 1] the contractions' error word, then the block
 // counters of the passes whose last block finishes their sums (zero between launches)
-enum CounterSlot { CT_DIR = SI_COUNT + 2, CT_LINE, CT_PAIR, CT_NORM };
+enum CounterSlot { CT_LINE = SI_COUNT + 2, CT_PAIR, CT_DIR };   // CT_DIR: 1 + kLbClusters of them
 
-// compact L-BFGS: pairs per inner-product pass, and the partial storage for
-// the largest memory (32 pairs; value by value, kRedBlocks partials each), followed
-// by one slab of <g, g> partials
-constexpr int kLbGroup = 10;
-constexpr long long kLbGGOff = (long long)kRedBlocks * 5 * kLbGroup * ((32 + kLbGroup - 1) / kLbGroup);
-constexpr long long kLbPartDoubles = kLbGGOff + kRedBlocks;
+// compact L-BFGS: pairs per inner-product pass; a block leaves kLbVals partials (a
+// row of kLbRow), the last block of every kLbCluster adds its cluster's up
+constexpr int kLbGroup = 10, kLbGroups = (32 + kLbGroup - 1) / kLbGroup;
+constexpr int kLbVals = 5 * kLbGroup + 1, kLbRow = kLbVals + 1;
+constexpr int kLbCluster = 16, kLbClusters = (kRedBlocks + kLbCluster - 1) / kLbCluster;
+constexpr long long kLbSumOff = (long long)kLbGroups * kRedBlocks * kLbRow;
+constexpr long long kLbPartDoubles = kLbSumOff + (long long)kLbGroups * kLbClusters * kLbRow;
 
 struct SolverDev {
     long long n2;        // floats per theta-space vector (2 * n_theta)
@@ -36,7 +37,9 @@ struct SolverDev {
     double* acoef;       // [64] direction coefficients: [j] of s_j, [32 + j] of y_j (j-th newest)
     double* SYm;         // [ring * ring] <s_a, y_b> by slot
     double* YYm;         // [ring * ring] <y_a, y_b> by slot
-    double* lbpart;      // partials of the direction's inner products
+    double* lbpart;      // partials of the direction's inner products ...
+    double* lbsum;       // ... and their cluster sums
+    unsigned* lbctr;     // block counters: [0] clusters, [1 + i] blocks of cluster i (zero between launches)
     double* sc;          // ScalarSlot values
     int* ints;           // IntSlot values
     double* fhist;       // [TLR_MAX_HIST]
@@ -48,7 +51,7 @@ struct SolverDev {
 // blocks of a reduction over n values: enough work for 256 threads each, at most
 // kRedBlocks (a function of n alone, so the order of every sum is fixed)
 inline int red_blocks(long long n) {
-    const long long b = (n + 2047) / 2048;
+    const long long b = (n + 1023) / 1024;
     return (int)(b < 1 ? 1 : b > kRedBlocks ? kRedBlocks : b);
 }
 
