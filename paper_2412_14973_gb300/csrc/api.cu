@@ -229,6 +229,36 @@ struct HostStats {
     double fhist[TLR_MAX_HIST];
 };
 
+// Pinned blocks for the statistics of solves: mapping and unmapping one per handle
+// took 0.2 ms.  At most kMostPinned idle ones are kept; tlr_mdd_trim_pool frees them.
+constexpr size_t kMostPinned = 16;
+std::mutex g_pinned_mu;
+std::vector<HostStats*> g_pinned;
+
+cudaError_t pinned_get(HostStats** p) {
+    {
+        std::lock_guard<std::mutex> lk(g_pinned_mu);
+        if (!g_pinned.empty()) {
+            *p = g_pinned.back();
+            g_pinned.pop_back();
+            return cudaSuccess;
+        }
+    }
+    // usable from every device's context
+    return cudaHostAlloc((void**)p, sizeof(HostStats), cudaHostAllocPortable);
+}
+void pinned_put(HostStats* p) {
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lk(g_pinned_mu);
+        if (g_pinned.size() < kMostPinned) {
+            g_pinned.push_back(p);
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
 struct GraphKey {
     double lam0 = -1, decay = 0, rho = 0;
     int stages = -1, admm = -1, lbfgs = -1, mem = -1, timing = -1, flags = -1;
@@ -816,7 +846,9 @@ int build_tables(tlr_mdd_s* h, char* tab_base, std::vector<HostTable>* keep) {
     const long long ns = L.ns;
     const size_t slot = ((sizeof(GProb) * (3 * (size_t)L.N + 1)) + 255) & ~size_t(255);
     int ti = 0;
+    std::vector<char> img(8 * slot);   // all tables, copied at once
     auto upload = [&](GemmLaunch& G, std::vector<GProb>& v, int am, int bm, int epi) -> int {
+        char* const at = img.data() + slot * ti;
         GProb* dst = reinterpret_cast<GProb*>(tab_base + slot * ti++);
         G.d_probs = dst;
         G.nprob = (int)v.size();
@@ -834,10 +866,7 @@ int build_tables(tlr_mdd_s* h, char* tab_base, std::vector<HostTable>* keep) {
         G.prec = h->d.precision;
         G.persistent = tensor_core(G.prec) && ((persist_classes() >> G.cls) & 1);
         G.err = h->ints + SI_COUNT + 1;
-        if (!v.empty()) {
-            cudaError_t e = cudaMemcpyAsync(dst, v.data(), v.size() * sizeof(GProb), cudaMemcpyHostToDevice, h->st);
-            if (e != cudaSuccess) return -1;
-        }
+        if (!v.empty()) memcpy(at, v.data(), v.size() * sizeof(GProb));
         if (keep) keep->push_back(HostTable{&G, v});
         return 0;
     };
@@ -986,7 +1015,7 @@ int build_tables(tlr_mdd_s* h, char* tab_base, std::vector<HostTable>* keep) {
         h->Lp.kchunk = h->kchunk;
         h->Lp.part_stride = L.nth;
     }
-    return 0;
+    return cudaMemcpyAsync(tab_base, img.data(), img.size(), cudaMemcpyHostToDevice, h->st) == cudaSuccess ? 0 : -1;
 }
 
 // ---------------------------------------------------------------------------
@@ -1062,8 +1091,22 @@ int build_tc(tlr_mdd_s* h, std::vector<HostTable>& tabs) {
             }
     h->packed_size = total;
     CK(h, ws_alloc((void**)&h->packed, std::max<size_t>(total, 256), h->st));
-    // padding rows and k-slots of every packed operand stay zero from here on
-    CK(h, cudaMemsetAsync(h->packed, 0, std::max<size_t>(total, 256), h->st));
+    // padding rows and k-slots of every packed operand stay zero from here on (an
+    // operand without padding is written whole before it is read); neighbouring
+    // operands are cleared together
+    {
+        size_t lo = 0, hi = 0;
+        for (auto& ko : order) {
+            const PackKey& k = ko.first;
+            if (k.R % k.TR == 0 && k.K % 16 == 0) continue;
+            if (ko.second != hi) {
+                if (hi > lo) CK(h, cudaMemsetAsync(h->packed + lo, 0, hi - lo, h->st));
+                lo = ko.second;
+            }
+            hi = ko.second + (size_t)((packed_bytes(k.R, k.K, k.TR) + 1023) & ~1023LL);
+        }
+        if (hi > lo) CK(h, cudaMemsetAsync(h->packed + lo, 0, hi - lo, h->st));
+    }
     auto job_of = [&](const PackKey& k, size_t off) {
         PackJob j;
         j.src = (const cf*)k.src;
@@ -1270,9 +1313,13 @@ int build_tc(tlr_mdd_s* h, std::vector<HostTable>& tabs) {
     const size_t rpo = bytes;
     bytes += (2 * (size_t)L.N * sizeof(char*) + 255) & ~size_t(255);
     CK(h, ws_alloc((void**)&h->tcp_tables, std::max<size_t>(bytes, 256), h->st));
+    std::vector<char> img(std::max<size_t>(bytes, 256));   // all tables, copied at once
+    auto put = [&](size_t at, const void* src, size_t n) {
+        if (n) memcpy(img.data() + at, src, n);
+    };
     if (vpack) {
         char** d_rowptr = reinterpret_cast<char**>(h->tcp_tables + ro);
-        CK(h, cudaMemcpyAsync(d_rowptr, rowptr.data(), rowptr.size() * sizeof(char*), cudaMemcpyHostToDevice, h->st));
+        put(ro, rowptr.data(), rowptr.size() * sizeof(char*));
         for (size_t ti = 0; ti < tabs.size(); ++ti)
             if (tabs[ti].G == &h->Lc_v) {
                 for (auto& f : vfix) pp[ti][f.first].rowptr = d_rowptr + f.second;
@@ -1285,23 +1332,19 @@ int build_tc(tlr_mdd_s* h, std::vector<HostTable>& tabs) {
         G.d_jobs = reinterpret_cast<PackJob*>(h->tcp_tables + jo[ti]);
         G.njobs = (int)jobs[ti].size();
         G.max_items = maxit[ti];
-        if (!pp[ti].empty())
-            CK(h, cudaMemcpyAsync(G.d_pprobs, pp[ti].data(), pp[ti].size() * sizeof(PProb), cudaMemcpyHostToDevice,
-                                  h->st));
-        if (!jobs[ti].empty())
-            CK(h, cudaMemcpyAsync(G.d_jobs, jobs[ti].data(), jobs[ti].size() * sizeof(PackJob),
-                                  cudaMemcpyHostToDevice, h->st));
+        put(po[ti], pp[ti].data(), pp[ti].size() * sizeof(PProb));
+        put(jo[ti], jobs[ti].data(), jobs[ti].size() * sizeof(PackJob));
     }
     if (rfuse) {
         h->d_rkn = reinterpret_cast<char**>(h->tcp_tables + rpo);
         h->d_rmk = h->d_rkn + L.N;
-        CK(h, cudaMemcpyAsync(h->d_rkn, rkn.data(), L.N * sizeof(char*), cudaMemcpyHostToDevice, h->st));
-        CK(h, cudaMemcpyAsync(h->d_rmk, rmk.data(), L.N * sizeof(char*), cudaMemcpyHostToDevice, h->st));
+        put(rpo, rkn.data(), L.N * sizeof(char*));
+        put(rpo + L.N * sizeof(char*), rmk.data(), L.N * sizeof(char*));
         h->rstep_on = true;
     }
     if (!ttp.empty()) {
         TPackTile* d_ttp = reinterpret_cast<TPackTile*>(h->tcp_tables + tpo);
-        CK(h, cudaMemcpyAsync(d_ttp, ttp.data(), ttp.size() * sizeof(TPackTile), cudaMemcpyHostToDevice, h->st));
+        put(tpo, ttp.data(), ttp.size() * sizeof(TPackTile));
         h->Le_a1.d_gpack = d_ttp;
         h->Le_a1.n_gpack = (int)ttp.size();
         h->Le_a1.gpack_src = h->Tp;
@@ -1309,15 +1352,13 @@ int build_tc(tlr_mdd_s* h, std::vector<HostTable>& tabs) {
     }
     h->d_tpack = reinterpret_cast<TPackTile*>(h->tcp_tables + to);
     h->n_tpack = (int)tt.size();
-    if (!tt.empty())
-        CK(h, cudaMemcpyAsync(h->d_tpack, tt.data(), tt.size() * sizeof(TPackTile), cudaMemcpyHostToDevice, h->st));
+    put(to, tt.data(), tt.size() * sizeof(TPackTile));
     h->d_static_jobs = reinterpret_cast<PackJob*>(h->tcp_tables + so);
     h->n_static_jobs = (int)sjobs.size();
     h->static_items = smax;
-    if (!sjobs.empty())
-        CK(h, cudaMemcpyAsync(h->d_static_jobs, sjobs.data(), sjobs.size() * sizeof(PackJob), cudaMemcpyHostToDevice,
-                              h->st));
-    CK(h, cudaStreamSynchronize(h->st));   // host vectors go out of scope
+    put(so, sjobs.data(), sjobs.size() * sizeof(PackJob));
+    // (pageable memory is staged before the call returns)
+    CK(h, cudaMemcpyAsync(h->tcp_tables, img.data(), bytes, cudaMemcpyHostToDevice, h->st));
     return TLR_OK;
 }
 
@@ -1466,6 +1507,12 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
         if (h->packed) cudaFreeAsync(h->packed, h->st);
         if (h->tcp_tables) cudaFreeAsync(h->tcp_tables, h->st);
         if (h->arena) cudaFreeAsync(h->arena, h->st);
+        if (h->ev0) cudaEventDestroy(h->ev0);
+        if (h->ev1) cudaEventDestroy(h->ev1);
+        if (h->hstats) {
+            cudaStreamSynchronize(h->st);
+            pinned_put(h->hstats);
+        }
         delete h;
         return code;
     };
@@ -1503,11 +1550,15 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
     } else {
         long long n = 1;
         while (n < d->nx || n < d->ny) n <<= 1;
-        int32_t* slot = nullptr;
-        CKF(cudaMallocAsync((void**)&slot, (size_t)(n * n) * sizeof(int32_t), h->st));
-        cudaError_t e = hilbert_perm(d->nx, d->ny, h->perm, slot, h->st);
-        cudaFreeAsync(slot, h->st);
-        CKF(e);
+        // its slots (n^2 of them) in the work panels, or of their own where those are too small
+        const size_t need = (size_t)(n * n) * sizeof(int32_t);
+        Scratch own;
+        int32_t* slot = reinterpret_cast<int32_t*>(h->R);
+        if (need > (size_t)(reinterpret_cast<char*>(h->Zs) - reinterpret_cast<char*>(h->R))) {
+            CKF(own.get(need, h->st));
+            slot = reinterpret_cast<int32_t*>(own.ptr());
+        }
+        CKF(hilbert_perm(d->nx, d->ny, h->perm, slot, h->st));
     }
     {
         int rc = load_data(h, D, U, d->input_memory);
@@ -1516,24 +1567,27 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
             return fail(rc);
         }
     }
-    // maps
-    if (L.Ktot > 0)
-        CKF(cudaMemcpyAsync(h->d_partner, L.partner.data(), L.Ktot * sizeof(int), cudaMemcpyHostToDevice, h->st));
-    if (L.general && L.KtotB > 0)
-        CKF(cudaMemcpyAsync(h->d_partnerB, L.partnerB.data(), L.KtotB * sizeof(int), cudaMemcpyHostToDevice, h->st));
-    if (L.ncol > 0) {
-        CKF(cudaMemcpyAsync((void*)h->pm.colsrc, L.colsrc.data(), L.ncol * sizeof(long long), cudaMemcpyHostToDevice, h->st));
-        CKF(cudaMemcpyAsync((void*)h->pm.colstride, L.colstride.data(), L.ncol * sizeof(int), cudaMemcpyHostToDevice, h->st));
-        CKF(cudaMemcpyAsync((void*)h->pm.colpan, L.colpan.data(), L.ncol * sizeof(long long), cudaMemcpyHostToDevice, h->st));
-        CKF(cudaMemcpyAsync((void*)h->pm.panstride, L.panstride.data(), L.ncol * sizeof(int), cudaMemcpyHostToDevice, h->st));
-        CKF(cudaMemcpyAsync((void*)h->pm.colrows, L.colrows.data(), L.ncol * sizeof(int), cudaMemcpyHostToDevice, h->st));
+    // maps: adjacent in the arena (carve), copied at once
+    {
+        char* const lo = reinterpret_cast<char*>(h->d_partner);
+        std::vector<char> img(reinterpret_cast<char*>(h->d_roff + L.N + 1) - lo);
+        auto put = [&](const void* at, const auto& v) {
+            if (!v.empty()) memcpy(img.data() + (reinterpret_cast<const char*>(at) - lo), v.data(), v.size() * sizeof(v[0]));
+        };
+        put(h->d_partner, L.partner);
+        if (L.general) put(h->d_partnerB, L.partnerB);
+        put(h->pm.colsrc, L.colsrc);
+        put(h->pm.colstride, L.colstride);
+        put(h->pm.colpan, L.colpan);
+        put(h->pm.panstride, L.panstride);
+        put(h->pm.colrows, L.colrows);
+        put(h->pm.zsrc, L.zsrc);
+        put(h->pm.zoff, L.zoff);
+        put(h->pm.zdim, L.zdim);
+        const std::vector<long long> roff(L.roff.begin(), L.roff.end());
+        put(h->d_roff, roff);
+        CKF(cudaMemcpyAsync(lo, img.data(), img.size(), cudaMemcpyHostToDevice, h->st));
     }
-    if (L.ndense > 0) {
-        CKF(cudaMemcpyAsync((void*)h->pm.zsrc, L.zsrc.data(), L.ndense * sizeof(long long), cudaMemcpyHostToDevice, h->st));
-        CKF(cudaMemcpyAsync((void*)h->pm.zoff, L.zoff.data(), L.ndense * sizeof(long long), cudaMemcpyHostToDevice, h->st));
-        CKF(cudaMemcpyAsync((void*)h->pm.zdim, L.zdim.data(), L.ndense * sizeof(int), cudaMemcpyHostToDevice, h->st));
-    }
-    CKF(cudaMemcpyAsync(h->d_roff, L.roff.data(), (L.N + 1) * sizeof(long long), cudaMemcpyHostToDevice, h->st));
     // solver counters and the contraction kernels' error word start at zero
     CKF(cudaMemsetAsync(h->ints, 0, kIntSlots * sizeof(int), h->st));
     std::vector<HostTable> tabs;
@@ -1552,13 +1606,14 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
     }
     CKF(cudaEventCreate(&h->ev0));
     CKF(cudaEventCreate(&h->ev1));
-    CKF(cudaMallocHost((void**)&h->hstats, sizeof(HostStats)));
+    CKF(pinned_get(&h->hstats));
     if (tensor_core(d->precision))
         CKF(gemm_tc_prepare());
     else
         CKF(gemm_f32_prepare());
+    CKF(cudaMemcpyAsync(h->hstats->sc, h->scal, sizeof(double), cudaMemcpyDeviceToHost, h->st));
     CKF(cudaStreamSynchronize(h->st));
-    CKF(cudaMemcpy(&h->alpha, h->scal, sizeof(double), cudaMemcpyDeviceToHost));
+    h->alpha = h->hstats->sc[0];
 #undef CKF
     *out = h;
     return TLR_OK;
@@ -2339,6 +2394,12 @@ int tlr_mdd_trim_pool(int64_t keep_bytes, int64_t* reserved) {
     cudaMemPool_t p = nullptr;
     CK((tlr_mdd_s*)nullptr, ws_pool(&p));
     CK((tlr_mdd_s*)nullptr, cudaMemPoolTrimTo(p, (size_t)keep_bytes));
+    std::vector<HostStats*> idle;
+    {
+        std::lock_guard<std::mutex> lk(g_pinned_mu);
+        idle.swap(g_pinned);
+    }
+    for (HostStats* q : idle) cudaFreeHost(q);
     if (reserved) {
         unsigned long long r = 0;
         CK((tlr_mdd_s*)nullptr, cudaMemPoolGetAttribute(p, cudaMemPoolAttrReservedMemCurrent, &r));
@@ -2362,7 +2423,6 @@ int tlr_mdd_destroy(tlr_mdd_t* h) {
         cudaEventDestroy(t.a);
         cudaEventDestroy(t.b);
     }
-    if (h->hstats) cudaFreeHost(h->hstats);
     if (h->ring) cudaFreeAsync(h->ring, h->st);
     if (h->packed) cudaFreeAsync(h->packed, h->st);
     if (h->tcp_tables) cudaFreeAsync(h->tcp_tables, h->st);
@@ -2370,6 +2430,7 @@ int tlr_mdd_destroy(tlr_mdd_t* h) {
     if (h->ev0) cudaEventDestroy(h->ev0);
     if (h->ev1) cudaEventDestroy(h->ev1);
     cudaError_t e = cudaStreamSynchronize(h->st);
+    pinned_put(h->hstats);   // no copy into it is in flight any more
     delete h;
     return e == cudaSuccess ? TLR_OK : TLR_ERR_CUDA;
 }
