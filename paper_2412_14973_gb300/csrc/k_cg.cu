@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(256) k_cg_dir(cf* __restrict__ x, cf* __restri
     if (c >= n) return;   // the packing's padding stays zero
     const bool vec = (n & 1) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;   // x is the caller's buffer
     const int nkc = (n + 15) >> 4;
-    char* const tile = pk + ((long long)blockIdx.y * nkc + blockIdx.x) * kPackTile + ((lane & 7) >> 2) * 128 + (lane & 3) * 4;
+    char* const tile = pk + ((long long)blockIdx.y * nkc + blockIdx.x) * kPackTile;
     float4 rv[4], pv[4], xv[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -210,7 +210,8 @@ __global__ void __launch_bounds__(256) k_cg_dir(cf* __restrict__ x, cf* __restri
                 p[o + 1] = make_float2(q.z, q.w);
             }
         }
-        if (pk) pk_store2(tile + row_off(kFmtBF16X3, rl), make_float2(q.x, q.y), make_float2(q.z, q.w));
+        if (pk)
+            pk_store2(tile + row_off(kFmtBF16X3, rl), kFmtBF16X3, lane & 7, make_float2(q.x, q.y), make_float2(q.z, q.w));
     }
 }
 

@@ -59,8 +59,16 @@ __device__ __forceinline__ void pk_store8(char* row, int fmt, int kg, const floa
         *reinterpret_cast<uint4*>(dst + q * 4096) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
 }
 
-// Two neighbouring values (even k) of a BF16x3 row, 4 bytes per plane, at their place
-__device__ __forceinline__ void pk_store2(char* dst, float2 a, float2 b) {
+// Two neighbouring values, k = 2 q and 2 q + 1 (q < 8) of a row of a packed tile, row
+// as for pk_store8: 4 bytes per plane (BF16x3) or 8 (TF32)
+__device__ __forceinline__ void pk_store2(char* row, int fmt, int q, float2 a, float2 b) {
+    if (fmt == kFmtTF32) {
+        char* d = row + (q >> 1) * 128 + (q & 1) * 8;
+        *reinterpret_cast<uint2*>(d) = make_uint2(tf32_rna(a.x), tf32_rna(b.x));
+        *reinterpret_cast<uint2*>(d + 8192) = make_uint2(tf32_rna(a.y), tf32_rna(b.y));
+        return;
+    }
+    char* dst = row + (q >> 2) * 128 + (q & 3) * 4;
     const float x[2][2] = {{a.x, b.x}, {a.y, b.y}};
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
