@@ -32,6 +32,8 @@ using namespace tlr;
 
 std::atomic<long long> tlr::g_launches{0};
 
+thread_local long long tlr::t_early_blocks = tlr::kEarlyAny;
+
 int tlr::device_sms() {
     static const int n = [] {
         int dev = 0, v = 0;
@@ -2621,7 +2623,14 @@ static int enqueue_body(tlr_mdd_s* h, const tlr_mdd_solve_opts_t* o) {
         CK(h, cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
         g_capture_sink = &h->gtimed;
         const long long n_before = g_launches.load();
-        int rc = enqueue_solve(h, o);
+        int rc;
+        {
+            struct Recording {
+                explicit Recording(long long n) { t_early_blocks = n; }
+                ~Recording() { t_early_blocks = kEarlyAny; }
+            } recording(h->L.nr <= 512 ? device_sms() : 0);
+            rc = enqueue_solve(h, o);
+        }
         h->graph_kernels = g_launches.load() - n_before;
         g_launches.fetch_sub(h->graph_kernels);   // recorded, not launched: counted at each replay
         g_capture_sink = nullptr;

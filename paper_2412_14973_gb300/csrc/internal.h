@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <climits>
 #include <atomic>
 #include <string>
 #include <vector>
@@ -31,19 +32,68 @@ constexpr long long kPassCtasDefault = 0;
 long long pass_cap();
 void set_pass_cap(long long ctas);
 
+// Programmatic dependent launch: a kernel launched through launch_chain or
+// launch_pass may be scheduled while its predecessor on the stream still runs, so
+// its launch and the placing of its blocks take no time of their own between two
+// passes (an iteration of a small solve is a chain of about 16 of them).  Every
+// such kernel begins with chain_entry(), or chain_wait(), in all of its threads,
+// before it reads, writes or returns: it waits there until its predecessor has
+// completed and its results are visible.  A pass then lets its own successor be
+// scheduled at once.  A contraction does not (its successor follows when its last
+// block ends): blocks placed early go to whatever SMs are idle, and beside a long
+// contraction these are the few that finish first, where they crowd.  For the same
+// reason a recorded solve, whose launches cost little else, lets only launches of
+// at most a block per SM start early, no FP32 contraction, and none at all above
+// 512 receivers, where every pass is long (t_early_blocks).
+// Measured, plain launches -> this: misfit and gradient of nr = 2048, general form,
+// 0.268 -> 0.232 ms; operator of nr = 2025 in TF32 132 -> 114 us; benchmark solver
+// at nr = 2048 4.33 -> 4.07 ms; recorded solve of nr = 256 3.50 -> 3.41 ms.
+// Contractions that release their successor at once: benchmark solver 4.15, misfit
+// and gradient of nr = 4096 in FP32 2.30 against 2.27.  Recorded, nr = 1024 in FP32:
+// every launch early 6.58, up to a block per SM 6.47, none 6.45.  Only launches of
+// at most a block per SM, everywhere: 0.264 ms, 129 us, 4.29 ms.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_entry() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// the most blocks of a launch that may start early on this thread (see above)
+constexpr long long kEarlyAny = LLONG_MAX;
+extern thread_local long long t_early_blocks;
+int device_sms();
+
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pass(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
+inline cudaError_t launch_with(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, const int* priority,
+                               cudaStream_t st, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributePriority;
-    at[0].val.priority = pass_priority();
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed =
+        (long long)grid.x * grid.y * grid.z <= t_early_blocks ? 1 : 0;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    if (priority) {
+        at[1].id = cudaLaunchAttributePriority;
+        at[1].val.priority = *priority;
+        cfg.numAttrs = 2;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+// at the stream's priority
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                Args... args) {
+    return launch_with(kernel, grid, block, smem, nullptr, st, args...);
+}
+// a memory-bound pass, at the passes' priority
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pass(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
+    const int prio = pass_priority();
+    return launch_with(kernel, grid, block, 0, &prio, st, args...);
 }
 
 // ---------------------------------------------------------------------------
@@ -261,8 +311,6 @@ cudaError_t gemm_tcp(const GemmLaunch& L, cudaStream_t st);
 cudaError_t gemm_f32(const GemmLaunch& L, cudaStream_t st);
 cudaError_t gemm_f32_prepare();
 int gemm_f32_split(long long tiles, long long K, long long most);
-// SMs of the current device (api.cu)
-int device_sms();
 // tcgen05 path (k_gemm_tc.cu): BF16x3 split, 3M complex, FP32 accumulation in TMEM
 cudaError_t gemm_tc(const GemmLaunch& L, cudaStream_t st);
 // one-time kernel attributes (shared-memory size), outside any stream capture

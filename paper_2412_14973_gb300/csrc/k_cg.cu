@@ -44,6 +44,7 @@ __device__ __forceinline__ double sum_fixed(const double* part, int n, double (*
 __global__ void __launch_bounds__(256) k_cg_sym(const cf* __restrict__ y, const cf* __restrict__ p, float s2,
                                                 cf* __restrict__ out, int n, double* __restrict__ part,
                                                 double* __restrict__ sc) {
+    chain_entry();
     __shared__ cf t[CG_T][CG_T + 1];
     __shared__ double sh[1][256];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;     // 8 rows per pass
@@ -100,6 +101,7 @@ __global__ void __launch_bounds__(256) k_cg_sym(const cf* __restrict__ y, const 
 __global__ void __launch_bounds__(kRedThreads) k_cg_step(cf* __restrict__ r, const cf* __restrict__ Ap, long long n2,
                                                          double tol, double* __restrict__ sc,
                                                          double* __restrict__ part) {
+    chain_entry();
     __shared__ double sh[1][256];
     const float a = Ap ? (float)sc[CG_ALPHA] : 0.f;
     Acc acc;
@@ -156,6 +158,7 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_step(cf* __restrict__ r, con
 // at n = 2048, the reads touching 16 lines per instruction).
 __global__ void __launch_bounds__(256) k_cg_dir(cf* __restrict__ x, cf* __restrict__ p, const cf* __restrict__ r,
                                                 int n, const double* __restrict__ sc, char* __restrict__ pk) {
+    chain_entry();
     if (sc[CG_ALPHA] == 0.0) return;   // converged earlier: p and its packing stand
     const float al = (float)sc[CG_ALPHA], be = (float)sc[CG_BETA];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -221,9 +224,8 @@ int cg_partials(int) { return std::max(kSymBlocks, kRedBlocks); }
 
 cudaError_t cg_sym(const cf* y, const cf* p, float s2, cf* out, int n, double* part, double* sc, cudaStream_t st) {
     const int t = (n + CG_T - 1) / CG_T;
-    k_cg_sym<<<std::min(t * t, kSymBlocks), 256, 0, st>>>(y, p, s2, out, n, part, sc);
     counted(1);
-    return cudaGetLastError();
+    return launch_chain(k_cg_sym, dim3(std::min(t * t, kSymBlocks)), dim3(256), 0, st, y, p, s2, out, n, part, sc);
 }
 
 // start: x = 0, r = p = b (r holds b on entry), sc cleared, rr = ||b||^2
@@ -233,19 +235,18 @@ cudaError_t cg_start(cf* x, cf* r, cf* p, int n, double* part, double* sc, cudaS
     if (e == cudaSuccess) e = cudaMemcpyAsync(p, r, n2 * sizeof(cf), cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(sc, 0, 8 * sizeof(double), st);
     if (e != cudaSuccess) return e;
-    k_cg_step<<<kRedBlocks, kRedThreads, 0, st>>>(r, nullptr, n2, 0.0, sc, part);
     counted(1);
-    return cudaGetLastError();
+    return launch_chain(k_cg_step, dim3(kRedBlocks), dim3(kRedThreads), 0, st, r, (const cf*)nullptr, n2, 0.0, sc, part);
 }
 
 cudaError_t cg_iteration_tail(cf* x, cf* r, cf* p, const cf* Ap, int n, double tol, double* part, double* sc, char* pk,
                               cudaStream_t st) {
     const long long n2 = (long long)n * n;
-    k_cg_step<<<kRedBlocks, kRedThreads, 0, st>>>(r, Ap, n2, tol, sc, part);
-    counted(1);
-    k_cg_dir<<<dim3((n + 15) / 16, (n + 127) / 128), 256, 0, st>>>(x, p, r, n, sc, pk);
-    counted(1);
-    return cudaGetLastError();
+    counted(2);
+    const cudaError_t e = launch_chain(k_cg_step, dim3(kRedBlocks), dim3(kRedThreads), 0, st, r, Ap, n2, tol, sc, part);
+    if (e != cudaSuccess) return e;
+    return launch_chain(k_cg_dir, dim3((n + 15) / 16, (n + 127) / 128), dim3(256), 0, st, x, p, (const cf*)r, n,
+                        (const double*)sc, pk);
 }
 
 }  // namespace tlr

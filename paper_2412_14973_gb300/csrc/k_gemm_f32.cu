@@ -443,6 +443,7 @@ __device__ __forceinline__ bool write_tile(const Item& it, int epi, long long pa
 template <int AM, int BMD>
 __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ Launch L, int epi,
                                                        long long part_stride, int* err) {
+    chain_wait();
     extern __shared__ __align__(1024) char smem[];
     if (*(volatile int*)err != 0) return;   // an earlier contraction gave up: do no more work
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + CTRL_OFF);   // operand stage split (one arrival per worker warp)
@@ -659,9 +660,12 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
 
 template <int AM, int BMD>
 cudaError_t launch(const GemmLaunch& G, const Launch& L, unsigned grid, cudaStream_t st) {
-    k_cgemm_f32<AM, BMD><<<grid, NTHR, SMEM_BYTES, st>>>(L, G.epi, G.part_stride, G.err);
     counted(1);
-    return cudaGetLastError();
+    if (t_early_blocks != kEarlyAny) {   // recorded: a CTA takes a whole SM, early ones crowd (see chain_entry)
+        k_cgemm_f32<AM, BMD><<<grid, NTHR, SMEM_BYTES, st>>>(L, G.epi, G.part_stride, G.err);
+        return cudaGetLastError();
+    }
+    return launch_chain(k_cgemm_f32<AM, BMD>, dim3(grid), dim3(NTHR), SMEM_BYTES, st, L, G.epi, G.part_stride, G.err);
 }
 
 }  // namespace

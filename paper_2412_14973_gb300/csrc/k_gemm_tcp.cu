@@ -143,12 +143,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, float* v) {
 // pairs fill 64 contiguous bytes of each plane.  The job is copied to registers
 // first (through the pointer every store would make its fields be read again).
 // Small jobs are latency: 16 loads of a thread in flight, one round of them.
-// A solve of 256 receivers 4.03 -> 3.61 ms, the operator on 2499 x 1901 in TF32
+// A solve of 256 receivers 4.03 -> 3.61 ms, the operator on 2025 receivers x 1501 sources in TF32
 // 139 -> 131 us, misfit and gradient of 5525 x 6343 1.103 -> 1.043 ms; before, a
 // thread took a row's 16 values from 256 rows, each read touching 32 lines.
 constexpr int PACK_KC = 2;
 
 __global__ void __launch_bounds__(256) k_pack(const PackJob* __restrict__ jobs) {
+    chain_entry();
     const PackJob J = jobs[blockIdx.y];
     if (J.TR != 128) return;   // both formats are laid out on 128-row tiles
     const int nkc = (J.K + KC - 1) / KC, nrb = (J.R + 127) >> 7;
@@ -261,6 +262,7 @@ __device__ __forceinline__ void transpose8(float2* a) {
 __global__ void __launch_bounds__(256) k_tpack(const TPackTile* __restrict__ tiles, cf* __restrict__ T,
                                                const cf* __restrict__ Tp, const double* __restrict__ alpha,
                                                int ns, int gx, long long ntiles) {
+    chain_entry();
     const float a = alpha ? (float)alpha[0] : 0.f;
     constexpr int plane = 128 * 16 * 2;   // bytes of one BF16 plane of a 128 x 16 tile
     const int n = threadIdx.x & (TP_N - 1), kg = threadIdx.x >> 7;
@@ -342,6 +344,7 @@ __global__ void __launch_bounds__(256) k_rstep(cf* __restrict__ R, const cf* __r
                                                int b, char* const* __restrict__ kn, char* const* __restrict__ mk,
                                                double* __restrict__ part, const long long* __restrict__ roff,
                                                int nblk, int fmt, int gx, long long ntiles) {
+    chain_entry();
     __shared__ double sh[1][256];
     constexpr int plane = 128 * 16 * 2;
     const float a = alpha ? (float)alpha[0] : 0.f;
@@ -521,6 +524,7 @@ __global__ void __launch_bounds__(NTHR, CTAS_PER_SM + 1) k_cgemm_tcp(const PProb
                                                        const ZItem* __restrict__ zmap, int nsplit, int kchunk,
                                                        int epi, long long part_stride, int* err, int fmt,
                                                        int mfast) {
+    chain_wait();
     extern __shared__ __align__(1024) char smem[];
     // slice z: problem and split (uniform, or each problem its own through zmap)
     int prob, chunk;
@@ -781,6 +785,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_tcp_pers(const PProb* __restr
                                                             const ZItem* __restrict__ zmap, int nsplit, int kchunk,
                                                             int epi, long long part_stride, int* err, int fmt,
                                                             int nx, int ny, long long nitems) {
+    chain_wait();
     extern __shared__ __align__(1024) char smem[];
     if (*(volatile int*)err != 0) return;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + P_CTRL_OFF);
@@ -1096,20 +1101,18 @@ cudaError_t gemm_tcp(const GemmLaunch& L, cudaStream_t st) {
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             sms = 152;
         const unsigned g = (unsigned)std::min<long long>(sms, nitems);
-        k_cgemm_tcp_pers<<<g, NTHR, P_SMEM_BYTES, st>>>(L.d_pprobs, L.d_zmap, L.nsplit, kchunk, L.epi,
-                                                        L.part_stride, L.err, pack_fmt(L.prec), nx, ny, nitems);
         counted(1);
-        return cudaGetLastError();
+        return launch_chain(k_cgemm_tcp_pers, dim3(g), dim3(NTHR), P_SMEM_BYTES, st, (const PProb*)L.d_pprobs, L.d_zmap,
+                            L.nsplit, kchunk, L.epi, L.part_stride, L.err, pack_fmt(L.prec), nx, ny, nitems);
     }
     const unsigned mt = (unsigned)((L.maxM + TM - 1) / TM), nt = (unsigned)((L.maxN + TN - 1) / TN);
     const int mfast = nt <= 65535u ? 1 : 0;
     const unsigned nzs = (unsigned)(L.d_zmap ? L.nz : L.nprob * L.nsplit);
     if (nzs == 0) return cudaSuccess;
     dim3 grid(mfast ? mt : nt, mfast ? nt : mt, nzs);
-    k_cgemm_tcp<<<grid, NTHR, SMEM_BYTES, st>>>(L.d_pprobs, L.d_zmap, L.nsplit, kchunk, L.epi, L.part_stride, L.err,
-                                                 pack_fmt(L.prec), mfast);
     counted(1);
-    return cudaGetLastError();
+    return launch_chain(k_cgemm_tcp, grid, dim3(NTHR), SMEM_BYTES, st, (const PProb*)L.d_pprobs, L.d_zmap, L.nsplit, kchunk,
+                        L.epi, L.part_stride, L.err, pack_fmt(L.prec), mfast);
 }
 
 }  // namespace tlr

@@ -75,6 +75,7 @@ __device__ __forceinline__ double sum_slabs(const double* part, int n, double* s
 template <bool TO_PANEL>
 __global__ void __launch_bounds__(256) k_panel_map(PanelMap m, const cf* __restrict__ src, cf* __restrict__ dst,
                                                    int gcols, int grows) {
+    chain_entry();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const long long nlb = (long long)gcols * grows;
     for (long long e = blockIdx.x; e < nlb; e += gridDim.x) {
@@ -157,6 +158,7 @@ __device__ __forceinline__ bool dense_tile(long long e, long long b, const long 
 __global__ void k_sym_dense(const cf* __restrict__ pan, long long zbase, long long ndense, long long b,
                             cf* __restrict__ Zs, int general, const long long* __restrict__ zoff,
                             const int* __restrict__ zdim) {
+    chain_entry();
     GRID_STRIDE(e, ndense * b * b) {
         long long base, n, r, c;
         if (!dense_tile(e, b, zoff, zdim, base, n, r, c)) continue;
@@ -208,6 +210,7 @@ __device__ __forceinline__ cf split_sum_dense(const cf* __restrict__ part, int n
 __global__ void k_reduce_grad(const cf* __restrict__ part, int nsplit, long long stride, long long nlr,
                               long long ndense, long long b, cf* __restrict__ grad, int general,
                               const long long* __restrict__ zoff, const int* __restrict__ zdim) {
+    chain_entry();
     GRID_STRIDE(e, nlr) grad[e] = split_sum(part, nsplit, stride, e);
     GRID_STRIDE(e, ndense * b * b) {
         long long base, n, r, q;
@@ -230,6 +233,7 @@ cudaError_t reduce_grad(const cf* part, int nsplit, long long stride, long long 
 // FP64 inner products
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_sum_partials(const double* part, long long n, double scale, double* out) {
+    chain_entry();
     __shared__ double sh[1][256];
     const double v = sum_part(part, n, sh);
     if (threadIdx.x == 0) out[0] = scale * v;
@@ -267,6 +271,7 @@ __device__ __forceinline__ void dots6_group(float* t, float rx, float ry, float 
 __global__ void __launch_bounds__(kRedThreads) k_step_residual(cf* __restrict__ R, const cf* __restrict__ A1,
                                                               const cf* __restrict__ A2, long long n,
                                                               const double* __restrict__ alpha, double* part) {
+    chain_entry();
     __shared__ double sh[1][256];
     const float a = (float)alpha[0];
     const float a2 = (float)(alpha[0] * alpha[0]);
@@ -288,6 +293,7 @@ __global__ void __launch_bounds__(kRedThreads) k_step_residual(cf* __restrict__ 
 
 __global__ void k_axpy_dev(float* __restrict__ x, const float* __restrict__ y, long long n2,
                            const double* __restrict__ alpha) {
+    chain_entry();
     const float a = (float)alpha[0];
     if (a == 0.f) return;
     GRID_STRIDE(i, n2) x[i] = fmaf(a, y[i], x[i]);
@@ -305,6 +311,7 @@ cudaError_t axpy_dev(float* x, const float* y, long long n2, const double* alpha
 
 // partials of ||R||^2
 __global__ void __launch_bounds__(kRedThreads) k_norm_part(const cf* __restrict__ R, long long n, double* part) {
+    chain_entry();
     __shared__ double sh[1][256];
     Acc s;
     GRID_STRIDE(i, n) {
@@ -318,6 +325,7 @@ __global__ void __launch_bounds__(kRedThreads) k_norm_part(const cf* __restrict_
 
 // g = gf + rho (x - v); history cleared (start of an x-update)
 __global__ void k_xupdate_start(SolverDev S, double rho) {
+    chain_entry();
     const float r = (float)rho;
     GRID_STRIDE(i, S.n2) S.g[i] = S.gf[i] + r * (S.x[i] - S.v[i]);
     if (blockIdx.x == 0 && threadIdx.x == 0) S.ints[SI_CNT] = 0;
@@ -364,6 +372,7 @@ inline int lb_blocks(long long n2) {
 // this part, so the block sums its 51 values 8 lanes each (72 cycles a value; a
 // shuffle tree per warp and value took 320).
 __global__ void __launch_bounds__(kLbThreads, 4) k_lb_dots(SolverDev S, int j0, int last) {
+    chain_entry();
     __shared__ __align__(16) float shv[kLbVals * kLbLd];
     const int cnt = S.ints[SI_CNT];
     if (j0 < cnt) {
@@ -548,6 +557,7 @@ __device__ void lb_solve(const SolverDev& S, int cnt, int ncl, double* val, doub
 // 3 + k); four floats per thread and four pairs per step in flight (the vectors
 // start 16-byte aligned when n2 is a multiple of 4, else a scalar loop)
 __global__ void __launch_bounds__(kRedThreads) k_lb_dir(SolverDev S) {
+    chain_entry();
     __shared__ float cs[32], cy[32];
     __shared__ const float* ps[32];
     __shared__ const float* py[32];
@@ -771,6 +781,7 @@ __device__ __forceinline__ void dots6_end(const SolverDev& S, const Acc* s, int 
 // is even; the buffers start 256-byte aligned)
 __global__ void __launch_bounds__(kRedThreads) k_dots6(SolverDev S, const cf* __restrict__ R, const cf* __restrict__ A1,
                                                       const cf* __restrict__ A2, long long n, int nb3, double rho) {
+    chain_entry();
     __shared__ double sh[6][256];
     Acc s[6];
     if ((n & 1) == 0) {
@@ -816,6 +827,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dots6(SolverDev S, const cf* __
 __global__ void __maxnreg__(48) k_dots6p(SolverDev S, char* const* __restrict__ kn, const cf* __restrict__ A1,
                                          const cf* __restrict__ A2, int ns, int nr, int b,
                                          const long long* __restrict__ roff, int nblk, int fmt, int nb3, double rho) {
+    chain_entry();
     __shared__ double sh[6][256];
     constexpr int plane = 128 * 16 * 2;
     const int gx = (ns + kFuseCols - 1) / kFuseCols;
@@ -849,6 +861,7 @@ __global__ void __maxnreg__(48) k_dots6p(SolverDev S, char* const* __restrict__ 
 
 // x += a d ; s_free = a d (two floats at a time: n2 is even)
 __global__ void k_step_theta(SolverDev S) {
+    chain_entry();
     const double ad = S.sc[SC_ALPHA];
     const float a = (float)ad;
     const int R = S.ring;
@@ -876,6 +889,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gradient_pair(SolverDev S, cons
                                                               const long long* __restrict__ zoff,
                                                               const int* __restrict__ zdim, double rho,
                                                               const double* __restrict__ partf, long long nf) {
+    chain_entry();
     __shared__ double sh[3][256];
     const float r = (float)rho;
     const int R = S.ring;
@@ -936,6 +950,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gradient_pair(SolverDev S, cons
 
 // ADMM z- and dual updates (eq. 23, 24 in scaled form) and v = z - u
 __global__ void k_admm_zu(SolverDev S, double lam, double rho) {
+    chain_entry();
     const float den = (float)(1.0 / (1.0 + 2.0 * lam / rho));
     GRID_STRIDE(i, S.n2) {
         const float x = S.x[i], u = S.u[i];
@@ -949,6 +964,7 @@ __global__ void k_admm_zu(SolverDev S, double lam, double rho) {
 
 // start of the solve: z = x, u = 0, v = x, counters cleared
 __global__ void k_admm_init(SolverDev S) {
+    chain_entry();
     GRID_STRIDE(i, S.n2) {
         const float x = S.x[i];
         S.z[i] = x;
@@ -967,6 +983,7 @@ __global__ void k_admm_init(SolverDev S) {
 
 // resumed solve: v = z - u from the stored split; counters cleared
 __global__ void k_admm_resume(SolverDev S) {
+    chain_entry();
     GRID_STRIDE(i, S.n2) S.v[i] = S.z[i] - S.u[i];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         S.ints[SI_CNT] = 0;
@@ -980,6 +997,7 @@ __global__ void k_admm_resume(SolverDev S) {
 
 // f0 = f = 0.5 ||R||^2
 __global__ void __launch_bounds__(256) k_record_f0(SolverDev S, const double* partf, long long np) {
+    chain_entry();
     __shared__ double sh[1][256];
     const double rr = sum_part(partf, np, sh);
     if (threadIdx.x != 0) return;
