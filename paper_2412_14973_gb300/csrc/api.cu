@@ -32,7 +32,26 @@ using namespace tlr;
 
 std::atomic<long long> tlr::g_launches{0};
 
-thread_local long long tlr::t_early_blocks = tlr::kEarlyAny;
+thread_local long long tlr::t_early_blocks = 0;
+
+// Lets the launches of a call start early (chain_entry) while in scope.
+namespace {
+class Early {
+public:
+    explicit Early(long long blocks) : before_(t_early_blocks) { t_early_blocks = blocks; }
+    ~Early() { t_early_blocks = before_; }
+    Early(const Early&) = delete;
+    Early& operator=(const Early&) = delete;
+
+private:
+    long long before_;
+};
+// a single product, gradient or benchmark solve: where its panels are small
+constexpr long long kEarlyEntries = 1ll << 23;
+long long early_product(long long rows, long long cols) { return rows * cols <= kEarlyEntries ? kEarlyAny : 0; }
+// a solve: up to 512 receivers, launches of at most a block per SM
+long long early_solve(long long nr) { return nr <= 512 ? device_sms() : 0; }
+}  // namespace
 
 int tlr::device_sms() {
     static const int n = [] {
@@ -1680,6 +1699,7 @@ int tlr_mdd_apply(tlr_mdd_t* h, const void* theta, void* Y) {
     if (!h) FAIL(h, TLR_ERR_STATE, "handle is NULL");
     if (!theta || !Y) FAIL(h, TLR_ERR_ARG, "theta or Y is NULL");
     const Layout& L = h->L;
+    const Early early(early_product(L.nr, L.ns));
     CK(h, theta_to_panel(h->pm, (const cf*)theta, h->x, h->st));
     int rc = forward(h, true);
     if (rc) return rc;
@@ -1691,6 +1711,7 @@ int tlr_mdd_grad(tlr_mdd_t* h, const void* theta, void* grad, double* f) {
     if (!h) FAIL(h, TLR_ERR_STATE, "handle is NULL");
     if (!theta || !grad) FAIL(h, TLR_ERR_ARG, "theta or grad is NULL");
     const Layout& L = h->L;
+    const Early early(early_product(L.nr, L.ns));
     CK(h, theta_to_panel(h->pm, (const cf*)theta, h->x, h->st));
     int rc = forward(h, false);
     if (rc) return rc;
@@ -1722,6 +1743,7 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     if (!V || !G) FAIL(h, TLR_ERR_ARG, "V or G is NULL");
     const Layout& L = h->L;
     const long long nr = L.nr, ns = L.ns;
+    const Early early(early_product(nr, ns));
     const bool tc = tensor_core(h->d.precision);
     const long long t128 = (nr + 127) / 128, t64 = (nr + 63) / 64;
     int ns_split = tc ? choose_split(t64 * t64, ns) : gemm_f32_split(t128 * t128, ns, 32);
@@ -1834,6 +1856,7 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
     if (h->pending) FAIL(h, TLR_ERR_STATE, "a solve is pending on this handle");
     const Layout& L = h->L;
     const int n = (int)L.nr, ns = (int)L.ns;
+    const Early early(early_product(n, std::max(n, ns)));
     const size_t n2 = (size_t)n * n;
     const bool tc = tensor_core(h->d.precision);   // BF16x3 packed products for both tensor-core modes
     const int np = cg_partials(n);
@@ -2487,6 +2510,7 @@ static SolverDev solver_dev(tlr_mdd_s* h, int m) {
 
 static int enqueue_solve(tlr_mdd_s* h, const tlr_mdd_solve_opts_t* o) {
     const Layout& L = h->L;
+    const Early early(early_solve(L.nr));
     const long long nrs = (long long)L.nr * L.ns;
     const SolverDev S = solver_dev(h, o->memory);
     const double rho = o->rho;
@@ -2623,14 +2647,7 @@ static int enqueue_body(tlr_mdd_s* h, const tlr_mdd_solve_opts_t* o) {
         CK(h, cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
         g_capture_sink = &h->gtimed;
         const long long n_before = g_launches.load();
-        int rc;
-        {
-            struct Recording {
-                explicit Recording(long long n) { t_early_blocks = n; }
-                ~Recording() { t_early_blocks = kEarlyAny; }
-            } recording(h->L.nr <= 512 ? device_sms() : 0);
-            rc = enqueue_solve(h, o);
-        }
+        int rc = enqueue_solve(h, o);
         h->graph_kernels = g_launches.load() - n_before;
         g_launches.fetch_sub(h->graph_kernels);   // recorded, not launched: counted at each replay
         g_capture_sink = nullptr;

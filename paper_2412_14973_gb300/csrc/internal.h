@@ -41,17 +41,20 @@ void set_pass_cap(long long ctas);
 // completed and its results are visible.  A pass then lets its own successor be
 // scheduled at once.  A contraction does not (its successor follows when its last
 // block ends): blocks placed early go to whatever SMs are idle, and beside a long
-// contraction these are the few that finish first, where they crowd.  For the same
-// reason a recorded solve, whose launches cost little else, lets only launches of
-// at most a block per SM start early, no FP32 contraction, and none at all above
-// 512 receivers, where every pass is long (t_early_blocks).
+// contraction these are the few that finish first, where they crowd.
+// Blocks that wait also hold room that other streams' contractions would use: with
+// every launch early, four streams of nr = 9216 solves fell from 3.67 to 2.95
+// freq-solves/s (one stream 3.25).  So a launch starts early only where a call asks
+// for it (t_early_blocks, 0 unless set): single products, gradients and benchmark
+// solves on panels of up to 2^23 elements, whose kernels last microseconds; and
+// solves up to 512 receivers, there launches of at most a block per SM and no FP32
+// contraction (recorded, nr = 1024 in FP32: every launch early 6.58 ms, up to a
+// block per SM 6.47, none 6.45).
 // Measured, plain launches -> this: misfit and gradient of nr = 2048, general form,
 // 0.268 -> 0.232 ms; operator of nr = 2025 in TF32 132 -> 114 us; benchmark solver
 // at nr = 2048 4.33 -> 4.07 ms; recorded solve of nr = 256 3.50 -> 3.41 ms.
-// Contractions that release their successor at once: benchmark solver 4.15, misfit
-// and gradient of nr = 4096 in FP32 2.30 against 2.27.  Recorded, nr = 1024 in FP32:
-// every launch early 6.58, up to a block per SM 6.47, none 6.45.  Only launches of
-// at most a block per SM, everywhere: 0.264 ms, 129 us, 4.29 ms.
+// Contractions that release their successor at once: benchmark solver 4.15.  Only
+// launches of at most a block per SM, everywhere: 0.264 ms, 129 us, 4.29 ms.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_entry() {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
 template <int AM, int BMD>
 cudaError_t launch(const GemmLaunch& G, const Launch& L, unsigned grid, cudaStream_t st) {
     counted(1);
-    if (t_early_blocks != kEarlyAny) {   // recorded: a CTA takes a whole SM, early ones crowd (see chain_entry)
+    if (t_early_blocks != kEarlyAny) {   // in a solve: a CTA takes a whole SM, early ones crowd (see chain_entry)
         k_cgemm_f32<AM, BMD><<<grid, NTHR, SMEM_BYTES, st>>>(L, G.epi, G.part_stride, G.err);
         return cudaGetLastError();
     }
