@@ -919,7 +919,7 @@ def secondary_leg(T, torch, args, dev):
     step()          # plain launches (a handle's first solve)
     step()          # records the solve graphs
     ms = sum(step() for _ in range(args.secondary))
-    # the same step on every 8th frequency, tensor cores and the FP32 SIMT
+    # the same step on every 8th frequency, tensor cores and the FP32
     # path, on handles of their own (8 solves on the streams overlap little:
     # the pass grid is left uncapped; a recorded graph keeps the grid it was
     # recorded with)
@@ -1046,7 +1046,7 @@ def serving_leg(T, torch, n, seed, dev, fp32_loads=(), multi_ctas=0):
     """The serving mix: n per-frequency solve requests, nr = ns uniform over
     {1024, 2048, 4096, 8192}, tile over {128, 256, 512}, rank log-uniform
     2-64, BF16x3 tensor cores, 30-iteration solves.  Measured: one request at
-    a time on the tensor cores (all n) and on the FP32 SIMT path (the first
+    a time on the tensor cores (all n) and on the FP32 path (the first
     m of them), then the whole stream served with continuous batching (4
     slots, 120 GB budget, shape-keyed handle reuse) at Poisson arrivals of 90%
     of the tensor cores' one-at-a-time capacity: solves/s, p50 / p99 latency

@@ -244,9 +244,10 @@ int tlr_mdd_solve_wait(tlr_mdd_t* h, tlr_mdd_stats_t* stats);
  * the result X = P Z = Z is written to X: DEVICE complex64 nr x nr, Hilbert
  * order (like X_h), row-major.  D-hat^H D-hat is formed once; every
  * iteration is one nr x nr x nr complex product in the handle's precision.
- * Work memory (6 nr^2 complex64, plus packed operands on the tensor-core
- * path) is allocated on the handle's stream and released before return; the
- * call synchronises.  lambda < 0 or non-finite, iters < 0, tol < 0, X NULL:
+ * Work memory (4 nr^2 complex64 plus packed operands on the tensor-core path,
+ * 5 nr^2 in FP32) comes from the library's pool on the handle's stream and goes
+ * back before return (the pool keeps at most 256 MB of it); the iterates are
+ * built in X; the call synchronises.  lambda < 0 or non-finite, iters < 0, tol < 0, X NULL:
  * TLR_ERR_ARG; a pending solve on the handle: TLR_ERR_STATE.
  * stats (HOST, may be NULL): iterations taken, final ||r|| / ||b||, device
  * time of the whole call. */
@@ -326,8 +327,10 @@ int tlr_mdd_set_state(tlr_mdd_t* h, const void* z, const void* u);
  * (f0 + nf <= nt / 2 + 1).  freq_to_time: the inverse real DFT of the band
  * (bins outside it zero, the imaginary parts of bins 0 and nt/2 ignored), with
  * the factor 1 / nt, so freq_to_time(time_to_freq(x)) = x when the band is the
- * whole spectrum.  Real FFTs by cuFFT over chunks of traces (work memory about
- * 256 MB plus cuFFT's own, allocated and released per call); synchronises.
+ * whole spectrum.  Lengths nt <= 4096 with prime factors up to 13, and any nt <=
+ * 2048, are transformed in shared memory (work memory: tables of a few KB); others
+ * by cuFFT over chunks of traces (about 256 MB plus cuFFT's own, allocated and
+ * released per call); synchronises.
  * Invalid sizes: TLR_ERR_ARG. */
 int tlr_mdd_time_to_freq(const float* x_t, int64_t ntr, int64_t nt, int64_t f0, int64_t nf, void* X_w,
                          void* stream);
