@@ -117,6 +117,14 @@ cudaError_t ws_alloc(void** ptr, size_t bytes, cudaStream_t st) {
     return cudaMallocFromPoolAsync(ptr, bytes, p, st);
 }
 
+// Waits for the stream, whatever e is (an asynchronous copy from pageable memory may
+// read its source until then, and the caller's host tables go out of scope after
+// it); the first error.
+cudaError_t settle(cudaError_t e, cudaStream_t st) {
+    const cudaError_t w = cudaStreamSynchronize(st);
+    return e != cudaSuccess ? e : w;
+}
+
 // Per-call scratch, from the same pool: mapping fresh device memory on every
 // call cost as much as the work it served (0.9 of 5.9 ms of a benchmark solve at
 // nr = 2048).  When it is given back the pool keeps at most kScratchKeep bytes
@@ -690,6 +698,8 @@ struct tlr_mdd_s {
     bool pending = false;
     bool pending_graph = false;
     void* pending_host_theta = nullptr;
+    // host sides of the uploads of tlr_mdd_create, until it has waited for the stream
+    std::vector<std::vector<char>> uploads;
 };
 
 #define FAIL(h, code, msg)                  \
@@ -867,7 +877,8 @@ int build_tables(tlr_mdd_s* h, char* tab_base, std::vector<HostTable>* keep) {
     const long long ns = L.ns;
     const size_t slot = ((sizeof(GProb) * (3 * (size_t)L.N + 1)) + 255) & ~size_t(255);
     int ti = 0;
-    std::vector<char> img(8 * slot);   // all tables, copied at once
+    h->uploads.emplace_back(8 * slot);   // all tables, copied at once
+    std::vector<char>& img = h->uploads.back();
     auto upload = [&](GemmLaunch& G, std::vector<GProb>& v, int am, int bm, int epi) -> int {
         char* const at = img.data() + slot * ti;
         GProb* dst = reinterpret_cast<GProb*>(tab_base + slot * ti++);
@@ -1334,7 +1345,8 @@ int build_tc(tlr_mdd_s* h, std::vector<HostTable>& tabs) {
     const size_t rpo = bytes;
     bytes += (2 * (size_t)L.N * sizeof(char*) + 255) & ~size_t(255);
     CK(h, ws_alloc((void**)&h->tcp_tables, std::max<size_t>(bytes, 256), h->st));
-    std::vector<char> img(std::max<size_t>(bytes, 256));   // all tables, copied at once
+    h->uploads.emplace_back(std::max<size_t>(bytes, 256));   // all tables, copied at once
+    std::vector<char>& img = h->uploads.back();
     auto put = [&](size_t at, const void* src, size_t n) {
         if (n) memcpy(img.data() + at, src, n);
     };
@@ -1378,7 +1390,6 @@ int build_tc(tlr_mdd_s* h, std::vector<HostTable>& tabs) {
     h->n_static_jobs = (int)sjobs.size();
     h->static_items = smax;
     put(so, sjobs.data(), sjobs.size() * sizeof(PackJob));
-    // (pageable memory is staged before the call returns)
     CK(h, cudaMemcpyAsync(h->tcp_tables, img.data(), bytes, cudaMemcpyHostToDevice, h->st));
     return TLR_OK;
 }
@@ -1400,8 +1411,7 @@ static int load_data(tlr_mdd_s* h, const void* D, const void* U, int memory) {
         Usrc = h->A1;
     }
     if (d->alpha > 0.0) {
-        const double al = d->alpha;
-        CK(h, cudaMemcpyAsync(h->scal, &al, sizeof(double), cudaMemcpyHostToDevice, h->st));
+        CK(h, cudaMemcpyAsync(h->scal, &d->alpha, sizeof(double), cudaMemcpyHostToDevice, h->st));
     } else {
         CK(h, max_abs2(Dsrc, (long long)nrs, h->dpart, kRedBlocks, h->scal, h->st));
     }
@@ -1530,10 +1540,8 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
         if (h->arena) cudaFreeAsync(h->arena, h->st);
         if (h->ev0) cudaEventDestroy(h->ev0);
         if (h->ev1) cudaEventDestroy(h->ev1);
-        if (h->hstats) {
-            cudaStreamSynchronize(h->st);
-            pinned_put(h->hstats);
-        }
+        cudaStreamSynchronize(h->st);   // copies may still read h->uploads, D, U or write the statistics
+        if (h->hstats) pinned_put(h->hstats);
         delete h;
         return code;
     };
@@ -1591,7 +1599,8 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
     // maps: adjacent in the arena (carve), copied at once
     {
         char* const lo = reinterpret_cast<char*>(h->d_partner);
-        std::vector<char> img(reinterpret_cast<char*>(h->d_roff + L.N + 1) - lo);
+        h->uploads.emplace_back(reinterpret_cast<char*>(h->d_roff + L.N + 1) - lo);
+        std::vector<char>& img = h->uploads.back();
         auto put = [&](const void* at, const auto& v) {
             if (!v.empty()) memcpy(img.data() + (reinterpret_cast<const char*>(at) - lo), v.data(), v.size() * sizeof(v[0]));
         };
@@ -1634,6 +1643,7 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
         CKF(gemm_f32_prepare());
     CKF(cudaMemcpyAsync(h->hstats->sc, h->scal, sizeof(double), cudaMemcpyDeviceToHost, h->st));
     CKF(cudaStreamSynchronize(h->st));
+    h->uploads.clear();
     h->alpha = h->hstats->sc[0];
 #undef CKF
     *out = h;
@@ -1837,8 +1847,7 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     if (e == cudaSuccess) e = run_gemm(G1, h->st);
     if (e == cudaSuccess && ns_split > 1) e = reduce_grad(part, ns_split, nr * nr, nr * nr, 0, 1, (cf*)G, h->st);
     if (own) cudaFreeAsync(part, h->st);
-    CK(h, e);
-    CK(h, cudaStreamSynchronize(h->st));  // tab lives on this stack frame
+    CK(h, settle(e, h->st));   // tab lives on this stack frame
     return TLR_OK;
 }
 
@@ -1889,8 +1898,12 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
     };
     // three products: G = conj(D) D^T, Bm = conj(D) U^T, y = G p
     GemmLaunch GL[3];
+    // host sides of the tables, until the stream has been waited for
+    GProb qf[3] = {blank(), blank(), blank()};
+    PProb qp[3];
+    PackJob J[5];
     if (!tc) {
-        GProb q[3] = {blank(), blank(), blank()};
+        GProb(&q)[3] = qf;
         q[0].t[0] = term(h->Dt, ns, h->Dt, ns, nullptr, ns, true, false);
         q[1].t[0] = term(h->Dt, ns, h->Ut, ns, nullptr, ns, true, false);
         q[2].t[0] = term(G, n, pv, n, nullptr, n, false, false);
@@ -1917,7 +1930,6 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
     } else {
         // pack jobs: 0 conj(D) (A, MK) -> pkA; 1 D (B, rows n) -> pkB; 2 U (B) -> pkB;
         // 3 G (A, MK) -> pkA; 4 p (B; p is symmetric, so its rows serve) -> pkB
-        PackJob J[5];
         const cf* src[5] = {h->Dt, h->Dt, h->Ut, G, pv};
         const int Ks[5] = {ns, ns, ns, n, n};
         for (int i = 0; i < 5; ++i) {
@@ -1933,7 +1945,7 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
             J[i].dst = (i == 0 || i == 3) ? (void*)pkA : (void*)pkB;
             J[i].fmt = kFmtBF16X3;
         }
-        PProb q[3];
+        PProb(&q)[3] = qp;
         memset(q, 0, sizeof(q));
         cf* outs[3] = {G, y, y};
         for (int i = 0; i < 3; ++i) {
@@ -1996,7 +2008,7 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
     if (e == cudaSuccess) e = cudaMemcpyAsync(hs, sc, sizeof(hs), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&werr, h->ints + SI_COUNT + 1, sizeof(int), cudaMemcpyDeviceToHost, h->st);
     buf.release();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
+    e = settle(e, h->st);   // the host tables above go out of scope
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
     if (e0) cudaEventDestroy(e0);
@@ -2060,7 +2072,7 @@ int tile_ranks_impl(const cf* X, int64_t nr, int64_t b, double eps, std::vector<
     if (e == cudaSuccess) e = cudaMemcpyAsync(ranks.data(), dr, nt * sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hv0, dv0, sizeof(double), cudaMemcpyDeviceToHost, st);
     buf.release();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = settle(e, st);
     if (e != cudaSuccess) {
         err = std::string("tile ranks: ") + cudaGetErrorString(e);
         return TLR_ERR_CUDA;
@@ -2202,8 +2214,7 @@ int tlr_mdd_warm_start(tlr_mdd_t* h, const void* X, void* theta) {
         e = tile_svd((const cf*)X, L.nr, dtl, nsvd, bmax, work, true, 30, 1e-5f, sig, ord, nullptr, h->st);
     if (e == cudaSuccess) e = warm_fill((const cf*)X, L.nr, dwt, nw, bmax, work, sig, ord, (cf*)theta, h->st);
     buf.release();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);   // the host tables above go out of scope
-    CK(h, e);
+    CK(h, settle(e, h->st));   // the host tables above go out of scope
     return TLR_OK;
 }
 
@@ -2344,8 +2355,7 @@ int tlr_mdd_unpermute_dense(tlr_mdd_t* h, const void* theta, void* X) {
         e = assemble_dense((const cf*)theta, nr, L.dmax, L.N, dt, Xh, h->st, L.general, L.b > 0 ? nullptr : h->d_roff);
     if (e == cudaSuccess) e = unpermute_dense(Xh, nr, h->perm, (cf*)X, h->st);
     buf.release();
-    CK(h, e);
-    CK(h, cudaStreamSynchronize(h->st));
+    CK(h, settle(e, h->st));   // the table above goes out of scope
     return TLR_OK;
 }
 
@@ -2764,10 +2774,11 @@ namespace {
 
 // One merged launch of contraction kind `kind` over every member: problem
 // tables and pack jobs concatenated (device-to-device), one slice per
-// member problem and split in a map.  Returns false when the members'
-// launches of this kind differ in epilogue or format (they then run apart).
+// member problem and split in a map (its host side zm has to live until the
+// stream is waited for).  Returns false when the members' launches of this
+// kind differ in epilogue or format (they then run apart).
 bool plan_merged(tlr_mdd_batch_s* b, GemmLaunch tlr_mdd_s::*kind, GemmLaunch& M, size_t& off, bool size_only,
-                 cudaStream_t st, cudaError_t& e) {
+                 cudaStream_t st, cudaError_t& e, std::vector<ZItem>& zm) {
     const GemmLaunch& G0 = b->hs[0]->*kind;
     int nprob = 0, njobs = 0, nz = 0;
     for (auto* h : b->hs) {
@@ -2800,7 +2811,6 @@ bool plan_merged(tlr_mdd_batch_s* b, GemmLaunch tlr_mdd_s::*kind, GemmLaunch& M,
     M.prec = G0.prec;
     M.persistent = (persist_classes() >> G0.cls) & 1;
     M.err = b->err;
-    std::vector<ZItem> zm;
     int pbase = 0, jbase = 0;
     for (auto* h : b->hs) {
         const GemmLaunch& G = h->*kind;
@@ -3074,9 +3084,10 @@ int tlr_mdd_batch_create(tlr_mdd_batch_t** out, tlr_mdd_t* const* hs, int32_t n,
     size_t off = 256;   // the error word first
     cudaError_t e = cudaSuccess;
     bool merged[6];
+    std::vector<ZItem> zm[6];
     for (int k = 0; k < 6; ++k) {
         GemmLaunch tmp;
-        merged[k] = plan_merged(b, kBatchKinds[k], tmp, off, true, b->st, e);
+        merged[k] = plan_merged(b, kBatchKinds[k], tmp, off, true, b->st, e, zm[k]);
     }
     if (ws_alloc((void**)&b->tables, off, b->st) != cudaSuccess) {
         b->tables = nullptr;
@@ -3086,8 +3097,8 @@ int tlr_mdd_batch_create(tlr_mdd_batch_t** out, tlr_mdd_t* const* hs, int32_t n,
     e = cudaMemsetAsync(b->tables, 0, 256, b->st);
     off = 256;
     for (int k = 0; k < 6 && e == cudaSuccess; ++k)
-        if (merged[k]) plan_merged(b, kBatchKinds[k], b->*kBatchMerged[k], off, false, b->st, e);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
+        if (merged[k]) plan_merged(b, kBatchKinds[k], b->*kBatchMerged[k], off, false, b->st, e, zm[k]);
+    e = settle(e, b->st);
     if (e != cudaSuccess) return fail(TLR_ERR_CUDA, cudaGetErrorString(e));
     *out = b;
     return TLR_OK;

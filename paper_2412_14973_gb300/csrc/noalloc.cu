@@ -114,15 +114,15 @@ extern "C" int tlr_mdd_adjoint_noalloc(const void* V, const void* Dt, int64_t nr
     L.flops = 8.0 * (double)nr * (double)nr * (double)ns;
     // Every partial slab is written in full by the GEMM before the reduction
     // reads it, so no part of the array has to start at zero.
-    if (cudaMemcpyAsync(base, &p, sizeof(GProb), cudaMemcpyHostToDevice, st) != cudaSuccess) return TLR_ERR_CUDA;
     L.err = err;
-    if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) return TLR_ERR_CUDA;
-    if (run_gemm(L, st) != cudaSuccess) return TLR_ERR_CUDA;
-    if (reduce_grad(part, nsplit, nr * nr, nr * nr, 0, 1, (cf*)G, st) != cudaSuccess) return TLR_ERR_CUDA;
-    // p lives on this stack frame; the copy above was staged before return,
-    // but wait for the stream so the caller may reuse V, Dt and G at once.
     int werr = 0;
-    if (cudaMemcpyAsync(&werr, err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return TLR_ERR_CUDA;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return TLR_ERR_CUDA;
+    cudaError_t e = cudaMemcpyAsync(base, &p, sizeof(GProb), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
+    if (e == cudaSuccess) e = run_gemm(L, st);
+    if (e == cudaSuccess) e = reduce_grad(part, nsplit, nr * nr, nr * nr, 0, 1, (cf*)G, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&werr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    // p and werr live on this stack frame, and the caller may reuse V, Dt and G at once
+    const cudaError_t w = cudaStreamSynchronize(st);
+    if (e != cudaSuccess || w != cudaSuccess) return TLR_ERR_CUDA;
     return werr == 0 ? TLR_OK : TLR_ERR_TIMEOUT;
 }
