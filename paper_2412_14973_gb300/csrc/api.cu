@@ -894,6 +894,7 @@ int build_tables(tlr_mdd_s* h, char* tab_base, std::vector<HostTable>* keep) {
             G.maxN = std::max(G.maxN, p.N);
             for (int t = 0; t < p.nt; ++t) G.flops += 8.0 * p.M * (double)p.N * p.t[t].K;
         }
+        G.shallow = std::any_of(v.begin(), v.end(), [](const GProb& p) { return gemm_f32_shallow(p, 1, 0); });
         G.cls = am == A_KM ? 0 : (bm == B_KN ? 1 : 2);
         G.prec = h->d.precision;
         G.persistent = tensor_core(G.prec) && ((persist_classes() >> G.cls) & 1);
@@ -1046,6 +1047,8 @@ int build_tables(tlr_mdd_s* h, char* tab_base, std::vector<HostTable>* keep) {
         h->Lp.nsplit = h->nsplit;
         h->Lp.kchunk = h->kchunk;
         h->Lp.part_stride = L.nth;
+        h->Lp.shallow = std::any_of(v.begin(), v.end(),
+                                    [&](const GProb& p) { return gemm_f32_shallow(p, h->nsplit, h->kchunk); });
     }
     return cudaMemcpyAsync(tab_base, img.data(), img.size(), cudaMemcpyHostToDevice, h->st) == cudaSuccess ? 0 : -1;
 }
@@ -1815,6 +1818,7 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     G1.kchunk = (int)(((ns + ns_split - 1) / ns_split + 15) / 16 * 16);
     G1.part_stride = nr * nr;
     G1.epi = ns_split > 1 ? EPI_PARTIAL : EPI_STORE;
+    G1.shallow = gemm_f32_shallow(p, ns_split, G1.kchunk);
     tab.g = p;
     if (packed) {
         for (int i = 0; i < 2; ++i) {
@@ -1925,6 +1929,7 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
             GL[i].bmode = i < 2 ? B_NK : B_KN;
             GL[i].epi = EPI_STORE;
             GL[i].prec = TLR_PREC_FP32;
+            GL[i].shallow = gemm_f32_shallow(q[i], 1, 0);
             GL[i].err = h->ints + SI_COUNT + 1;
         }
     } else {

@@ -204,7 +204,8 @@ struct GemmLaunch {
     bool persistent = false;    // packed path: the persistent, double-buffered kernel
     const ZItem* d_zmap = nullptr;   // persistent only: per-slice problem, split and partial offset
     int nz = 0;                      // slices in d_zmap (replaces nprob x nsplit)
-    int* err = nullptr;         // device error word (tensor-core path: bounded-wait timeouts)
+    int* err = nullptr;         // device error word (bounded-wait timeouts)
+    bool shallow = true;        // FP32 path: an output may be a sum of 1 .. kF32Shallow products (gemm_f32_shallow)
     // packed tensor-core path: problems on packed operands and the packs to run first
     PProb* d_pprobs = nullptr;
     PackJob* d_jobs = nullptr;
@@ -313,6 +314,10 @@ cudaError_t gemm_tcp(const GemmLaunch& L, cudaStream_t st);
 // `tiles` 128 x 128 output tiles, at most `most`.
 cudaError_t gemm_f32(const GemmLaunch& L, cudaStream_t st);
 cudaError_t gemm_f32_prepare();
+// Outputs that are sums of at most this many products are computed without the tensor
+// cores; gemm_f32_shallow: whether a problem has any, split over K like this.
+constexpr int kF32Shallow = 12;
+bool gemm_f32_shallow(const GProb& p, int nsplit, int kchunk);
 int gemm_f32_split(long long tiles, long long K, long long most);
 // tcgen05 path (k_gemm_tc.cu): BF16x3 split, 3M complex, FP32 accumulation in TMEM
 cudaError_t gemm_tc(const GemmLaunch& L, cudaStream_t st);

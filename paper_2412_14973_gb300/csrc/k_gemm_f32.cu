@@ -3,7 +3,7 @@
 // expand Y = F T~ (+ P Z Dfrak), the factor-gradient projections (eq. 25-27)
 // and the dense adjoint G = V Dfrak^H, on FP32 operands in place.
 //
-// Arithmetic.  Every FP32 value is split exactly into three BF16 values
+// Arithmetic.  Every FP32 value from 2^-109 up is split exactly into three BF16 values
 // x = h + m + l (h = RN(x), m = RN(x - h), l = x - h - m: 8 + 8 + 8 significant
 // bits), and every real product takes the six of the nine BF16 products that
 // are not below 2^-24 of it: hh, hm, mh, hl, mm, lh.  A complex product is four
@@ -35,10 +35,12 @@
 // Persistent: one CTA per SM walks the output tiles, its pipeline running
 // across tile ends.
 //
-// Values beyond the split (Inf, NaN, or a magnitude that rounds to Inf in BF16)
-// make a tile's results non-finite; every non-finite result is recomputed with
-// plain FP32 fused multiply-adds before it is stored, so Inf and NaN come out
-// as FP32 arithmetic gives them.
+// Values beyond the split: Inf, NaN or a magnitude that rounds to Inf in BF16 make a
+// tile's results non-finite; a value other than zero below 2^-109 has a third part
+// below BF16's smallest and is found while it is split.  What they touch is computed
+// again with plain FP32 fused multiply-adds (plain_tile): the non-finite results, results
+// below 2^-100, or the whole tile.  So Inf, NaN and small values come out as FP32
+// arithmetic gives them.
 //
 // Every barrier wait is bounded (2 s); a timeout is recorded in the error word.
 #include <cuda_bf16.h>
@@ -148,8 +150,17 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     return r;
 }
 
+// least = min(least, |x0|, |x1|) and most = max(most, |x0|, |x1|), a NaN kept by the latter
+__device__ __forceinline__ void min_abs(float& least, float x0, float x1) {
+    asm("min.abs.f32 %0, %0, %1, %2;" : "+f"(least) : "f"(x0), "f"(x1));
+}
+__device__ __forceinline__ void max_abs(float& most, float x0, float x1) {
+    asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(most) : "f"(x0), "f"(x1));
+}
+
 // h, m, l of two FP32 values as BF16 pairs (x0 in the low half)
-__device__ __forceinline__ void split2(float x0, float x1, uint32_t* w) {
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t* w, float& least) {
+    min_abs(least, x0, x1);
     uint64_t x = pair(x0, x1);
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
@@ -174,6 +185,9 @@ struct Launch {
     const GProb* probs;
     int nsplit, kchunk, nx, ny;
     int nitems;         // below 2^31 - grid (gemm_f32)
+    int epi;
+    int shallow;        // 0: no item has 1 .. SHALLOW products per output
+    long long part_stride;
 };
 
 __device__ __forceinline__ bool item_at(const Launch& L, int i, Item& it) {
@@ -197,7 +211,24 @@ __device__ __forceinline__ void k_range(const Launch& L, const Item& it, int K, 
     }
 }
 
+// An item's products per output: up to SHALLOW of them are left to plain FP32
+// multiply-adds (plain_tile), which round less often than the drained chunk's 24 MMAs
+// do: 1 product 3.0e-8 against 4.7e-8, 8 same-signed ones 4.6e-8 against 4.8e-8, 16
+// already 6.1e-8 against 4.6e-8 (relative error in norm).
+constexpr int SHALLOW = kF32Shallow;
+__device__ __forceinline__ int depth_of(const Launch& L, const Item& it) {
+    int d = 0;
+    for (int t = 0; t < it.P->nt; ++t) {
+        int kb, ke;
+        k_range(L, it, it.P->t[t].K, kb, ke);
+        d += max(0, ke - kb);
+    }
+    return d;
+}
+
+// the chunks that an item gives the tensor cores
 __device__ __forceinline__ int chunks_of(const Launch& L, const Item& it) {
+    if (L.shallow && depth_of(L, it) <= SHALLOW) return 0;
     int C = 0;
     for (int t = 0; t < it.P->nt; ++t) {
         int kb, ke;
@@ -307,9 +338,12 @@ __device__ __forceinline__ void copy_chunk(const Opnd& o, int k0, int ke, int w,
 // 8 different columns, or consecutive rows) and the 8-byte stores (rows 8 to 15
 // of 16 take the other half of the k-group: together all banks) are free of
 // bank conflicts.  k contiguous: thread = (row, half of each k-group); rows
-// contiguous: thread = (row, k-group).
+// contiguous: thread = (row, k-group).  True where a value other than zero is below
+// 2^-109, so that its split may not be exact (half an instruction per value finds the
+// smallest magnitude; where that is below, zeros are told from the rest).
 template <bool KCONTIG>
-__device__ __forceinline__ void split_chunk(char* tile, const char* raw, int t8) {
+__device__ __forceinline__ bool split_chunk(char* tile, const char* raw, int t8) {
+    float least = 1.f;
     const int r = KCONTIG ? (t8 >> 5) * 16 + (t8 & 15) : t8 & 127;
     const int odd = (r >> 3) & 1;
     char* const d = tile + (r >> 3) * 256 + (r & 7) * 16;
@@ -332,62 +366,136 @@ __device__ __forceinline__ void split_chunk(char* tile, const char* raw, int t8)
         }
         char* const o = d + kg * 128 + h * 8;
         uint32_t w[2][3];
-        split2(v[0].x, v[1].x, w[0]);
-        split2(v[2].x, v[3].x, w[1]);
+        split2(v[0].x, v[1].x, w[0], least);
+        split2(v[2].x, v[3].x, w[1], least);
 #pragma unroll
         for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(o + p * PLANE) = make_uint2(w[0][p], w[1][p]);
-        split2(v[0].y, v[1].y, w[0]);
-        split2(v[2].y, v[3].y, w[1]);
+        split2(v[0].y, v[1].y, w[0], least);
+        split2(v[2].y, v[3].y, w[1], least);
 #pragma unroll
         for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(o + (3 + p) * PLANE) = make_uint2(w[0][p], w[1][p]);
     }
-}
-
-// one output by plain FP32 fused multiply-adds
-template <int AM, int BMD>
-__device__ __forceinline__ float2 plain_dot(const Launch& L, const Item& it, int m, int n) {
-    float2 c = make_float2(0.f, 0.f);
-    for (int ti = 0; ti < it.P->nt; ++ti) {
-        const GTerm& t = it.P->t[ti];
-        int kb, ke;
-        k_range(L, it, t.K, kb, ke);
-        for (int k = kb; k < ke; ++k) {
-            float2 a = AM == A_KM ? t.A[(long long)k * t.lda + m] : t.A[(long long)m * t.lda + k];
-            const long long row = BMD == B_KN ? (t.g ? t.g[k] : k) : (t.g ? t.g[n] : n);
-            float2 b = BMD == B_KN ? t.B[row * t.ldb + n] : t.B[row * t.ldb + k];
-            a.y *= t.sa;
-            b.y *= t.sb;
-            c.x = fmaf(a.x, b.x, c.x);
-            c.x = fmaf(-a.y, b.y, c.x);
-            c.y = fmaf(a.x, b.y, c.y);
-            c.y = fmaf(a.y, b.x, c.y);
+    if (!(least < 0x1p-109f)) return false;
+    bool small = false;
+    const float2* q = reinterpret_cast<const float2*>(raw);
+#pragma unroll 1
+    for (int i = 0; i < 8; ++i) {   // the same values again
+        float2 v;
+        if (KCONTIG) {
+            const int kg = i >> 2, h = ((t8 >> 4) & 1) ^ odd;
+            v = q[(raw_pos(r, kg * 4 + h * 2 + ((i >> 1) & 1)) >> 3) + (i & 1)];
+        } else {
+            v = q[((t8 >> 7) * 8 + i) * 128 + r];
         }
+        small = small || (v.x != 0.f && fabsf(v.x) < 0x1p-109f) || (v.y != 0.f && fabsf(v.y) < 0x1p-109f);
     }
-    return c;
+    return small;
 }
 
-__device__ __forceinline__ bool finite2(float2 v) { return isfinite(v.x) && isfinite(v.y); }
+// A result that the tensor cores gave as plain FP32 multiply-adds would, up to its
+// rounding: zero, or from 2^-100 up and finite (below, the sums' own rounding nears
+// FP32's smallest values, which the tensor core meets 24 times a chunk).
+__device__ __forceinline__ bool good(float x) {
+    const uint32_t u = __float_as_uint(x) & 0x7fffffffu, lo = (uint32_t)(127 - 100) << 23;
+    return u == 0u || u - lo < 0x7f800000u - lo;
+}
 
-// Recomputes the non-finite results among a thread's row of 32 columns just
-// written (not inlined: called once the accumulators are dead).
+// a magnitude's bits, doubled, less one: zero becomes the largest
+__device__ __forceinline__ uint32_t twice(float x) { return 2u * __float_as_uint(x) - 1u; }
+
+// Recomputes results of a warp's 32 x 32 part of a tile just written by plain FP32
+// fused multiply-adds along k: all of them, or those that are not good().  The warp
+// works on 32 x 16 at a time, a lane on 4 rows (8 apart) and 4 columns (4 apart), so
+// an operand row read from L1 or L2 serves 4 products (one lane per row, an output
+// after the other, read each operand row for one).  
 template <int AM, int BMD>
-__device__ __noinline__ void mend_row(const Launch& L, int item, int epi, long long part_stride, int lg, int cg,
-                                      int lane) {
+__device__ __forceinline__ void plain_tile(const Launch& L, int item, bool all) {
+    const int lane = threadIdx.x & 31, lg = (threadIdx.x >> 5) & 3, cg = threadIdx.x >> 7, epi = L.epi;
     Item it;
     item_at(L, item, it);
     const GProb& P = *it.P;
-    const int m = it.m0 + lg * 32 + lane, nb = it.n0 + cg * 32;
-    if (m >= P.M) return;
-    cf* const Cp = P.C + (epi == EPI_PARTIAL ? it.chunk * part_stride : 0) + (long long)m * P.ldc;
-    for (int n = nb; n < min(P.N, nb + 32); ++n) {
-        if (finite2(Cp[n])) continue;
-        float2 v = plain_dot<AM, BMD>(L, it, m, n);
-        if (epi == EPI_SUB) {
-            const float2 s = P.S[(long long)m * P.ldc + n];
-            v.x -= s.x;
-            v.y -= s.y;
+    const int m0 = it.m0 + lg * 32 + (lane & 7);
+    cf* const C = P.C + (epi == EPI_PARTIAL ? it.chunk * L.part_stride : 0);
+    __syncwarp();   // the other lanes' results are read below
+    for (int half = 0; half < 2; ++half) {
+        const int n0 = it.n0 + cg * 32 + half * 16 + (lane >> 3);
+        unsigned todo = 0;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int m = m0 + (e >> 2) * 8, n = n0 + (e & 3) * 4;
+            if (m < P.M && n < P.N) {
+                bool again = all;
+                if (!all) {
+                    const float2 v = C[(long long)m * P.ldc + n];
+                    again = !good(v.x) || !good(v.y);
+                }
+                if (again) todo |= 1u << e;
+            }
         }
-        Cp[n] = v;
+        if (!__any_sync(0xffffffffu, todo != 0u)) continue;
+        float2 c[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) c[e] = make_float2(0.f, 0.f);
+        for (int ti = 0; ti < P.nt; ++ti) {
+            const GTerm& t = P.t[ti];
+            int kb, ke;
+            k_range(L, it, t.K, kb, ke);
+            const cf* a[4];
+            const cf* b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {   // rows and columns beyond the operands read the last
+                const int m = min(m0 + i * 8, P.M - 1), n = min(n0 + i * 4, P.N - 1);
+                a[i] = AM == A_KM ? t.A + m : t.A + (long long)m * t.lda;
+                b[i] = BMD == B_KN ? t.B + n : t.B + (long long)(t.g ? t.g[n] : n) * t.ldb;
+            }
+            const float sa = t.sa, sb = t.sb;
+            for (int k = kb; k < ke; ++k) {
+                const long long ao = AM == A_KM ? (long long)k * t.lda : k;
+                const long long bo = BMD == B_KN ? (long long)(t.g ? t.g[k] : k) * t.ldb : k;
+                float2 x[4], y[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    x[i] = a[i][ao];
+                    x[i].y *= sa;
+                    y[i] = b[i][bo];
+                    y[i].y *= sb;
+                }
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    const float2 u = x[e >> 2], v = y[e & 3];
+                    c[e].x = fmaf(u.x, v.x, c[e].x);
+                    c[e].x = fmaf(-u.y, v.y, c[e].x);
+                    c[e].y = fmaf(u.x, v.y, c[e].y);
+                    c[e].y = fmaf(u.y, v.x, c[e].y);
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            if (!(todo >> e & 1u)) continue;
+            const long long o = (long long)(m0 + (e >> 2) * 8) * P.ldc + n0 + (e & 3) * 4;
+            if (epi == EPI_SUB) {
+                const float2 s = P.S[o];
+                c[e].x -= s.x;
+                c[e].y -= s.y;
+            }
+            C[o] = c[e];
+        }
+    }
+}
+
+// A warp's part of this CTA's items: those without chunks and those with any of the
+// chunks span[0] .. span[1] as a whole, of the items span[2] .. span[3] what is not good()
+template <int AM, int BMD>
+__device__ __noinline__ void plain_items(const Launch& L, const int* span) {
+    int c = 0;
+    for (int i = blockIdx.x; i < L.nitems; i += gridDim.x) {
+        Item it;
+        if (!item_at(L, i, it)) continue;
+        const int C = chunks_of(L, it);
+        const bool all = C == 0 || (c <= span[1] && c + C > span[0]);
+        if (all || (i >= span[2] && i <= span[3])) plain_tile<AM, BMD>(L, i, all);
+        c += C;
     }
 }
 
@@ -395,16 +503,18 @@ __device__ __noinline__ void mend_row(const Launch& L, int item, int epi, long l
 // imaginary parts) to the tile's destination, 16 bytes at a time; consecutive
 // stores fill the row's 32-byte sectors.  (No room for a staging transpose in
 // shared memory; the stores run beside the next tile's first MMAs.)  True if
-// any value is not finite.
-__device__ __forceinline__ bool write_tile(const Item& it, int epi, long long part_stride, const uint64_t* acc, int lg,
-                                           int cg, int lane) {
+// any value is not good().
+__device__ __forceinline__ bool write_tile(const Launch& L, const Item& it, const uint64_t* acc, int lg, int cg,
+                                           int lane) {
+    const int epi = L.epi;
     const GProb& P = *it.P;
     const int m = it.m0 + lg * 32 + lane, nb = it.n0 + cg * 32, N = P.N;
     if (m >= P.M) return false;
-    cf* const Cp = P.C + (epi == EPI_PARTIAL ? it.chunk * part_stride : 0) + (long long)m * P.ldc + nb;
+    cf* const Cp = P.C + (epi == EPI_PARTIAL ? it.chunk * L.part_stride : 0) + (long long)m * P.ldc + nb;
     const cf* const Sp = epi == EPI_SUB ? P.S + (long long)m * P.ldc + nb : nullptr;
     const bool vec = ((reinterpret_cast<uintptr_t>(Cp) | reinterpret_cast<uintptr_t>(Sp)) & 15) == 0;
-    bool bad = false;
+    float most = 0.f;
+    uint32_t least = ~0u;
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
         if (nb + 2 * q < N) {
@@ -428,7 +538,12 @@ __device__ __forceinline__ bool write_tile(const Item& it, int epi, long long pa
                     }
                 }
             }
-            bad |= !(isfinite(v.x) && isfinite(v.y)) || (two && !(isfinite(v.z) && isfinite(v.w)));
+            // of a single column twice the same value
+            const float z = two ? v.z : v.x, w = two ? v.w : v.y;
+            max_abs(most, v.x, v.y);
+            max_abs(most, z, w);
+            least = __vimin3_u32(least, twice(v.x), twice(v.y));
+            least = __vimin3_u32(least, twice(z), twice(w));
             if (vec && two) {
                 *reinterpret_cast<float4*>(Cp + 2 * q) = v;
             } else {
@@ -437,12 +552,11 @@ __device__ __forceinline__ bool write_tile(const Item& it, int epi, long long pa
             }
         }
     }
-    return bad;
+    return least < 2u * ((uint32_t)(127 - 100) << 23) - 1u || !(most < INFINITY);
 }
 
 template <int AM, int BMD>
-__global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ Launch L, int epi,
-                                                       long long part_stride, int* err) {
+__global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ Launch L, int* err) {
     chain_wait();
     extern __shared__ __align__(1024) char smem[];
     if (*(volatile int*)err != 0) return;   // an earlier contraction gave up: do no more work
@@ -454,6 +568,9 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
     uint64_t* rempty = rfull + NRAW;        // [NRAW] raw chunk read (one arrival per worker warp)
     uint32_t* tslot = reinterpret_cast<uint32_t*>(rempty + NRAW);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+    // what is computed again: the first and last of this CTA's chunks with a value whose
+    // split may not be exact, the first and last item with results that are not good(), any
+    int* const again = reinterpret_cast<int*>(tslot + 2);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < NSTAGE; ++s) {
@@ -470,7 +587,14 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *abort_flag = 0;
+        again[0] = again[2] = INT_MAX;
+        again[1] = again[3] = -1;
+        again[4] = 0;
     }
+    // ones where no copy goes (rows beyond an operand), so that nothing left there by
+    // another kernel is taken for a small value
+    for (int e = threadIdx.x; e < NRAW * 2 * RAW_OP / 16; e += NTHR)
+        reinterpret_cast<float4*>(smem + RAW_OFF)[e] = make_float4(1.f, 1.f, 1.f, 1.f);
     if (warp == WMMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"(TMEM_COLS)
@@ -488,7 +612,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
             int c = 0;
             for (int i = blockIdx.x; i < L.nitems && !*abort_flag; i += gridDim.x) {
                 Item it;
-                if (!item_at(L, i, it)) continue;
+                if (!item_at(L, i, it) || (L.shallow && depth_of(L, it) <= SHALLOW)) continue;
                 // a ragged last N tile computes only its 16-column groups
                 const uint32_t idesc = IDESC | ((uint32_t)(min(TN, (it.P->N - it.n0 + 15) & ~15) >> 3) << 17);
                 for (int t = 0; t < it.P->nt && !*abort_flag; ++t) {
@@ -536,7 +660,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
         int c = 0;
         for (int i = blockIdx.x; i < L.nitems && !*abort_flag; i += gridDim.x) {
             Item it;
-            if (!item_at(L, i, it)) continue;
+            if (!item_at(L, i, it) || (L.shallow && depth_of(L, it) <= SHALLOW)) continue;
             for (int t = 0; t < it.P->nt && !*abort_flag; ++t) {
                 const GTerm& T = it.P->t[t];
                 int k0, ke;
@@ -565,14 +689,22 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
         const int t8 = threadIdx.x & 255;
         const int lg = warp & 3, cg = warp >> 2;   // TMEM lanes 32 lg .., columns 32 cg ..
         const uint32_t tm0 = tmem + ((uint32_t)(lg * 32) << 16) + cg * 32;
+        // the chunks of this CTA in all (the split runs ahead of the drain, across items)
+        int total = 0;
+        for (int i = blockIdx.x; i < L.nitems; i += gridDim.x) {
+            Item it;
+            if (!item_at(L, i, it)) continue;
+            const int C = chunks_of(L, it);
+            total += C;
+            if (C == 0) *(volatile int*)(again + 4) = 1;
+        }
         uint64_t acc[32];   // real parts of 32 columns in pairs, then imaginary parts
 #pragma unroll
         for (int j = 0; j < 32; ++j) acc[j] = 0;
         // the item whose chunks are being added up, its chunks still to split and to drain
         int ci = (int)blockIdx.x - (int)gridDim.x;
         bool cols = false;   // it has columns in this warp's group
-        // moves to the next item with chunks (returns their number, 0 at the
-        // end); items without chunks are written as zeros on the way
+        // moves to the next item with chunks (returns their number, 0 at the end)
         auto next_item = [&]() -> int {
             for (;;) {
                 ci += gridDim.x;
@@ -582,15 +714,8 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
                 const int C = chunks_of(L, it);
                 cols = it.n0 + cg * 32 < it.P->N;
                 if (C > 0) return C;
-                write_tile(it, epi, part_stride, acc, lg, cg, lane);
             }
         };
-        // chunks of this CTA in all (the split runs ahead of the drain, across items)
-        int total = 0;
-        for (int i = blockIdx.x; i < L.nitems; i += gridDim.x) {
-            Item it;
-            if (item_at(L, i, it)) total += chunks_of(L, it);
-        }
         int left = next_item();
         int produced = 0, drained = 0;
         while (drained < total) {
@@ -604,10 +729,12 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
                 }
                 char* tile = smem + s * STAGE + (isB ? TILE : 0);
                 const char* raw = smem + RAW_OFF + (2 * r + (isB ? 1 : 0)) * RAW_OP;
-                if (isB)
-                    split_chunk<BMD == B_NK>(tile, raw, t8);
-                else
-                    split_chunk<AM == A_MK>(tile, raw, t8);
+                const bool t = isB ? split_chunk<BMD == B_NK>(tile, raw, t8) : split_chunk<AM == A_MK>(tile, raw, t8);
+                if (t) {
+                    atomicMin(again, produced);
+                    atomicMax(again + 1, produced);
+                    *(volatile int*)(again + 4) = 1;
+                }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) {
@@ -642,8 +769,11 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
             if (--left == 0) {
                 Item it;
                 item_at(L, ci, it);
-                const bool bad = write_tile(it, epi, part_stride, acc, lg, cg, lane);
-                if (__any_sync(0xffffffffu, bad)) mend_row<AM, BMD>(L, ci, epi, part_stride, lg, cg, lane);
+                if (write_tile(L, it, acc, lg, cg, lane)) {
+                    atomicMin(again + 2, ci);
+                    atomicMax(again + 3, ci);
+                    *(volatile int*)(again + 4) = 1;
+                }
 #pragma unroll
                 for (int j = 0; j < 32; ++j) acc[j] = 0;
                 left = next_item();
@@ -654,18 +784,20 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
     __syncthreads();
     if (*abort_flag && threadIdx.x == 0) atomicExch(err, TLR_ERR_TIMEOUT);
     if (warp == WMMA) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tslot), "r"(TMEM_COLS) : "memory");
     }
+    // what the split does not hold, and sums of few products
+    if (warp < NW && again[4] && !*abort_flag) plain_items<AM, BMD>(L, again);
 }
 
 template <int AM, int BMD>
 cudaError_t launch(const GemmLaunch& G, const Launch& L, unsigned grid, cudaStream_t st) {
     counted(1);
     if (t_early_blocks != kEarlyAny) {   // in a solve: a CTA takes a whole SM, early ones crowd (see chain_entry)
-        k_cgemm_f32<AM, BMD><<<grid, NTHR, SMEM_BYTES, st>>>(L, G.epi, G.part_stride, G.err);
+        k_cgemm_f32<AM, BMD><<<grid, NTHR, SMEM_BYTES, st>>>(L, G.err);
         return cudaGetLastError();
     }
-    return launch_chain(k_cgemm_f32<AM, BMD>, dim3(grid), dim3(NTHR), SMEM_BYTES, st, L, G.epi, G.part_stride, G.err);
+    return launch_chain(k_cgemm_f32<AM, BMD>, dim3(grid), dim3(NTHR), SMEM_BYTES, st, L, G.err);
 }
 
 }  // namespace
@@ -696,6 +828,16 @@ cudaError_t gemm_f32_prepare() {
     return e;
 }
 
+bool gemm_f32_shallow(const GProb& p, int nsplit, int kchunk) {
+    for (int c = 0; c < nsplit; ++c) {
+        long long d = 0;
+        for (int t = 0; t < p.nt; ++t)
+            d += nsplit == 1 ? p.t[t].K : std::max(0LL, std::min<long long>(p.t[t].K - (long long)c * kchunk, kchunk));
+        if (d > 0 && d <= SHALLOW) return true;
+    }
+    return false;
+}
+
 cudaError_t gemm_f32(const GemmLaunch& G, cudaStream_t st) {
     if (G.nprob == 0 || G.maxM == 0 || G.maxN == 0) return cudaSuccess;
     if (!G.err) return cudaErrorInvalidValue;
@@ -708,6 +850,9 @@ cudaError_t gemm_f32(const GemmLaunch& G, cudaStream_t st) {
     const long long nitems = (long long)L.nx * L.ny * G.nprob * G.nsplit;
     if (nitems > 0x7fff0000LL) return cudaErrorInvalidValue;
     L.nitems = (int)nitems;
+    L.epi = G.epi;
+    L.shallow = G.shallow ? 1 : 0;
+    L.part_stride = G.part_stride;
     const unsigned grid = (unsigned)std::min<long long>(device_sms(), nitems);
     if (G.amode == A_KM && G.bmode == B_KN) return launch<A_KM, B_KN>(G, L, grid, st);
     if (G.amode == A_MK && G.bmode == B_KN) return launch<A_MK, B_KN>(G, L, grid, st);

@@ -110,6 +110,7 @@ extern "C" int tlr_mdd_adjoint_noalloc(const void* V, const void* Dt, int64_t nr
     L.kchunk = (int)(((ns + nsplit - 1) / nsplit + 15) / 16 * 16);
     L.part_stride = nr * nr;
     L.epi = EPI_PARTIAL;
+    L.shallow = gemm_f32_shallow(p, nsplit, L.kchunk);
     L.cls = 2;                                           // diagnostics class: project / adjoint
     L.flops = 8.0 * (double)nr * (double)nr * (double)ns;
     // Every partial slab is written in full by the GEMM before the reduction
