@@ -196,18 +196,23 @@ int tlr_mdd_create(tlr_mdd_t** h, const tlr_mdd_desc_t* d, const void* D, const 
 int tlr_mdd_set_data(tlr_mdd_t* h, const void* D, const void* U, int32_t input_memory);
 
 /* Y = X_h Dfrak (receiver-major, Hilbert order), nr x ns complex64 DEVICE.
- * X_h = C(theta) by eq. (6)-(9), (15); theta DEVICE complex64 [n_theta]. */
+ * X_h = C(theta) by eq. (6)-(9), (15); theta DEVICE complex64 [n_theta].
+ * Asynchronous: a contraction that gives up on a bounded wait (the handle's
+ * later ones then do nothing) shows at the handle's next synchronising product
+ * or solve (tlr_mdd_grad with f, tlr_mdd_adjoint, tlr_mdd_solve,
+ * tlr_mdd_solve_wait, tlr_mdd_batch_wait, tlr_mdd_benchmark_solve), which returns
+ * TLR_ERR_TIMEOUT and leaves the handle usable. */
 int tlr_mdd_apply(tlr_mdd_t* h, const void* theta, void* Y);
 
 /* G = V Dfrak^H, nr x nr complex64 DEVICE, for V nr x ns complex64 DEVICE.
  * With V = X_h Dfrak - Ufrak this is W^T, W = D^H (D X - U) (Derivatives
- * paragraph); W' = G + G^T. */
+ * paragraph); W' = G + G^T.  Synchronises. */
 int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G);
 
 /* f = 0.5 ||D-hat C(theta) - U-hat||_F^2 (eq. 17a) and its factor gradients
  * (eq. 25-27) stacked like theta in grad (DEVICE complex64 [n_theta]); the
  * convention is grad = df/dRe(theta) + i df/dIm(theta).  f: HOST double
- * (the call synchronises the stream), or NULL. */
+ * (the call synchronises the stream), or NULL (asynchronous, as tlr_mdd_apply). */
 int tlr_mdd_grad(tlr_mdd_t* h, const void* theta, void* grad, double* f);
 
 /* ADMM with an L-BFGS x-update and exact line search (eq. 18-24), lambda

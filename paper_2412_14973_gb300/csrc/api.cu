@@ -1668,6 +1668,14 @@ int tlr_mdd_set_data(tlr_mdd_t* h, const void* D, const void* U, int32_t input_m
     return TLR_OK;
 }
 
+// A contraction of this handle gave up on a bounded wait (those after it returned at
+// once): report it and clear the word, so that the handle can be used again.
+static int timed_out(tlr_mdd_s* h) {
+    CK(h, cudaMemsetAsync(h->ints + SI_COUNT + 1, 0, sizeof(int), h->st));
+    CK(h, cudaStreamSynchronize(h->st));
+    FAIL(h, TLR_ERR_TIMEOUT, "a tensor-core contraction timed out on a barrier wait");
+}
+
 static int forward(tlr_mdd_s* h, bool plain_apply) {
     const Layout& L = h->L;
     CK(h, sym_dense(h->x, L.nlr, L.ndense, L.dmax, h->Zs, h->st, L.general, h->pm.zoff, h->pm.zdim));
@@ -1741,11 +1749,7 @@ int tlr_mdd_grad(tlr_mdd_t* h, const void* theta, void* grad, double* f) {
         CK(h, cudaMemcpyAsync(&rr, h->scal + 1, sizeof(double), cudaMemcpyDeviceToHost, h->st));
         CK(h, cudaMemcpyAsync(&werr, h->ints + SI_COUNT + 1, sizeof(int), cudaMemcpyDeviceToHost, h->st));
         CK(h, cudaStreamSynchronize(h->st));
-        if (werr != 0) {
-            CK(h, cudaMemsetAsync(h->ints + SI_COUNT + 1, 0, sizeof(int), h->st));
-            CK(h, cudaStreamSynchronize(h->st));
-            FAIL(h, TLR_ERR_TIMEOUT, "a tensor-core contraction timed out on a barrier wait");
-        }
+        if (werr != 0) return timed_out(h);
         *f = 0.5 * rr;
     }
     return TLR_OK;
@@ -1850,9 +1854,11 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     G1.err = h->ints + SI_COUNT + 1;
     if (e == cudaSuccess) e = run_gemm(G1, h->st);
     if (e == cudaSuccess && ns_split > 1) e = reduce_grad(part, ns_split, nr * nr, nr * nr, 0, 1, (cf*)G, h->st);
+    int werr = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&werr, h->ints + SI_COUNT + 1, sizeof(int), cudaMemcpyDeviceToHost, h->st);
     if (own) cudaFreeAsync(part, h->st);
-    CK(h, settle(e, h->st));   // tab lives on this stack frame
-    return TLR_OK;
+    CK(h, settle(e, h->st));   // tab and werr live on this stack frame
+    return werr != 0 ? timed_out(h) : TLR_OK;
 }
 
 // Benchmark solver of eq. (4) on the handle's data: conjugate gradients on
@@ -2019,11 +2025,7 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     CK(h, e);
-    if (werr != 0) {
-        CK(h, cudaMemsetAsync(h->ints + SI_COUNT + 1, 0, sizeof(int), h->st));
-        CK(h, cudaStreamSynchronize(h->st));
-        FAIL(h, TLR_ERR_TIMEOUT, "a tensor-core contraction timed out on a barrier wait");
-    }
+    if (werr != 0) return timed_out(h);
     // slots of k_cg.cu: rr 0, <p,Ap> 1, alpha 2, beta 3, ||b||^2 4, done 5, iterations 6
     const double rel = hs[4] > 0.0 ? std::sqrt(hs[0] / hs[4]) : 0.0;
     const int status = std::isfinite(hs[0]) ? TLR_OK : TLR_ERR_NONFINITE;
@@ -2736,12 +2738,7 @@ int tlr_mdd_solve_wait(tlr_mdd_t* h, tlr_mdd_stats_t* stats) {
         stats->f0 = hs.sc[SC_F0];
         stats->gpu_ms = ms;
     }
-    if (hs.ints[SI_COUNT + 1] != 0) {
-        // a tensor-core contraction gave up on a bounded wait: report and re-arm
-        CK(h, cudaMemsetAsync(h->ints + SI_COUNT + 1, 0, sizeof(int), h->st));
-        CK(h, cudaStreamSynchronize(h->st));
-        FAIL(h, TLR_ERR_TIMEOUT, "a tensor-core contraction timed out on a barrier wait");
-    }
+    if (hs.ints[SI_COUNT + 1] != 0) return timed_out(h);
     if (hs.ints[SI_STATUS] != 0) FAIL(h, TLR_ERR_NONFINITE, "non-finite value met during the solve");
     return TLR_OK;
 }
@@ -3191,9 +3188,14 @@ int tlr_mdd_batch_wait(tlr_mdd_batch_t* b, tlr_mdd_stats_t* stats) {
             s.gpu_ms = ms;
         }
         if (hs.ints[SI_STATUS] != 0) worst = TLR_ERR_NONFINITE;
+        if (hs.ints[SI_COUNT + 1] != 0) {   // a contraction of this member's own
+            BCK(cudaMemset(b->hs[m]->ints + SI_COUNT + 1, 0, sizeof(int)));
+            werr = hs.ints[SI_COUNT + 1];
+        }
     }
     if (werr != 0) {
         BCK(cudaMemset(b->err, 0, sizeof(int)));
+        BCK(cudaStreamSynchronize(nullptr));   // before anything on the members' and the batch's streams
         FAIL((tlr_mdd_s*)nullptr, TLR_ERR_TIMEOUT, "a tensor-core contraction timed out on a barrier wait");
     }
     if (worst) FAIL((tlr_mdd_s*)nullptr, worst, "non-finite value met during a member's solve");
