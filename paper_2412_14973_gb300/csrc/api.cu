@@ -27,6 +27,7 @@
 #include <mutex>
 #include <set>
 #include <tuple>
+#include <unordered_map>
 
 using namespace tlr;
 
@@ -109,12 +110,40 @@ cudaError_t ws_pool(cudaMemPool_t* out) {
     return cudaSuccess;
 }
 
+// What handles have taken from each device's pool, and the most of it since the
+// reserve was last handed back: the part of the reserve that is meant to stay.
+struct Taken {
+    unsigned long long now = 0, most = 0;
+};
+Taken g_taken[kMaxPoolDevices];
+std::unordered_map<void*, std::pair<int, size_t>> g_blocks;   // handles' blocks: device, bytes
+
 // stream-ordered allocation of handle workspace from the library's pool
 cudaError_t ws_alloc(void** ptr, size_t bytes, cudaStream_t st) {
     cudaMemPool_t p = nullptr;
+    int dev = 0;
     cudaError_t e = ws_pool(&p);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(ptr, bytes, p, st);
     if (e != cudaSuccess) return e;
-    return cudaMallocFromPoolAsync(ptr, bytes, p, st);
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    g_blocks[*ptr] = {dev, bytes};
+    g_taken[dev].now += bytes;
+    g_taken[dev].most = std::max(g_taken[dev].most, g_taken[dev].now);
+    return cudaSuccess;
+}
+
+void ws_free(void* ptr, cudaStream_t st) {
+    if (!ptr) return;
+    {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        auto it = g_blocks.find(ptr);
+        if (it != g_blocks.end()) {
+            g_taken[it->second.first].now -= it->second.second;
+            g_blocks.erase(it);
+        }
+    }
+    cudaFreeAsync(ptr, st);
 }
 
 // Waits for the stream, whatever e is (an asynchronous copy from pageable memory may
@@ -127,8 +156,8 @@ cudaError_t settle(cudaError_t e, cudaStream_t st) {
 
 // Per-call scratch, from the same pool: mapping fresh device memory on every
 // call cost as much as the work it served (0.9 of 5.9 ms of a benchmark solve at
-// nr = 2048).  When it is given back the pool keeps at most kScratchKeep bytes
-// more than it held reserved before the call.
+// nr = 2048).  Once it is given back the pool holds at most kScratchKeep bytes more
+// than handles have taken, however many calls there were.
 constexpr unsigned long long kScratchKeep = 256ull << 20;
 
 class Scratch {
@@ -139,7 +168,7 @@ public:
     cudaError_t get(size_t bytes, cudaStream_t st) {
         st_ = st;
         cudaError_t e = ws_pool(&pool_);
-        if (e == cudaSuccess) e = cudaMemPoolGetAttribute(pool_, cudaMemPoolAttrReservedMemCurrent, &before_);
+        if (e == cudaSuccess) e = cudaGetDevice(&dev_);
         if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)&p_, bytes, pool_, st);
         if (e != cudaSuccess) p_ = nullptr;
         return e;
@@ -155,16 +184,20 @@ public:
     }
     ~Scratch() {
         release();
-        unsigned long long now = 0;
-        if (freed_ && cudaMemPoolGetAttribute(pool_, cudaMemPoolAttrReservedMemCurrent, &now) == cudaSuccess &&
-            now > before_ + kScratchKeep)
-            cudaMemPoolTrimTo(pool_, (size_t)(before_ + kScratchKeep));
+        if (!freed_) return;
+        unsigned long long now = 0, keep;
+        {
+            std::lock_guard<std::mutex> lk(g_pool_mu);
+            keep = g_taken[dev_].most + kScratchKeep;
+        }
+        if (cudaMemPoolGetAttribute(pool_, cudaMemPoolAttrReservedMemCurrent, &now) == cudaSuccess && now > keep)
+            cudaMemPoolTrimTo(pool_, (size_t)keep);
     }
 
 private:
     cudaMemPool_t pool_ = nullptr;
     cudaStream_t st_ = nullptr;
-    unsigned long long before_ = 0;
+    int dev_ = 0;
     char* p_ = nullptr;
     bool freed_ = false;
 };
@@ -1538,9 +1571,9 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
     h->arena_bytes = a.used;
     auto fail = [&](int code) {
         g_last_error = h->err;
-        if (h->packed) cudaFreeAsync(h->packed, h->st);
-        if (h->tcp_tables) cudaFreeAsync(h->tcp_tables, h->st);
-        if (h->arena) cudaFreeAsync(h->arena, h->st);
+        ws_free(h->packed, h->st);
+        ws_free(h->tcp_tables, h->st);
+        ws_free(h->arena, h->st);
         if (h->ev0) cudaEventDestroy(h->ev0);
         if (h->ev1) cudaEventDestroy(h->ev1);
         cudaStreamSynchronize(h->st);   // copies may still read h->uploads, D, U or write the statistics
@@ -1567,6 +1600,7 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
             return fail(e_ == cudaErrorMemoryAllocation ? TLR_ERR_NOMEM : TLR_ERR_CUDA); \
         }                                                                          \
     } while (0)
+    Scratch own;   // of the receiver order, given back once the stream has been waited for
     // receiver order
     if (d->perm) {
         std::vector<char> seen(L.nr, 0);
@@ -1584,7 +1618,6 @@ int tlr_mdd_create(tlr_mdd_t** out, const tlr_mdd_desc_t* d, const void* D, cons
         while (n < d->nx || n < d->ny) n <<= 1;
         // its slots (n^2 of them) in the work panels, or of their own where those are too small
         const size_t need = (size_t)(n * n) * sizeof(int32_t);
-        Scratch own;
         int32_t* slot = reinterpret_cast<int32_t*>(h->R);
         if (need > (size_t)(reinterpret_cast<char*>(h->Zs) - reinterpret_cast<char*>(h->R))) {
             CKF(own.get(need, h->st));
@@ -2436,6 +2469,14 @@ int tlr_mdd_trim_pool(int64_t keep_bytes, int64_t* reserved) {
     cudaMemPool_t p = nullptr;
     CK((tlr_mdd_s*)nullptr, ws_pool(&p));
     CK((tlr_mdd_s*)nullptr, cudaMemPoolTrimTo(p, (size_t)keep_bytes));
+    {
+        int dev = 0;
+        CK((tlr_mdd_s*)nullptr, cudaGetDevice(&dev));
+        unsigned long long left = 0;
+        CK((tlr_mdd_s*)nullptr, cudaMemPoolGetAttribute(p, cudaMemPoolAttrReservedMemCurrent, &left));
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        g_taken[dev].most = std::max(g_taken[dev].now, std::min(g_taken[dev].most, left));
+    }
     std::vector<HostStats*> idle;
     {
         std::lock_guard<std::mutex> lk(g_pinned_mu);
@@ -2465,10 +2506,10 @@ int tlr_mdd_destroy(tlr_mdd_t* h) {
         cudaEventDestroy(t.a);
         cudaEventDestroy(t.b);
     }
-    if (h->ring) cudaFreeAsync(h->ring, h->st);
-    if (h->packed) cudaFreeAsync(h->packed, h->st);
-    if (h->tcp_tables) cudaFreeAsync(h->tcp_tables, h->st);
-    if (h->arena) cudaFreeAsync(h->arena, h->st);
+    ws_free(h->ring, h->st);
+    ws_free(h->packed, h->st);
+    ws_free(h->tcp_tables, h->st);
+    ws_free(h->arena, h->st);
     if (h->ev0) cudaEventDestroy(h->ev0);
     if (h->ev1) cudaEventDestroy(h->ev1);
     cudaError_t e = cudaStreamSynchronize(h->st);
@@ -2606,7 +2647,7 @@ static int enqueue_body(tlr_mdd_s* h, const tlr_mdd_solve_opts_t* o) {
             cudaGraphExecDestroy(h->gexec);
             h->gexec = nullptr;
         }
-        if (h->ring) cudaFreeAsync(h->ring, h->st);
+        ws_free(h->ring, h->st);
         h->ring = nullptr;
         h->ring_m = 0;
         CK(h, ws_alloc((void**)&h->ring, (size_t)2 * (o->memory + 1) * n2 * sizeof(float), h->st));
@@ -3038,7 +3079,7 @@ void b_free(tlr_mdd_batch_s* b) {
     if (b->ev0) cudaEventDestroy(b->ev0);
     if (b->ev1) cudaEventDestroy(b->ev1);
     if (b->tables) {
-        cudaFreeAsync(b->tables, b->st);
+        ws_free(b->tables, b->st);
         cudaStreamSynchronize(b->st);
     }
     delete b;
@@ -3129,7 +3170,7 @@ int tlr_mdd_batch_solve_async(tlr_mdd_batch_t* b, void* const* thetas, const tlr
                 cudaGraphExecDestroy(h->gexec);
                 h->gexec = nullptr;
             }
-            if (h->ring) cudaFreeAsync(h->ring, b->ms[m]);
+            ws_free(h->ring, b->ms[m]);
             h->ring = nullptr;
             h->ring_m = 0;
             BCK(ws_alloc((void**)&h->ring, (size_t)2 * (o->memory + 1) * n2 * sizeof(float), b->ms[m]));
