@@ -350,27 +350,28 @@ __device__ __forceinline__ int ring_idx(const SolverDev& S, int j) {
 
 // partials per block: for pair j of the group, <s_j,g>, <y_j,g>, <s_j,y_n>,
 // <s_n,y_j>, <y_j,y_n> (n = the newest pair).  Per-thread sums are plain FP32
-// multiply-adds (a thread sums a few dozen terms at these sizes), combined in FP64
-// across threads and blocks: these products only set the direction's coefficients,
-// whose rounding the exact line search and the descent test absorb.
+// multiply-adds (one term per 77824 values: a few dozen at the large sizes), combined
+// in FP64 across threads and blocks: these products only set the direction's
+// coefficients, whose rounding the exact line search and the descent test absorb.
 // 128 threads of <= 128 registers: a CTA fits beside the two GEMM CTAs of an SM
 constexpr int kLbThreads = 128;
 constexpr int kLbLd = kLbThreads + 8;   // row length of the block's sums: 4 rows read together lie in different banks
 
 __device__ void lb_solve(const SolverDev& S, int cnt, int ncl, double* val, double* mat);
 
-// Blocks of the direction's inner products: 4 values of each vector per thread (a
-// round of its 23 loads is a memory latency, a block's sums are 2 us of FP64 adds)
-// until there are kRedBlocks
+// Blocks of the direction's inner products: one value of each vector per thread until
+// there are kRedBlocks, so that up to 77824 values every product goes to the FP64 sums
+// by itself
 inline int lb_blocks(long long n2) {
-    const long long b = (n2 + 4 * kLbThreads - 1) / (4 * kLbThreads);
+    const long long b = (n2 + kLbThreads - 1) / kLbThreads;
     return (int)(b < 1 ? 1 : b > kRedBlocks ? kRedBlocks : b);
 }
 
 // last != 0: the launch over the last group of pairs, whose last block finishes
-// the direction's coefficients (lb_solve).  FP64 adds run at 2 lanes per cycle on
-// this part, so the block sums its 51 values 8 lanes each (72 cycles a value; a
-// shuffle tree per warp and value took 320).
+// the direction's coefficients (lb_solve).  FP64 adds and conversions run at 2 lanes
+// per cycle on this part, so a lane adds its 16 terms of a value up as an exact FP32
+// sum with its errors (Acc2: no fewer bits than FP64) and 8 lanes meet in FP64.  With
+// FP64 adds throughout, a solve of 256 receivers took 3.64 ms (3.37 here).
 __global__ void __launch_bounds__(kLbThreads, 4) k_lb_dots(SolverDev S, int j0, int last) {
     chain_entry();
     __shared__ __align__(16) float shv[kLbVals * kLbLd];
@@ -420,9 +421,14 @@ __global__ void __launch_bounds__(kLbThreads, 4) k_lb_dots(SolverDev S, int j0, 
         for (int v0 = 0; v0 < kLbVals; v0 += kLbThreads / 8) {
             const int v = v0 + (threadIdx.x >> 3);   // 8 lanes per value
             const float* row = shv + min(v, kLbVals - 1) * kLbLd;
-            double r = 0.0;
+            Acc2 a;
 #pragma unroll
-            for (int i = 0; i < kLbThreads / 8; ++i) r += (double)row[l8 + 8 * i];
+            for (int i = 0; i < kLbThreads / 8; ++i) a.add(row[l8 + 8 * i]);
+            double r = a.val();
+            if (!isfinite(r)) {   // Inf, NaN or sums beyond FP32
+                r = 0.0;
+                for (int i = 0; i < kLbThreads / 8; ++i) r += (double)row[l8 + 8 * i];
+            }
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o, 8);
             if (l8 == 0 && v < kLbVals) mine[v] = r;
