@@ -8,15 +8,16 @@
 // (unnormalised), k = 0 .. nt/2; the inverse puts the band [f0, f0 + nf) back
 // (zero elsewhere) and divides by nt.
 //
-// Lengths up to 4096 with prime factors up to 13, and any length up to 2048, take
-// one kernel per direction: a CTA transforms a few pairs of traces (a pair as the
+// Lengths up to 4096 with prime factors up to 13, and lengths up to 2048 with one above
+// 127, take one kernel per direction (where own_transform says that it is as accurate as
+// the library's): a CTA transforms a few pairs of traces (a pair as the
 // real and imaginary part of one complex transform) in shared memory and writes
 // the band of the frequency-major stack (stack[f][tr], one ns x nr panel per
 // frequency) or the traces themselves, so a trace is read once and its band
 // written once: 244 MB each way for 40000 traces of 1125 samples, 200 bins,
 // where a library transform between a spectrum in memory and a gather moved
-// 1.5 GB and its plans were made (and destroyed) on every call: 3.55 ms for both
-// directions against 0.46 here (kernels 233 + 189 us).  Bound by shared-memory
+// 1.5 GB and its plans were made (and destroyed) on every call: 3.5 to 4.9 ms for both
+// directions, as the host makes the plans, against 0.46 here (kernels 233 + 189 us).  Bound by shared-memory
 // traffic (two passes per factor); the bytes alone would take 72 us.
 //
 // Other lengths: cuFFT plans over a chunk of traces, with the band gather /
@@ -290,9 +291,10 @@ __global__ void __launch_bounds__(FFT_T) k_fft_chirp(const __grid_constant__ Fft
 // either stays relative to its own norm, and a trace of zeros stays zeros).
 // From every thread's squared norms s1, s2 over values of its pair (n1, n2: any
 // of them not zero): the scales up[], down[] per trace of the CTA.  Lanes `b` apart
-// share a pair (warp: one pair per warp).  Returns whether a trace cannot be
-// scaled (Inf, NaN, or a squared norm outside 1e-30 .. 1e30): then the traces are
-// transformed one at a time.
+// share a pair (warp: one pair per warp).  Returns whether a trace's norm is not to
+// be had (Inf, NaN, or a squared norm outside 1e-30 .. 1e30): then the traces are
+// transformed one at a time, such a one scaled by 2^-64 or 2^64, which keeps the
+// sums of a chirp in range.
 __device__ __forceinline__ bool pair_scales(float s1, float s2, bool n1, bool n2, int pair, int apart_by, int B,
                                             float* up, float* down) {
     __shared__ float red[FFT_T / 32][16], nzr[FFT_T / 32][16];
@@ -321,7 +323,7 @@ __device__ __forceinline__ bool pair_scales(float s1, float s2, bool n1, bool n2
             nz += nzr[i][threadIdx.x];
         }
         odd = nz != 0.f && !(ss > 1e-30f && ss < 1e30f);
-        const int e = nz != 0.f && !odd ? ilogbf(ss) / 2 : 0;
+        const int e = nz == 0.f ? 0 : !odd ? ilogbf(ss) / 2 : ss <= 1e-30f ? -64 : 64;
         up[threadIdx.x] = ldexpf(1.f, -e);
         down[threadIdx.x] = nz != 0.f ? ldexpf(1.f, e) : 0.f;
     }
@@ -355,7 +357,8 @@ __global__ void __launch_bounds__(FFT_T, 3) k_fft_forward(const __grid_constant_
             s2 = fmaf(v.y, v.y, s2);
             n1 = n1 || v.x != 0.f;
             n2 = n2 || v.y != 0.f;
-            if (pass == 1) v = make_float2(v.y, 0.f);
+            if (pass == 0) v.x *= up[2 * pr];
+            if (pass == 1) v = make_float2(v.y * up[2 * pr + 1], 0.f);
             a[pr * ld + t] = v;
         }
     };
@@ -383,7 +386,8 @@ __global__ void __launch_bounds__(FFT_T, 3) k_fft_forward(const __grid_constant_
             const cf u = z[b * ld + k], v = z[b * ld + kc];
             const long long tr = t0 + 2 * b, o = (long long)f * ntr + tr;
             if (apart) {
-                if (tr + pass < ntr) out[o + pass] = u;
+                const float h = down[2 * b + pass];
+                if (tr + pass < ntr) out[o + pass] = make_float2(u.x * h, u.y * h);
                 continue;
             }
             // z = x1 + i x2: X1 = (Z_k + conj Z_{n-k}) / 2, X2 = (Z_k - conj Z_{n-k}) / 2i
@@ -443,7 +447,12 @@ __global__ void __launch_bounds__(FFT_T, 3) k_fft_inverse(const __grid_constant_
         }
         apart = pair_scales(s1, s2, n1, n2, b, B, B, up, down);
     }
-    const float s = 1.f / (float)n;
+    // v / n: a product with the rounded 1 / n would be an error that all values share
+    const float s = 1.f / (float)n, nn = (float)n;
+    auto over_n = [&](float v) {
+        const float q = v * s;
+        return fmaf(fmaf(-q, nn, v), s, q);
+    };
     for (int pass = apart ? 0 : -1; pass < (apart ? 2 : 0); ++pass) {
         for (int e = threadIdx.x; e < B * ld; e += FFT_T) sm[e] = make_float2(0.f, 0.f);
         __syncthreads();
@@ -452,6 +461,7 @@ __global__ void __launch_bounds__(FFT_T, 3) k_fft_inverse(const __grid_constant_
             bin(f, p, q);
             if (apart) {
                 if (pass == 1) p = q;
+                p = make_float2(p.x * up[2 * b + pass], p.y * up[2 * b + pass]);
                 q = make_float2(0.f, 0.f);
             } else {   // the spectra are scaled here: a bin mixes both traces
                 p = make_float2(p.x * up[2 * b], p.y * up[2 * b]);
@@ -476,10 +486,10 @@ __global__ void __launch_bounds__(FFT_T, 3) k_fft_inverse(const __grid_constant_
             for (int t = threadIdx.x; t < n; t += FFT_T) {
                 const cf v = z[r * ld + t];   // the conjugate of n (x1 + i x2)
                 if (apart) {
-                    if (pass ? in2 : in1) (pass ? xb : xa)[t] = v.x * s;
+                    if (pass ? in2 : in1) (pass ? xb : xa)[t] = over_n(v.x) * down[2 * r + pass];
                 } else {
-                    if (in1) xa[t] = v.x * s * down[2 * r];
-                    if (in2) xb[t] = -v.y * s * down[2 * r + 1];
+                    if (in1) xa[t] = over_n(v.x) * down[2 * r];
+                    if (in2) xb[t] = over_n(-v.y) * down[2 * r + 1];
                 }
             }
         }
@@ -520,6 +530,28 @@ bool fft_plan(long long n, FftPlan& P) {
     P.B = 8;
     while (P.B > 2 && 2 * P.B * (P.M + 1) * (int)sizeof(cf) > 74 * 1024) P.B /= 2;
     return true;
+}
+
+// Whether the transform in shared memory is at least as accurate as the library's.
+// Measured, error against 64 bits of white traces over every length with factors to
+// 13 up to 4096 and 560 others up to 2048, own / library: chirps 0.6 to 0.77 where the
+// largest prime factor is above 127, up to 1.6 below (there the library has factors for
+// it); powers of two from 64 on 0.66 to 0.9; forward 0.5 to 0.95 from length 100 on (up
+// to 1.2 below); inverse 0.5 to 1.0 for even lengths above 1296 and odd ones from 1000 on
+// but powers of a prime (1.09 at 3125), up to 1.3 below (1.036 at 1080).
+bool own_transform(const FftPlan& P, bool forward) {
+    int most = 1, rest = P.n;
+    bool power = true;   // of one prime
+    for (int f = 2; rest > 1; ++f)
+        for (; rest % f == 0; rest /= f) {
+            power = power && (most == 1 || most == f);
+            most = f;
+        }
+    if (P.chirp) return most > 127;
+    if (P.n <= 2) return true;
+    if (power && most == 2) return P.n >= 64;
+    if (forward) return P.n >= 100;
+    return !power && (P.n % 2 == 0 ? P.n > 1296 : P.n >= 1000);
 }
 
 // both directions in shared memory (see the top of this file)
@@ -563,11 +595,13 @@ const char* cufft_msg(cufftResult r) {
     }
 }
 
-// traces per chunk: the chunk's real and complex buffers within ~256 MB
+// traces per chunk: the chunk's real and complex buffers within ~256 MB; an even
+// number of them, so that every chunk starts on 8 bytes like the first (cuFFT refuses
+// real arrays that do not)
 long long chunk_traces(long long ntr, long long nt) {
     const long long per = nt * 4 + (nt / 2 + 1) * 8;
     long long c = std::max(1LL, (256LL << 20) / per);
-    return std::min(ntr, c);
+    return std::min(ntr, c + (c & 1));
 }
 
 }  // namespace
@@ -577,11 +611,8 @@ size_t fft_scratch_bytes(long long nt) {
     return fft_plan(nt, P) ? (size_t)(2 * P.M + P.n) * sizeof(cf) : 0;
 }
 
-int fft_stack(bool forward, const float* x_t_in, const cf* X_in, long long ntr, long long nt, long long f0,
-              long long nf, cf* X_out, float* x_t_out, char* scratch, cudaStream_t st, std::string& err) {
-    FftPlan P;
-    if (scratch && fft_plan(nt, P) && ntr <= 0x7fffffffLL)
-        return fft_shared(P, forward, x_t_in, X_in, ntr, f0, nf, X_out, x_t_out, scratch, st, err);
+static int fft_library(bool forward, const float* x_t_in, const cf* X_in, long long ntr, long long nt, long long f0,
+                       long long nf, cf* X_out, float* x_t_out, cudaStream_t st, std::string& err) {
     const long long nh = nt / 2 + 1;
     const long long C = chunk_traces(ntr, nt);
     cf* spec = nullptr;
@@ -643,6 +674,21 @@ int fft_stack(bool forward, const float* x_t_in, const cf* X_in, long long ntr, 
     if (plan_tail) cufftDestroy(plan_tail);
     cudaFreeAsync(spec, st);
     return rc;
+}
+
+int fft_stack(bool forward, const float* x_t_in, const cf* X_in, long long ntr, long long nt, long long f0,
+              long long nf, cf* X_out, float* x_t_out, char* scratch, cudaStream_t st, std::string& err) {
+    FftPlan P;
+    const bool own = scratch && fft_plan(nt, P) && ntr <= 0x7fffffffLL;
+    // (cuFFT takes real arrays that start on 8 bytes)
+    const bool aligned = (reinterpret_cast<uintptr_t>(forward ? x_t_in : x_t_out) & 7) == 0;
+    if (!own || (aligned && !own_transform(P, forward))) {
+        const int rc = fft_library(forward, x_t_in, X_in, ntr, nt, f0, nf, X_out, x_t_out, st, err);
+        if (!own || rc != TLR_ERR_NOMEM) return rc;
+        (void)cudaGetLastError();   // no room for its work memory
+        err.clear();
+    }
+    return fft_shared(P, forward, x_t_in, X_in, ntr, f0, nf, X_out, x_t_out, scratch, st, err);
 }
 
 }  // namespace tlr
