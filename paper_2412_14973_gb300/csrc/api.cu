@@ -730,6 +730,7 @@ struct tlr_mdd_s {
     std::vector<TimedLaunch> gtimed;
     bool pending = false;
     bool pending_graph = false;
+    bool in_batch = false;             // a batched solve uses the work panels, on streams of its own
     void* pending_host_theta = nullptr;
     // host sides of the uploads of tlr_mdd_create, until it has waited for the stream
     std::vector<std::vector<char>> uploads;
@@ -1808,6 +1809,7 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     // forward product, gradient or solve, all of them on this stream); only
     // partials that do not fit there are allocated.  Allocating them on each
     // call cost 0.5 ms at nr = 2048 (fresh mappings), as much as the product.
+    // While a batched solve runs on them, scratch of the call's own.
     Arena w;
     w.base = reinterpret_cast<char*>(h->R);
     w.cap = (size_t)(reinterpret_cast<char*>(h->Zs) - w.base);
@@ -1818,19 +1820,25 @@ int tlr_mdd_adjoint(tlr_mdd_t* h, const void* V, void* G) {
     };
     AdjTab tab;
     memset(&tab, 0, sizeof(tab));
+    const size_t pk = (size_t)packed_bytes(nr, ns, kPackTRA);
+    const size_t npart = (size_t)ns_split * nr * nr;
+    Scratch tmp;
+    if (h->in_batch) {
+        w.cap = sizeof(AdjTab) + 2 * pk + (ns_split > 1 ? npart * sizeof(cf) : 0) + 4 * 256;
+        CK(h, tmp.get(w.cap, h->st));
+        w.base = tmp.ptr();
+    }
     AdjTab* dtab = w.take<AdjTab>(1);
     GProb* dp = &dtab->g;
     // tensor-core handles: V and conj(Dfrak) packed first, then the packed
     // contraction (the same MMAs in the same order as the on-the-fly kernel, which
     // its split of the operands in every tile holds to 109 TFLOP/s at nr = ns =
     // 4096; the two packs cost 2 x 268 MB there), where both operands fit
-    const size_t pk = (size_t)packed_bytes(nr, ns, kPackTRA);
     const bool packed = tc && h->tcp_tables && w.used + 2 * (pk + 256) <= w.cap;
     char* pka = packed ? w.take<char>(pk) : nullptr;
     char* pkb = packed ? w.take<char>(pk) : nullptr;
     cf* part = nullptr;
     bool own = false;
-    const size_t npart = (size_t)ns_split * nr * nr;
     if (ns_split > 1 && w.used + npart * sizeof(cf) <= w.cap) {
         part = w.take<cf>(npart);
     } else if (ns_split > 1) {
@@ -3073,6 +3081,8 @@ void b_free(tlr_mdd_batch_s* b) {
             cudaStreamSynchronize(s);
             cudaStreamDestroy(s);
         }
+    if (b->pending)   // never waited for
+        for (tlr_mdd_s* h : b->hs) h->in_batch = false;
     for (auto e : b->evm)
         if (e) cudaEventDestroy(e);
     if (b->evj) cudaEventDestroy(b->evj);
@@ -3194,6 +3204,7 @@ int tlr_mdd_batch_solve_async(tlr_mdd_batch_t* b, void* const* thetas, const tlr
     if (rc) return rc;
     BCK(cudaEventRecord(b->ev1, b->st));
     b->pending = true;
+    for (tlr_mdd_s* h : b->hs) h->in_batch = true;
     return TLR_OK;
 }
 
@@ -3211,6 +3222,7 @@ int tlr_mdd_batch_wait(tlr_mdd_batch_t* b, tlr_mdd_stats_t* stats) {
     if (!b->pending) FAIL((tlr_mdd_s*)nullptr, TLR_ERR_STATE, "no batched solve is pending");
     b->pending = false;
     BCK(cudaEventSynchronize(b->ev1));
+    for (tlr_mdd_s* h : b->hs) h->in_batch = false;
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, b->ev0, b->ev1) != cudaSuccess) (void)cudaGetLastError();
     int werr = 0;

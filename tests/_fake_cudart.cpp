@@ -35,6 +35,7 @@ std::map<std::string, long long> launches;
 std::string fail_name;
 int fail_arg = 0, fail_code = 0;
 long long stale_uploads = 0, uploads = 0;
+const void* last_upload = nullptr;
 thread_local struct {
     dim3 g, b;
     size_t s;
@@ -76,6 +77,7 @@ cudaError_t copy(void* dst, const void* src, size_t n, cudaMemcpyKind kind, cuda
         return cudaSuccess;
     }
     ++uploads;
+    last_upload = dst;
     std::vector<char> now((const char*)src, (const char*)src + n);
     queues[st].push_back([=] {
         if (memcmp(now.data(), src, n) != 0) ++stale_uploads;
@@ -116,6 +118,12 @@ void fake_fill_freed(int on) {
 }
 long long fake_stale_uploads() { return stale_uploads; }
 long long fake_uploads() { return uploads; }
+// the start of the block that the last upload went to
+const void* fake_last_upload_block() {
+    LOCK;
+    auto it = blocks.upper_bound(const_cast<void*>(last_upload));
+    return it == blocks.begin() ? nullptr : (--it)->first;
+}
 long long fake_default_pool_most() { return (long long)dflt.most; }
 long long fake_launches(const char* name) {
     LOCK;

@@ -44,6 +44,7 @@ def fake():
         F = T.lib()
         F.fake_fail.argtypes = [C.c_char_p, C.c_int, C.c_int]
         F.fake_launches.argtypes = [C.c_char_p]
+        F.fake_last_upload_block.restype = C.c_void_p
         for f in ("fake_stale_uploads", "fake_uploads", "fake_default_pool_most", "fake_launches"):
             getattr(F, f).restype = C.c_longlong
         yield F
