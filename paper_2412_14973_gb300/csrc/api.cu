@@ -692,10 +692,9 @@ struct tlr_mdd_s {
     long long* d_roff = nullptr; // [N + 1] first row of each block
     PanelMap pm{};
     // theta-space vectors
-    cf *x = nullptr, *z = nullptr, *u = nullptr, *v = nullptr, *g = nullptr, *gf = nullptr, *dd = nullptr,
-       *q = nullptr;
+    cf *x = nullptr, *z = nullptr, *u = nullptr, *v = nullptr, *g = nullptr, *gf = nullptr, *dd = nullptr;
     // solver small state
-    double *rho_h = nullptr, *sy_h = nullptr, *yy_h = nullptr, *acoef = nullptr, *sc = nullptr, *fhist = nullptr;
+    double *acoef = nullptr, *sc = nullptr, *fhist = nullptr;
     double *lbm = nullptr, *lbpart = nullptr;   // compact L-BFGS: S^T Y and Y^T Y by slot; partials
     int* ints = nullptr;
     // ring (allocated on first solve)
@@ -811,11 +810,7 @@ void carve(tlr_mdd_s* h, Arena& a) {
     h->g = a.take<cf>(nth);
     h->gf = a.take<cf>(nth);
     h->dd = a.take<cf>(nth);
-    h->q = a.take<cf>(nth);
     h->th_io = a.take<cf>(nth);
-    h->rho_h = a.take<double>(64);
-    h->sy_h = a.take<double>(64);
-    h->yy_h = a.take<double>(64);
     h->acoef = a.take<double>(64);
     h->sc = a.take<double>(SC_COUNT + 8);
     h->ints = a.take<int>(kIntSlots);
@@ -1919,7 +1914,7 @@ int tlr_mdd_benchmark_solve(tlr_mdd_t* h, double lambda, int32_t iters, double t
     const Early early(early_product(n, std::max(n, ns)));
     const size_t n2 = (size_t)n * n;
     const bool tc = tensor_core(h->d.precision);   // BF16x3 packed products for both tensor-core modes
-    const int np = cg_partials(n);
+    const int np = cg_partials();
     // work arrays: G, r, p, y and (FP32) Ap, which takes G's place once G is packed;
     // x is built in X; partials; scalars; tables; packed operands (tensor cores)
     const size_t pk = tc ? (size_t)std::max(packed_bytes(n, ns, kPackTRA), packed_bytes(n, n, kPackTRA)) : 0;
@@ -2553,12 +2548,8 @@ static SolverDev solver_dev(tlr_mdd_s* h, int m) {
     S.g = (float*)h->g;
     S.gf = (float*)h->gf;
     S.d = (float*)h->dd;
-    S.q = (float*)h->q;
     S.sh = h->ring;
     S.yh = h->ring + (size_t)S.ring * n2;
-    S.rho_h = h->rho_h;
-    S.sy_h = h->sy_h;
-    S.yy_h = h->yy_h;
     S.acoef = h->acoef;
     S.SYm = h->lbm;
     S.YYm = h->lbm + 33 * 33;

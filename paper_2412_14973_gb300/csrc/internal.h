@@ -133,7 +133,7 @@ struct GProb {
 // EPI_PACKNK (packed tensor-core path only): row m of the product is written in
 // the packed BF16-plane format as row rowptr[m] of an NK-packed B operand
 // (16 columns = one 16-deep chunk of that operand), not as FP32.
-enum Epi { EPI_STORE = 0, EPI_SUB = 1, EPI_ACCUM = 2, EPI_PARTIAL = 3, EPI_PACKNK = 4 };
+enum Epi { EPI_STORE = 0, EPI_SUB = 1, EPI_PARTIAL = 3, EPI_PACKNK = 4 };
 enum AMode { A_KM = 0, A_MK = 1 };
 enum BMode { B_KN = 0, B_NK = 1 };
 
@@ -257,8 +257,8 @@ cudaError_t rstep(cf* R, const cf* A1, const cf* A2, const double* alpha, int nr
 // iteration (step, beta, direction; pk != nullptr: the new p as a packed BF16x3
 // B operand, its padding untouched) on device scalars sc[8] (slots in k_cg.cu:
 // rr, <p,Ap>, alpha, beta, ||b||^2, done, iterations, a block counter).
-// cg_partials(n) = partial slots needed.
-int cg_partials(int n);
+// cg_partials() = partial slots needed.
+int cg_partials();
 cudaError_t cg_sym(const cf* y, const cf* p, float s2, cf* out, int n, double* part, double* sc, cudaStream_t st);
 cudaError_t cg_start(cf* x, cf* r, cf* p, int n, double* part, double* sc, cudaStream_t st);
 cudaError_t cg_iteration_tail(cf* x, cf* r, cf* p, const cf* Ap, int n, double tol, double* part, double* sc, char* pk,

@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(256) k_cg_dir(cf* __restrict__ x, cf* __restri
 
 }  // namespace
 
-int cg_partials(int) { return std::max(kSymBlocks, kRedBlocks); }
+int cg_partials() { return std::max(kSymBlocks, kRedBlocks); }
 
 cudaError_t cg_sym(const cf* y, const cf* p, float s2, cf* out, int n, double* part, double* sc, cudaStream_t st) {
     const int t = (n + CG_T - 1) / CG_T;

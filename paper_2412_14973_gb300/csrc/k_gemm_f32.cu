@@ -840,7 +840,7 @@ bool gemm_f32_shallow(const GProb& p, int nsplit, int kchunk) {
 
 cudaError_t gemm_f32(const GemmLaunch& G, cudaStream_t st) {
     if (G.nprob == 0 || G.maxM == 0 || G.maxN == 0) return cudaSuccess;
-    if (!G.err) return cudaErrorInvalidValue;
+    if (!G.err || (G.epi != EPI_STORE && G.epi != EPI_SUB && G.epi != EPI_PARTIAL)) return cudaErrorInvalidValue;
     Launch L;
     L.probs = G.d_probs;
     L.nsplit = G.nsplit;

@@ -487,10 +487,6 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_tc(const GProb* __restrict__ 
                         const cf sv = P.S[o];
                         v.x -= sv.x;
                         v.y -= sv.y;
-                    } else if (epi == EPI_ACCUM) {
-                        const cf cv = Cp[o];
-                        v.x += cv.x;
-                        v.y += cv.y;
                     }
                     Cp[o] = v;
                 }

@@ -494,15 +494,6 @@ __device__ __forceinline__ void epi_drain(const PProb& P, int m0, int n0, long l
                         v1.x -= s1.x;
                         v1.y -= s1.y;
                     }
-                } else if (epi == EPI_ACCUM) {
-                    const cf c0 = Cp[o];
-                    v0.x += c0.x;
-                    v0.y += c0.y;
-                    if (two) {
-                        const cf c1 = Cp[o + 1];
-                        v1.x += c1.x;
-                        v1.y += c1.y;
-                    }
                 }
                 if (two && ((reinterpret_cast<uintptr_t>(Cp + o) & 15) == 0)) {
                     *reinterpret_cast<float4*>(Cp + o) = make_float4(v0.x, v0.y, v1.x, v1.y);

@@ -948,9 +948,6 @@ __global__ void __launch_bounds__(kRedThreads) k_gradient_pair(SolverDev S, cons
     if (S.sc[SC_ALPHA] > 0.0 && dsy > 1e-12 * sqrt(dss * dyy)) {
         S.ints[SI_NEWEST] = fr;
         S.ints[SI_CNT] = min(S.ints[SI_CNT] + 1, S.m);
-        S.rho_h[fr] = 1.0 / dsy;
-        S.sy_h[fr] = dsy;
-        S.yy_h[fr] = dyy;
     }
 }
 

@@ -12,21 +12,6 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Block-wide sum of v (blockDim.x a multiple of 32, at most 1024); result valid in thread 0.
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-    v = warp_sum(v);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (w == 0) {
-        r = (l < (int)(blockDim.x >> 5)) ? sh[l] : 0.0;
-        r = warp_sum(r);
-    }
-    __syncthreads();
-    return r;
-}
-
 // Block-wide sums of K values per thread (256 threads); thread k < K returns sum k,
 // the others 0.  FP64 adds run at 2 lanes per cycle and SM on this part, so the
 // tree is folded through shared memory first (8 values per thread, 32 lanes per

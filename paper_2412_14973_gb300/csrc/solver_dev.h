@@ -29,11 +29,8 @@ struct SolverDev {
     long long n2;        // floats per theta-space vector (2 * n_theta)
     int m;               // L-BFGS memory
     int ring;            // m + 1 slots: the slot after the newest is always free
-    float *x, *z, *u, *v, *g, *gf, *d, *q;
+    float *x, *z, *u, *v, *g, *gf, *d;
     float *sh, *yh;      // ring of s and y vectors, ring * n2 floats each
-    double* rho_h;       // [ring] 1 / <s, y>
-    double* sy_h;        // [ring] <s, y>
-    double* yy_h;        // [ring] <y, y>
     double* acoef;       // [64] direction coefficients: [j] of s_j, [32 + j] of y_j (j-th newest)
     double* SYm;         // [ring * ring] <s_a, y_b> by slot
     double* YYm;         // [ring * ring] <y_a, y_b> by slot
