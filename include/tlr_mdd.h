@@ -332,12 +332,10 @@ int tlr_mdd_set_state(tlr_mdd_t* h, const void* z, const void* u);
  * (f0 + nf <= nt / 2 + 1).  freq_to_time: the inverse real DFT of the band
  * (bins outside it zero, the imaginary parts of bins 0 and nt/2 ignored), with
  * the factor 1 / nt, so freq_to_time(time_to_freq(x)) = x when the band is the
- * whole spectrum.  Lengths nt <= 4096 with prime factors up to 13, and nt <= 2048
- * with one above 127, are transformed in shared memory where that is no less
- * accurate than cuFFT (work memory: tables of a few KB; always so for powers of two
- * from 64 on, forward from nt = 100 on, both ways above nt = 1296 but for powers of an
- * odd prime); others by cuFFT over chunks of traces (about 256 MB plus cuFFT's own,
- * allocated and released per call).  Synchronises.
+ * whole spectrum.  Lengths nt <= 4096 with prime factors up to 13, and any nt from 64
+ * to 2048, are transformed in shared memory (work memory: tables of up to 160 KB), at
+ * errors no larger than those of cuFFT's FP32 transforms; others by cuFFT over chunks of
+ * traces (about 256 MB plus cuFFT's own, allocated and released per call); synchronises.
  * Invalid sizes: TLR_ERR_ARG. */
 int tlr_mdd_time_to_freq(const float* x_t, int64_t ntr, int64_t nt, int64_t f0, int64_t nf, void* X_w,
                          void* stream);

@@ -66,9 +66,9 @@ def test_magnitudes_at_the_ends_of_the_range(nt):
         assert np.linalg.norm(y[i] - x[i]) <= 1e-6 * np.linalg.norm(x[i].astype(np.float64)), i
 
 
-@pytest.mark.parametrize("nt,ntr", [(85, 800001), (247, 300001), (4097, 16385)])
-def test_library_lengths_over_several_chunks_of_odd_traces(nt, ntr):
-    # chunks of the library's transforms start on 8 bytes
+@pytest.mark.parametrize("nt,ntr", [(51, 800001), (85, 800001), (247, 300001), (4097, 16385)])
+def test_many_traces_of_odd_lengths(nt, ntr):
+    # several chunks of the library's transforms (51, 4097) start on 8 bytes each
     torch.manual_seed(1)
     nf = 9
     x = torch.randn(ntr, nt, device="cuda")
@@ -84,8 +84,9 @@ def test_library_lengths_over_several_chunks_of_odd_traces(nt, ntr):
     assert _rel(y[ntr - 100:].double(), torch.fft.irfft(S, n=nt, dim=1)) <= 1e-6
 
 
-def test_library_lengths_of_traces_that_start_on_four_bytes():
-    nt, ntr, nf = 68, 7, 35
+@pytest.mark.parametrize("nt", [51, 68])
+def test_traces_that_start_on_four_bytes(nt):
+    ntr, nf = 7, nt // 2 + 1
     x = torch.randn(ntr * nt + 1, device="cuda")[1:]
     X = torch.empty(nf, ntr, dtype=torch.complex64, device="cuda")
     T.tlr_mdd_time_to_freq(x, ntr, nt, 0, nf, X)
