@@ -150,17 +150,18 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     return r;
 }
 
-// least = min(least, |x0|, |x1|) and most = max(most, |x0|, |x1|), a NaN kept by the latter
-__device__ __forceinline__ void min_abs(float& least, float x0, float x1) {
-    asm("min.abs.f32 %0, %0, %1, %2;" : "+f"(least) : "f"(x0), "f"(x1));
-}
+// most = max(most, |x0|, |x1|), NaN if any is
 __device__ __forceinline__ void max_abs(float& most, float x0, float x1) {
     asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(most) : "f"(x0), "f"(x1));
 }
 
-// h, m, l of two FP32 values as BF16 pairs (x0 in the low half)
-__device__ __forceinline__ void split2(float x0, float x1, uint32_t* w, float& least) {
-    min_abs(least, x0, x1);
+// a magnitude's bits, doubled, less one: zero becomes the largest
+__device__ __forceinline__ uint32_t twice(float x) { return 2u * __float_as_uint(x) - 1u; }
+
+// h, m, l of two FP32 values as BF16 pairs (x0 in the low half); least: the smallest
+// twice() so far
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t* w, uint32_t& least) {
+    least = __vimin3_u32(least, twice(x0), twice(x1));
     uint64_t x = pair(x0, x1);
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
@@ -339,11 +340,12 @@ __device__ __forceinline__ void copy_chunk(const Opnd& o, int k0, int ke, int w,
 // of 16 take the other half of the k-group: together all banks) are free of
 // bank conflicts.  k contiguous: thread = (row, half of each k-group); rows
 // contiguous: thread = (row, k-group).  True where a value other than zero is below
-// 2^-109, so that its split may not be exact (half an instruction per value finds the
-// smallest magnitude; where that is below, zeros are told from the rest).
+// 2^-109, so that its split may not be exact (1.5 instructions a value; the smallest
+// magnitude by floating-point minima takes half of one, but zeros have to be told apart
+// then, which cost more where there are any).
 template <bool KCONTIG>
 __device__ __forceinline__ bool split_chunk(char* tile, const char* raw, int t8) {
-    float least = 1.f;
+    uint32_t least = ~0u;
     const int r = KCONTIG ? (t8 >> 5) * 16 + (t8 & 15) : t8 & 127;
     const int odd = (r >> 3) & 1;
     char* const d = tile + (r >> 3) * 256 + (r & 7) * 16;
@@ -375,21 +377,7 @@ __device__ __forceinline__ bool split_chunk(char* tile, const char* raw, int t8)
 #pragma unroll
         for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(o + (3 + p) * PLANE) = make_uint2(w[0][p], w[1][p]);
     }
-    if (!(least < 0x1p-109f)) return false;
-    bool small = false;
-    const float2* q = reinterpret_cast<const float2*>(raw);
-#pragma unroll 1
-    for (int i = 0; i < 8; ++i) {   // the same values again
-        float2 v;
-        if (KCONTIG) {
-            const int kg = i >> 2, h = ((t8 >> 4) & 1) ^ odd;
-            v = q[(raw_pos(r, kg * 4 + h * 2 + ((i >> 1) & 1)) >> 3) + (i & 1)];
-        } else {
-            v = q[((t8 >> 7) * 8 + i) * 128 + r];
-        }
-        small = small || (v.x != 0.f && fabsf(v.x) < 0x1p-109f) || (v.y != 0.f && fabsf(v.y) < 0x1p-109f);
-    }
-    return small;
+    return least < 2u * ((uint32_t)(127 - 109) << 23) - 1u;
 }
 
 // A result that the tensor cores gave as plain FP32 multiply-adds would, up to its
@@ -399,9 +387,6 @@ __device__ __forceinline__ bool good(float x) {
     const uint32_t u = __float_as_uint(x) & 0x7fffffffu, lo = (uint32_t)(127 - 100) << 23;
     return u == 0u || u - lo < 0x7f800000u - lo;
 }
-
-// a magnitude's bits, doubled, less one: zero becomes the largest
-__device__ __forceinline__ uint32_t twice(float x) { return 2u * __float_as_uint(x) - 1u; }
 
 // Recomputes results of a warp's 32 x 32 part of a tile just written by plain FP32
 // fused multiply-adds along k: all of them, or those that are not good().  The warp
