@@ -540,7 +540,7 @@ __device__ __forceinline__ bool pair_scales(float s1, float s2, bool n1, bool n2
 
 // stack[f][tr] = the bins f0 .. f0 + nf - 1 of the traces; a CTA takes P.B pairs
 template <bool EX>
-__global__ void __launch_bounds__(FFT_T, EX ? 2 : 3)
+__global__ void __launch_bounds__(FFT_T, 3)
     k_fft_forward(const __grid_constant__ FftPlan P, const float* __restrict__ x, long long ntr, int f0, int nf,
                   const cf* __restrict__ tab, cf* __restrict__ out) {
     extern __shared__ __align__(16) cf sm[];
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(FFT_T, EX ? 2 : 3)
 // bins 0 and n / 2 ignored), times 1 / n.  The band is read twice, once for the
 // norms (the second time from L2).
 template <bool EX>
-__global__ void __launch_bounds__(FFT_T, EX ? 2 : 3)
+__global__ void __launch_bounds__(FFT_T, 3)
     k_fft_inverse(const __grid_constant__ FftPlan P, const cf* __restrict__ in, long long ntr, int f0, int nf,
                   const cf* __restrict__ tab, float* __restrict__ x) {
     extern __shared__ __align__(16) cf sm[];
