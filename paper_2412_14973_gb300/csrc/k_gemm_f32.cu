@@ -574,7 +574,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
         *abort_flag = 0;
         again[0] = again[2] = INT_MAX;
         again[1] = again[3] = -1;
-        again[4] = 0;
+        again[4] = again[5] = 0;   // (the last stays zero: a wait that nobody ends early)
     }
     // ones where no copy goes (rows beyond an operand), so that nothing left there by
     // another kernel is taken for a small value
@@ -636,6 +636,10 @@ __global__ void __launch_bounds__(NTHR, 1) k_cgemm_f32(const __grid_constant__ L
                     }
                 }
             }
+            // after a timeout: the MMAs in flight end (or two seconds pass) before their
+            // operands and accumulators are given up
+            if (*abort_flag && c > 0)
+                (void)mbar_wait(smem_u32(&tfull[(c - 1) & 1]), (uint32_t)(((c - 1) >> 1) & 1), again + 5);
         }
         __syncwarp();
     } else if (warp >= WCOPY) {
