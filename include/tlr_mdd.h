@@ -47,7 +47,8 @@ extern "C" {
 #define TLR_ERR_STATE       -8  /* call out of order (e.g. destroyed handle) */
 
 /* ---- precision of the complex contractions ---- */
-#define TLR_PREC_FP32   0  /* FP32: exact three-way BF16 split on the tensor cores, FP32 accumulation */
+#define TLR_PREC_FP32   0  /* FP32: three-way BF16 split on the tensor cores (exact from 2^-109 up; smaller values,
+                              sums of up to 12 products and non-finite results by FP32 multiply-adds), FP32 accumulation */
 #define TLR_PREC_BF16X3 1  /* tcgen05 tensor cores: BF16 hi/lo split (3 products), 4M complex, FP32 accumulation */
 #define TLR_PREC_TF32   2  /* tcgen05 tensor cores: operands rounded to TF32 (RN, ties away; 10 mantissa bits),
                               4M complex, FP32 accumulation.  The dense adjoint (tlr_mdd_adjoint) and the
@@ -251,7 +252,8 @@ int tlr_mdd_solve_wait(tlr_mdd_t* h, tlr_mdd_stats_t* stats);
  * iteration is one nr x nr x nr complex product in the handle's precision.
  * Work memory (4 nr^2 complex64 plus packed operands on the tensor-core path,
  * 5 nr^2 in FP32) comes from the library's pool on the handle's stream and goes
- * back before return (the pool keeps at most 256 MB of it); the iterates are
+ * back before return (the pool keeps at most 256 MB above what handles have
+ * taken, over all calls); the iterates are
  * built in X; the call synchronises.  lambda < 0 or non-finite, iters < 0, tol < 0, X NULL:
  * TLR_ERR_ARG; a pending solve on the handle: TLR_ERR_STATE.
  * stats (HOST, may be NULL): iterations taken, final ||r|| / ||b||, device
@@ -420,7 +422,7 @@ int64_t tlr_mdd_launch_count(void);
  * the same options for every member; enqueued on `stream` (plain launches,
  * no graph); thetas must stay valid until the wait.  query: 1 done, 0
  * running.  wait: stats (HOST array [n], may be NULL) as for a single solve,
- * gpu_ms the whole batch's device time; returns TLR_ERR_TIMEOUT if a merged
+ * gpu_ms the whole batch's device time; returns TLR_ERR_TIMEOUT if a
  * contraction timed out, TLR_ERR_NONFINITE if a member met a non-finite
  * value.  A member must not be used otherwise while a batched solve is
  * pending; destroy does not destroy the members. */

@@ -16,7 +16,7 @@
 // written once: 244 MB each way for 40000 traces of 1125 samples, 200 bins,
 // where a library transform between a spectrum in memory and a gather moved
 // 1.5 GB and its plans were made (and destroyed) on every call: 3.5 to 4.9 ms for both
-// directions, as the host makes the plans, against 0.46 here (kernels 233 + 189 us).  Bound by shared-memory
+// directions, as the host makes the plans, against 0.47 here (kernels 233 + 189 us).  Bound by shared-memory
 // traffic (two passes per factor); the bytes alone would take 72 us.
 //
 // Other lengths: cuFFT plans over a chunk of traces, with the band gather /
