@@ -394,7 +394,7 @@ __device__ __forceinline__ bool good(float x) {
 // fused multiply-adds along k: all of them, or those that are not good().  The warp
 // works on 32 x 16 at a time, a lane on 4 rows (8 apart) and 4 columns (4 apart), so
 // an operand row read from L1 or L2 serves 4 products (one lane per row, an output
-// after the other, read each operand row for one).  
+// after the other, read each operand row for one).
 template <int AM, int BMD>
 __device__ __forceinline__ void plain_tile(const Launch& L, int item, bool all) {
     const int lane = threadIdx.x & 31, lg = (threadIdx.x >> 5) & 3, cg = threadIdx.x >> 7, epi = L.epi;
